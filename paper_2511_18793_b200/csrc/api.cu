@@ -273,7 +273,7 @@ size_t carve(nezha_ctx* c) {
   e.tok_row = cv.take<int>(c->Ms); e.tok_pos = cv.take<int>(c->Ms); e.tok_id = cv.take<int>(c->Ms);
   e.tok_ctx_len = cv.take<int>(c->Ms); e.tok_kv_dst = cv.take<long long>(c->Ms);
   e.tok_ext = cv.take<long long>((size_t)c->Mv_max * c->L);
-  e.row_tok_count = cv.take<int>(c->Bmax); e.n_tokens = cv.take<int>(1);
+  e.row_tok_count = cv.take<int>(c->Bmax); e.n_tokens = cv.take<int>(1); e.pf_n_tokens = cv.take<int>(1);
   e.row_tok_start = cv.take<int>(c->Bmax); e.pf_row_start = cv.take<int>(c->Bmax); e.pf_row_count = cv.take<int>(c->Bmax);
   e.req_info = cv.take<int4>(c->Bmax); e.pf_req_info = cv.take<int4>(c->Bmax);
   e.h_f32 = c->h_f32;
@@ -840,18 +840,18 @@ nezha_status nezha_prefill(nezha_ctx* c, const int32_t* hist_codes, const int32_
   const int S_call = 1 + max_n * c->L + c->L;
   for (int b0 = 0; b0 < batch; b0 += c->chunk_rows) {
     const int rows = (batch - b0 < c->chunk_rows) ? batch - b0 : c->chunk_rows;
-    const long long M = (long long)rows * S_call;
+    const long long M = (long long)rows * S_call;      // bound; the histories' real lengths are known on the device (pf_n_tokens)
     // a prompt chunk of at most kSkinnyRows tokens in an engine of the weight-streaming class (one short history): the same
     // kernel as its decode passes.  The prefill is shared by all decode modes, so their equality is not touched.
     c->skinny_now = c->skinny_decode && M <= kSkinnyRows ? 1 : 0;
     launch_prefill_tokens(e, hist_codes, n_hist, b0, rows, max_n, S_call, c->S, c->h_rows, c->st);
     if (c->fused) {
-      launch_embed_norm(c->embed, e.tok_id, (int)M, nullptr, c->d, c->resid, c->layers[0].attn_norm, c->xn, c->ss_e, c->st);
+      launch_embed_norm(c->embed, e.tok_id, (int)M, e.pf_n_tokens, c->d, c->resid, c->layers[0].attn_norm, c->xn, c->ss_e, c->st);
       const float* ss; int parts;
-      run_layers_fused(c, M, nullptr, false, rows, S_call, &ss, &parts);
+      run_layers_fused(c, M, e.pf_n_tokens, false, rows, S_call, &ss, &parts);
     } else {
-      launch_embed(c->embed, c->bf16, e.tok_id, (int)M, nullptr, c->d, c->resid, c->st);
-      run_layers(c, M, nullptr, false, rows, S_call);
+      launch_embed(c->embed, c->bf16, e.tok_id, (int)M, e.pf_n_tokens, c->d, c->resid, c->st);
+      run_layers(c, M, e.pf_n_tokens, false, rows, S_call);
     }
     const size_t ho = (size_t)b0 * (c->L + 1) * c->d;
     launch_rmsnorm(c->resid, c->d, c->h_rows, c->final_norm, c->bf16, (char*)c->h_act + ho * c->esz, c->h_f32 + ho,

@@ -1171,43 +1171,58 @@ void launch_copy_logits(const float* src, long long row_stride, int col_off, con
                                                       idx_stride, T, dst);
 }
 
-// Prompt tokens of a chunk of requests: [BOS, history codes item by item, SP_1..SP_L], padded with BOS up to
-// S_call positions (padding sits after the real tokens, so causal attention never shows it to them).
-__global__ void prefill_tokens_kernel(EngineState e, const int* hist, const int* n_hist, int b0, int rows, int max_n,
-                                      int S_call, int S_cap, int* h_rows) {
+// Prompt tokens of a chunk of requests: [BOS, history codes item by item, SP_1..SP_L], request after request with nothing in
+// between.  A call whose histories are of unequal length is given rows of max_n items, but a pass over all of them would
+// spend on padding what the longest history costs for every request; the token list holds the real tokens only and its
+// length stays on the device (pf_n_tokens: the row count of every kernel of the pass).  Grid = (requests, tiles of 256
+// positions); a block adds up the lengths of the requests before its own (a few thousand at most, one round of loads).
+__global__ void __launch_bounds__(256) prefill_tokens_kernel(EngineState e, const int* hist, const int* n_hist, int b0, int rows,
+                                                             int max_n, int S_cap, int* h_rows) {
   pdl_wait();
   pdl_launch();
-  const long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (idx >= (long long)rows * S_call) return;
-  const int lb = (int)(idx / S_call), p = (int)(idx % S_call), b = b0 + lb;
-  const int L = e.L;
-  int nh = n_hist[b];
-  if (nh < 0 || nh > max_n) { atomicOr(e.status, kStBadCode); nh = nh < 0 ? 0 : max_n; }
-  const int P = 1 + nh * L;
-  const int bos = e.li.vocab_codes + L;
-  int tok = bos;
-  if (p > 0 && p < P) {
+  const int lb = blockIdx.x, b = b0 + lb, L = e.L;
+  auto items = [&](int row) {
+    const int nh = n_hist[b0 + row];
+    return nh < 0 ? 0 : nh > max_n ? max_n : nh;
+  };
+  __shared__ int part[8];
+  int before = 0;
+  for (int i = threadIdx.x; i < lb; i += blockDim.x) before += items(i);
+  before = (int)__reduce_add_sync(0xffffffffu, (unsigned)before);
+  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = before;
+  __syncthreads();
+  before = 0;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) before += part[i];
+  const int nh = items(lb), P = 1 + nh * L, S = P + L;
+  const int start = lb * (1 + L) + before * L;     // first token of the request in the list
+  const int p = blockIdx.y * blockDim.x + threadIdx.x;
+  if (p == 0) {
+    if (n_hist[b] != nh) atomicOr(e.status, kStBadCode);
+    e.row_P[b] = P; e.pf_row_start[lb] = start; e.pf_row_count[lb] = S;
+    e.pf_req_info[lb] = make_int4(start, S, b, -1);
+    if (lb == rows - 1) *e.pf_n_tokens = start + S;
+  }
+  if (p >= S) return;
+  const int idx = start + p;
+  int tok = e.li.vocab_codes + L;                  // BOS
+  if (p >= P) {
+    tok = e.li.vocab_codes + (p - P);
+  } else if (p > 0) {
     const int item = (p - 1) / L, lv = (p - 1) % L;
     int code = hist[((long long)b * max_n + item) * L + lv];
     if (code < 0 || code >= e.li.T[lv]) { atomicOr(e.status, kStBadCode); code = 0; }
     tok = e.li.off[lv] + code;
-  } else if (p >= P && p < P + L) {
-    tok = e.li.vocab_codes + (p - P);
   }
   e.tok_id[idx] = tok; e.tok_pos[idx] = p; e.tok_row[idx] = b; e.tok_ctx_len[idx] = p + 1;
   e.tok_kv_dst[idx] = ((long long)b * e.Hkv * S_cap + p) * e.hd;
-  if (p == 0) {
-    e.row_P[b] = P; e.pf_row_start[lb] = lb * S_call; e.pf_row_count[lb] = S_call;
-    e.pf_req_info[lb] = make_int4(lb * S_call, S_call, b, -1);
-  }
-  if (p >= P - 1 && p <= P - 1 + L) h_rows[lb * (L + 1) + (p - (P - 1))] = (int)idx;
+  if (p >= P - 1) h_rows[lb * (L + 1) + (p - (P - 1))] = idx;
 }
 
 void launch_prefill_tokens(const EngineState& e, const int* hist, const int* n_hist, int b0, int rows, int max_n,
                            int S_call, int S_cap, int* h_rows, cudaStream_t st) {
-  const long long n = (long long)rows * S_call;
   LaunchScope ls(kcNodes, st);
-  launch_pdl(prefill_tokens_kernel, dim3((unsigned)((n + 255) / 256)), dim3(256), 0, st, e, hist, n_hist, b0, rows, max_n, S_call, S_cap, h_rows);
+  launch_pdl(prefill_tokens_kernel, dim3(rows, (S_call + 255) / 256), dim3(256), 0, st, e, hist, n_hist, b0, rows, max_n, S_cap, h_rows);
 }
 void launch_trace_beams(const EngineState& e, int batch, int K, const nezha_trace& tr, cudaStream_t st) {
   LaunchScope ls(kcMisc, st);

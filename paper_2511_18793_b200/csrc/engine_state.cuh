@@ -47,7 +47,8 @@ struct EngineState {
   int* pf_row_start; int* pf_row_count;   // [Bmax] the same for a prefill chunk (indexed by row within the chunk)
   int4* req_info; int4* pf_req_info;      // [Bmax] {first token, token count, cache row, context length or -1 = causal}:
                                           //        all the attention kernel needs to know about a request, in one load
-  int* n_tokens;        // [1]
+  int* n_tokens;        // [1] tokens of the verify pass
+  int* pf_n_tokens;     // [1] tokens of the prefill chunk
   int* counters;        // [8]: 0 unfinished rows, 1 primary tokens (round), 2 accepted levels (round), 3 drafted (round)
 
   const float* h_f32;   // [Bmax][L+1][d]
