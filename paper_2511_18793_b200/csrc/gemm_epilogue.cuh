@@ -19,6 +19,16 @@ __device__ __forceinline__ void tc_commit(uint32_t bar) {
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 
+// Output tile number `tile` of a launch with tiles_m x tiles_n tiles, in launch order: bands of `band` row tiles, inside a
+// band column by column.  The tiles that run at the same time then span about as many rows as columns of the product, so
+// an operand byte is fetched from HBM once per band and not once per wave.
+struct TileMN { int m, n; };
+__device__ __forceinline__ TileMN tile_of(int tile, int tiles_m, int tiles_n, int band) {
+  const int per_band = band * tiles_n, g = tile / per_band, r = tile - g * per_band;
+  const int m_first = g * band, rows = min(band, tiles_m - m_first), n = r / rows;
+  return TileMN{m_first + r - n * rows, n};
+}
+
 // K-major operand tile, 128-byte swizzle: rows are 128 B apart, 8-row groups 1024 B apart (SBO), LBO unused (1),
 // descriptor version 1 (sm_100), layout type 2 (SWIZZLE_128B).
 __device__ __forceinline__ uint64_t smem_desc(uint32_t addr) {

@@ -109,6 +109,11 @@ __global__ void __launch_bounds__(kThreads) gemm_tc_pair_kernel(const __grid_con
   pdl_launch();
   const int M = a.M_dev ? min(a.M, *a.M_dev) : a.M;
   const int tiles_m = (M + 2 * BM - 1) / (2 * BM), tiles_n = (a.N + kBN2 - 1) / kBN2;
+  // 16 row tiles x 4-5 column tiles per wave of 74 pairs: 16 k rows x 4096 x 11008 ran at 1,020 TFLOP/s with all row tiles in
+  // one band (every wave streamed the whole of A from HBM), 1,177 / 1,176 / 1,230 / 1,109 in bands of 4 / 8 / 16 / 32;
+  // 16 k x 22016 x 4096 at 1,070, then 1,184 / 1,288 / 1,315 / 1,232.  With fewer than 16 column tiles a band of 8
+  // already spans a wave: 16 k x 896 x 4864 870 -> 1,011 (965 in bands of 16).
+  const int band = tiles_n >= 16 ? 16 : 8;
   const int n_tiles = tiles_m * tiles_n;             // tiles of the pair; a pair without a tile falls through every loop
   const int pair = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
 
@@ -119,8 +124,9 @@ __global__ void __launch_bounds__(kThreads) gemm_tc_pair_kernel(const __grid_con
       uint32_t round = 0;
       bool ok = true;
       for (int tile = pair; tile < n_tiles && ok; tile += n_pairs) {
-        const int m0 = (tile % tiles_m) * (2 * BM) + rank * BM;          // this CTA's rows
-        const int nb0 = (tile / tiles_m) * kBN2 + rank * (kBN2 / 2);     // this CTA's half of the W tile
+        const TileMN tt = tile_of(tile, tiles_m, tiles_n, band);
+        const int m0 = tt.m * (2 * BM) + rank * BM;                      // this CTA's rows
+        const int nb0 = tt.n * kBN2 + rank * (kBN2 / 2);                 // this CTA's half of the W tile
         for (int k = 0; k < k_iters; ++k) {
           // (round 0 never waits: the parity before a fresh barrier's first one counts as complete)
           if (!mbar_wait_or_abort(empty_bar(s), round ^ 1u, abort_flag)) { ok = false; break; }
@@ -165,7 +171,8 @@ __global__ void __launch_bounds__(kThreads) gemm_tc_pair_kernel(const __grid_con
     int t_local = 0;
     bool ok = true;
     for (int tile = pair; tile < n_tiles && ok; tile += n_pairs, ++t_local) {
-      const int m0 = (tile % tiles_m) * (2 * BM) + rank * BM, n0 = (tile / tiles_m) * kBN2;
+      const TileMN tt = tile_of(tile, tiles_m, tiles_n, band);
+      const int m0 = tt.m * (2 * BM) + rank * BM, n0 = tt.n * kBN2;
       const int b = t_local & 1;
       const EpiRow er = epilogue_row<EPI>(a, m0 + q * 32 + lane, M);
       ok = warp_wait(acc_full(b), (t_local >> 1) & 1, abort_flag, lane);
