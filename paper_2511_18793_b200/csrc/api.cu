@@ -141,9 +141,9 @@ bool check_config(const nezha_config* cfg, std::string* why) {
   return true;
 }
 
-unsigned long long bucket_count(size_t n_items, double lf) {
+unsigned long long bucket_count(size_t n_items, double lf, int slots_per_bucket) {
   double slots = ceil((double)(n_items ? n_items : 1) / lf);
-  unsigned long long nb = (unsigned long long)ceil(slots / kBucketSlots);
+  unsigned long long nb = (unsigned long long)ceil(slots / slots_per_bucket);
   return nb < 2 ? 2 : nb;
 }
 
@@ -180,8 +180,11 @@ size_t carve(nezha_ctx* c) {
   e.status = cv.take<int>(8);
   e.counters = cv.take<int>(8);
   c->n_unique_dev = cv.take<unsigned long long>(1);
-  e.hs.n_buckets = bucket_count(c->n_items, c->load_factor);
-  e.hs.slots = cv.take<unsigned long long>(e.hs.n_buckets * kBucketSlots);
+  // 32-bit slots where every packed key fits them (mult has become prod T here; see HashSetView)
+  e.hs.n_buckets = bucket_count(c->n_items, c->load_factor, 8);
+  e.hs.narrow = mult <= 1ull << 32 && e.hs.n_buckets < 1ull << 31 ? 1 : 0;
+  if (!e.hs.narrow) e.hs.n_buckets = bucket_count(c->n_items, c->load_factor, 4);
+  e.hs.slots = cv.take<unsigned long long>((e.hs.n_buckets + 1) * (kBucketBytes / 8));
   {  // prefix map: for every prefix length n < L at most one slot per item and per possible prefix, at the hash set's
      // load factor; slots hold the bit set of the widest codebook
     const double items = (double)(c->n_items ? c->n_items : 1);

@@ -74,7 +74,36 @@ inline int select_warps(const SelectArgs& a) {
   return a.in_stride < 8 ? 8 : a.in_stride > cap ? cap : a.in_stride;
 }
 
-template <int VPL>
+// Eq. 5 on the extensions of a beam that a lane answers for (codes lane, lane + 32, ...), 8 probes in flight: bit j = code
+// lane + 32 j continues the prefix to a valid ID.
+template <bool NARROW, int VPL>
+__device__ __forceinline__ unsigned probe_extensions(unsigned long long* slots, unsigned long long n_buckets,
+                                                  unsigned long long prefix_key, unsigned long long mult_n, int T) {
+  const HashSetView hs{slots, n_buckets, NARROW};
+  const int lane = threadIdx.x & 31;
+  constexpr int PB = VPL < 8 ? VPL : 8;
+  unsigned ok_mask = 0u;
+#pragma unroll 1
+  for (int j0 = 0; j0 < VPL; j0 += PB) {
+    unsigned long long pk[PB]; bool want[PB], ok[PB];
+#pragma unroll
+    for (int j = 0; j < PB; ++j) {
+      want[j] = lane + 32 * (j0 + j) < T;
+      pk[j] = prefix_key + (unsigned long long)(lane + 32 * (j0 + j)) * mult_n;
+    }
+    hs_contains_form<NARROW, PB>(hs, pk, want, ok);
+#pragma unroll
+    for (int j = 0; j < PB; ++j) ok_mask |= (ok[j] ? 1u : 0u) << (j0 + j);
+  }
+  return ok_mask;
+}
+
+// PROBE: Eq. 5 on every extension of a beam by hash probes (select_probes).  A form of its own because the selection kernels
+// are bound by instruction fetch and latency: the probes' straight-line code in all of them, where the default answers the
+// mask from the prefix map, cost 1.4 % (16 layers, one request) to 3 % (4 layers, 64 requests) of a whole decode.
+inline bool select_probes(const SelectArgs& a) { return a.filter && a.per_beam >= a.T && !a.prefix_filter && !a.final_mask_from_map; }
+
+template <int VPL, bool PROBE>
 __device__ __forceinline__ void select_body(const SelectArgs& a) {
   const int b = blockIdx.x;
   extern __shared__ unsigned char smem_raw[];
@@ -156,21 +185,12 @@ __device__ __forceinline__ void select_body(const SelectArgs& a) {
         const int t = lane + 32 * j;
         if (t < a.T && !pm_test(bits, t)) key[j] = -INFINITY;
       }
-    } else if (all_codes && a.filter) {                  // Eq. 5 on every extension of the beam, 8 probes in flight
-      constexpr int PB = VPL < 8 ? VPL : 8;
+    } else if (PROBE && all_codes && a.filter) {
+      const unsigned ok = a.hs.narrow ? probe_extensions<true, VPL>(a.hs.slots, a.hs.n_buckets, prefix_key, mult_n, a.T)
+                                      : probe_extensions<false, VPL>(a.hs.slots, a.hs.n_buckets, prefix_key, mult_n, a.T);
 #pragma unroll
-      for (int j0 = 0; j0 < VPL; j0 += PB) {
-        unsigned long long pk[PB]; bool want_probe[PB], ok[PB];
-#pragma unroll
-        for (int j = 0; j < PB; ++j) {
-          want_probe[j] = lane + 32 * (j0 + j) < a.T;
-          pk[j] = prefix_key + (unsigned long long)(lane + 32 * (j0 + j)) * mult_n;
-        }
-        hs_contains_many<PB>(a.hs, pk, want_probe, ok);
-#pragma unroll
-        for (int j = 0; j < PB; ++j)
-          if (want_probe[j] && !ok[j]) key[j0 + j] = -INFINITY;
-      }
+      for (int j = 0; j < VPL; ++j)
+        if (!((ok >> j) & 1u)) key[j] = -INFINITY;
     }
     int cnt = 0;
     if constexpr (VPL >= 16) {
@@ -345,11 +365,20 @@ __device__ __forceinline__ void select_body(const SelectArgs& a) {
   if (threadIdx.x == 0) a.out_count[b] = n_out;
 }
 
-template <int VPL>
+// Codes per lane of a codebook of T codes, as a constant.
+template <int V> struct Vpl { static constexpr int value = V; };
+template <typename F> void with_vpl(int T, F&& f) {
+  if (T <= 32) f(Vpl<1>{});
+  else if (T <= 256) f(Vpl<8>{});
+  else if (T <= 512) f(Vpl<16>{});
+  else f(Vpl<32>{});
+}
+
+template <int VPL, bool PROBE>
 __global__ void __launch_bounds__(select_max_threads(VPL)) select_kernel(SelectArgs a) {
   pdl_wait();
   pdl_launch();
-  select_body<VPL>(a);
+  select_body<VPL, PROBE>(a);
 }
 
 }  // namespace
@@ -369,11 +398,14 @@ cudaError_t select_configure(int max_beam) {
   int bytes = (int)select_smem_bytes(max_beam, max_beam);
   if (bytes <= configured_bytes[dev]) return cudaSuccess;
   configured_bytes[dev] = bytes;
-  cudaError_t e;
-  if ((e = cudaFuncSetAttribute(select_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes))) return e;
-  if ((e = cudaFuncSetAttribute(select_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes))) return e;
-  if ((e = cudaFuncSetAttribute(select_kernel<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes))) return e;
-  if ((e = cudaFuncSetAttribute(select_kernel<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes))) return e;
+  cudaError_t e = cudaSuccess;
+  auto set = [&](auto vpl) {
+    constexpr int V = decltype(vpl)::value;
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(select_kernel<V, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(select_kernel<V, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  };
+  set(Vpl<1>{}); set(Vpl<8>{}); set(Vpl<16>{}); set(Vpl<32>{});
+  if (e != cudaSuccess) return e;
   return select_step_configure(bytes);
 }
 
@@ -383,10 +415,10 @@ void launch_select(const SelectArgs& a, cudaStream_t st) {
   LaunchScope ls(kcSelect, st);
   const int warps = select_warps(a);   // a warp per beam where that fits
   const dim3 block(32 * warps);
-  if (a.T <= 32) launch_pdl(select_kernel<1>, dim3(a.batch), block, smem, st, a);
-  else if (a.T <= 256) launch_pdl(select_kernel<8>, dim3(a.batch), block, smem, st, a);
-  else if (a.T <= 512) launch_pdl(select_kernel<16>, dim3(a.batch), block, smem, st, a);
-  else launch_pdl(select_kernel<32>, dim3(a.batch), block, smem, st, a);
+  with_vpl(a.T, [&](auto vpl) {
+    constexpr int V = decltype(vpl)::value;
+    launch_pdl(select_probes(a) ? select_kernel<V, true> : select_kernel<V, false>, dim3(a.batch), block, smem, st, a);
+  });
 }
 
 // ====================================================================================================
@@ -666,7 +698,7 @@ __global__ void __launch_bounds__(select_max_threads(VPL)) select_step_kernel(Se
                                                           const float* __restrict__ bias, __nv_bfloat16* s_act) {
   pdl_wait();
   pdl_launch();
-  select_body<VPL>(a);
+  select_body<VPL, false>(a);                      // (an earlier level than the last: nothing to probe)
   __syncthreads();                                 // the block's own selection (global writes) is visible to all its threads
   for (int k = threadIdx.x >> 5; k < e.Kmax; k += blockDim.x >> 5)          // a warp per beam slot
     draft_step_slot(e, blockIdx.x, k, l, G, g_stride, t_cols, U, bias, s_act, threadIdx.x & 31, 32);
@@ -923,12 +955,12 @@ __global__ void advance_kernel(EngineState e, int batch, int n, int K, int* out_
   advance_body(e, n, K, out_codes, out_score, out_count);
 }
 // The selection of B_{n+1} and the step above in one launch (both act on the requests whose current level is n).
-template <int VPL>
+template <int VPL, bool PROBE>
 __global__ void __launch_bounds__(select_max_threads(VPL)) select_advance_kernel(SelectArgs a, EngineState e, int n, int K, int* out_codes,
                                                              float* out_score, int* out_count) {
   pdl_wait();
   pdl_launch();
-  select_body<VPL>(a);
+  select_body<VPL, PROBE>(a);
   __syncthreads();                                 // the block's own selection (global writes) is visible to all its threads
   advance_body(e, n, K, out_codes, out_score, out_count);
 }
@@ -1099,15 +1131,16 @@ void launch_draft_step(const EngineState& e, int batch, int l, const float* G, l
              (__nv_bfloat16*)s_act);
 }
 cudaError_t select_step_configure(int bytes) {
-  cudaError_t e;
-  if ((e = cudaFuncSetAttribute(select_advance_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes))) return e;
-  if ((e = cudaFuncSetAttribute(select_advance_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes))) return e;
-  if ((e = cudaFuncSetAttribute(select_advance_kernel<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes))) return e;
-  if ((e = cudaFuncSetAttribute(select_advance_kernel<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes))) return e;
-  if ((e = cudaFuncSetAttribute(select_step_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes))) return e;
-  if ((e = cudaFuncSetAttribute(select_step_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes))) return e;
-  if ((e = cudaFuncSetAttribute(select_step_kernel<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes))) return e;
-  return cudaFuncSetAttribute(select_step_kernel<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  cudaError_t e = cudaSuccess;
+  auto set = [&](auto vpl) {
+    constexpr int V = decltype(vpl)::value;
+    constexpr auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(select_advance_kernel<V, false>, attr, bytes);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(select_advance_kernel<V, true>, attr, bytes);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(select_step_kernel<V>, attr, bytes);
+  };
+  set(Vpl<1>{}); set(Vpl<8>{}); set(Vpl<16>{}); set(Vpl<32>{});
+  return e;
 }
 void launch_select_step(const SelectArgs& a, const EngineState& e, int l, const float* G, long long g_stride, int t_cols,
                         const float* U, const float* bias, void* s_act, cudaStream_t st) {
@@ -1117,10 +1150,9 @@ void launch_select_step(const SelectArgs& a, const EngineState& e, int l, const 
   const int warps = select_warps(a);
   const dim3 block(32 * warps), grid(a.batch);
   __nv_bfloat16* s = (__nv_bfloat16*)s_act;
-  if (a.T <= 32) launch_pdl(select_step_kernel<1>, grid, block, smem, st, a, e, l, G, g_stride, t_cols, U, bias, s);
-  else if (a.T <= 256) launch_pdl(select_step_kernel<8>, grid, block, smem, st, a, e, l, G, g_stride, t_cols, U, bias, s);
-  else if (a.T <= 512) launch_pdl(select_step_kernel<16>, grid, block, smem, st, a, e, l, G, g_stride, t_cols, U, bias, s);
-  else launch_pdl(select_step_kernel<32>, grid, block, smem, st, a, e, l, G, g_stride, t_cols, U, bias, s);
+  with_vpl(a.T, [&](auto vpl) {
+    launch_pdl(select_step_kernel<decltype(vpl)::value>, grid, block, smem, st, a, e, l, G, g_stride, t_cols, U, bias, s);
+  });
 }
 void launch_copy_logits_bias(const float* src, long long row_stride, int row_mul, int batch, int n_beams, int T,
                              const float* bias, long long bias_stride, float* dst, cudaStream_t st) {
@@ -1150,10 +1182,11 @@ void launch_select_advance(const SelectArgs& a, const EngineState& e, int n, int
   LaunchScope ls(kcSelect, st);
   const int warps = select_warps(a);
   const dim3 block(32 * warps), grid(a.batch);
-  if (a.T <= 32) launch_pdl(select_advance_kernel<1>, grid, block, smem, st, a, e, n, K, out_codes, out_score, out_count);
-  else if (a.T <= 256) launch_pdl(select_advance_kernel<8>, grid, block, smem, st, a, e, n, K, out_codes, out_score, out_count);
-  else if (a.T <= 512) launch_pdl(select_advance_kernel<16>, grid, block, smem, st, a, e, n, K, out_codes, out_score, out_count);
-  else launch_pdl(select_advance_kernel<32>, grid, block, smem, st, a, e, n, K, out_codes, out_score, out_count);
+  with_vpl(a.T, [&](auto vpl) {
+    constexpr int V = decltype(vpl)::value;
+    launch_pdl(select_probes(a) ? select_advance_kernel<V, true> : select_advance_kernel<V, false>, grid, block, smem, st, a, e, n,
+               K, out_codes, out_score, out_count);
+  });
 }
 void launch_round_end(const EngineState& e, int batch, int K, int round, const nezha_trace& tr, int adaptive, cudaStream_t st) {
   LaunchScope ls(kcAccept, st);

@@ -11,7 +11,7 @@
 namespace nz {
 
 constexpr int kMaxLevels = NEZHA_MAX_LEVELS;
-constexpr int kBucketSlots = 4;                  // 4 x 8 B = one 32-byte sector per bucket
+constexpr int kBucketBytes = 32;                 // one sector per bucket of the hash set: 4 wide or 8 narrow slots
 constexpr unsigned long long kEmptyKey = ~0ull;  // never a packed key: prod(T) < 2^64 - 1
 constexpr int kMaxProbeBuckets = 4096;           // bound of every probe / insert walk
 
@@ -77,11 +77,19 @@ __device__ __forceinline__ float warp_sum(float v) {
 }
 
 // --------------------------------------------------------------------------------------------------
-// hash set (Eq. 5): open addressing over 4-slot buckets, linear probing over buckets
+// hash set (Eq. 5): open addressing over 32-byte buckets (one sector), linear probing over buckets
 // --------------------------------------------------------------------------------------------------
+// Two slot widths.  A code space of at most 2^32 tuples (every configured workload: 256^4, 512^3, 32^3) is stored NARROW:
+// the key is sent through a bijection of the 32-bit integers and the slot holds the 32-bit image, so that a bucket has
+// eight slots and the table half the bytes at the same number of slots -- a random probe of a table beyond the L2 costs a
+// 64-byte DRAM access whatever it reads, so bytes of table are what a probe pays for (10M items at load factor 0.5: 160 MB
+// -> 80 MB; the probe kernel's figures stand at hs_probe_kernel).  Larger spaces hold the 64-bit keys themselves, four per
+// bucket.  The empty slot is all ones in both: no packed key in the wide form; in the narrow form one key may map to it,
+// whose membership is a word of its own behind the buckets.
 struct HashSetView {
-  unsigned long long* slots;       // [n_buckets * kBucketSlots]
-  unsigned long long n_buckets;
+  unsigned long long* slots;       // n_buckets buckets of kBucketBytes (+ one more that holds the special word, narrow form)
+  unsigned long long n_buckets;    // narrow: below 2^31
+  int narrow;
 };
 
 // 64-bit finalizer (the published murmur3 fmix64 constants), then multiply-shift range reduction so that
@@ -93,45 +101,84 @@ __device__ __forceinline__ unsigned long long hs_mix(unsigned long long k) {
 __device__ __forceinline__ unsigned long long hs_bucket(unsigned long long key, unsigned long long n_buckets) {
   return __umul64hi(hs_mix(key), n_buckets);
 }
+// The 32-bit finalizer of the same family (fmix32): a bijection (xor-shifts and odd multipliers).
+__device__ __forceinline__ unsigned hs_mix32(unsigned k) {
+  k ^= k >> 16; k *= 0x85ebca6bu; k ^= k >> 13; k *= 0xc2b2ae35u; k ^= k >> 16;
+  return k;
+}
+__device__ __forceinline__ const unsigned* hs_special(const HashSetView& hs) {
+  return reinterpret_cast<const unsigned*>(hs.slots) + hs.n_buckets * (kBucketBytes / 4);
+}
 
-// One thread walks the probe sequence alone, a whole bucket (one sector) per step.  The empty-slot sentinel is not a
-// packed key (Eq. 4 maps onto [0, prod T) and prod T < 2^64 - 1): it is never a member, although it equals every free slot.
-__device__ __forceinline__ bool hs_contains_thread(const HashSetView& hs, unsigned long long key) {
-  if (key == kEmptyKey) return false;
-  unsigned long long b = hs_bucket(key, hs.n_buckets);
-  for (int step = 0; step < kMaxProbeBuckets; ++step) {
-    const ulonglong2* p = reinterpret_cast<const ulonglong2*>(hs.slots + b * kBucketSlots);
-    ulonglong2 lo = __ldg(p), hi = __ldg(p + 1);
-    if (lo.x == key || lo.y == key || hi.x == key || hi.y == key) return true;
-    if (lo.x == kEmptyKey || lo.y == kEmptyKey || hi.x == kEmptyKey || hi.y == kEmptyKey) return false;
-    if (++b == hs.n_buckets) b = 0;
+struct __align__(32) Bucket { unsigned w[8]; };          // one bucket, narrow slots or the halves of wide ones
+__device__ __forceinline__ Bucket ld_bucket(const unsigned long long* slots, unsigned long long b) {
+  Bucket r;                                              // one 32-byte request
+  asm("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+      : "=r"(r.w[0]), "=r"(r.w[1]), "=r"(r.w[2]), "=r"(r.w[3]), "=r"(r.w[4]), "=r"(r.w[5]), "=r"(r.w[6]), "=r"(r.w[7])
+      : "l"(slots + b * (kBucketBytes / 8)));
+  return r;
+}
+// What a key is compared with: both halves of a wide slot, or (narrow) the image in every half.
+struct SlotValue { unsigned lo, hi; };
+template <bool NARROW> __device__ __forceinline__ SlotValue slot_value(unsigned long long key) {
+  if constexpr (NARROW) { const unsigned m = hs_mix32((unsigned)key); return SlotValue{m, m}; }
+  return SlotValue{(unsigned)key, (unsigned)(key >> 32)};
+}
+// What a bucket says about a key: 1 = it is here, 0 = it is nowhere (a free slot ends its walk), -1 = look further.
+template <bool NARROW> __device__ __forceinline__ int bucket_verdict(const Bucket& k, SlotValue v) {
+  bool hit = false, open = false;
+#pragma unroll
+  for (int i = 0; i < 8; i += 2) {
+    const bool e0 = k.w[i] == v.lo, e1 = k.w[i + 1] == v.hi, o0 = k.w[i] == ~0u, o1 = k.w[i + 1] == ~0u;
+    hit |= NARROW ? (e0 || e1) : (e0 && e1);
+    open |= NARROW ? (o0 || o1) : (o0 && o1);
+  }
+  return hit ? 1 : open ? 0 : -1;
+}
+template <bool NARROW> __device__ __forceinline__ unsigned long long home_bucket(const HashSetView& hs, unsigned long long key) {
+  if constexpr (NARROW) return __umulhi(hs_mix32((unsigned)key), (unsigned)hs.n_buckets);
+  return hs_bucket(key, hs.n_buckets);
+}
+// The walk on from a home bucket that is full without holding the key: rare at the load factors in use.
+template <bool NARROW>
+__device__ __forceinline__ bool hs_walk_on(unsigned long long* slots, unsigned long long n_buckets, unsigned long long b,
+                                               SlotValue v) {
+  const HashSetView hs{slots, n_buckets, NARROW};
+  for (int step = 1; step < kMaxProbeBuckets; ++step) {
+    if (++b == n_buckets) b = 0;
+    const int verdict = bucket_verdict<NARROW>(ld_bucket(hs.slots, b), v);
+    if (verdict >= 0) return verdict > 0;
   }
   return false;
 }
 
-// Membership of N keys per thread with the memory round trips overlapped: the home buckets of all keys are loaded
-// first (independent loads), and only a key whose home bucket is full without holding it walks on alone.
-template <int N>
-__device__ __forceinline__ void hs_contains_many(const HashSetView& hs, const unsigned long long* keys, const bool* want,
+// Membership of N keys per thread with the memory round trips overlapped: the home buckets of all keys are loaded first
+// (independent loads).
+template <bool NARROW, int N>
+__device__ __forceinline__ void hs_contains_form(const HashSetView& hs, const unsigned long long* keys, const bool* want,
                                                  bool* found) {
-  ulonglong2 lo[N], hi[N];
+  Bucket k[N];
 #pragma unroll
-  for (int j = 0; j < N; ++j) {
-    if (want[j]) {
-      const ulonglong2* p = reinterpret_cast<const ulonglong2*>(hs.slots + hs_bucket(keys[j], hs.n_buckets) * kBucketSlots);
-      lo[j] = __ldg(p); hi[j] = __ldg(p + 1);
-    }
-  }
+  for (int j = 0; j < N; ++j)
+    if (want[j]) k[j] = ld_bucket(hs.slots, home_bucket<NARROW>(hs, keys[j]));
 #pragma unroll
   for (int j = 0; j < N; ++j) {
     found[j] = false;
-    if (!want[j]) continue;
-    const unsigned long long k = keys[j];
-    if (k == kEmptyKey) continue;                      // the sentinel matches every free slot and is no key
-    if (lo[j].x == k || lo[j].y == k || hi[j].x == k || hi[j].y == k) found[j] = true;
-    else if (lo[j].x == kEmptyKey || lo[j].y == kEmptyKey || hi[j].x == kEmptyKey || hi[j].y == kEmptyKey) found[j] = false;
-    else found[j] = hs_contains_thread(hs, k);        // home bucket full: rare at the load factors in use
+    // outside the code space (narrow), or the free slots' value (wide): no member
+    if (!want[j] || (NARROW ? keys[j] >> 32 != 0ull : keys[j] == kEmptyKey)) continue;
+    const SlotValue v = slot_value<NARROW>(keys[j]);
+    if (NARROW && v.lo == ~0u) { found[j] = __ldg(hs_special(hs)) != 0u; continue; }
+    const int verdict = bucket_verdict<NARROW>(k[j], v);
+    found[j] = verdict >= 0 ? verdict > 0 : hs_walk_on<NARROW>(hs.slots, hs.n_buckets, home_bucket<NARROW>(hs, keys[j]), v);
   }
+}
+// One key, either form.
+__device__ __forceinline__ bool hs_contains_thread(const HashSetView& hs, unsigned long long key) {
+  const bool want[1] = {true};
+  bool found[1];
+  if (hs.narrow) hs_contains_form<true, 1>(hs, &key, want, found);
+  else hs_contains_form<false, 1>(hs, &key, want, found);
+  return found[0];
 }
 
 // --------------------------------------------------------------------------------------------------
@@ -179,13 +226,6 @@ struct LevelInfo {
   unsigned long long mult[kMaxLevels];   // Eq. 4 positional multipliers
   int vocab_codes;                 // sum(T)
 };
-
-// Eq. 4 on a code tuple held in registers / local memory.
-__device__ __forceinline__ unsigned long long pack_key(const LevelInfo& li, const int* codes) {
-  unsigned long long k = 0;
-  for (int l = 0; l < li.L; ++l) k += (unsigned long long)codes[l] * li.mult[l];
-  return k;
-}
 
 // --------------------------------------------------------------------------------------------------
 // GEMM:  C[M,N] (op)= A[M,K] * W[N,K]^T   (both operands K-major)
