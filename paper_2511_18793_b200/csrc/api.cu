@@ -14,12 +14,11 @@
 #include "engine_state.cuh"
 
 namespace nz {
-void launch_hs_clear(HashSetView hs, cudaStream_t st);
 void launch_hs_pack(const LevelInfo& li, const int* codes, unsigned long long n, unsigned long long* keys, int* status,
                     cudaStream_t st);
-void launch_hs_insert(const LevelInfo& li, HashSetView hs, const int* codes, unsigned long long n,
-                      unsigned long long* n_unique, int* status, cudaStream_t st);
-void launch_pm_build(const LevelInfo& li, PrefixMapView pm, const int* codes, unsigned long long n, int* status, cudaStream_t st);
+void launch_set_build(const LevelInfo& li, HashSetView hs, PrefixMapView pm, const int* codes, unsigned long long n,
+                      unsigned long long* n_unique, int* status, int n_sm, cudaStream_t st);
+int sm_count();
 void launch_hs_probe(HashSetView hs, const unsigned long long* keys, unsigned long long n, uint8_t* found,
                      cudaStream_t st);
 void launch_prefill_tokens(const EngineState& e, const int* hist, const int* n_hist, int b0, int rows, int max_n,
@@ -185,24 +184,25 @@ size_t carve(nezha_ctx* c) {
   e.hs.narrow = mult <= 1ull << 32 && e.hs.n_buckets < 1ull << 31 ? 1 : 0;
   if (!e.hs.narrow) e.hs.n_buckets = bucket_count(c->n_items, c->load_factor, 4);
   e.hs.slots = cv.take<unsigned long long>((e.hs.n_buckets + 1) * (kBucketBytes / 8));
-  {  // prefix map: for every prefix length n < L at most one slot per item and per possible prefix, at the hash set's
-     // load factor; slots hold the bit set of the widest codebook
+  {  // prefix map: for every prefix length n < L every possible prefix's bit set, or at most one slot per item at the hash
+     // set's load factor, whichever takes less (PrefixMapView)
     const double items = (double)(c->n_items ? c->n_items : 1);
     double prefixes = 1.0;
     unsigned long long total = 0;
+    e.pm.set_words = (c->Tmax + 63) / 64;
+    e.pm.stride = 2;
+    while (e.pm.stride < 1 + e.pm.set_words) e.pm.stride *= 2;
     for (int n = 0; n < g.L; ++n) {
       if (n > 0) prefixes *= (double)g.T[n - 1];
-      const double n_pref = prefixes < items ? prefixes : items;
+      const double slots = ceil((prefixes < items ? prefixes : items) / c->load_factor) + 1;
+      const bool direct = prefixes * e.pm.set_words <= slots * e.pm.stride;
       e.pm.level_off[n] = total;
-      e.pm.level_slots[n] = (unsigned long long)ceil(n_pref / c->load_factor) + 1;
-      total += e.pm.level_slots[n];
+      e.pm.level_slots[n] = direct ? 0 : (unsigned long long)slots;
+      total += direct ? (unsigned long long)prefixes * e.pm.set_words : (unsigned long long)slots * e.pm.stride;
     }
     for (int n = g.L; n < kMaxLevels; ++n) { e.pm.level_off[n] = 0; e.pm.level_slots[n] = 0; }
-    e.pm.n_slots = total;
-    int words = 1 + (c->Tmax + 63) / 64, stride = 2;
-    while (stride < words) stride *= 2;
-    e.pm.stride = stride;
-    e.pm.slots = cv.take<unsigned long long>(e.pm.n_slots * (unsigned long long)stride);
+    e.pm.n_words = total;
+    e.pm.slots = cv.take<unsigned long long>(e.pm.n_words);
   }
   // weights
   const size_t esz = c->esz;
@@ -506,10 +506,9 @@ void draft_phase(nezha_ctx* c, int batch, int K, bool from_scratch, int first_le
 }
 
 nezha_status pending_device_error(nezha_ctx* c) {
-  int st = 0;
   NZ_CUDA(c, cudaMemcpyAsync(c->host_counters + 8, c->es.status, 4 * sizeof(int), cudaMemcpyDeviceToHost, c->st));
   NZ_CUDA(c, cudaStreamSynchronize(c->st));
-  st = c->host_counters[8];
+  const int st = c->host_counters[8];
   if (st) NZ_CUDA(c, cudaMemsetAsync(c->es.status, 0, 4 * sizeof(int), c->st));
   if (st & kStHashFull) return fail(c, NEZHA_ERR_HASH_FULL, "hash set insertion exhausted its probe bound");
   if (st & kStBadCode) return fail(c, NEZHA_ERR_CATALOG, "a code outside [0, T_l) was given");
@@ -804,16 +803,12 @@ nezha_status nezha_create(const nezha_config* cfg, const nezha_weights* w, const
 
 nezha_status nezha_build_hashset(nezha_ctx* c, uint64_t* n_unique) {
   if (!c) return NEZHA_ERR_ARG;
-  NZ_CUDA(c, cudaMemsetAsync(c->n_unique_dev, 0, sizeof(unsigned long long), c->st));
-  launch_hs_clear(c->es.hs, c->st);
-  launch_hs_insert(c->es.li, c->es.hs, c->catalog, c->n_items, c->n_unique_dev, c->es.status, c->st);
-  launch_pm_build(c->es.li, c->es.pm, c->catalog, c->n_items, c->es.status, c->st);
-  unsigned long long nu = 0;
-  NZ_CUDA(c, cudaMemcpyAsync(&nu, c->n_unique_dev, sizeof(nu), cudaMemcpyDeviceToHost, c->st));
-  NZ_CUDA(c, cudaStreamSynchronize(c->st));
+  launch_set_build(c->es.li, c->es.hs, c->es.pm, c->catalog, c->n_items, c->n_unique_dev, c->es.status, sm_count(), c->st);
+  // (into pinned memory: the copy is queued with the status word's, and one wait serves both)
+  NZ_CUDA(c, cudaMemcpyAsync(c->host_counters, c->n_unique_dev, sizeof(unsigned long long), cudaMemcpyDeviceToHost, c->st));
   NZ_CUDA(c, cudaGetLastError());
-  if (n_unique) *n_unique = nu;
   nezha_status ps = pending_device_error(c);
+  if (n_unique) memcpy(n_unique, c->host_counters, sizeof(unsigned long long));
   if (ps != NEZHA_OK) return ps;
   if (c->state < 1) c->state = 1;
   return NEZHA_OK;

@@ -187,21 +187,26 @@ __device__ __forceinline__ bool hs_contains_thread(const HashSetView& hs, unsign
 // For every n in [0, L): the distinct n-code prefixes of the valid IDs, each with the bit set of the level-(n+1) codes t
 // such that some valid ID begins with (prefix, t).  For n = L - 1 that is Eq. 5 itself for all T_L extensions of a beam in
 // one look-up -- the same answers as T_L hash probes, bit for bit; for n < L - 1 it answers "does any valid ID begin with
-// these codes?", the validity filter at the earlier levels.  One table region per n (so a key needs no level tag), open
-// addressing with linear probing over slots of `stride` words inside the region: word 0 = prefix key + 1 (0 = empty),
-// words 1.. = the bit set.
+// these codes?", the validity filter at the earlier levels.  One table region per n (so a key needs no level tag), in one of
+// two forms, whichever takes fewer bytes for that n (launch-time constant, chosen where the arena is laid out):
+//   direct   the bit sets of all prod T[:n] possible prefixes, indexed by the prefix key.  The short prefixes always, and
+//            the longest ones of a catalogue that is dense in its prefix space (10M items over 256^3 prefixes: 537 MB
+//            against 1.28 GB hashed, and an insertion is one atomic with no slot to find first)
+//   hashed   open addressing with linear probing over slots of `stride` words: word 0 = prefix key + 1 (0 = empty), words
+//            1.. = the bit set (1M items over 256^3 prefixes: 128 MB)
 struct PrefixMapView {
-  unsigned long long* slots;       // [n_slots * stride]; null = not in use
-  unsigned long long n_slots;      // all regions together
-  int stride;                      // words per slot: a power of two >= 1 + ceil(max T / 64)
-  unsigned long long level_off[kMaxLevels];     // first slot of the region of prefixes with n codes
-  unsigned long long level_slots[kMaxLevels];   // its slot count
+  unsigned long long* slots;       // all regions, n_words words
+  unsigned long long n_words;
+  int stride, set_words;           // words per slot (a power of two >= 1 + set_words); words per bit set, ceil(max T / 64)
+  unsigned long long level_off[kMaxLevels];     // first word of the region of prefixes with n codes
+  unsigned long long level_slots[kMaxLevels];   // its slot count; 0 = direct
 };
-// The bit set of a prefix of n codes, or null if no valid ID begins with it.  Every lane of a warp may call this with the
-// same key (the loads are then broadcasts).
+// The bit set of a prefix of n codes, or null (an empty set counts as none) if no valid ID begins with it.  Every lane of a
+// warp may call this with the same key (the loads are then broadcasts).
 __device__ __forceinline__ const unsigned long long* pm_find(const PrefixMapView& pm, int n, unsigned long long prefix_key) {
   const unsigned long long ns = pm.level_slots[n];
-  const unsigned long long* region = pm.slots + pm.level_off[n] * pm.stride;
+  const unsigned long long* region = pm.slots + pm.level_off[n];
+  if (ns == 0) return region + prefix_key * pm.set_words;
   unsigned long long s = __umul64hi(hs_mix(prefix_key), ns);
   for (int step = 0; step < kMaxProbeBuckets; ++step) {
     const unsigned long long* slot = region + s * pm.stride;

@@ -18,6 +18,20 @@
 
 namespace nz {
 
+int sm_count() {                                  // of the current device
+  static std::mutex mu;
+  static int n[kMaxDevices] = {};
+  std::lock_guard<std::mutex> g(mu);
+  const int dev = current_device();
+  if (n[dev] == 0) {
+    int v = 0;
+    if (cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || v <= 0) v = 148;
+    cudaGetLastError();
+    n[dev] = v;
+  }
+  return n[dev];
+}
+
 namespace {
 
 using namespace gemm_detail;
@@ -186,20 +200,6 @@ __global__ void __launch_bounds__(kThreads + 32 * (ISS - 1)) gemm_tc_kernel(cons
 // ---------------------------------------------------------------------------------------------------
 // host side
 // ---------------------------------------------------------------------------------------------------
-int sm_count() {                                  // of the current device
-  static std::mutex mu;
-  static int n[kMaxDevices] = {};
-  std::lock_guard<std::mutex> g(mu);
-  const int dev = current_device();
-  if (n[dev] == 0) {
-    int v = 0;
-    if (cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || v <= 0) v = 148;
-    cudaGetLastError();
-    n[dev] = v;
-  }
-  return n[dev];
-}
-
 template <int BN, int EPI, int ISS>
 void launch(const GemmArgs& a, cudaStream_t st) {
   CUtensorMap ta, tb;
