@@ -5,9 +5,9 @@
 // 128 x 64 tile of W (16 KB per copy, the unit that has to be kept in flight), the rows of A are the MMA's N (MT = 32, 64
 // or 128), and the accumulator in TMEM is a 128 x MT block of C^T.  An output tile is 128 columns of C; the K range of a
 // tile is split over the CTAs of a thread-block cluster (up to 8) so that every SM streams a share of W, whatever N.
-// Each CTA leaves its partial block in its own shared memory; after a cluster barrier the 32 x 32 blocks of the tile are
-// dealt out to the cluster's CTAs, which add the parts in rank order, reading their peers' shared memory -- the bits
-// never depend on timing -- and run the same fused epilogue as the other tensor-core kernels.
+// Each CTA leaves its partial block in its own shared memory; after a cluster barrier pieces of the tile are dealt out to
+// the cluster's warps, which add the parts in rank order, reading their peers' shared memory -- the bits never depend on
+// timing -- and run the same fused epilogue as the other tensor-core kernels.
 // A CTA issues the weight copies of its first ring round BEFORE the launch's dependency on the preceding kernel is
 // resolved (W is constant data), and the kernel is sized for two CTAs per SM, so the weight stream of a launch starts
 // while its predecessor is still draining.
@@ -27,18 +27,14 @@ template <int MT> struct SkinnyCfg {
   static constexpr int kTileBytesX = MT * BK * 2;
   static constexpr int kStageBytes = kTileBytesW + kTileBytesX;
   static constexpr int kStages = MT == 32 ? 5 : MT == 64 ? 4 : 3;
-  static constexpr int kBlocks = 4 * (MT / 32);              // 32 x 32 blocks of the tile: (TMEM lane quarter, 32 rows of A)
-  static constexpr int kEpiWarps = MT == 32 ? 4 : 8;         // warp w: lane quarter w % 4, every (kEpiWarps / 4)-th row block
-  static constexpr int kBlocksPerWarp = kBlocks / kEpiWarps;
-  static constexpr int kThreads = 64 + 32 * kEpiWarps;
   static constexpr int kBarBytes = 128;
-  // (the epilogue's transpose tiles reuse the ring: a CTA has one tile, and the ring is idle once it is accumulated)
-  static constexpr int kSmemBytes = kStages * kStageBytes + 1024 /*alignment slack*/ + kBarBytes;
+  // (the accumulator's image reuses the ring: a CTA has one tile, and the ring is idle once it is accumulated)
+  static constexpr int kSmemBytes = kStages * kStageBytes + 1024 /*alignment slack*/ + kBarBytes + MT * 4 /*row scales*/;
   static constexpr int kTmemCols = MT;
   // kind::f16 instruction descriptor: D = f32, A = B = bf16, both K-major, N = MT, M = 128.
   static constexpr uint32_t kInstrDesc =
       (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(MT >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
-  static_assert(kBlocks * 4096 <= kStages * kStageBytes, "transpose tiles do not fit in the ring");
+  static_assert(MT * 512 <= kStages * kStageBytes, "the accumulator's image does not fit in the ring");
   static_assert(2 * (kSmemBytes + 1024) <= 228 * 1024, "two CTAs per SM");
 };
 
@@ -60,11 +56,31 @@ __device__ __forceinline__ float4 ld_peer_f4(uint32_t local, uint32_t rank) {
   asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(ra) : "memory");
   return v;
 }
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {
+  uint32_t r[16];
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr));
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+  for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
+}
 
-// grid = tiles x splits, clusters of `splits` CTAs (blockIdx.x = tile * splits + split, split = rank in the cluster).  Warp 0: TMA producer; warp 1: TMEM owner and MMA issuer;
-// warps 2 ..: epilogue, warp w on TMEM lane quarter w % 4 (columns n0 + 32 q ..) and the 32-row blocks c = (w - 2) / 4, + 1 or 2, .. of A.
+constexpr int kSkinnyEpiWarps = 8;
+constexpr int kSkinnyThreads = 64 + 32 * kSkinnyEpiWarps;
+
+// grid = (tiles x splits, row tiles), clusters of `splits` CTAs along x (blockIdx.x = tile * splits + split, split = rank in
+// the cluster).  Warp 0: TMA producer; warp 1: TMEM owner and MMA issuer; warps 2 .. 9: epilogue.
+// The epilogue is a chain of latencies behind the last MMA, so it is spread as thin as it goes: the tile's live rows are cut
+// into units of 4 rows x 32 columns (one float4 per lane) that are dealt out to all epilogue warps of the cluster; a unit is
+// one round of peer loads, and what it needs from memory is fetched before the accumulator is ready.  (One warp per 32 x 32
+// block, the blocks dealt out to the CTAs, each row's norm scale added up by one lane: per launch at 20 rows 11.8 instead of 9.1 us for
+// the output and down projections of the d = 2048 backbone, 7.8 instead of 5.4 for QKV.)
 template <int MT, int EPI>
-__global__ void __launch_bounds__(SkinnyCfg<MT>::kThreads, 2)
+__global__ void __launch_bounds__(kSkinnyThreads, 2)
     gemm_skinny_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmX, GemmArgs a,
                        int splits, int* status) {
   using C = SkinnyCfg<MT>;
@@ -73,16 +89,17 @@ __global__ void __launch_bounds__(SkinnyCfg<MT>::kThreads, 2)
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   uint8_t* gen_base = smem_raw + (base - smem_u32(smem_raw));
   const uint32_t bar_base = base + STAGES * C::kStageBytes;
-  // barriers: full[STAGES], empty[STAGES], acc_full; then the TMEM slot and the abort flag
+  // barriers: full[STAGES], empty[STAGES], acc_full; then the TMEM slot and the abort flag; then the rows' norm scales
   auto full_bar = [&](int s) { return bar_base + 8u * s; };
   auto empty_bar = [&](int s) { return bar_base + 8u * (STAGES + s); };
   const uint32_t acc_full = bar_base + 8u * (2 * STAGES);
   volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(gen_base + STAGES * C::kStageBytes + 8 * (2 * STAGES + 1));
   volatile uint32_t* abort_flag = tmem_slot + 1;
+  float* row_scale = reinterpret_cast<float*>(gen_base + STAGES * C::kStageBytes + C::kBarBytes);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int tile = blockIdx.x / splits, split = (int)cluster_rank();
-  const int n0 = tile * 128;
+  const int n0 = tile * 128, m0 = blockIdx.y * MT;
   // this CTA's share of the k-steps: contiguous, the first (k_iters % splits) shares one step longer
   const int k_iters = a.K / BK;
   const int k_base = k_iters / splits, k_rem = k_iters - k_base * splits;
@@ -96,11 +113,13 @@ __global__ void __launch_bounds__(SkinnyCfg<MT>::kThreads, 2)
     mbar_fence_init();
     tma_prefetch_map(&tmW);
     tma_prefetch_map(&tmX);
-    // the weight tiles of the first round: constant data, so they may be fetched while the predecessor still runs
-    for (int s = 0; s < pre; ++s) {
-      mbar_expect_tx(full_bar(s), C::kStageBytes);
-      tma_load_2d(base + s * C::kStageBytes, &tmW, (k_begin + s) * BK, n0, full_bar(s));
-    }
+    // the weight tiles of the first round: constant data, so they may be fetched while the predecessor still runs (only for
+    // the first row tile, which always goes through with its copies: whether the others have rows is not known yet)
+    if (blockIdx.y == 0)
+      for (int s = 0; s < pre; ++s) {
+        mbar_expect_tx(full_bar(s), C::kStageBytes);
+        tma_load_2d(base + s * C::kStageBytes, &tmW, (k_begin + s) * BK, n0, full_bar(s));
+      }
   }
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32((const void*)tmem_slot)),
@@ -114,18 +133,36 @@ __global__ void __launch_bounds__(SkinnyCfg<MT>::kThreads, 2)
   pdl_wait();
   pdl_launch();
   const int M = a.M_dev ? min(a.M, *a.M_dev) : a.M;
-  constexpr int BPW = C::kBlocksPerWarp, CSTEP = C::kEpiWarps / 4;
-  EpiRow er[BPW];                                // of the epilogue warps: the row the lane answers for in each of its blocks
-#pragma unroll
-  for (int bi = 0; bi < BPW; ++bi) er[bi] = EpiRow{1.f, 0, -1};
+  const bool live = blockIdx.y == 0 || m0 < M;    // the same in all CTAs of a cluster
+  const int rows = max(0, min(MT, M - m0));       // rows of this tile that exist
+  // units of the epilogue: unit u = columns n0 + 32 (u / quads) .., rows m0 + 4 (u % quads) ..
+  const int ew = warp - 2, quads = (rows + 3) >> 2, col_groups = min(4, (a.N - n0) >> 5), units = col_groups * quads;
+  const int u_step = splits * kSkinnyEpiWarps, u_first = split + splits * ew;     // (neighbouring units on different CTAs)
+  const int k8 = lane & 7, rsub = lane >> 3;
+  const bool mine = live && warp >= 2 && u_first < units;
+  EpiAux aux;                                     // what the warp's next unit needs from memory
+  int pos = 0;
+  long long kvd = -1;
+  auto fetch = [&](int u) {
+    const int n_chunk = n0 + 32 * (u / quads), r = 4 * (u % quads) + rsub;
+    if (EPI == kEpiRopeKV && r < rows) { pos = a.f.tok_pos[m0 + r]; kvd = a.f.kv_dst[m0 + r]; }
+    if (r < rows) aux = epi_prefetch<EPI>(a, chunk_ctx<EPI>(a, n_chunk, k8), m0 + r, n_chunk + 4 * k8, pos);
+  };
 
-  if (warp == 0) {
+  if (!live) {
+    // nothing to do for this row tile
+  } else if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer
     if (lane == 0) {
       bool ok = true;
       int issued = pre;                          // k-steps whose `full` barrier has been armed
-      for (int s = 0; s < pre; ++s)
-        tma_load_2d(base + s * C::kStageBytes + C::kTileBytesW, &tmX, (k_begin + s) * BK, 0, full_bar(s));
+      for (int s = 0; s < pre; ++s) {
+        if (blockIdx.y != 0) {
+          mbar_expect_tx(full_bar(s), C::kStageBytes);
+          tma_load_2d(base + s * C::kStageBytes, &tmW, (k_begin + s) * BK, n0, full_bar(s));
+        }
+        tma_load_2d(base + s * C::kStageBytes + C::kTileBytesW, &tmX, (k_begin + s) * BK, m0, full_bar(s));
+      }
       int s = 0;
       uint32_t round = 1;                        // parity bit of the round that k-step `pre` belongs to (pre = STAGES here)
       for (int k = pre; k < k_count; ++k, ++issued) {
@@ -133,7 +170,7 @@ __global__ void __launch_bounds__(SkinnyCfg<MT>::kThreads, 2)
         const uint32_t fb = full_bar(s), dst = base + s * C::kStageBytes;
         mbar_expect_tx(fb, C::kStageBytes);
         tma_load_2d(dst, &tmW, (k_begin + k) * BK, n0, fb);
-        tma_load_2d(dst + C::kTileBytesW, &tmX, (k_begin + k) * BK, 0, fb);
+        tma_load_2d(dst + C::kTileBytesW, &tmX, (k_begin + k) * BK, m0, fb);
         if (++s == STAGES) { s = 0; round ^= 1u; }
       }
       if (!ok) {                                 // drain: wait (bounded) for the copies still in flight
@@ -160,81 +197,77 @@ __global__ void __launch_bounds__(SkinnyCfg<MT>::kThreads, 2)
       else *abort_flag = 1;
     }
   } else {
-    // ------------------------------------------------------------------ epilogue
-    // block b = 4 c + q of the tile: columns n0 + 32 q .., rows 32 c .. of A; its transpose tile is slot b of the (idle) ring
-    const int q = warp & 3, c0 = (warp - 2) >> 2;
-    const int n_chunk = n0 + q * 32;
+    // ------------------------------------------------------------------ epilogue, first half: the accumulator into shared memory
+    // (under the main loop: the rows' norm scales, 8 lanes per row, each lane every eighth partial sum)
+    for (int r = ew * 4 + rsub; r < ((rows + 3) & ~3); r += 4 * kSkinnyEpiWarps) {
+      float ss = 0.f;
+      if (a.f.ss_in && r < rows)
+        for (int p = k8; p < a.f.ss_in_parts; p += 8) ss += a.f.ss_in[(long long)p * a.f.ss_ld + m0 + r];
 #pragma unroll
-    for (int bi = 0; bi < BPW; ++bi) {             // overlaps the main loop
-      const int c = c0 + bi * CSTEP;
-      if (splits == 1 || (c * 4 + q) % splits == split) er[bi] = epilogue_row<EPI>(a, c * 32 + lane, M);
+      for (int o = 1; o < 8; o <<= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
+      if (k8 == 0) row_scale[r] = a.f.ss_in ? rsqrtf(ss * a.f.inv_dim + a.f.eps) : 1.f;
     }
+    if (mine) fetch(u_first);
     const bool ok = warp_wait(acc_full, 0, abort_flag, lane);
     tc_fence_after();
+    if (ok) {
+      // TMEM lane = column n0 + 32 q + lane, TMEM column = row; each warp takes a half of the rows of its lane quarter.  The image
+      // of a 32 x 32 block is 32 lines of one row each, their 16-byte chunks swizzled by the row.
+      const int q = warp & 3, half = ew >> 2;
+      float* img = reinterpret_cast<float*>(gen_base) + q * 1024;
 #pragma unroll 1
-    for (int bi = 0; bi < BPW && ok; ++bi) {
-      const int c = c0 + bi * CSTEP, blk = c * 4 + q;
-      const int row0 = c * 32, rows_here = min(32, M - row0);   // rows of this block that exist (may be <= 0)
-      if (rows_here <= 0 || n_chunk >= a.N) continue;        // warp-uniform
-      float4* stg4 = reinterpret_cast<float4*>(gen_base) + blk * (32 * 8);
-      float* stg = reinterpret_cast<float*>(stg4);
-      float v[32];                               // lane = column n_chunk + lane, v[j] = row row0 + j
-      tmem_ld32(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(c * 32), v);
-      if (splits > 1) {
-        // the partial block stays in this CTA's shared memory, in the "8 lanes per row" image; the cluster adds the parts below
+      for (int r0 = half * (MT / 2); r0 < (half + 1) * (MT / 2) && r0 < rows; r0 += 16) {
+        float v[16];
+        tmem_ld16(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)r0, v);
+        float* blk = img + (r0 >> 5) * 4096;
 #pragma unroll
-        for (int j = 0; j < 32; ++j) stg[(j * 8 + ((lane >> 2) ^ (j & 7))) * 4 + (lane & 3)] = v[j];
-      } else {
-        // from lane = column to the "8 lanes per row" image: row j's 32 columns are one 128-byte line, chunks swizzled
-        const float rs_mine = bi == 0 ? er[0].rs : er[BPW - 1].rs;
-#pragma unroll
-        for (int j = 0; j < 32; ++j)
-          stg[(j * 8 + ((lane >> 2) ^ (j & 7))) * 4 + (lane & 3)] = v[j] * __shfl_sync(0xffffffffu, rs_mine, j);
-        __syncwarp();
-        epilogue_block<EPI>(a, stg4, lane, row0, rows_here, n_chunk, bi == 0 ? er[0] : er[BPW - 1]);
+        for (int j = 0; j < 16; ++j) {
+          const int r = (r0 & 31) + j;
+          blk[(r * 8 + ((lane >> 2) ^ (r & 7))) * 4 + (lane & 3)] = v[j];
+        }
       }
+    } else if (lane == 0) {
+      *abort_flag = 1;
     }
-    if (!ok && lane == 0) *abort_flag = 1;
   }
-  if (splits > 1) {
-    // The cluster's CTAs are the splits of one tile (rank = split).  Block b of the tile is finished by CTA b mod
-    // splits: it adds the parts in rank order, reading its peers' shared memory, and runs the epilogue on the sum.
-    cluster_sync_all();                          // all parts are in place (or their CTA has raised its abort flag)
-    if (warp >= 2 && !*abort_flag) {
-      const int q = warp & 3, c0 = (warp - 2) >> 2;
-      const int n_chunk = n0 + q * 32;
+  // All parts are in place behind this barrier (or their CTA has raised its abort flag).
+  if (splits > 1) cluster_sync_all();
+  else __syncthreads();
+  if (mine && !*abort_flag) {
+    // ------------------------------------------------------------------ epilogue, second half: the parts of a unit, added in rank order
 #pragma unroll 1
-      for (int bi = 0; bi < BPW; ++bi) {
-        const int c = c0 + bi * CSTEP, blk = c * 4 + q;
-        const int row0 = c * 32, rows_here = min(32, M - row0);
-        if (rows_here <= 0 || n_chunk >= a.N || blk % splits != split) continue;
-        const EpiRow& erb = bi == 0 ? er[0] : er[BPW - 1];
-        float4* stg4 = reinterpret_cast<float4*>(gen_base) + blk * (32 * 8);
-        const uint32_t img = base + (uint32_t)blk * 4096u + (uint32_t)lane * 16u;
-        float4 acc[8];
+    for (int u = u_first; u < units; u += u_step) {
+      const int g = u / quads, r = 4 * (u - g * quads) + rsub, n_chunk = n0 + 32 * g, row = m0 + r;
+      const ChunkCtx cc = chunk_ctx<EPI>(a, n_chunk, k8);
+      const uint32_t at = base + (uint32_t)(((r >> 5) * 4 + g) * 4096 + ((r & 31) * 8 + (k8 ^ (r & 7))) * 16);
+      float4 x;
+      if (splits > 1) {
+        float4 part[8];
 #pragma unroll
-        for (int i = 0; i < 8; ++i) acc[i] = ld_peer_f4(img + i * 512, 0);
-        for (int sp = 1; sp < splits; ++sp) {
+        for (int sp = 0; sp < 8; ++sp)
+          if (sp < splits) part[sp] = ld_peer_f4(at, (uint32_t)sp);
+        x = part[0];
 #pragma unroll
-          for (int i = 0; i < 8; ++i) {
-            const float4 t = ld_peer_f4(img + i * 512, (uint32_t)sp);
-            acc[i].x += t.x; acc[i].y += t.y; acc[i].z += t.z; acc[i].w += t.w;
-          }
-        }
-        __syncwarp();                            // (this CTA's own part is one of the sources)
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          const float rs = __shfl_sync(0xffffffffu, erb.rs, i * 4 + (lane >> 3));
-          stg4[i * 32 + lane] = make_float4(acc[i].x * rs, acc[i].y * rs, acc[i].z * rs, acc[i].w * rs);
-        }
-        __syncwarp();
-        epilogue_block<EPI>(a, stg4, lane, row0, rows_here, n_chunk, erb);
+        for (int sp = 1; sp < 8; ++sp)
+          if (sp < splits) { x.x += part[sp].x; x.y += part[sp].y; x.z += part[sp].z; x.w += part[sp].w; }
+      } else {
+        x = *reinterpret_cast<const float4*>(gen_base + (at - base));
       }
+      const float rs = row_scale[r];
+      x = make_float4(x.x * rs, x.y * rs, x.z * rs, x.w * rs);
+      const float4 back = epi_apply<EPI>(a, cc, r < rows, row, n_chunk + 4 * k8, k8, x, aux, kvd);
+      if (EPI == kEpiAddNorm) {
+        float ssq = back.x * back.x + back.y * back.y + back.z * back.z + back.w * back.w;
+#pragma unroll
+        for (int o = 1; o < 8; o <<= 1) ssq += __shfl_xor_sync(0xffffffffu, ssq, o);
+        if (k8 == 0 && r < rows) a.f.ss_out[(long long)(n_chunk >> 5) * a.f.ss_ld + row] = ssq;
+      }
+      if (u + u_step < units) fetch(u + u_step);
     }
-    cluster_sync_all();                          // no CTA leaves while a peer may still read its part
   }
   tc_fence_before();
-  __syncthreads();
+  if (splits > 1) cluster_sync_all();            // no CTA leaves while a peer may still read its part
+  else __syncthreads();
   if (warp == 1) {
     __syncwarp();
     tc_fence_after();
@@ -257,7 +290,7 @@ void launch(const GemmArgs& a, int tiles, int splits, cudaStream_t st) {
     cudaFuncSetAttribute(gemm_skinny_kernel<MT, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes);
   });
   cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(tiles * splits); cfg.blockDim = dim3(C::kThreads); cfg.dynamicSmemBytes = C::kSmemBytes; cfg.stream = st;
+  cfg.gridDim = dim3(tiles * splits, (a.M + MT - 1) / MT); cfg.blockDim = dim3(kSkinnyThreads); cfg.dynamicSmemBytes = C::kSmemBytes; cfg.stream = st;
   cudaLaunchAttribute at[2];
   at[0].id = cudaLaunchAttributeClusterDimension;
   at[0].val.clusterDim.x = splits; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
@@ -283,12 +316,13 @@ void launch_mt(const GemmArgs& a, int tiles, int splits, cudaStream_t st) {
 
 }  // namespace
 
-// Number of CTAs a tile's K range is split over (= the cluster size): as many as bring the grid to about one CTA per SM
-// (NEZHA_SKINNY_CTAS: another target), at most 8, each with at least four k-steps (64 KB of W per partial tile).
+// Number of CTAs a tile's K range is split over (= the cluster size): as many as bring the grid to about two CTAs per SM
+// (NEZHA_SKINNY_CTAS: another target), at most 8, each with at least four k-steps (64 KB of W per partial tile).  (One CTA
+// per SM: 2.5 % more for a whole decode of the 16-layer d = 2048 backbone; its gate/up projection then has one CTA per tile.)
 // A function of N, K and the device only -- never of the row count -- so a product's bits do not depend on its rows.
 int gemm_skinny_splits(int N, int K, int n_sm) {
   static const int forced = getenv("NEZHA_SKINNY_CTAS") ? atoi(getenv("NEZHA_SKINNY_CTAS")) : 0;
-  const int target = forced > 0 ? forced : n_sm;
+  const int target = forced > 0 ? forced : 2 * n_sm;
   const int tiles = (N + 127) / 128, k_iters = K / BK;
   int s = target / tiles;
   if (s > k_iters / 4) s = k_iters / 4;
