@@ -93,9 +93,10 @@ struct nezha_ctx {
   int m_expected;           // tokens the current verify pass is expected to hold (0 = unknown); shapes GEMM tiling only
   int m_seen[kMaxLevels + 1];   // tokens each round of the last decode call processed, rounded up to a row tile
   int chains_now;           // GemmArgs::chains of the products being queued: 2 inside a decode call, 0 otherwise
-  // Weight-streaming products: an engine none of whose decode passes can exceed kSkinnyRows rows runs every product of a
-  // decode call through that kernel (the choice is per engine, so both decode modes compute the same bits).
-  bool skinny_decode;
+  // Weight-streaming products: the most rows a pass of this engine's decode calls may have where that is at most
+  // kSkinnyClassRows, else 0.  Every product of a decode call is given this class (the choice of its kernel is per engine and
+  // product, so both decode modes compute the same bits).
+  int skinny_class;
   int skinny_now;           // GemmArgs::skinny of the products being queued
   int rounds_seen[3];       // rounds the last decode call of each mode needed: that many are launched without waiting
   int device;               // the GPU that was current at nezha_create
@@ -570,7 +571,7 @@ nezha_status decode_impl(nezha_ctx* c, int batch, int K, int mode, const int* dr
     nezha_ctx* c;
     explicit ChainScope(nezha_ctx* c_) : c(c_) {
       c->chains_now = 2;
-      c->skinny_now = c->skinny_decode ? 1 : 0;
+      c->skinny_now = c->skinny_class;
     }
     ~ChainScope() { c->chains_now = 0; c->skinny_now = 0; }
   } chain_scope(c);
@@ -738,7 +739,7 @@ nezha_status nezha_create(const nezha_config* cfg, const nezha_weights* w, const
   bool ok = cudaMemsetAsync(c->es.status, 0, 8 * sizeof(int), st) == cudaSuccess;
   {
     const long long pass_rows = c->Mv_max > (long long)c->Bmax * c->Kmax ? c->Mv_max : (long long)c->Bmax * c->Kmax;
-    c->skinny_decode = c->fused && pass_rows <= kSkinnyRows && !getenv("NEZHA_NO_SKINNY");
+    c->skinny_class = c->fused && pass_rows <= kSkinnyClassRows && !getenv("NEZHA_NO_SKINNY") ? (int)pass_rows : 0;
   }
   // the caches start as zeros: tiles may overhang into never-written rows, whose (masked) values must be finite
   ok = ok && cudaMemsetAsync(c->k_ctx, 0, (size_t)c->nl * c->ctx_layer_elems * c->esz, st) == cudaSuccess &&
@@ -839,9 +840,9 @@ nezha_status nezha_prefill(nezha_ctx* c, const int32_t* hist_codes, const int32_
   for (int b0 = 0; b0 < batch; b0 += c->chunk_rows) {
     const int rows = (batch - b0 < c->chunk_rows) ? batch - b0 : c->chunk_rows;
     const long long M = (long long)rows * S_call;      // bound; the histories' real lengths are known on the device (pf_n_tokens)
-    // a prompt chunk of at most kSkinnyRows tokens in an engine of the weight-streaming class (one short history): the same
-    // kernel as its decode passes.  The prefill is shared by all decode modes, so their equality is not touched.
-    c->skinny_now = c->skinny_decode && M <= kSkinnyRows ? 1 : 0;
+    // the prompt chunk of a few short histories in an engine of that kind: the same rule, with the chunk's own row bound as the
+    // class.  The prefill is shared by all decode modes, so their equality is not touched.
+    c->skinny_now = c->skinny_class && M <= kSkinnyClassRows ? (int)M : 0;
     launch_prefill_tokens(e, hist_codes, n_hist, b0, rows, max_n, S_call, c->S, c->h_rows, c->st);
     if (c->fused) {
       launch_embed_norm(c->embed, e.tok_id, (int)M, e.pf_n_tokens, c->d, c->resid, c->layers[0].attn_norm, c->xn, c->ss_e, c->st);
@@ -1013,7 +1014,7 @@ nezha_status nezha_gemm(nezha_ctx* c, const void* A, const void* W, void* C, int
   if (path == 4) {
     if (M > kSkinnyRows || !c->bf16)
       return fail(c, NEZHA_ERR_UNSUPPORTED, "nezha_gemm: the weight-streaming kernel takes bf16 products of at most 128 rows");
-    a.skinny = 1;
+    a.skinny = kSkinnyRows;
   }
   const bool tc_ok = c->bf16 && gemm_tc_supported(a);
   if (path >= 2 && !tc_ok) return fail(c, NEZHA_ERR_UNSUPPORTED, "nezha_gemm: shape not covered by the tcgen05 kernel");

@@ -259,7 +259,8 @@ struct GemmFuse {
   int Hq, Hkv, hd;
 };
 
-constexpr int kSkinnyRows = 128;    // most rows a launch of the weight-streaming GEMM kernel takes
+constexpr int kSkinnyRows = 128;         // engines whose passes have at most this many rows stream every product's weights
+constexpr int kSkinnyClassRows = 640;    // and at most this many: the products for which it pays (gemm_skinny_applies)
 
 struct GemmArgs {
   const void* A; long long lda;
@@ -278,11 +279,11 @@ struct GemmArgs {
   // differently: a caller that needs the same bits from launches of different sizes asks for the same value in all of
   // them (the tiling itself never changes the result).
   int chains;
-  // Non-zero: a launch of at most kSkinnyRows rows may run as the weight-streaming kernel (weights as the 128-row MMA
-  // operand, the rows as its N, the K range split over the CTAs of a cluster).  Its summation order differs from the
-  // other kernels' and depends on (N, K) and the device only: a caller that needs the same bits from two launches sets
-  // the flag in both or in neither.  W must be constant data (it is read before the launch's dependency on its
-  // predecessor is resolved).
+  // Row class, or 0: the most rows that any launch of the caller's family may have (at most kSkinnyClassRows).  The product
+  // may then run as the weight-streaming kernel (weights as the 128-row MMA operand, the rows as its N, the K range split
+  // over the CTAs of a cluster), by a rule on (N, K), the class and the device only.  Its summation order differs from the
+  // other kernels': a caller that needs the same bits from two launches gives both the same class.  W must be constant
+  // data (it is read before the launch's dependency on its predecessor is resolved).
   int skinny;
 };
 

@@ -1,4 +1,4 @@
-// Weight-streaming GEMM for launches of at most 128 rows:  C[M,N] (op)= A[M,K] * W[N,K]^T  with the operands' roles
+// Weight-streaming GEMM for launches of few rows (at most 128, or a few row tiles of 128: gemm_skinny_applies):  C[M,N] (op)= A[M,K] * W[N,K]^T  with the operands' roles
 // swapped on the tensor core.
 //
 // With a handful of rows the product is bound by reading W once from HBM.  The 128-row MMA operand is therefore a
@@ -316,14 +316,17 @@ void launch_mt(const GemmArgs& a, int tiles, int splits, cudaStream_t st) {
 
 }  // namespace
 
-// Number of CTAs a tile's K range is split over (= the cluster size): as many as bring the grid to about two CTAs per SM
-// (NEZHA_SKINNY_CTAS: another target), at most 8, each with at least four k-steps (64 KB of W per partial tile).  (One CTA
-// per SM: 2.5 % more for a whole decode of the 16-layer d = 2048 backbone; its gate/up projection then has one CTA per tile.)
-// A function of N, K and the device only -- never of the row count -- so a product's bits do not depend on its rows.
-int gemm_skinny_splits(int N, int K, int n_sm) {
+// ---- which products of an engine run here, and how their K range is split.  Both are functions of N, K, the device and the
+// engine's row class (the most rows a pass of it may have) only -- never of a launch's row count -- so a product's bits do not
+// depend on its rows.
+// Number of CTAs a tile's K range is split over (= the cluster size): as many as bring the grid of the class's row tiles to
+// about two CTAs per SM (NEZHA_SKINNY_CTAS: another target), at most 8, each with at least four k-steps (64 KB of W per
+// partial tile).  (One CTA per SM: 2.5 % more for a whole decode of the 16-layer d = 2048 backbone; its gate/up projection
+// then has one CTA per tile.)
+int gemm_skinny_splits(int N, int K, int row_class, int n_sm) {
   static const int forced = getenv("NEZHA_SKINNY_CTAS") ? atoi(getenv("NEZHA_SKINNY_CTAS")) : 0;
   const int target = forced > 0 ? forced : 2 * n_sm;
-  const int tiles = (N + 127) / 128, k_iters = K / BK;
+  const int tiles = (N + 127) / 128 * ((row_class + 127) / 128), k_iters = K / BK;
   int s = target / tiles;
   if (s > k_iters / 4) s = k_iters / 4;
   if (s > 8) s = 8;                              // the portable cluster size
@@ -331,13 +334,24 @@ int gemm_skinny_splits(int N, int K, int n_sm) {
   return s;
 }
 
+// Up to 128 rows every product is bound by reading W, and this kernel keeps more of it in flight.  With more rows W is
+// shared by several row tiles and the general kernel's wider tiles win again -- except where its k-loop is the bound: one
+// CTA walks all of K at 0.29 us per k-step (0.17 with two issuers, N <= 1024), however few tiles there are, while here K is
+// split.  Measured at 256 / 512 rows, general -> this kernel: 2048 x 8192 41 -> 17 / 41 -> 34 us, 1536 x 8960 45 -> 17 /
+// 46 -> 31, 896 x 4864 17 -> 10 / 18 -> 13; but 16384 x 2048 21 -> 37 / 33 -> 66, 6144 x 4096 25 -> 36.
 bool gemm_skinny_applies(const GemmArgs& a, int n_sm) {
-  (void)n_sm;
-  return a.skinny && a.M <= kSkinnyRows && (long long)((a.N + 127) / 128) * 8 <= 0x7fffffff;
+  if (!a.skinny || a.M > a.skinny || a.skinny > kSkinnyClassRows) return false;
+  if (a.skinny <= kSkinnyRows) return true;
+  const int tiles = (a.N + 127) / 128 * ((a.skinny + 127) / 128), k_iters = a.K / BK;
+  const int s = gemm_skinny_splits(a.N, a.K, a.skinny, n_sm);
+  const int waves = (tiles * s + 2 * n_sm - 1) / (2 * n_sm), k_cta = (k_iters + s - 1) / s;
+  const double here = waves * (7.0 + 0.75 * k_cta);
+  const double there = 4.0 + (a.chains == 2 && a.N <= 1024 ? 0.17 : 0.29) * k_iters;      // (its least: one wave of tiles)
+  return here < 0.9 * there;
 }
 
 void launch_gemm_skinny(const GemmArgs& a, int n_sm, cudaStream_t st) {
-  const int tiles = (a.N + 127) / 128, splits = gemm_skinny_splits(a.N, a.K, n_sm);
+  const int tiles = (a.N + 127) / 128, splits = gemm_skinny_splits(a.N, a.K, a.skinny, n_sm);
   if (a.M <= 32) launch_mt<32>(a, tiles, splits, st);      // (the bound, not the expected count: no row may be dropped)
   else if (a.M <= 64) launch_mt<64>(a, tiles, splits, st);
   else launch_mt<128>(a, tiles, splits, st);
