@@ -5,7 +5,6 @@
 #include <stdlib.h>
 #include <string.h>
 
-#include <array>
 #include <map>
 #include <string>
 #include <vector>
@@ -84,7 +83,7 @@ struct nezha_ctx {
   int* host_counters;       // pinned
   // CUDA graphs of the decode segments (one per round), keyed by everything that shapes the launch sequence
   struct Segment { int seen; cudaGraphExec_t exec; long long launches[kcCount]; };
-  std::map<std::array<uintptr_t, 16>, Segment> segments;
+  std::map<std::vector<uintptr_t>, Segment> segments;
   bool use_graphs;
   int opt_transition, opt_inputs, opt_filter;   // nezha_set_option (ablations of the draft head)
   int opt_mask;             // nezha_set_option: 0 = the primary model's last-level mask probes the hash set, 1 (default) = it reads the prefix map
@@ -471,7 +470,9 @@ void draft_level_step(nezha_ctx* c, int batch, int l) {
 
 // Algorithm 3's inference loop (from the empty beam), or its continuation from the true beams (Algorithm 2's drafting step).
 // `first_level` = smallest level any request can still need drafting at (levels below are teacher-forced only).
-void draft_phase(nezha_ctx* c, int batch, int K, bool from_scratch, int first_level, bool filter) {
+// out_*: the last level's beams go straight to these buffers (mode 0), with the status words to the host.
+void draft_phase(nezha_ctx* c, int batch, int K, bool from_scratch, int first_level, bool filter, int* out_codes = nullptr,
+                 float* out_scores = nullptr, int* out_count = nullptr) {
   const EngineState& e = c->es;
   const bool fast = draft_fast(c);
   launch_draft_init(e, batch, from_scratch ? 1 : 0, fast ? c->draft_sact : nullptr, c->st);
@@ -492,6 +493,10 @@ void draft_phase(nezha_ctx* c, int batch, int K, bool from_scratch, int first_le
       s.gate = e.d_m; s.gate_mode = 2; s.gate_value = l;
       s.out_codes = e.dw_codes + lv_out * c->L; s.out_score = e.dw_score + lv_out; s.out_parent = e.dw_parent + lv_out;
       s.out_token = nullptr; s.out_count = e.dw_count + (size_t)l * c->Bmax;
+      if (out_codes && l == c->L) {
+        s.out_codes = out_codes; s.out_score = out_scores; s.out_count = out_count; s.out_parent = nullptr; s.out_stride = K;
+        s.status = e.status; s.host_status = c->host_counters + 8;
+      }
       // The selection and the state update it feeds in one launch -- where a launch is what costs (narrow models).  The
       // fused kernel is one CTA per request; at d = 4096 its 20 x 4096 state elements per request take 64 us on 32 SMs
       // against 14 us for the update spread over (request, beam) CTAs.
@@ -506,26 +511,30 @@ void draft_phase(nezha_ctx* c, int batch, int K, bool from_scratch, int first_le
   }
 }
 
-nezha_status pending_device_error(nezha_ctx* c) {
-  NZ_CUDA(c, cudaMemcpyAsync(c->host_counters + 8, c->es.status, 4 * sizeof(int), cudaMemcpyDeviceToHost, c->st));
-  NZ_CUDA(c, cudaStreamSynchronize(c->st));
-  const int st = c->host_counters[8];
+// The status words as they stand in `words` (host memory), reported and cleared.
+nezha_status device_error(nezha_ctx* c, const int* words) {
+  const int st = words[0];
   if (st) NZ_CUDA(c, cudaMemsetAsync(c->es.status, 0, 4 * sizeof(int), c->st));
   if (st & kStHashFull) return fail(c, NEZHA_ERR_HASH_FULL, "hash set insertion exhausted its probe bound");
   if (st & kStBadCode) return fail(c, NEZHA_ERR_CATALOG, "a code outside [0, T_l) was given");
   if (st)      // a kernel that records where it gave up leaves three more words (0 if it does not)
     return fail(c, NEZHA_ERR_CUDA, "a bounded device-side wait expired (kernel gave up and returned); where: " +
-                                       std::to_string(c->host_counters[9]) + " " + std::to_string(c->host_counters[10]) + " " +
-                                       std::to_string(c->host_counters[11]));
+                                       std::to_string(words[1]) + " " + std::to_string(words[2]) + " " + std::to_string(words[3]));
   return NEZHA_OK;
 }
+nezha_status pending_device_error(nezha_ctx* c) {
+  NZ_CUDA(c, cudaMemcpyAsync(c->host_counters + 8, c->es.status, 4 * sizeof(int), cudaMemcpyDeviceToHost, c->st));
+  NZ_CUDA(c, cudaStreamSynchronize(c->st));
+  return device_error(c, c->host_counters + 8);
+}
 
-// Runs one segment of a decode call (the part before the rounds, or one round).  The launch sequence of a segment
+using SegmentKey = std::vector<uintptr_t>;
+// Runs one segment of a decode call (the part before the rounds and the rounds expected, or one round).  The launch sequence of a segment
 // is fixed by its key, so after one eager run it is captured into a CUDA graph and replayed from then on: one
-// launch per round instead of dozens, and no launch gaps between its kernels.  Eager when the stream cannot be
+// launch per call instead of dozens, and no launch gaps between its kernels.  Eager when the stream cannot be
 // captured, while per-launch event timing is on, or if capture fails.
 template <typename F>
-nezha_status run_segment(nezha_ctx* c, const std::array<uintptr_t, 16>& key, F&& body) {
+nezha_status run_segment(nezha_ctx* c, const SegmentKey& key, F&& body) {
   if (!c->use_graphs || profile_is_on()) { body(); return NEZHA_OK; }
   nezha_ctx::Segment& sg = c->segments[key];
   if (sg.exec) {
@@ -579,35 +588,25 @@ nezha_status decode_impl(nezha_ctx* c, int batch, int K, int mode, const int* dr
   if (trace) tr = *trace;
   nezha_decode_stats sd{};
   const int R = L - 1;
-  auto key_of = [&](int segment) {
-    std::array<uintptr_t, 16> k{};
-    k[0] = (uintptr_t)segment; k[1] = (uintptr_t)batch; k[2] = (uintptr_t)K; k[3] = (uintptr_t)(mode | c->opt_transition << 8 | c->opt_inputs << 12 | c->opt_filter << 16 | c->opt_mask << 20 | (is_tree ? 1 : 0) << 24 | c->opt_level_filter << 25 | c->opt_adaptive << 26);
-    k[4] = (uintptr_t)drafts; k[5] = (uintptr_t)n_draft; k[6] = (uintptr_t)out_codes; k[7] = (uintptr_t)out_scores;
-    k[8] = (uintptr_t)out_count; k[9] = (uintptr_t)tr.drafts; k[10] = (uintptr_t)tr.n_draft; k[11] = (uintptr_t)tr.accepted_len;
-    k[12] = (uintptr_t)tr.level_reached; k[13] = (uintptr_t)tr.beams ^ ((uintptr_t)tr.tree_codes << 1);
-    k[14] = (uintptr_t)tr.beam_scores ^ ((uintptr_t)tr.tree_count << 1);
-    k[15] = (uintptr_t)c->m_seen[segment];           // the expected token count shapes the tiling of the round's GEMMs
+  const uintptr_t opts = (uintptr_t)(mode | c->opt_transition << 8 | c->opt_inputs << 12 | c->opt_filter << 16 | c->opt_mask << 20 |
+                                     (is_tree ? 1 : 0) << 24 | c->opt_level_filter << 25 | c->opt_adaptive << 26);
+  // A segment covers rounds first .. last (0 = the part before the rounds).
+  auto key_of = [&](int first, int last) {
+    SegmentKey k{(uintptr_t)first, (uintptr_t)last, (uintptr_t)batch, (uintptr_t)K, opts,
+                 (uintptr_t)drafts, (uintptr_t)n_draft, (uintptr_t)out_codes, (uintptr_t)out_scores, (uintptr_t)out_count,
+                 (uintptr_t)tr.drafts, (uintptr_t)tr.n_draft, (uintptr_t)tr.accepted_len, (uintptr_t)tr.level_reached,
+                 (uintptr_t)tr.beams ^ ((uintptr_t)tr.tree_codes << 1), (uintptr_t)tr.beam_scores ^ ((uintptr_t)tr.tree_count << 1)};
+    for (int r = first > 1 ? first : 1; r <= last; ++r) k.push_back((uintptr_t)c->m_seen[r]);   // shapes the round's tiling
     return k;
   };
-  nezha_status rs = run_segment(c, key_of(0), [&] {
-    if (tr.drafts) launch_fill_i32(tr.drafts, (long long)R * batch * K * L, -1, c->st);
-    if (tr.n_draft) launch_fill_i32(tr.n_draft, (long long)R * batch, -1, c->st);
-    if (tr.accepted_len) launch_fill_i32(tr.accepted_len, (long long)R * batch * K, -1, c->st);
-    if (tr.level_reached) launch_fill_i32(tr.level_reached, (long long)R * batch, -1, c->st);
-    if (tr.tree_codes) launch_fill_i32(tr.tree_codes, (long long)R * L * batch * K * L, -1, c->st);
-    if (tr.tree_count) launch_fill_i32(tr.tree_count, (long long)R * L * batch, -1, c->st);
-    launch_fill_i32(out_codes, (long long)batch * K * L, -1, c->st);
-    launch_fill_f32(out_scores, (long long)batch * K, -INFINITY, c->st);
-    launch_fill_i32(out_count, batch, 0, c->st);
-    launch_init_decode(e, batch, c->st);
+  auto begin = [&] {
+    launch_decode_begin(e, batch, K, out_codes, out_scores, out_count, tr, c->st);
     if (mode == NEZHA_MODE_DRAFT) {
-      draft_phase(c, batch, K, true, 1, c->opt_filter != 0);
-      const size_t lv = (size_t)L * c->Bmax * c->Kmax;
-      launch_write_out(e.dw_codes + lv * L, e.dw_score + lv, e.dw_count + (size_t)L * c->Bmax, c->Kmax, L, batch, K,
-                       out_codes, out_scores, out_count, c->st);
+      draft_phase(c, batch, K, true, 1, c->opt_filter != 0, out_codes, out_scores, out_count);
       return;
     }
-    // B_1 from the prefill hidden state h_0 (Algorithm 1's LM head, top-K and pruning at l = 1)
+    // B_1 from the prefill hidden state h_0 (Algorithm 1's LM head, top-K and pruning at l = 1), settled at once
+    // (for L == 1 this also writes the result)
     gemm(c, c->h_act, (long long)(L + 1) * c->d, c->lm_head, c->d, c->logits0, c->cfg.T[0], batch, nullptr, c->cfg.T[0], c->d,
          kEpiStoreF32);
     SelectArgs s = select_base(c, batch, K);
@@ -618,68 +617,69 @@ nezha_status decode_impl(nezha_ctx* c, int batch, int K, int mode, const int* dr
     s.prefix_filter = (c->opt_level_filter && L > 1) ? 1 : 0;
     s.out_codes = e.tb_codes + lv_out * L; s.out_score = e.tb_score + lv_out; s.out_parent = e.tb_parent + lv_out;
     s.out_count = e.tb_count + (size_t)1 * c->Bmax;
-    launch_select(s, c->st);
-    // settle level 1 (for L == 1 this also writes the result)
-    launch_fill_i32(e.row_cur, batch, 0, c->st);
-    launch_advance(e, batch, 0, K, out_codes, out_scores, out_count, c->st);
-  });
-  if (rs != NEZHA_OK) return rs;
-  if (mode == NEZHA_MODE_DRAFT) {
-    nezha_status ps = pending_device_error(c);
-    if (stats) *stats = sd;
-    return ps;
-  }
-  for (int round = 1; round <= R; ++round) {
+    s.status = e.status; s.host_status = c->host_counters + 8;
+    launch_select_advance(s, e, 0, K, out_codes, out_scores, out_count, RoundEnd{}, c->st);
+  };
+  auto run_round = [&](int round) {
     // drafts are mostly rejected or mostly accepted in a steady workload, so the round's token count repeats: tile for it
     c->m_expected = c->m_seen[round];
-    rs = run_segment(c, key_of(round), [&] {
-      if (mode == NEZHA_MODE_AR) launch_draft_set(e, batch, K, nullptr, nullptr, c->st);
-      else if (round == 1 && drafts && is_tree) launch_draft_tree_set(e, batch, K, drafts, n_draft, c->st);
-      else if (round == 1 && drafts) launch_draft_set(e, batch, K, drafts, n_draft, c->st);
-      else draft_phase(c, batch, K, round == 1, round == 1 ? 1 : round + 1, c->opt_filter != 0);
-      launch_build_nodes(e, batch, c->st);
-      verify_pass(c, (long long)batch * K * (L - round), batch, K * (L - round));
-      for (int n = round; n < L; ++n) {
-        SelectArgs s = select_base(c, batch, K);
-        const size_t lv_in = (size_t)n * c->Bmax * c->Kmax, lv_out = (size_t)(n + 1) * c->Bmax * c->Kmax;
-        s.logits = c->logits_v; s.row_stride = c->Nv; s.col_off = e.li.off[n] - e.li.off[1];
-        s.src_row = e.tb_src + lv_in; s.src_mul = 0;
-        s.in_codes = e.tb_codes + lv_in * L; s.in_score = e.tb_score + lv_in; s.in_count = e.tb_count + (size_t)n * c->Bmax;
-        s.n = n; s.T = c->cfg.T[n]; s.per_beam = s.T; s.filter = (n + 1 == L) ? 1 : 0;
-        s.prefix_filter = (c->opt_level_filter && n + 1 < L) ? 1 : 0;
-        s.gate = e.row_cur; s.gate_mode = 1; s.gate_value = n;
-        s.out_codes = e.tb_codes + lv_out * L; s.out_score = e.tb_score + lv_out; s.out_parent = e.tb_parent + lv_out;
-        s.out_count = e.tb_count + (size_t)(n + 1) * c->Bmax;
-        launch_select_advance(s, e, n, K, out_codes, out_scores, out_count, c->st);
-      }
-      launch_round_end(e, batch, K, round, tr, mode == NEZHA_MODE_VERIFIED ? c->opt_adaptive : 0, c->st);
-      cudaMemcpyAsync(c->host_counters + 16 + 8 * round, e.counters, 8 * sizeof(int), cudaMemcpyDeviceToHost, c->st);
-    });
+    if (mode == NEZHA_MODE_AR) launch_draft_set(e, batch, K, nullptr, nullptr, c->st);
+    else if (round == 1 && drafts && is_tree) launch_draft_tree_set(e, batch, K, drafts, n_draft, c->st);
+    else if (round == 1 && drafts) launch_draft_set(e, batch, K, drafts, n_draft, c->st);
+    else draft_phase(c, batch, K, round == 1, round == 1 ? 1 : round + 1, c->opt_filter != 0);
+    launch_build_nodes(e, batch, c->st);
+    verify_pass(c, (long long)batch * K * (L - round), batch, K * (L - round));
+    for (int n = round; n < L; ++n) {
+      SelectArgs s = select_base(c, batch, K);
+      const size_t lv_in = (size_t)n * c->Bmax * c->Kmax, lv_out = (size_t)(n + 1) * c->Bmax * c->Kmax;
+      s.logits = c->logits_v; s.row_stride = c->Nv; s.col_off = e.li.off[n] - e.li.off[1];
+      s.src_row = e.tb_src + lv_in; s.src_mul = 0;
+      s.in_codes = e.tb_codes + lv_in * L; s.in_score = e.tb_score + lv_in; s.in_count = e.tb_count + (size_t)n * c->Bmax;
+      s.n = n; s.T = c->cfg.T[n]; s.per_beam = s.T; s.filter = (n + 1 == L) ? 1 : 0;
+      s.prefix_filter = (c->opt_level_filter && n + 1 < L) ? 1 : 0;
+      s.gate = e.row_cur; s.gate_mode = 1; s.gate_value = n;
+      s.out_codes = e.tb_codes + lv_out * L; s.out_score = e.tb_score + lv_out; s.out_parent = e.tb_parent + lv_out;
+      s.out_count = e.tb_count + (size_t)(n + 1) * c->Bmax;
+      RoundEnd re{};
+      if (n + 1 == L)
+        re = RoundEnd{c->host_counters + 16 + 8 * round, round, mode == NEZHA_MODE_VERIFIED ? c->opt_adaptive : 0, tr};
+      launch_select_advance(s, e, n, K, out_codes, out_scores, out_count, re, c->st);
+    }
     c->m_expected = 0;
+  };
+  // Whether another round is needed is known only from a round's counters.  A steady workload needs the same number of rounds
+  // call after call, so the part before the rounds and the rounds the last call (of the same mode) needed are one segment:
+  // one graph, no host wait and no gap in between.  A round queued for nothing finds every request finished and each of its
+  // kernels returns at once; what is missing follows round by round.
+  int queued = mode == NEZHA_MODE_DRAFT ? 0 : c->rounds_seen[mode] < 1 ? (R < 1 ? R : 1) : c->rounds_seen[mode] < R ? c->rounds_seen[mode] : R;
+  nezha_status rs = run_segment(c, key_of(0, queued), [&] {
+    begin();
+    for (int r = 1; r <= queued; ++r) run_round(r);
+  });
+  bool finished = R < 1 || mode == NEZHA_MODE_DRAFT;
+  for (;;) {
     if (rs != NEZHA_OK) return rs;
-    // Whether another round is needed is known only from this round's counters.  A steady workload needs the same
-    // number of rounds call after call, so the rounds the last call needed are queued without waiting in between;
-    // a round queued for nothing finds every request finished and each of its kernels returns at once.
-    if (round < R && round < c->rounds_seen[mode]) continue;
     NZ_CUDA(c, cudaStreamSynchronize(c->st));
     NZ_CUDA(c, cudaGetLastError());
-    bool finished = false;
-    for (int r = sd.rounds + 1; r <= round && !finished; ++r) {
+    for (int r = sd.rounds + 1; r <= queued && !finished; ++r) {
       const int* hc = c->host_counters + 16 + 8 * r;
-      c->m_seen[r] = (hc[1] + 127) / 128 * 128;
+      // (the tiling hint keeps still while the count stays within a quarter of it: every value is a graph of its own)
+      const int m = (hc[1] + 127) / 128 * 128;
+      if (m > c->m_seen[r] || 4 * m < 3 * c->m_seen[r]) c->m_seen[r] = m;
       sd.rounds = r;
       sd.primary_tokens += hc[1];
       sd.accepted_levels += hc[2];
       if (r == 1) sd.drafted = hc[3];
       finished = hc[0] == 0;
     }
-    if (finished) break;
+    if (finished || queued >= R) break;
+    ++queued;
+    rs = run_segment(c, key_of(queued, queued), [&] { run_round(queued); });
   }
-  c->rounds_seen[mode] = sd.rounds;
+  if (mode != NEZHA_MODE_DRAFT) c->rounds_seen[mode] = sd.rounds;
   if (tr.beams || tr.beam_scores) launch_trace_beams(e, batch, K, tr, c->st);
-  nezha_status ps = pending_device_error(c);
   if (stats) *stats = sd;
-  return ps;
+  return device_error(c, queued > 0 ? c->host_counters + 16 + 8 * queued + 4 : c->host_counters + 8);
 }
 
 }  // namespace
@@ -953,7 +953,7 @@ nezha_status nezha_draft_logits(nezha_ctx* c, int32_t batch, int32_t n_beams, in
     return fail(c, NEZHA_ERR_ARG, "nezha_draft_logits: bad argument");
   const EngineState& e = c->es;
   // start set = the given prefixes at level `level`; teacher-force the transitions, then Eq. 2 for the next level
-  launch_init_decode(e, batch, c->st);
+  launch_decode_begin(e, batch, 0, nullptr, nullptr, nullptr, nezha_trace{}, c->st);
   launch_fill_i32(e.d_m, batch, level, c->st);
   launch_fill_i32(e.dw_count + (size_t)level * c->Bmax, batch, n_beams, c->st);
   if (level > 0) {

@@ -363,6 +363,10 @@ __device__ __forceinline__ void select_body(const SelectArgs& a) {
     }
   }
   if (threadIdx.x == 0) a.out_count[b] = n_out;
+  if (a.host_status && b == 0 && threadIdx.x < 4) {      // (what the kernels before this one reported)
+    a.host_status[threadIdx.x] = *(volatile int*)(a.status + threadIdx.x);
+    __threadfence_system();
+  }
 }
 
 // Codes per lane of a codebook of T codes, as a constant.
@@ -432,53 +436,57 @@ __global__ void fill_i32_kernel(int* p, long long n, int v) {
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
     p[i] = v;
 }
-__global__ void fill_f32_kernel(float* p, long long n, float v) {
-  pdl_wait();
-  pdl_launch();
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-    p[i] = v;
-}
 
-// B_0 = { empty beam, score 0 } for every request; nothing settled.
-__global__ void init_decode_kernel(EngineState e, int batch) {
+// Start of a decode call, one block per request: B_0 = { empty beam, score 0 }, nothing settled, and the fill values of the
+// call's outputs (out_* and the trace's pointers may be null; their slots of rounds that do not run keep these values).
+__global__ void __launch_bounds__(128) decode_begin_kernel(EngineState e, int batch, int K, int* out_codes, float* out_scores,
+                                                           int* out_count, nezha_trace tr) {
   pdl_wait();
   pdl_launch();
-  const int b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b == 0) {
-    for (int i = 0; i < 8; ++i) e.counters[i] = 0;
-    *e.draft_rows = batch * e.Kmax;
+  const int b = blockIdx.x, L = e.L, R = e.L - 1;
+  if (b == 0 && threadIdx.x < 8) e.counters[threadIdx.x] = 0;
+  if (b == 0 && threadIdx.x == 0) { *e.draft_rows = batch * e.Kmax; *e.n_tokens = 0; }
+  if (threadIdx.x == 0) {
+    e.tb_count[0 * e.Bmax + b] = 1;
+    e.tb_score[lvl_bk(e, 0, b, 0)] = 0.f;
+    e.tb_parent[lvl_bk(e, 0, b, 0)] = -1;
+    e.tb_src[lvl_bk(e, 0, b, 0)] = -1;
+    e.row_m[b] = 0;
+    e.row_cur[b] = 0;
+    e.row_spec[b] = 1;
+    e.row_m_start[b] = 0;
+    e.d_m[b] = L;
+    if (out_count) out_count[b] = 0;
   }
-  if (b >= batch) return;
-  e.tb_count[0 * e.Bmax + b] = 1;
-  e.tb_score[lvl_bk(e, 0, b, 0)] = 0.f;
-  e.tb_parent[lvl_bk(e, 0, b, 0)] = -1;
-  e.tb_src[lvl_bk(e, 0, b, 0)] = -1;
-  e.row_m[b] = 0;
-  e.row_cur[b] = -1;
-  e.row_spec[b] = 1;
-  e.row_m_start[b] = 0;
-  e.d_m[b] = e.L;
-  for (int l = 0; l <= e.L; ++l) e.dw_count[(long long)l * e.Bmax + b] = 0;     // no draft tree yet
+  for (int l = threadIdx.x; l <= L; l += blockDim.x) e.dw_count[(long long)l * e.Bmax + b] = 0;     // no draft tree yet
+  if (out_scores) for (int i = threadIdx.x; i < K; i += blockDim.x) out_scores[(long long)b * K + i] = -INFINITY;
+  auto fill = [&](int* p, int slices, int per) {       // [slices][batch][per]
+    if (!p) return;
+    for (int r = 0; r < slices; ++r)
+      for (int i = threadIdx.x; i < per; i += blockDim.x) p[((long long)r * batch + b) * per + i] = -1;
+  };
+  fill(out_codes, 1, K * L);
+  fill(tr.drafts, R, K * L); fill(tr.n_draft, R, 1); fill(tr.accepted_len, R, K); fill(tr.level_reached, R, 1);
+  fill(tr.tree_codes, R * L, K * L); fill(tr.tree_count, R * L, 1);
 }
 
 // Start of a round's drafting (Algorithm 2's drafting step): the draft head continues from the true beams B_m, or from
 // the empty beam in the first round (Algorithm 3's initialisation).
 // Also clears the round's counters (this is the first kernel of a drafting round) and, when s_act is given, starts
-// every beam slot's draft state at s_1 = h_0 (Eq. 1).
-__global__ void draft_init_kernel(EngineState e, int batch, int from_scratch, __nv_bfloat16* s_act) {
+// every beam slot's draft state at s_1 = h_0 (Eq. 1).  Grid = (requests, beam slots); slot 0's block does the bookkeeping.
+// (One block per request for all of its slots took 9 us at one request of d = 2048 and 30 us at d = 4096, beam 20.)
+__global__ void __launch_bounds__(128) draft_init_kernel(EngineState e, int batch, int from_scratch, __nv_bfloat16* s_act) {
   pdl_wait();
   pdl_launch();
   const int b = blockIdx.x;
-  if (b == 0 && threadIdx.x < 8) e.counters[threadIdx.x] = 0;
-  if (b >= batch) return;
   if (s_act) {
     const float* h0 = e.h_f32 + (long long)b * (e.L + 1) * e.d;
-    __nv_bfloat16* dst = s_act + (long long)b * e.Kmax * e.d;
-    for (int c = threadIdx.x; c < e.d; c += blockDim.x) {
-      const __nv_bfloat16 v = __float2bfloat16_rn(h0[c]);
-      for (int k = 0; k < e.Kmax; ++k) dst[(long long)k * e.d + c] = v;
-    }
+    __nv_bfloat16* dst = s_act + ((long long)b * e.Kmax + blockIdx.y) * e.d;
+    for (int c = threadIdx.x; c < e.d; c += blockDim.x) dst[c] = __float2bfloat16_rn(h0[c]);
   }
+  if (blockIdx.y != 0) return;
+  if (b == 0 && threadIdx.x < 8) e.counters[threadIdx.x] = 0;
+  if (b == 0 && threadIdx.x == 0) *e.n_tokens = 0;
   const int m = e.row_m[b];
   if (m >= e.L || !e.row_spec[b]) {              // finished, or its drafting is switched off: an empty tree this round
     if (threadIdx.x == 0) e.d_m[b] = e.L;
@@ -505,6 +513,7 @@ __global__ void draft_set_kernel(EngineState e, int batch, int K, const int* dra
   pdl_launch();
   const int b = blockIdx.x;
   if (b == 0 && threadIdx.x < 8) e.counters[threadIdx.x] = 0;      // first kernel of the round: clear its counters
+  if (b == 0 && threadIdx.x == 0) *e.n_tokens = 0;
   if (b >= batch) return;
   const int L = e.L, k = threadIdx.x;
   __shared__ int s_slot[2][128];                 // slot of tuple k's prefix in the previous / the current level
@@ -561,6 +570,7 @@ __global__ void draft_tree_set_kernel(EngineState e, int batch, int K, const int
   pdl_launch();
   const int b = blockIdx.x;
   if (b == 0 && threadIdx.x < 8) e.counters[threadIdx.x] = 0;
+  if (b == 0 && threadIdx.x == 0) *e.n_tokens = 0;
   if (b >= batch) return;
   const int L = e.L, k = threadIdx.x;
   const bool row_live = e.row_m[b] < L;
@@ -714,45 +724,51 @@ __global__ void copy_logits_bias_kernel(const float* src, long long row_stride, 
   for (int t = threadIdx.x; t < T; t += blockDim.x) dst[(long long)blockIdx.x * T + t] = z[t] + bias[(long long)b * bias_stride + t];
 }
 
+// Eq. 4 on the first n codes: two tuples of valid codes agree on them exactly when these keys are equal.
+__device__ __forceinline__ unsigned long long prefix_key_of(const EngineState& e, const int* codes, int n) {
+  unsigned long long k = 0;
+  for (int l = 0; l < n; ++l) k += (unsigned long long)(unsigned)codes[l] * e.li.mult[l];
+  return k;
+}
+
 // ----------------------------------------------------------------------------------------------------
 // verify-pass token list (the nodes M_p runs on this round)
 // ----------------------------------------------------------------------------------------------------
 // Request with m levels settled: nodes = the level-m code of every beam of B_m (slot = beam rank) and, for the levels
 // m+1..L-1, the last code of every alive node of the round's draft tree (slot = the node's slot in its level): one token
 // per distinct drafted prefix.  A level-m node of the tree is alive if its codes are a beam of B_m; a higher node if its
-// parent is alive.  Tokens of a request are contiguous; requests are laid out in order (each block sums the counts of the
-// requests before it).
-__global__ void nodes_count_kernel(EngineState e, int batch) {
+// parent is alive.  Tokens of a request are contiguous; the requests take their place in the list in the order in which
+// their blocks get there (no row of a pass depends on where it stands).
+__global__ void __launch_bounds__(128) nodes_kernel(EngineState e, int batch) {
   pdl_wait();
   pdl_launch();
   const int b = blockIdx.x;
+  const int L = e.L, Kmax = e.Kmax;
+  __shared__ int s_off, n_alive, s_rank[kMaxLevels][128], s_level_start[kMaxLevels + 1];
+  __shared__ unsigned long long s_key[128];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, n_warps = blockDim.x >> 5;
   const int m = e.row_m[b];
-  const int L = e.L;
-  __shared__ int n_alive;
-  if (threadIdx.x == 0) n_alive = 0;
   if (b == 0 && threadIdx.x == 0) *e.draft_rows = 0;     // this round's drafting is over; round_end raises it again if needed
-  __syncthreads();
   if (m >= L) {
     if (threadIdx.x == 0) { e.row_tok_count[b] = 0; e.row_cur[b] = -1; e.req_info[b] = make_int4(0, 0, b, 0); }
     return;
   }
   const int nb = e.tb_count[m * e.Bmax + b];
+  if (threadIdx.x == 0) n_alive = 0;
+  for (int r = threadIdx.x; r < nb; r += blockDim.x) s_key[r] = prefix_key_of(e, e.tb_codes + lvl_bk(e, m, b, r) * L, m);
+  __syncthreads();
   for (int j = m; j < L; ++j) {
-    const int cnt = min(e.dw_count[(long long)j * e.Bmax + b], e.Kmax);
-    for (int k = threadIdx.x; k < e.Kmax; k += blockDim.x) {
+    const int cnt = min(e.dw_count[(long long)j * e.Bmax + b], Kmax);
+    for (int k = threadIdx.x; k < Kmax; k += blockDim.x) {
       int beta = -1;
       if (k < cnt) {
         if (j == m) {
-          const int* dc = e.dw_codes + lvl_bk(e, m, b, k) * L;
-          for (int r = 0; r < nb && beta < 0; ++r) {
-            const int* bc = e.tb_codes + lvl_bk(e, m, b, r) * L;
-            bool eq = true;
-            for (int l = 0; l < m; ++l) eq &= (dc[l] == bc[l]);
-            if (eq) beta = r;
-          }
+          const unsigned long long key = prefix_key_of(e, e.dw_codes + lvl_bk(e, m, b, k) * L, m);
+          for (int r = nb - 1; r >= 0; --r)
+            if (s_key[r] == key) beta = r;
         } else {
           const int p = e.dw_parent[lvl_bk(e, j, b, k)];
-          if (p >= 0 && p < e.Kmax) beta = e.d_beam[lvl_bk(e, j - 1, b, p)];
+          if (p >= 0 && p < Kmax) beta = e.d_beam[lvl_bk(e, j - 1, b, p)];
           if (beta >= 0) atomicAdd(&n_alive, 1);
         }
       }
@@ -761,27 +777,11 @@ __global__ void nodes_count_kernel(EngineState e, int batch) {
     __syncthreads();                               // level j's answers (global, this block's own) before level j + 1 reads them
   }
   if (threadIdx.x == 0) {
-    e.row_tok_count[b] = nb + n_alive;
-    e.row_cur[b] = m;
-    e.row_m_start[b] = m;
-  }
-}
-
-__global__ void __launch_bounds__(128) nodes_fill_kernel(EngineState e, int batch) {
-  pdl_wait();
-  pdl_launch();
-  const int b = blockIdx.x;
-  const int L = e.L, Kmax = e.Kmax;
-  __shared__ int s_off, s_rank[kMaxLevels][128], s_level_start[kMaxLevels + 1];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, n_warps = blockDim.x >> 5;
-  const int m = e.row_m[b];
-  if (threadIdx.x == 0) {
-    int off = 0;
-    for (int i = 0; i < b; ++i) off += e.row_tok_count[i];
+    const int n_tok = nb + n_alive, off = atomicAdd(e.n_tokens, n_tok);
     s_off = off;
-    e.row_tok_start[b] = off;
-    if (e.row_tok_count[b] > 0) e.req_info[b] = make_int4(off, e.row_tok_count[b], b, e.row_P[b]);
-    if (b == batch - 1) *e.n_tokens = off + e.row_tok_count[b];
+    e.row_tok_count[b] = n_tok; e.row_tok_start[b] = off;
+    e.row_cur[b] = m; e.row_m_start[b] = m;
+    e.req_info[b] = make_int4(off, n_tok, b, n_tok > 0 ? e.row_P[b] : 0);
   }
   for (int i = threadIdx.x; i < L * Kmax; i += blockDim.x) e.node_index[(long long)b * L * Kmax + i] = -1;
   // rank of every alive node within its level (a warp per level: ballots over its <= 128 slots)
@@ -797,8 +797,6 @@ __global__ void __launch_bounds__(128) nodes_fill_kernel(EngineState e, int batc
     if (lane == 0) s_level_start[j] = base;        // the level's count for now; turned into a start below
   }
   __syncthreads();
-  if (m >= L) return;
-  const int nb = e.tb_count[m * e.Bmax + b];
   if (threadIdx.x == 0) {
     int start = nb;
     for (int j = m + 1; j < L; ++j) { const int c = s_level_start[j]; s_level_start[j] = start; start += c; }
@@ -912,24 +910,24 @@ __device__ __forceinline__ void advance_body(const EngineState& e, int n, int K,
     return;
   }
   __shared__ int all_matched;
+  __shared__ unsigned long long s_node[128];       // keys of the alive nodes of level n + 1 (a dead one: no key)
   if (threadIdx.x == 0) all_matched = 1;
-  __syncthreads();
   const int nd = min(e.dw_count[(long long)n1 * e.Bmax + b], Kmax);
+  for (int k = threadIdx.x; k < nd; k += blockDim.x) {
+    const long long s = lvl_bk(e, n1, b, k);
+    s_node[k] = e.d_beam[s] < 0 ? kEmptyKey : prefix_key_of(e, e.dw_codes + s * L, n1);
+  }
+  __syncthreads();
   for (int r = threadIdx.x; r < cnt; r += blockDim.x) {
     const long long bi = lvl_bk(e, n1, b, r);
     const int parent = e.tb_parent[bi];
     const long long pi = lvl_bk(e, n, b, parent);
     for (int i = 0; i + 1 < n; ++i) e.tb_anc[bi * L + i] = e.tb_anc[pi * L + i];
     if (n >= 1) e.tb_anc[bi * L + (n - 1)] = e.tb_self[pi];
-    const int* bc = e.tb_codes + bi * L;
+    const unsigned long long key = prefix_key_of(e, e.tb_codes + bi * L, n1);
     int match = -1;
-    for (int k = 0; k < nd && match < 0; ++k) {
-      if (e.d_beam[lvl_bk(e, n1, b, k)] < 0) continue;
-      const int* dc = e.dw_codes + lvl_bk(e, n1, b, k) * L;
-      bool eq = true;
-      for (int l = 0; l < n1; ++l) eq &= (dc[l] == bc[l]);
-      if (eq) match = k;
-    }
+    for (int k = nd - 1; k >= 0; --k)
+      if (s_node[k] == key) match = k;
     if (match >= 0) {
       e.tb_src[bi] = e.node_index[((long long)b * L + n1) * Kmax + match];
       e.tb_self[bi] = match;
@@ -949,56 +947,44 @@ __device__ __forceinline__ void advance_body(const EngineState& e, int n, int K,
     }
   }
 }
-__global__ void advance_kernel(EngineState e, int batch, int n, int K, int* out_codes, float* out_score, int* out_count) {
-  pdl_wait();
-  pdl_launch();
-  advance_body(e, n, K, out_codes, out_score, out_count);
-}
-// The selection of B_{n+1} and the step above in one launch (both act on the requests whose current level is n).
-template <int VPL, bool PROBE>
-__global__ void __launch_bounds__(select_max_threads(VPL)) select_advance_kernel(SelectArgs a, EngineState e, int n, int K, int* out_codes,
-                                                             float* out_score, int* out_count) {
-  pdl_wait();
-  pdl_launch();
-  select_body<VPL, PROBE>(a);
-  __syncthreads();                                 // the block's own selection (global writes) is visible to all its threads
-  advance_body(e, n, K, out_codes, out_score, out_count);
-}
-
 // End of a round: accepted length of every draft = the largest i <= (level reached) with D[k][0..i) in B_i;
-// trace outputs; counters for the host (unfinished requests, primary tokens, accepted levels).
+// trace outputs; counters for the host (unfinished requests, primary tokens, accepted levels), which the last block to get
+// here writes to the host's pinned memory together with the status word (a copy node behind every round costs 10 us).
 // adaptive: a request whose round settled only the one level that the pass settles anyway gained nothing from its drafts
 // and stops drafting (its remaining rounds are plain autoregressive steps).
-__global__ void round_end_kernel(EngineState e, int batch, int K, int round, nezha_trace tr, int adaptive) {
-  pdl_wait();
-  pdl_launch();
-  const int b = blockIdx.x;
+__device__ __forceinline__ void round_end_body(const EngineState& e, int K, const RoundEnd& re) {
+  const int b = blockIdx.x, batch = gridDim.x, round = re.round;
   const int L = e.L, Kmax = e.Kmax;
+  const nezha_trace& tr = re.tr;
+  __shared__ int acc_sum;
+  __shared__ unsigned long long s_beam[128];
   const int took_part = e.row_tok_count[b] > 0;
   const int m_now = e.row_m[b];
   const int nd = took_part ? e.dw_count[(long long)L * e.Bmax + b] : 0;
   const long long tro = ((long long)(round - 1) * batch + b);
-  __shared__ int acc_sum;
   if (threadIdx.x == 0) acc_sum = 0;
-  __syncthreads();
-  for (int k = threadIdx.x; k < K; k += blockDim.x) {
-    int acc = -1;
-    if (k < nd) {
-      const int* dc = e.dw_codes + lvl_bk(e, L, b, k) * L;
-      acc = 0;
-      for (int i = 1; i <= m_now; ++i) {
-        const int nbi = e.tb_count[i * e.Bmax + b];
-        bool in = false;
-        for (int r = 0; r < nbi && !in; ++r) {
-          const int* bc = e.tb_codes + lvl_bk(e, i, b, r) * L;
-          bool eq = true;
-          for (int l = 0; l < i; ++l) eq &= (dc[l] == bc[l]);
-          in = eq;
-        }
-        if (in) acc = i; else break;
-      }
-      atomicAdd(&acc_sum, acc);
+  // thread k answers for drafted tuple k (K <= 128 <= threads)
+  const int k = threadIdx.x;
+  const bool mine = k < K && k < nd;
+  int acc = mine ? 0 : -1;
+  if (nd > 0) {
+    const int* dc = e.dw_codes + lvl_bk(e, L, b, mine ? k : 0) * L;
+    unsigned long long key = 0;
+    for (int i = 1; i <= m_now; ++i) {
+      const int nbi = e.tb_count[i * e.Bmax + b];
+      __syncthreads();
+      if (k < nbi) s_beam[k] = prefix_key_of(e, e.tb_codes + lvl_bk(e, i, b, k) * L, i);
+      __syncthreads();
+      if (mine) key += (unsigned long long)(unsigned)dc[i - 1] * e.li.mult[i - 1];
+      bool in = false;
+      if (mine && acc == i - 1)
+        for (int r = 0; r < nbi; ++r) in |= s_beam[r] == key;
+      if (in) acc = i;
     }
+  }
+  __syncthreads();
+  if (mine && acc > 0) atomicAdd(&acc_sum, acc);
+  if (k < K) {
     if (tr.accepted_len) tr.accepted_len[tro * K + k] = acc;
     if (tr.drafts)
       for (int l = 0; l < L; ++l)
@@ -1017,27 +1003,39 @@ __global__ void round_end_kernel(EngineState e, int batch, int K, int round, nez
   if (threadIdx.x == 0) {
     if (tr.n_draft) tr.n_draft[tro] = took_part ? nd : -1;
     if (tr.level_reached) tr.level_reached[tro] = took_part ? m_now : -1;
-    if (took_part && adaptive) e.row_spec[b] = (m_now - e.row_m_start[b] >= 2) ? 1 : 0;
-    if (m_now < L && e.row_spec[b]) atomicMax(e.draft_rows, batch * Kmax);   // somebody drafts next round
+    int spec = e.row_spec[b];
+    if (took_part && re.adaptive) { spec = (m_now - e.row_m_start[b] >= 2) ? 1 : 0; e.row_spec[b] = spec; }
+    if (m_now < L && spec) atomicMax(e.draft_rows, batch * Kmax);            // somebody drafts next round
     if (m_now < L) atomicAdd(&e.counters[0], 1);
-    atomicAdd(&e.counters[1], e.row_tok_count[b]);
-    atomicAdd(&e.counters[2], acc_sum);
-    if (round == 1) atomicAdd(&e.counters[3], nd);
+    if (took_part) atomicAdd(&e.counters[1], e.row_tok_count[b]);
+    if (acc_sum) atomicAdd(&e.counters[2], acc_sum);
+    if (round == 1 && nd) atomicAdd(&e.counters[3], nd);
+    __threadfence();
+    if (atomicAdd(&e.counters[7], 1) == batch - 1) {
+      __threadfence();
+      for (int i = 0; i < 4; ++i) {
+        re.host[i] = *(volatile int*)(e.counters + i);
+        re.host[4 + i] = *(volatile int*)(e.status + i);
+      }
+      __threadfence_system();
+    }
   }
 }
 
-__global__ void write_out_kernel(const int* codes, const float* score, const int* count, int stride, int L, int K,
-                                 int* out_codes, float* out_score, int* out_count) {
+// The selection of B_{n+1}, the step above (both act on the requests whose current level is n) and, behind the last level,
+// the end of the round, in one launch.
+template <int VPL, bool PROBE>
+__global__ void __launch_bounds__(select_max_threads(VPL)) select_advance_kernel(SelectArgs a, EngineState e, int n, int K, int* out_codes,
+                                                             float* out_score, int* out_count, RoundEnd re) {
   pdl_wait();
   pdl_launch();
-  const int b = blockIdx.x;
-  const int cnt = min(count[b], K);
-  for (int k = threadIdx.x; k < K; k += blockDim.x) {
-    const long long s = (long long)b * stride + k;
-    out_score[(long long)b * K + k] = k < cnt ? score[s] : -INFINITY;
-    for (int l = 0; l < L; ++l) out_codes[((long long)b * K + k) * L + l] = k < cnt ? codes[s * L + l] : -1;
+  select_body<VPL, PROBE>(a);
+  __syncthreads();                                 // the block's own selection (global writes) is visible to all its threads
+  advance_body(e, n, K, out_codes, out_score, out_count);
+  if (re.host) {
+    __syncthreads();
+    round_end_body(e, K, re);
   }
-  if (threadIdx.x == 0) out_count[b] = cnt;
 }
 
 // dst[b, r, :] = src[row(b, r), col_off : col_off + T],
@@ -1077,18 +1075,14 @@ void launch_fill_i32(int* p, long long n, int v, cudaStream_t st) {
   LaunchScope ls(kcMisc, st);
   launch_pdl(fill_i32_kernel, dim3((unsigned)((n + 255) / 256 < 1184 ? (n + 255) / 256 : 1184)), dim3(256), 0, st, p, n, v);
 }
-void launch_fill_f32(float* p, long long n, float v, cudaStream_t st) {
-  if (n <= 0) return;
+void launch_decode_begin(const EngineState& e, int batch, int K, int* out_codes, float* out_scores, int* out_count,
+                         const nezha_trace& tr, cudaStream_t st) {
   LaunchScope ls(kcMisc, st);
-  launch_pdl(fill_f32_kernel, dim3((unsigned)((n + 255) / 256 < 1184 ? (n + 255) / 256 : 1184)), dim3(256), 0, st, p, n, v);
-}
-void launch_init_decode(const EngineState& e, int batch, cudaStream_t st) {
-  LaunchScope ls(kcMisc, st);
-  launch_pdl(init_decode_kernel, dim3((batch + 127) / 128), dim3(128), 0, st, e, batch);
+  launch_pdl(decode_begin_kernel, dim3(batch), dim3(128), 0, st, e, batch, K, out_codes, out_scores, out_count, tr);
 }
 void launch_draft_init(const EngineState& e, int batch, int from_scratch, void* s_act, cudaStream_t st) {
   LaunchScope ls(kcDraftGlue, st);
-  launch_pdl(draft_init_kernel, dim3(batch), dim3(128), 0, st, e, batch, from_scratch, (__nv_bfloat16*)s_act);
+  launch_pdl(draft_init_kernel, dim3(batch, s_act ? e.Kmax : 1), dim3(128), 0, st, e, batch, from_scratch, (__nv_bfloat16*)s_act);
 }
 void launch_draft_set(const EngineState& e, int batch, int K, const int* drafts, const int* n_draft, cudaStream_t st) {
   LaunchScope ls(kcDraftGlue, st);
@@ -1161,22 +1155,16 @@ void launch_copy_logits_bias(const float* src, long long row_stride, int row_mul
              bias_stride, dst);
 }
 void launch_build_nodes(const EngineState& e, int batch, cudaStream_t st) {
-  LaunchScope ls(kcNodes, st, 2);
-  launch_pdl(nodes_count_kernel, dim3(batch), dim3(64), 0, st, e, batch);
-  launch_pdl(nodes_fill_kernel, dim3(batch), dim3(128), 0, st, e, batch);
+  LaunchScope ls(kcNodes, st);
+  launch_pdl(nodes_kernel, dim3(batch), dim3(128), 0, st, e, batch);
 }
 void launch_nodes_from_prefixes(const EngineState& e, int batch, int n_beams, int level, const int* prefixes,
                                 cudaStream_t st) {
   LaunchScope ls(kcNodes, st);
   launch_pdl(nodes_from_prefixes_kernel, dim3(batch), dim3(128), 0, st, e, batch, n_beams, level, prefixes);
 }
-void launch_advance(const EngineState& e, int batch, int n, int K, int* out_codes, float* out_score, int* out_count,
-                    cudaStream_t st) {
-  LaunchScope ls(kcAccept, st);
-  launch_pdl(advance_kernel, dim3(batch), dim3(64), 0, st, e, batch, n, K, out_codes, out_score, out_count);
-}
 void launch_select_advance(const SelectArgs& a, const EngineState& e, int n, int K, int* out_codes, float* out_score,
-                           int* out_count, cudaStream_t st) {
+                           int* out_count, const RoundEnd& re, cudaStream_t st) {
   if (a.batch <= 0) return;
   const size_t smem = select_smem_bytes(a.in_stride, a.K);
   LaunchScope ls(kcSelect, st);
@@ -1185,17 +1173,8 @@ void launch_select_advance(const SelectArgs& a, const EngineState& e, int n, int
   with_vpl(a.T, [&](auto vpl) {
     constexpr int V = decltype(vpl)::value;
     launch_pdl(select_probes(a) ? select_advance_kernel<V, true> : select_advance_kernel<V, false>, grid, block, smem, st, a, e, n,
-               K, out_codes, out_score, out_count);
+               K, out_codes, out_score, out_count, re);
   });
-}
-void launch_round_end(const EngineState& e, int batch, int K, int round, const nezha_trace& tr, int adaptive, cudaStream_t st) {
-  LaunchScope ls(kcAccept, st);
-  launch_pdl(round_end_kernel, dim3(batch), dim3(64), 0, st, e, batch, K, round, tr, adaptive);
-}
-void launch_write_out(const int* codes, const float* score, const int* count, int stride, int L, int batch, int K,
-                      int* out_codes, float* out_score, int* out_count, cudaStream_t st) {
-  LaunchScope ls(kcMisc, st);
-  launch_pdl(write_out_kernel, dim3(batch), dim3(64), 0, st, codes, score, count, stride, L, K, out_codes, out_score, out_count);
 }
 void launch_copy_logits(const float* src, long long row_stride, int col_off, const int* row_index, int row_mul,
                         int beam_mul, int batch, int n_beams, int idx_stride, int T, float* dst, cudaStream_t st) {

@@ -49,7 +49,8 @@ struct EngineState {
                                           //        all the attention kernel needs to know about a request, in one load
   int* n_tokens;        // [1] tokens of the verify pass
   int* pf_n_tokens;     // [1] tokens of the prefill chunk
-  int* counters;        // [8]: 0 unfinished rows, 1 primary tokens (round), 2 accepted levels (round), 3 drafted (round)
+  int* counters;        // [8]: 0 unfinished rows, 1 primary tokens (round), 2 accepted levels (round), 3 drafted (round),
+                        //      7 blocks that have closed the round
 
   const float* h_f32;   // [Bmax][L+1][d]
 };
@@ -73,18 +74,25 @@ struct SelectArgs {
   PrefixMapView pm;
   int final_mask_from_map;              // 1: the last-level mask of a beam (all T_L extensions) reads the prefix map; 0: hash probes
   int prefix_filter;                    // 1: this is an earlier level and candidates that begin no valid ID are dropped
+  const int* status; int* host_status;  // optional: the status words are copied to pinned host memory
 };
 void launch_select(const SelectArgs& a, cudaStream_t st);
-// launch_select (gated on row_cur == n) followed, in the same launch, by launch_advance of level n
+// What closes a round, behind its last selection (host == null: not this one): the trace's outputs and, in pinned host memory,
+// the counters (words 0-3) and the status words (4-7).
+struct RoundEnd { int* host; int round, adaptive; nezha_trace tr; };
+// launch_select (gated on row_cur == n) followed, in the same launch, by the accept / roll-back step of level n and, behind
+// the last level, the end of the round
 void launch_select_advance(const SelectArgs& a, const EngineState& e, int n, int K, int* out_codes, float* out_score,
-                           int* out_count, cudaStream_t st);
+                           int* out_count, const RoundEnd& re, cudaStream_t st);
 // launch_select followed, in the same launch, by launch_draft_step of level l (same arguments as there)
 void launch_select_step(const SelectArgs& a, const EngineState& e, int l, const float* G, long long g_stride, int t_cols,
                         const float* U, const float* bias, void* s_act, cudaStream_t st);
 size_t select_smem_bytes(int in_stride, int K);
 cudaError_t select_configure(int max_beam);
 
-void launch_init_decode(const EngineState& e, int batch, cudaStream_t st);
+// out_* and every pointer of tr may be null
+void launch_decode_begin(const EngineState& e, int batch, int K, int* out_codes, float* out_scores, int* out_count,
+                         const nezha_trace& tr, cudaStream_t st);
 void launch_draft_init(const EngineState& e, int batch, int from_scratch, void* s_act, cudaStream_t st);   // s_act may be null
 void launch_draft_set(const EngineState& e, int batch, int K, const int* drafts, const int* n_draft, cudaStream_t st);
 // the whole tree given by the caller: tree_codes [L][batch][K][L], tree_count [L][batch]
@@ -102,15 +110,9 @@ void launch_copy_logits_bias(const float* src, long long row_stride, int row_mul
 void launch_build_nodes(const EngineState& e, int batch, cudaStream_t st);
 void launch_nodes_from_prefixes(const EngineState& e, int batch, int n_beams, int level, const int* prefixes,
                                 cudaStream_t st);
-void launch_advance(const EngineState& e, int batch, int n, int K, int* out_codes, float* out_score, int* out_count,
-                    cudaStream_t st);
-void launch_round_end(const EngineState& e, int batch, int K, int round, const nezha_trace& tr, int adaptive, cudaStream_t st);
-void launch_write_out(const int* codes, const float* score, const int* count, int stride, int L, int batch, int K,
-                      int* out_codes, float* out_score, int* out_count, cudaStream_t st);
 void launch_copy_logits(const float* src, long long row_stride, int col_off, const int* row_index, int row_mul,
                         int beam_mul, int batch, int n_beams, int idx_stride, int T, float* dst, cudaStream_t st);
 void launch_fill_i32(int* p, long long n, int v, cudaStream_t st);
-void launch_fill_f32(float* p, long long n, float v, cudaStream_t st);
 void launch_trace_beams(const EngineState& e, int batch, int K, const nezha_trace& tr, cudaStream_t st);
 
 }  // namespace nz
