@@ -14,6 +14,9 @@ namespace {
 template <typename T, int HD>
 __global__ void __launch_bounds__(128) attn_simt_kernel(AttnArgs a) {
   constexpr int DPL = HD / 8;
+  constexpr int U = HD <= 32 ? 4 : 2;              // positions of a group in flight: their K and V rows are all asked for at once
+  pdl_wait();
+  pdl_launch();
   const int m = a.M_dev ? min(a.M, *a.M_dev) : a.M;
   const long long w = blockIdx.x * (long long)(blockDim.x >> 5) + (threadIdx.x >> 5);
   const int i = (int)(w / a.Hq), h = (int)(w % a.Hq);
@@ -26,19 +29,39 @@ __global__ void __launch_bounds__(128) attn_simt_kernel(AttnArgs a) {
   for (int j = 0; j < DPL; ++j) { qv[j] = to_f32(qp[j]) * a.scale; acc[j] = 0.f; }
   float m_run = -INFINITY, l_run = 0.f;
 
-  auto visit = [&](const T* kp, const T* vp) {
-    float s = 0.f;
+  // U positions (k / v: their rows, null = none) into the running softmax of the lane's group
+  auto visit = [&](const T* const* kp, const T* const* vp) {
+    float kv[U][DPL], vv[U][DPL], s[U];
 #pragma unroll
-    for (int j = 0; j < DPL; ++j) s = fmaf(qv[j], to_f32(kp[j]), s);
-    return s;
-  };
-  auto update = [&](float s, const T* vp) {
-    const float m_new = fmaxf(m_run, s);
+    for (int u = 0; u < U; ++u)
+#pragma unroll
+      for (int j = 0; j < DPL; ++j) {
+        kv[u][j] = kp[u] ? to_f32(kp[u][j]) : 0.f;
+        vv[u][j] = kp[u] ? to_f32(vp[u][j]) : 0.f;
+      }
+    float m_new = m_run;
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      s[u] = 0.f;
+#pragma unroll
+      for (int j = 0; j < DPL; ++j) s[u] = fmaf(qv[j], kv[u][j], s[u]);
+      s[u] += __shfl_xor_sync(0xffffffffu, s[u], 1);
+      s[u] += __shfl_xor_sync(0xffffffffu, s[u], 2);
+      s[u] += __shfl_xor_sync(0xffffffffu, s[u], 4);
+      if (kp[u]) m_new = fmaxf(m_new, s[u]);
+    }
+    if (m_new == -INFINITY) return;                // (nothing seen yet; the same in the group's 8 lanes)
     const float corr = (m_run == -INFINITY) ? 0.f : expf(m_run - m_new);
-    const float pw = expf(s - m_new);
-    l_run = l_run * corr + pw;
+    l_run *= corr;
 #pragma unroll
-    for (int j = 0; j < DPL; ++j) acc[j] = acc[j] * corr + pw * to_f32(vp[j]);
+    for (int j = 0; j < DPL; ++j) acc[j] *= corr;
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const float pw = kp[u] ? expf(s[u] - m_new) : 0.f;
+      l_run += pw;
+#pragma unroll
+      for (int j = 0; j < DPL; ++j) acc[j] = fmaf(pw, vv[u][j], acc[j]);
+    }
     m_run = m_new;
   };
 
@@ -46,25 +69,27 @@ __global__ void __launch_bounds__(128) attn_simt_kernel(AttnArgs a) {
   const long long base = (long long)a.tok_row[i] * a.ctx_row_stride + (long long)kvh * a.ctx_head_stride + sub * DPL;
   const T* kc = reinterpret_cast<const T*>(a.k_ctx) + base;
   const T* vc = reinterpret_cast<const T*>(a.v_ctx) + base;
-  for (int p0 = 0; p0 < ctx_len; p0 += 4) {
-    const int p = p0 + pg;
-    const bool valid = p < ctx_len;
-    float s = valid ? visit(kc + (long long)p * HD, nullptr) : 0.f;
-    s += __shfl_xor_sync(0xffffffffu, s, 1);
-    s += __shfl_xor_sync(0xffffffffu, s, 2);
-    s += __shfl_xor_sync(0xffffffffu, s, 4);
-    if (valid) update(s, vc + (long long)p * HD);
+  for (int p0 = 0; p0 < ctx_len; p0 += 4 * U) {
+    const T *kp[U], *vp[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int p = p0 + 4 * u + pg;
+      kp[u] = p < ctx_len ? kc + (long long)p * HD : nullptr;
+      vp[u] = vc + (long long)p * HD;
+    }
+    visit(kp, vp);
   }
-  for (int e0 = 0; e0 < a.n_ext_max; e0 += 4) {
-    const int e = e0 + pg;
-    const long long off = (e < a.n_ext_max) ? a.tok_ext[(long long)i * a.n_ext_max + e] : -1;
-    const bool valid = off >= 0;
-    const long long eo = off + (long long)kvh * a.ext_head_stride + sub * DPL;
-    float s = valid ? visit(reinterpret_cast<const T*>(a.k_ext) + eo, nullptr) : 0.f;
-    s += __shfl_xor_sync(0xffffffffu, s, 1);
-    s += __shfl_xor_sync(0xffffffffu, s, 2);
-    s += __shfl_xor_sync(0xffffffffu, s, 4);
-    if (valid) update(s, reinterpret_cast<const T*>(a.v_ext) + eo);
+  for (int e0 = 0; e0 < a.n_ext_max; e0 += 4 * U) {
+    const T *kp[U], *vp[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int e = e0 + 4 * u + pg;
+      const long long off = (e < a.n_ext_max) ? a.tok_ext[(long long)i * a.n_ext_max + e] : -1;
+      const long long eo = off + (long long)kvh * a.ext_head_stride + sub * DPL;
+      kp[u] = off >= 0 ? reinterpret_cast<const T*>(a.k_ext) + eo : nullptr;
+      vp[u] = reinterpret_cast<const T*>(a.v_ext) + eo;
+    }
+    visit(kp, vp);
   }
   // merge the 4 position groups
 #pragma unroll
@@ -96,10 +121,10 @@ void dispatch(const AttnArgs& a, cudaStream_t st) {
   const int wpb = 4;
   dim3 grid((unsigned)((warps + wpb - 1) / wpb));
   switch (a.hd) {
-    case 16: attn_simt_kernel<T, 16><<<grid, wpb * 32, 0, st>>>(a); break;
-    case 32: attn_simt_kernel<T, 32><<<grid, wpb * 32, 0, st>>>(a); break;
-    case 64: attn_simt_kernel<T, 64><<<grid, wpb * 32, 0, st>>>(a); break;
-    case 128: attn_simt_kernel<T, 128><<<grid, wpb * 32, 0, st>>>(a); break;
+    case 16: launch_pdl(attn_simt_kernel<T, 16>, grid, dim3(wpb * 32), 0, st, a); break;
+    case 32: launch_pdl(attn_simt_kernel<T, 32>, grid, dim3(wpb * 32), 0, st, a); break;
+    case 64: launch_pdl(attn_simt_kernel<T, 64>, grid, dim3(wpb * 32), 0, st, a); break;
+    case 128: launch_pdl(attn_simt_kernel<T, 128>, grid, dim3(wpb * 32), 0, st, a); break;
     default: break;
   }
 }

@@ -8,6 +8,8 @@ namespace nz {
 template <typename T>
 __global__ void embed_kernel(const T* __restrict__ table, const int* __restrict__ tokens, int M, const int* M_dev,
                              int d, float* __restrict__ resid) {
+  pdl_wait();
+  pdl_launch();
   const int m = M_dev ? min(M, *M_dev) : M;
   const int i = blockIdx.x;
   if (i >= m) return;
@@ -16,26 +18,60 @@ __global__ void embed_kernel(const T* __restrict__ table, const int* __restrict_
   for (int c = threadIdx.x; c < d; c += blockDim.x) dst[c] = to_f32(src[c]);
 }
 
-// out[i, :] = x[row, :] / sqrt(mean(x^2) + eps) * gain,  row = row_index ? row_index[i] : i.  One warp per row.
-template <typename T>
-__global__ void rmsnorm_kernel(const float* __restrict__ x, long long x_stride, const int* __restrict__ row_index,
+// out[i, :] = x[row, :] / sqrt(mean(x^2) + eps) * gain,  row = row_index ? row_index[i] : i.  `wpr` warps per row, 8 warps
+// per block; a lane takes 4 columns at a time (VEC: d % 4 == 0, so rows start on 16-byte boundaries).  A wide row on one
+// warp is a long chain of loads: 10 us at one request of d = 2048.
+template <typename T, bool VEC>
+__global__ void __launch_bounds__(256) rmsnorm_kernel(const float* __restrict__ x, long long x_stride, const int* __restrict__ row_index,
                                const T* __restrict__ gain, T* __restrict__ out, float* __restrict__ out_f32, int M,
-                               const int* M_dev, int d, float eps) {
+                               const int* M_dev, int d, float eps, int wpr) {
+  pdl_wait();
+  pdl_launch();
   const int m = M_dev ? min(M, *M_dev) : M;
-  const int i = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
-  if (i >= m) return;
-  const long long row = row_index ? row_index[i] : i;
-  if (row < 0) return;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int i = blockIdx.x * (8 / wpr) + warp / wpr;
+  const int t = (warp % wpr) * 32 + lane, n_thr = wpr * 32;      // this thread among the row's
+  const long long row = i < m ? (row_index ? row_index[i] : i) : -1;
   const float* src = x + row * x_stride;
+  __shared__ float part[8];
   float ss = 0.f;
-  for (int c = lane; c < d; c += 32) { float v = src[c]; ss += v * v; }
+  if (row >= 0) {
+    if constexpr (VEC) {
+#pragma unroll 4
+      for (int c = 4 * t; c < d; c += 4 * n_thr) {
+        const float4 v = *reinterpret_cast<const float4*>(src + c);
+        ss += v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w;
+      }
+    } else {
+      for (int c = t; c < d; c += n_thr) { const float v = src[c]; ss += v * v; }
+    }
+  }
   ss = warp_sum(ss);
+  if (wpr > 1) {
+    if (lane == 0) part[warp] = ss;
+    __syncthreads();
+    ss = 0.f;
+    for (int w = 0; w < wpr; ++w) ss += part[warp / wpr * wpr + w];
+  }
+  if (row < 0) return;
   const float r = rsqrtf(ss / (float)d + eps);
-  for (int c = lane; c < d; c += 32) {
-    float v = src[c] * r * to_f32(gain[c]);
-    if (out) out[(long long)i * d + c] = from_f32<T>(v);
-    if (out_f32) out_f32[(long long)i * d + c] = v;
+  if constexpr (VEC) {
+#pragma unroll 4
+    for (int c = 4 * t; c < d; c += 4 * n_thr) {
+      const float4 v = *reinterpret_cast<const float4*>(src + c);
+      float y[4] = {v.x * r * to_f32(gain[c]), v.y * r * to_f32(gain[c + 1]), v.z * r * to_f32(gain[c + 2]), v.w * r * to_f32(gain[c + 3])};
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        if (out) out[(long long)i * d + c + e] = from_f32<T>(y[e]);
+        if (out_f32) out_f32[(long long)i * d + c + e] = y[e];
+      }
+    }
+  } else {
+    for (int c = t; c < d; c += n_thr) {
+      const float v = src[c] * r * to_f32(gain[c]);
+      if (out) out[(long long)i * d + c] = from_f32<T>(v);
+      if (out_f32) out_f32[(long long)i * d + c] = v;
+    }
   }
 }
 
@@ -43,6 +79,8 @@ __global__ void rmsnorm_kernel(const float* __restrict__ x, long long x_stride, 
 // k and v of the token are appended to the cache.  One block per token, threads over (head, pair).
 template <typename T>
 __global__ void rope_append_kernel(RopeAppendArgs a) {
+  pdl_wait();
+  pdl_launch();
   const int m = a.M_dev ? min(a.M, *a.M_dev) : a.M;
   const int i = blockIdx.x;
   if (i >= m) return;
@@ -80,6 +118,8 @@ __global__ void rope_append_kernel(RopeAppendArgs a) {
 // act[i, f] = silu(gu[i, f]) * gu[i, F + f]
 template <typename T>
 __global__ void swiglu_kernel(const T* __restrict__ gu, T* __restrict__ act, int M, const int* M_dev, int F) {
+  pdl_wait();
+  pdl_launch();
   const int m = M_dev ? min(M, *M_dev) : M;
   const long long total = (long long)m * F;
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < total;
@@ -91,8 +131,9 @@ __global__ void swiglu_kernel(const T* __restrict__ gu, T* __restrict__ act, int
 }
 
 // Embedding gather fused with the first layer's RMSNorm input: resid = e (fp32), xg = e * gain (bf16, the first
-// GEMM's A operand) and ss[i] = sum(e^2) (the row scale is applied in that GEMM's epilogue).  One block per token.
-__global__ void embed_norm_kernel(const __nv_bfloat16* __restrict__ table, const int* __restrict__ tokens, int M,
+// GEMM's A operand) and ss[i] = sum(e^2) (the row scale is applied in that GEMM's epilogue).  One block per token, 8
+// columns per thread and step (d is a multiple of 64 here): one column per step took 11 us at d = 2048.
+__global__ void __launch_bounds__(256) embed_norm_kernel(const __nv_bfloat16* __restrict__ table, const int* __restrict__ tokens, int M,
                                   const int* M_dev, int d, float* __restrict__ resid,
                                   const __nv_bfloat16* __restrict__ gain, __nv_bfloat16* __restrict__ xg,
                                   float* __restrict__ ss) {
@@ -103,17 +144,33 @@ __global__ void embed_norm_kernel(const __nv_bfloat16* __restrict__ table, const
   if (i >= m) return;
   const __nv_bfloat16* src = table + (long long)tokens[i] * d;
   float part = 0.f;
-  for (int c = threadIdx.x; c < d; c += blockDim.x) {
-    const float v = __bfloat162float(src[c]);
-    resid[(long long)i * d + c] = v;
-    xg[(long long)i * d + c] = __float2bfloat16_rn(v * __bfloat162float(gain[c]));
-    part += v * v;
+  for (int c = 8 * threadIdx.x; c < d; c += 8 * blockDim.x) {
+    const uint4 ev = *reinterpret_cast<const uint4*>(src + c), gv = *reinterpret_cast<const uint4*>(gain + c);
+    const __nv_bfloat162 *ep = reinterpret_cast<const __nv_bfloat162*>(&ev), *gp = reinterpret_cast<const __nv_bfloat162*>(&gv);
+    float2 e[4];
+    uint4 xo;
+    __nv_bfloat162* xp = reinterpret_cast<__nv_bfloat162*>(&xo);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      e[j] = __bfloat1622float2(ep[j]);
+      const float2 g = __bfloat1622float2(gp[j]);
+      xp[j] = __floats2bfloat162_rn(e[j].x * g.x, e[j].y * g.y);
+      part += e[j].x * e[j].x + e[j].y * e[j].y;
+    }
+    float4* rp = reinterpret_cast<float4*>(resid + (long long)i * d + c);
+    rp[0] = make_float4(e[0].x, e[0].y, e[1].x, e[1].y);
+    rp[1] = make_float4(e[2].x, e[2].y, e[3].x, e[3].y);
+    *reinterpret_cast<uint4*>(xg + (long long)i * d + c) = xo;
   }
-  __shared__ float red[4];
+  __shared__ float red[8];
   part = warp_sum(part);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = part;
   __syncthreads();
-  if (threadIdx.x == 0) ss[i] = red[0] + red[1] + red[2] + red[3];
+  if (threadIdx.x == 0) {
+    float sum = 0.f;
+    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) sum += red[w];
+    ss[i] = sum;
+  }
 }
 
 // Weight re-layouts of the fused tensor-core path (run once, at context creation).  The GEMM epilogue hands every
@@ -141,7 +198,8 @@ void launch_embed_norm(const void* table, const int* tokens, int M, const int* M
                        const void* gain, void* xg, float* ss, cudaStream_t st) {
   if (M <= 0) return;
   LaunchScope ls(kcEmbed, st);
-  launch_pdl(embed_norm_kernel, dim3(M), dim3(128), 0, st, (const __nv_bfloat16*)table, tokens, M, M_dev, d, resid,
+  const int threads = (d / 8 + 31) / 32 * 32;
+  launch_pdl(embed_norm_kernel, dim3(M), dim3(threads < 256 ? threads : 256), 0, st, (const __nv_bfloat16*)table, tokens, M, M_dev, d, resid,
                                        (const __nv_bfloat16*)gain, (__nv_bfloat16*)xg, ss);
 }
 void launch_permute_rotary_rows(const void* src, void* dst, int rows, int hd, int cols, cudaStream_t st) {
@@ -158,29 +216,34 @@ void launch_embed(const void* table, bool bf16, const int* tokens, int M, const 
                   cudaStream_t st) {
   if (M <= 0) return;
   LaunchScope ls(kcEmbed, st);
-  if (bf16) embed_kernel<__nv_bfloat16><<<M, 128, 0, st>>>((const __nv_bfloat16*)table, tokens, M, M_dev, d, resid);
-  else embed_kernel<float><<<M, 128, 0, st>>>((const float*)table, tokens, M, M_dev, d, resid);
+  if (bf16) launch_pdl(embed_kernel<__nv_bfloat16>, dim3(M), dim3(128), 0, st, (const __nv_bfloat16*)table, tokens, M, M_dev, d, resid);
+  else launch_pdl(embed_kernel<float>, dim3(M), dim3(128), 0, st, (const float*)table, tokens, M, M_dev, d, resid);
 }
 
 void launch_rmsnorm(const float* x, long long x_stride, const int* row_index, const void* gain, bool bf16, void* out,
                     float* out_f32, int M, const int* M_dev, int d, float eps, cudaStream_t st) {
   if (M <= 0) return;
-  const int wpb = 8;
+  const int wpr = d >= 2048 ? 8 : d >= 1024 ? 4 : d >= 512 ? 2 : 1;
   LaunchScope ls(kcNorm, st);
-  dim3 grid((M + wpb - 1) / wpb);
-  if (bf16)
-    rmsnorm_kernel<__nv_bfloat16><<<grid, wpb * 32, 0, st>>>(x, x_stride, row_index, (const __nv_bfloat16*)gain,
-                                                             (__nv_bfloat16*)out, out_f32, M, M_dev, d, eps);
-  else
-    rmsnorm_kernel<float><<<grid, wpb * 32, 0, st>>>(x, x_stride, row_index, (const float*)gain, (float*)out, out_f32,
-                                                     M, M_dev, d, eps);
+  const dim3 grid((M + 8 / wpr - 1) / (8 / wpr));
+  const bool vec = d % 4 == 0 && x_stride % 4 == 0;
+  auto go = [&](auto kernel, auto* g, auto* o) {
+    launch_pdl(kernel, grid, dim3(256), 0, st, x, x_stride, row_index, g, o, out_f32, M, M_dev, d, eps, wpr);
+  };
+  if (bf16) {
+    if (vec) go(rmsnorm_kernel<__nv_bfloat16, true>, (const __nv_bfloat16*)gain, (__nv_bfloat16*)out);
+    else go(rmsnorm_kernel<__nv_bfloat16, false>, (const __nv_bfloat16*)gain, (__nv_bfloat16*)out);
+  } else {
+    if (vec) go(rmsnorm_kernel<float, true>, (const float*)gain, (float*)out);
+    else go(rmsnorm_kernel<float, false>, (const float*)gain, (float*)out);
+  }
 }
 
 void launch_rope_append(const RopeAppendArgs& a, bool bf16, cudaStream_t st) {
   if (a.M <= 0) return;
   LaunchScope ls(kcRope, st);
-  if (bf16) rope_append_kernel<__nv_bfloat16><<<a.M, 128, 0, st>>>(a);
-  else rope_append_kernel<float><<<a.M, 128, 0, st>>>(a);
+  if (bf16) launch_pdl(rope_append_kernel<__nv_bfloat16>, dim3(a.M), dim3(128), 0, st, a);
+  else launch_pdl(rope_append_kernel<float>, dim3(a.M), dim3(128), 0, st, a);
 }
 
 void launch_swiglu(const void* gu, void* act, int M, const int* M_dev, int F, bool bf16, cudaStream_t st) {
@@ -188,8 +251,8 @@ void launch_swiglu(const void* gu, void* act, int M, const int* M_dev, int F, bo
   long long total = (long long)M * F;
   LaunchScope ls(kcSwiglu, st);
   int blocks = (int)((total + 255) / 256 < 148 * 16 ? (total + 255) / 256 : 148 * 16);
-  if (bf16) swiglu_kernel<__nv_bfloat16><<<blocks, 256, 0, st>>>((const __nv_bfloat16*)gu, (__nv_bfloat16*)act, M, M_dev, F);
-  else swiglu_kernel<float><<<blocks, 256, 0, st>>>((const float*)gu, (float*)act, M, M_dev, F);
+  if (bf16) launch_pdl(swiglu_kernel<__nv_bfloat16>, dim3(blocks), dim3(256), 0, st, (const __nv_bfloat16*)gu, (__nv_bfloat16*)act, M, M_dev, F);
+  else launch_pdl(swiglu_kernel<float>, dim3(blocks), dim3(256), 0, st, (const float*)gu, (float*)act, M, M_dev, F);
 }
 
 }  // namespace nz
