@@ -9,6 +9,8 @@
 //   RW = 4, KW = 1   64 rows per CTA, every warp walks all tiles                       (many query rows per request)
 //   RW = 1, KW = 4   16 rows per CTA, the four warps take every fourth tile and their   (few rows: one beam set of a
 //                    softmax states are merged through shared memory at the end          small model, plain decode)
+// Where that leaves SMs idle -- few requests, whatever their context -- the tiles are also split over the CTAs of a cluster,
+// which merge their softmax states through distributed shared memory (SPLIT, see launch_attention_tc).
 // Ring slots are handed back to the producer with per-slot "empty" mbarriers, so warps never wait for each other.
 // The draft-token KV rows (a token sees its own tuple's drafted codes, at most L of them) are not gathered per token:
 // the request's whole block of draft positions -- every beam's, every level's, contiguous in the cache for one KV head --
@@ -58,6 +60,18 @@ __device__ __forceinline__ uint32_t kv_addr(uint32_t tile, int pos, int chunk) {
   return tile + sub * (kPos * 128) + pos * 128 + ((c ^ (pos & 7)) << 4);
 }
 
+__device__ __forceinline__ void cluster_sync_all() {       // every thread of every CTA of the cluster, on every path
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ float ld_peer(uint32_t local, uint32_t rank) {
+  uint32_t ra;
+  float v;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(local), "r"(rank));
+  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(ra) : "memory");
+  return v;
+}
+
 template <int HD, int RW, int KW>
 struct AttnCfg {
   static constexpr int kStages = KW == 1 ? 3 : KW;                // a multiple of KW: slot s always serves warp group s % KW
@@ -70,7 +84,8 @@ struct AttnCfg {
   static constexpr int kSmemBytes = kStages * kStageBytes + 1024 + 128 + kMergeBytes;
 };
 
-template <int HD, int RW, int KW>
+// SPLIT: blockIdx.x = KV head * cluster size + rank, a power of two of at most 8 CTAs per cluster; RW = 1.
+template <int HD, int RW, int KW, bool SPLIT>
 __global__ void __launch_bounds__(AttnCfg<HD, RW, KW>::kThreads) attn_tc_kernel(const __grid_constant__ CUtensorMap tmK,
                                                                                const __grid_constant__ CUtensorMap tmV,
                                                                                const __grid_constant__ CUtensorMap tmKx,
@@ -88,14 +103,19 @@ __global__ void __launch_bounds__(AttnCfg<HD, RW, KW>::kThreads) attn_tc_kernel(
   // the row tile is the slowest grid index: tiles beyond a request's rows (the grid covers the largest row count a
   // call may have) are scheduled after every tile that has work, instead of holding its place in the first wave
   // (a causal prefill has no such tiles to speak of, and its last tiles see the most context: those go first)
-  const int req_local = blockIdx.y, kvh = blockIdx.x;
+  uint32_t n_split = 1, rank = 0;
+  if constexpr (SPLIT) {
+    asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(n_split));
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+  }
+  const int req_local = blockIdx.y, kvh = SPLIT ? (int)(blockIdx.x / n_split) : (int)blockIdx.x;
   const int tile = a.n_ext_max > 0 ? (int)blockIdx.z : (int)(gridDim.z - 1 - blockIdx.z);
   const int G = a.Hq / a.Hkv;
   const int4 info = a.req_info[req_local];          // {first token, token count, cache row, context length or -1}
   const int tok0 = info.x, n_tok = info.y, request = info.z;
   const int R = n_tok * G;                          // query rows of this (request, kv head)
   const int r0 = tile * kRows;
-  if (r0 >= R) return;
+  if (r0 >= R) return;                              // (all CTAs of a cluster alike)
   // context positions this tile needs: all of them, or (causal prefill) up to its last token's own position
   const int max_ctx = info.w >= 0 ? info.w : min((r0 + kRows - 1) / G, n_tok - 1) + 1;
   const int n_tiles = (max_ctx + kPos - 1) / kPos;
@@ -104,7 +124,9 @@ __global__ void __launch_bounds__(AttnCfg<HD, RW, KW>::kThreads) attn_tc_kernel(
   // among them, through a per-row bit mask.  Rows nobody sees are finite (the cache is zeroed when the engine is made),
   // so their P = 0 contributes exactly nothing.
   const int n_xt = a.n_ext_max > 0 ? (a.ext_positions + kPos - 1) / kPos : 0;
-  const int NT = n_tiles + n_xt;
+  // this CTA's share of the tiles: all, or the cluster's in order of rank
+  const int t0 = SPLIT ? (int)((n_tiles + n_xt) * rank / n_split) : 0;
+  const int NT = (SPLIT ? (int)((n_tiles + n_xt) * (rank + 1) / n_split) : n_tiles + n_xt) - t0;
   const int kv_row0 = (int)(((long long)request * a.Hkv + kvh) * (a.ctx_head_stride / HD));   // first cache row
 
   extern __shared__ uint8_t smem_raw[];
@@ -144,11 +166,11 @@ __global__ void __launch_bounds__(AttnCfg<HD, RW, KW>::kThreads) attn_tc_kernel(
 #pragma unroll
         for (int h = 0; h < NH; ++h) {
           const uint32_t kd = base + s * C::kStageBytes + h * (kPos * 128), vd = kd + C::kTileBytes;
-          if (t < n_tiles) {
-            tma_load_2d(kd, &tmK, h * 64, kv_row0 + t * kPos, full_bar(s));
-            tma_load_2d(vd, &tmV, h * 64, kv_row0 + t * kPos, full_bar(s));
+          if (t0 + t < n_tiles) {
+            tma_load_2d(kd, &tmK, h * 64, kv_row0 + (t0 + t) * kPos, full_bar(s));
+            tma_load_2d(vd, &tmV, h * 64, kv_row0 + (t0 + t) * kPos, full_bar(s));
           } else {                                   // [positions, kv heads * hd]: this head's columns of 64 draft positions
-            const int y = request * a.ext_positions + (t - n_tiles) * kPos;
+            const int y = request * a.ext_positions + (t0 + t - n_tiles) * kPos;
             tma_load_2d(kd, &tmKx, kvh * HD + h * 64, y, full_bar(s));
             tma_load_2d(vd, &tmVx, kvh * HD + h * 64, y, full_bar(s));
           }
@@ -198,9 +220,9 @@ __global__ void __launch_bounds__(AttnCfg<HD, RW, KW>::kThreads) attn_tc_kernel(
         xpos[i][e] = off >= 0 ? (int)((off - (long long)request * a.ext_req_stride) / a.ext_pos_stride) : -1;
       }
 
-    for (int t = g; t < NT; t += KW) {
-      const int s = t % S;
-      const bool got = mbar_wait_or_abort(full_bar(s), (t / S) & 1, abort_flag);
+    for (int tl = g; tl < NT; tl += KW) {
+      const int s = tl % S, t = t0 + tl;
+      const bool got = mbar_wait_or_abort(full_bar(s), (tl / S) & 1, abort_flag);
       if (!__all_sync(0xffffffffu, got)) { if (lane == 0) *abort_flag = 1; break; }
       const uint32_t kt = base + s * C::kStageBytes, vt = kt + C::kTileBytes;
 
@@ -305,13 +327,11 @@ __global__ void __launch_bounds__(AttnCfg<HD, RW, KW>::kThreads) attn_tc_kernel(
     }
   }
   __syncthreads();
-  if (*abort_flag) {
-    if (threadIdx.x == 0) atomicOr(status, kStInternal);
-    return;
-  }
-  if (warp >= RW) return;                            // the rest is warp group 0's
+  const bool aborted = *abort_flag != 0;
+  if (aborted && threadIdx.x == 0) atomicOr(status, kStInternal);
+  if (!SPLIT && (aborted || warp >= RW)) return;     // the rest is warp group 0's
 
-  if (KW > 1) {
+  if (KW > 1 && warp < RW) {
 #pragma unroll 1
     for (int og = 1; og < KW; ++og) {
       const float* src = merge + ((size_t)((og - 1) * RW + rw) * C::kMergeFloats) * 32 + lane;
@@ -333,6 +353,66 @@ __global__ void __launch_bounds__(AttnCfg<HD, RW, KW>::kThreads) attn_tc_kernel(
     }
   }
 
+  if constexpr (SPLIT) {
+    // The cluster's states: every CTA leaves its own (o, m, l) where its ring was (all tiles are consumed), and finishes
+    // NB / n_split of the output's 8-column blocks over all ranks.
+    float* mine = reinterpret_cast<float*>(gen_base) + (size_t)rw * C::kMergeFloats * 32 + lane;
+    if (warp < RW) {
+#pragma unroll
+      for (int j = 0; j < NB; ++j)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) mine[(j * 4 + e) * 32] = o[j][e];
+      mine[(NB * 4 + 0) * 32] = m_run[0]; mine[(NB * 4 + 1) * 32] = m_run[1];
+      mine[(NB * 4 + 2) * 32] = l_run[0]; mine[(NB * 4 + 3) * 32] = l_run[1];
+    }
+    cluster_sync_all();
+    if (warp < RW && !aborted) {
+      const uint32_t at = base + (uint32_t)((rw * C::kMergeFloats * 32 + lane) * 4);
+      float wgt[8][2], m_all[2] = {-INFINITY, -INFINITY}, l_all[2] = {0.f, 0.f};
+#pragma unroll
+      for (int p = 0; p < 8; ++p)
+        if (p < (int)n_split)
+#pragma unroll
+          for (int i = 0; i < 2; ++i) {
+            wgt[p][i] = ld_peer(at + (NB * 4 + i) * 128, p);
+            m_all[i] = fmaxf(m_all[i], wgt[p][i]);
+          }
+#pragma unroll
+      for (int p = 0; p < 8; ++p)
+        if (p < (int)n_split)
+#pragma unroll
+          for (int i = 0; i < 2; ++i) {
+            wgt[p][i] = ex2(wgt[p][i] - (m_all[i] == -INFINITY ? 0.f : m_all[i]));
+            l_all[i] += wgt[p][i] * ld_peer(at + (NB * 4 + 2 + i) * 128, p);
+          }
+      __nv_bfloat16* out = reinterpret_cast<__nv_bfloat16*>(a.out);
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        l_all[i] += __shfl_xor_sync(0xffffffffu, l_all[i], 1);
+        l_all[i] += __shfl_xor_sync(0xffffffffu, l_all[i], 2);
+      }
+      const int share = NB / (int)n_split;
+#pragma unroll 2
+      for (int j = (int)rank * share; j < ((int)rank + 1) * share; ++j) {
+        float v[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+        for (int p = 0; p < 8; ++p)
+          if (p < (int)n_split)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) v[e] += wgt[p][e >> 1] * ld_peer(at + (j * 4 + e) * 128, p);
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+          if (live[i] && l_all[i] > 0.f) {
+            const float inv = 1.f / l_all[i];
+            __nv_bfloat16* op = out + (long long)tok[i] * a.out_stride + (long long)head[i] * HD + qc * 2;
+            *reinterpret_cast<__nv_bfloat162*>(op + j * 8) = __floats2bfloat162_rn(v[i * 2] * inv, v[i * 2 + 1] * inv);
+          }
+      }
+    }
+    cluster_sync_all();                              // no CTA leaves while a peer may still read its state
+    return;
+  }
+
   // ---- normalise and store
   __nv_bfloat16* out = reinterpret_cast<__nv_bfloat16*>(a.out);
 #pragma unroll
@@ -349,15 +429,16 @@ __global__ void __launch_bounds__(AttnCfg<HD, RW, KW>::kThreads) attn_tc_kernel(
   }
 }
 
-template <int HD, int RW, int KW>
-void launch(const CUtensorMap* tk, const CUtensorMap* tv, const AttnArgs& a, cudaStream_t st) {
+// splits > 1: the SPLIT form in clusters of that many CTAs.
+template <int HD, int RW, int KW, bool SPLIT = false>
+void launch(const CUtensorMap* tk, const CUtensorMap* tv, const AttnArgs& a, cudaStream_t st, int splits = 1) {
   using C = AttnCfg<HD, RW, KW>;
   static PerDeviceOnce configured;
   configured.run([] {
-    cudaFuncSetAttribute(attn_tc_kernel<HD, RW, KW>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes);
+    cudaFuncSetAttribute(attn_tc_kernel<HD, RW, KW, SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes);
   });
   const int G = a.Hq / a.Hkv;
-  dim3 grid(a.Hkv, a.n_rows, (a.max_tokens_per_row * G + 16 * RW - 1) / (16 * RW));
+  dim3 grid(a.Hkv * splits, a.n_rows, (a.max_tokens_per_row * G + 16 * RW - 1) / (16 * RW));
   // the layer's draft-token caches as [positions of all requests, kv heads * hd] (a prefill has none: any valid map)
   CUtensorMap tkx = *tk, tvx = *tv;
   if (a.n_ext_max > 0) {
@@ -368,7 +449,22 @@ void launch(const CUtensorMap* tk, const CUtensorMap* tv, const AttnArgs& a, cud
       return;
     }
   }
-  launch_pdl(attn_tc_kernel<HD, RW, KW>, dim3(grid), dim3(C::kThreads), C::kSmemBytes, st, *tk, *tv, tkx, tvx, a, a.status);
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid; cfg.blockDim = dim3(C::kThreads); cfg.dynamicSmemBytes = C::kSmemBytes; cfg.stream = st;
+  cudaLaunchAttribute at[2];
+  int n = 0;
+  if (SPLIT) {
+    at[n].id = cudaLaunchAttributeClusterDimension;
+    at[n].val.clusterDim.x = splits; at[n].val.clusterDim.y = 1; at[n].val.clusterDim.z = 1;
+    ++n;
+  }
+  if (pdl_enabled()) {
+    at[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[n].val.programmaticStreamSerializationAllowed = 1;
+    ++n;
+  }
+  cfg.attrs = at; cfg.numAttrs = n;
+  cudaLaunchKernelEx(&cfg, attn_tc_kernel<HD, RW, KW, SPLIT>, *tk, *tv, tkx, tvx, a, a.status);
 }
 
 }  // namespace
@@ -397,7 +493,21 @@ void launch_attention_tc(const AttnArgs& a, cudaStream_t st) {
   const int G = a.Hq / a.Hkv;
   const long long r_bound = (long long)a.max_tokens_per_row * G;
   const long long r = a.rows_expected > 0 && a.rows_expected < r_bound ? a.rows_expected : r_bound;
-  if (r <= 32) {                                     // 16-row CTAs whose two consumer warps split the KV tiles
+  // Few requests (16-row CTAs that all fit the SMs twice over): short CTAs whatever the number of rows, their tiles split over a
+  // cluster where the context is long.  K/V is then streamed once per 16 rows, from L2, by SMs that would be idle otherwise;
+  // the tcgen05 kernel's CTA of 128 rows is one chain of 8 us at two tiles and 45 us at 30.  Measured per decode, before ->
+  // without / with the split: 7B shape, one request of 1,853 positions 10.3 -> 9.9 / 8.5 ms; 1.5B shape, two of 601 9.5 -> 9.1
+  // / 8.9; 0.5B shape, five of 361 3.94 -> 3.56 / 3.62; 1B-sized backbone, one of 37 2.50 -> 2.38 ms (no split: a cluster
+  // costs 2 us a launch).
+  const long long ctas = (long long)a.Hkv * a.n_rows * ((r + 15) / 16);
+  const int tiles = (a.ctx_bound + kPos - 1) / kPos + (a.n_ext_max > 0 ? (a.ext_positions + kPos - 1) / kPos : 0);
+  int splits = tiles >= 24 ? 8 : tiles >= 10 ? 4 : 1;
+  while (splits > 1 && splits * ctas > 296) splits /= 2;
+  if (splits > 1) {
+    if (a.hd == 64) launch<64, 1, 2, true>(tk, tv, a, st, splits); else launch<128, 1, 2, true>(tk, tv, a, st, splits);
+    return;
+  }
+  if (r <= 32 || (ctas <= 296 && a.ctx_bound > 0)) {  // 16-row CTAs whose two consumer warps split the KV tiles
     if (a.hd == 64) launch<64, 1, 2>(tk, tv, a, st); else launch<128, 1, 2>(tk, tv, a, st);
     return;
   }
