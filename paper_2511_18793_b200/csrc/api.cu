@@ -91,7 +91,6 @@ struct nezha_ctx {
   int opt_level_filter;     // nezha_set_option: 1 = validity filter at every level (prefixes of valid IDs), 0 (default) = last level only
   int m_expected;           // tokens the current verify pass is expected to hold (0 = unknown); shapes GEMM tiling only
   int m_seen[kMaxLevels + 1];   // tokens each round of the last decode call processed, rounded up to a row tile
-  int chains_now;           // GemmArgs::chains of the products being queued: 2 inside a decode call, 0 otherwise
   // Weight-streaming products: the most rows a pass of this engine's decode calls may have where that is at most
   // kSkinnyClassRows, else 0.  Every product of a decode call is given this class (the choice of its kernel is per engine and
   // product, so both decode modes compute the same bits).
@@ -287,7 +286,6 @@ size_t carve(nezha_ctx* c) {
 void gemm(nezha_ctx* c, const void* A, long long lda, const void* W, long long ldw, void* C, long long ldc, long long M,
           const int* M_dev, int N, int K, int epi, const float* bias = nullptr) {
   GemmArgs a{A, lda, W, ldw, C, ldc, (int)M, M_dev, N, K, epi, bias, c->es.status};
-  a.chains = c->chains_now;
   a.skinny = c->skinny_now;
   if (c->bf16 && gemm_tc_supported(a)) launch_gemm_tc(a, c->st);
   else launch_gemm_simt(a, c->bf16, c->st);
@@ -302,7 +300,6 @@ int gemm_fused(nezha_ctx* c, const void* A, long long lda, const void* W, void* 
   if (extra) a.f = *extra;
   a.f.ss_in = ss_in; a.f.ss_in_parts = ss_parts; a.f.ss_ld = c->Ms; a.f.inv_dim = 1.f / (float)c->d; a.f.eps = c->cfg.rms_eps;
   a.M_expected = c->m_expected;
-  a.chains = c->chains_now;
   a.skinny = c->skinny_now;
   launch_gemm_tc(a, c->st);
   return N / 32;
@@ -576,17 +573,13 @@ nezha_status decode_impl(nezha_ctx* c, int batch, int K, int mode, const int* dr
     return fail(c, NEZHA_ERR_ARG, "nezha_decode: bad batch / beam_width / mode / output pointer");
   const EngineState& e = c->es;
   const int L = c->L;
-  // Every product of a decode call asks for the two-partial-sum order on narrow outputs (two MMA issuers): the
-  // choice is per call path, never per launch, so that the speculative and the autoregressive mode, whose passes differ
-  // in size, still compute the same bits.  The prefill keeps the plain order and the widest tiles.
-  struct ChainScope {
+  // Every product of a decode call is given the engine's row class: the choice of its kernel is per engine and product, never
+  // per launch, so that the speculative and the autoregressive mode, whose passes differ in size, compute the same bits.
+  struct ClassScope {
     nezha_ctx* c;
-    explicit ChainScope(nezha_ctx* c_) : c(c_) {
-      c->chains_now = 2;
-      c->skinny_now = c->skinny_class;
-    }
-    ~ChainScope() { c->chains_now = 0; c->skinny_now = 0; }
-  } chain_scope(c);
+    explicit ClassScope(nezha_ctx* c_) : c(c_) { c->skinny_now = c->skinny_class; }
+    ~ClassScope() { c->skinny_now = 0; }
+  } class_scope(c);
   nezha_trace tr{};
   if (trace) tr = *trace;
   nezha_decode_stats sd{};
@@ -718,7 +711,6 @@ nezha_status nezha_create(const nezha_config* cfg, const nezha_weights* w, const
   c->m_expected = 0;
   for (int i = 0; i <= kMaxLevels; ++i) c->m_seen[i] = 0;
   for (int i = 0; i < 3; ++i) c->rounds_seen[i] = 0;
-  c->chains_now = 0;
   c->skinny_now = 0;
   c->opt_transition = 0; c->opt_inputs = 0; c->opt_filter = 1; c->opt_mask = 1; c->opt_level_filter = 0; c->opt_adaptive = 0;
   const size_t need = carve(c);
@@ -1014,7 +1006,6 @@ nezha_status nezha_gemm(nezha_ctx* c, const void* A, const void* W, void* C, int
       path > 4)
     return fail(c, NEZHA_ERR_ARG, "nezha_gemm: bad argument");
   GemmArgs a{A, K, W, K, C, N, M, nullptr, N, K, epilogue, bias, c->es.status};
-  a.chains = path == 3 ? 2 : 0;
   if (path == 4) {
     if (M > kSkinnyRows || !c->bf16)
       return fail(c, NEZHA_ERR_UNSUPPORTED, "nezha_gemm: the weight-streaming kernel takes bf16 products of at most 128 rows");

@@ -156,30 +156,27 @@ __global__ void __launch_bounds__(AttnCfg<HD, RW, KW>::kThreads) attn_tc_kernel(
 
   if (warp == C::kConsumers) {
     // ------------------------------------------------------------------ TMA producer
-    if (lane == 0) {
-      int t = 0;
-      bool ok = true;
-      for (; t < NT; ++t) {
-        const int s = t % S;
-        if (t >= S && !mbar_wait_or_abort(empty_bar(s), ((t / S) - 1) & 1, abort_flag)) { ok = false; break; }
-        mbar_expect_tx(full_bar(s), C::kStageBytes);
+    const uint32_t leader = elect_one();
+    int t = 0;
+    bool ok = true;
+    for (; t < NT; ++t) {
+      const int s = t % S;
+      if (t >= S && !warp_wait_uniform(empty_bar(s), ((t / S) - 1) & 1, abort_flag)) { ok = false; break; }
+      mbar_expect_tx_if(full_bar(s), C::kStageBytes, leader);
+      // a context tile, or 64 draft positions of [positions, kv heads * hd]: this head's columns
+      const bool ctx_tile = t0 + t < n_tiles;
+      const int y = ctx_tile ? kv_row0 + (t0 + t) * kPos : request * a.ext_positions + (t0 + t - n_tiles) * kPos;
+      const int x0 = ctx_tile ? 0 : kvh * HD;
 #pragma unroll
-        for (int h = 0; h < NH; ++h) {
-          const uint32_t kd = base + s * C::kStageBytes + h * (kPos * 128), vd = kd + C::kTileBytes;
-          if (t0 + t < n_tiles) {
-            tma_load_2d(kd, &tmK, h * 64, kv_row0 + (t0 + t) * kPos, full_bar(s));
-            tma_load_2d(vd, &tmV, h * 64, kv_row0 + (t0 + t) * kPos, full_bar(s));
-          } else {                                   // [positions, kv heads * hd]: this head's columns of 64 draft positions
-            const int y = request * a.ext_positions + (t0 + t - n_tiles) * kPos;
-            tma_load_2d(kd, &tmKx, kvh * HD + h * 64, y, full_bar(s));
-            tma_load_2d(vd, &tmVx, kvh * HD + h * 64, y, full_bar(s));
-          }
-        }
+      for (int h = 0; h < NH; ++h) {
+        const uint32_t kd = base + s * C::kStageBytes + h * (kPos * 128), vd = kd + C::kTileBytes;
+        tma_load_2d_if(kd, ctx_tile ? &tmK : &tmKx, x0 + h * 64, y, full_bar(s), leader);
+        tma_load_2d_if(vd, ctx_tile ? &tmV : &tmVx, x0 + h * 64, y, full_bar(s), leader);
       }
-      if (!ok) {                                     // drain the copies still in flight before the CTA's smem goes away
-        *abort_flag = 1;
-        for (int j = max(0, t - S); j < t; ++j) mbar_wait(full_bar(j % S), (j / S) & 1);
-      }
+    }
+    if (!ok && lane == 0) {                          // drain the copies still in flight before the CTA's smem goes away
+      *abort_flag = 1;
+      for (int j = max(0, t - S); j < t; ++j) mbar_wait(full_bar(j % S), (j / S) & 1);
     }
   } else {
     // ------------------------------------------------------------------ consumers

@@ -61,12 +61,12 @@ template <int HD, bool PT> struct UmmaCfg {
 
 // D[tmem] (+)= A[tmem] * B[smem]: the A operand (128 rows = lanes, K along the columns, two bf16 per 32-bit cell) is read
 // from tensor memory.
-__device__ __forceinline__ void tc_mma_a_tmem(uint32_t tmem_d, uint32_t tmem_a, uint64_t db, uint32_t idesc, uint32_t accumulate) {
+__device__ __forceinline__ void tc_mma_a_tmem(uint32_t tmem_d, uint32_t tmem_a, uint64_t db, uint32_t idesc, uint32_t accumulate, uint32_t leader) {
   asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
-      ::"r"(tmem_d), "r"(tmem_a), "l"(db), "r"(idesc), "r"(accumulate) : "memory");
+      "{\n\t.reg .pred p, q;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 q, %5, 0;\n\t"
+      "@q tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
+      ::"r"(tmem_d), "r"(tmem_a), "l"(db), "r"(idesc), "r"(accumulate), "r"(leader) : "memory");
 }
 __device__ __forceinline__ void tmem_st32_bits(uint32_t taddr, const uint32_t* v) {
   asm volatile(
@@ -240,51 +240,51 @@ __global__ void __launch_bounds__(kThreadsU, UmmaCfg<HD, PT>::kCtasPerSm) attn_u
 
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer
-    if (lane == 0) {
-      int t = 0, k_issued = 0, v_issued = 0;
-      bool ok = true;
-      for (; t < NT; ++t) {
-        const int sk = t % SK, sv = t % SV;
-        const bool ctx_tile = t < n_tiles;
-        const int y = ctx_tile ? kv_row0 + t * kPosU : request * a.ext_positions + (t - n_tiles) * kPosU;
-        const int x0 = ctx_tile ? 0 : kvh * HD;      // the draft cache is [positions, kv heads * hd]: this head's columns
-        if (t >= SK && !mbar_wait_or_abort(k_empty(sk), (uint32_t)((t / SK) - 1) & 1u, abort_flag)) { gave_up(1, t); ok = false; break; }
-        mbar_expect_tx(k_full(sk), C::kTileBytes);
+    const uint32_t leader = elect_one();
+    int t = 0, k_issued = 0, v_issued = 0;
+    bool ok = true;
+    for (; t < NT; ++t) {
+      const int sk = t % SK, sv = t % SV;
+      const bool ctx_tile = t < n_tiles;
+      const int y = ctx_tile ? kv_row0 + t * kPosU : request * a.ext_positions + (t - n_tiles) * kPosU;
+      const int x0 = ctx_tile ? 0 : kvh * HD;        // the draft cache is [positions, kv heads * hd]: this head's columns
+      if (t >= SK && !warp_wait_uniform(k_empty(sk), (uint32_t)((t / SK) - 1) & 1u, abort_flag)) { if (leader) gave_up(1, t); ok = false; break; }
+      mbar_expect_tx_if(k_full(sk), C::kTileBytes, leader);
 #pragma unroll
-        for (int h = 0; h < NH; ++h)
-          tma_load_2d(k_base + sk * C::kTileBytes + h * (kPosU * 128), ctx_tile ? &tmK : &tmKx, x0 + h * 64, y, k_full(sk));
-        ++k_issued;
-        if (t >= SV && !mbar_wait_or_abort(v_empty(sv), (uint32_t)((t / SV) - 1) & 1u, abort_flag)) { gave_up(2, t); ok = false; break; }
-        mbar_expect_tx(v_full(sv), C::kTileBytes);
+      for (int h = 0; h < NH; ++h)
+        tma_load_2d_if(k_base + sk * C::kTileBytes + h * (kPosU * 128), ctx_tile ? &tmK : &tmKx, x0 + h * 64, y, k_full(sk), leader);
+      ++k_issued;
+      if (t >= SV && !warp_wait_uniform(v_empty(sv), (uint32_t)((t / SV) - 1) & 1u, abort_flag)) { if (leader) gave_up(2, t); ok = false; break; }
+      mbar_expect_tx_if(v_full(sv), C::kTileBytes, leader);
 #pragma unroll
-        for (int h = 0; h < NH; ++h)
-          tma_load_2d(v_base + sv * C::kTileBytes + h * (kPosU * 128), ctx_tile ? &tmV : &tmVx, x0 + h * 64, y, v_full(sv));
-        ++v_issued;
-      }
-      if (!ok) {                                     // drain the copies still in flight before the CTA's memory goes away
-        *abort_flag = 1;
-        for (int j = max(0, k_issued - SK); j < k_issued; ++j) mbar_wait(k_full(j % SK), (j / SK) & 1);
-        for (int j = max(0, v_issued - SV); j < v_issued; ++j) mbar_wait(v_full(j % SV), (j / SV) & 1);
-      }
+      for (int h = 0; h < NH; ++h)
+        tma_load_2d_if(v_base + sv * C::kTileBytes + h * (kPosU * 128), ctx_tile ? &tmV : &tmVx, x0 + h * 64, y, v_full(sv), leader);
+      ++v_issued;
+    }
+    if (!ok && lane == 0) {                          // drain the copies still in flight before the CTA's memory goes away
+      *abort_flag = 1;
+      for (int j = max(0, k_issued - SK); j < k_issued; ++j) mbar_wait(k_full(j % SK), (j / SK) & 1);
+      for (int j = max(0, v_issued - SV); j < v_issued; ++j) mbar_wait(v_full(j % SV), (j / SV) & 1);
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer
-    if (lane == 0) {
+    const uint32_t leader = elect_one();
+    {
       bool ok = true;
       auto issue_s = [&](int j) {                    // S_j = Q K_j^T into S buffer (PT ? j & 1 : 0)
         const int s = j % SK, b = PT ? (j & 1) : 0;
-        if (!mbar_wait_or_abort(k_full(s), (uint32_t)(j / SK) & 1u, abort_flag)) { gave_up(3, j); return false; }
+        if (!warp_wait_uniform(k_full(s), (uint32_t)(j / SK) & 1u, abort_flag)) { if (leader) gave_up(3, j); return false; }
         // plain: the scores of tile j - 1 must be in registers.  PT: buffer b last held S_{j-2} / P_{j-2}, whose P V product
         // was issued before this one, and the tensor core runs a CTA's products in issue order: nothing to wait for.
-        if (!PT && j >= 1 && !mbar_wait_or_abort(s_free, (uint32_t)(j - 1) & 1u, abort_flag)) { gave_up(4, j); return false; }
+        if (!PT && j >= 1 && !warp_wait_uniform(s_free, (uint32_t)(j - 1) & 1u, abort_flag)) { if (leader) gave_up(4, j); return false; }
         tc_fence_after();
         const uint32_t kt = k_base + s * C::kTileBytes;
 #pragma unroll
         for (int ks = 0; ks < KS; ++ks)
           tc_mma(tmem_base + 64u * b, smem_desc(q_base + (ks >> 2) * (kRowsU * 128) + (ks & 3) * 32),
-                 smem_desc(kt + (ks >> 2) * (kPosU * 128) + (ks & 3) * 32), C::kIdescS, ks > 0 ? 1u : 0u);
-        tc_commit(k_empty(s));                       // K_j may be overwritten
-        tc_commit(s_full(b));
+                 smem_desc(kt + (ks >> 2) * (kPosU * 128) + (ks & 3) * 32), C::kIdescS, ks > 0 ? 1u : 0u, leader);
+        tc_commit_if(k_empty(s), leader);                       // K_j may be overwritten
+        tc_commit_if(s_full(b), leader);
         return true;
       };
       if (NT > 0) ok = issue_s(0);
@@ -292,22 +292,22 @@ __global__ void __launch_bounds__(kThreadsU, UmmaCfg<HD, PT>::kCtasPerSm) attn_u
       for (int j = 0; j < NT && ok; ++j) {
         if (!PT && j + 1 < NT && !issue_s(j + 1)) { ok = false; break; }   // runs under the softmax of tile j
         const int b = PT ? (j & 1) : 0;
-        if (!mbar_wait_or_abort(p_full(b), (uint32_t)(PT ? (j >> 1) : j) & 1u, abort_flag)) { gave_up(5, j); ok = false; break; }
-        if (!mbar_wait_or_abort(v_full(j % SV), (uint32_t)(j / SV) & 1u, abort_flag)) { gave_up(6, j); ok = false; break; }
+        if (!warp_wait_uniform(p_full(b), (uint32_t)(PT ? (j >> 1) : j) & 1u, abort_flag)) { if (leader) gave_up(5, j); ok = false; break; }
+        if (!warp_wait_uniform(v_full(j % SV), (uint32_t)(j / SV) & 1u, abort_flag)) { if (leader) gave_up(6, j); ok = false; break; }
         tc_fence_after();
         const uint32_t vt = v_base + (j % SV) * C::kTileBytes;
 #pragma unroll
         for (int ks = 0; ks < kPosU / 16; ++ks) {
           const uint64_t dv = smem_desc_nmajor(vt + ks * (16 * 128), kPosU * 128);
           const uint32_t acc = (j > 0 || ks > 0) ? 1u : 0u;
-          if (PT) tc_mma_a_tmem(tmem_base + kColO, tmem_base + 64u * b + 8u * ks, dv, C::kIdescPV, acc);
-          else tc_mma(tmem_base + kColO, smem_desc(p_base + ks * 32), dv, C::kIdescPV, acc);
+          if (PT) tc_mma_a_tmem(tmem_base + kColO, tmem_base + 64u * b + 8u * ks, dv, C::kIdescPV, acc, leader);
+          else tc_mma(tmem_base + kColO, smem_desc(p_base + ks * 32), dv, C::kIdescPV, acc, leader);
         }
-        tc_commit(v_empty(j % SV));                  // V_j may be overwritten
-        tc_commit(pv_done(j));                       // O holds tiles 0..j (and, plain, P may be overwritten)
+        tc_commit_if(v_empty(j % SV), leader);                  // V_j may be overwritten
+        tc_commit_if(pv_done(j), leader);                       // O holds tiles 0..j (and, plain, P may be overwritten)
         if (PT && j + 2 < NT && !issue_s(j + 2)) { ok = false; break; }   // behind P_j V_j, into the buffer it has just read
       }
-      if (!ok) *abort_flag = 1;
+      if (!ok && leader) *abort_flag = 1;
     }
   } else {
     // ------------------------------------------------------------------ softmax, one thread per row

@@ -274,11 +274,6 @@ struct GemmArgs {
   int* status;           // device status word (bounded waits report here)
   GemmFuse f;            // zero-initialised unless a fused epilogue is asked for
   int M_expected;        // 0, or the row count the caller expects on the device (<= M): only shapes the tiling
-  // 0: the K range is accumulated in order.  2: products with N <= 1024 accumulate it in two interleaved partial sums
-  // (k-step k goes to sum k mod 2), added at the end, so that two MMA issuers can run the k-loop.  The two orders round
-  // differently: a caller that needs the same bits from launches of different sizes asks for the same value in all of
-  // them (the tiling itself never changes the result).
-  int chains;
   // Row class, or 0: the most rows that any launch of the caller's family may have (at most kSkinnyClassRows).  The product
   // may then run as the weight-streaming kernel (weights as the 128-row MMA operand, the rows as its N, the K range split
   // over the CTAs of a cluster), by a rule on (N, K), the class and the device only.  Its summation order differs from the

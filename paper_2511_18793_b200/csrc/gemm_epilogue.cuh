@@ -13,8 +13,12 @@ constexpr int kEpiWarps = 8;
 constexpr int kThreads = 64 + 32 * kEpiWarps;
 constexpr int kTransposeBytes = kEpiWarps * 32 * 32 * 4;   // per epilogue warp: a 32 x 32 fp32 block, chunks swizzled
 
-__device__ __forceinline__ void tc_commit(uint32_t bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+// (`leader`: see elect_one)
+__device__ __forceinline__ void tc_commit_if(uint32_t bar, uint32_t leader) {
+  asm volatile(
+      "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %1, 0;\n\t"
+      "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}"
+      ::"r"(bar), "r"(leader) : "memory");
 }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
@@ -35,30 +39,31 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t addr) {
   return (uint64_t)((addr >> 4) & 0x3FFF) | (1ull << 16) | (64ull << 32) | (1ull << 46) | (2ull << 61);
 }
 
-__device__ __forceinline__ void tc_mma(uint32_t tmem_d, uint64_t da, uint64_t db, uint32_t idesc, uint32_t accumulate) {
+__device__ __forceinline__ void tc_mma(uint32_t tmem_d, uint64_t da, uint64_t db, uint32_t idesc, uint32_t accumulate, uint32_t leader) {
   asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-      ::"r"(tmem_d), "l"(da), "l"(db), "r"(idesc), "r"(accumulate) : "memory");
+      "{\n\t.reg .pred p, q;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 q, %5, 0;\n\t"
+      "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+      ::"r"(tmem_d), "l"(da), "l"(db), "r"(idesc), "r"(accumulate), "r"(leader) : "memory");
 }
 
 // The four MMAs of one 64-deep k-step (K = 16 each) in one statement: the operands' descriptors advance by 32 bytes
-// (2 in the descriptor's 16-byte address units) per MMA; only the first may overwrite the accumulator.  One thread
-// issues every MMA of a CTA, so the instructions around each one are the floor of a short k-loop.
-__device__ __forceinline__ void tc_mma_kstep(uint32_t tmem_d, uint64_t da, uint64_t db, uint32_t idesc, uint32_t accumulate_first) {
+// (2 in the descriptor's 16-byte address units) per MMA; only the first may overwrite the accumulator.
+__device__ __forceinline__ void tc_mma_kstep(uint32_t tmem_d, uint64_t da, uint64_t db, uint32_t idesc, uint32_t accumulate_first,
+                                             uint32_t leader) {
   asm volatile(
-      "{\n\t.reg .pred p, t;\n\t.reg .b64 a1, b1, a2, b2, a3, b3;\n\t"
+      "{\n\t.reg .pred p, t, q;\n\t.reg .b64 a1, b1, a2, b2, a3, b3;\n\t"
       "setp.ne.b32 p, %4, 0;\n\t"
       "setp.eq.b32 t, %4, %4;\n\t"
+      "setp.ne.b32 q, %5, 0;\n\t"
       "add.s64 a1, %1, 2;\n\tadd.s64 b1, %2, 2;\n\t"
       "add.s64 a2, %1, 4;\n\tadd.s64 b2, %2, 4;\n\t"
       "add.s64 a3, %1, 6;\n\tadd.s64 b3, %2, 6;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], a1, b1, %3, t;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], a2, b2, %3, t;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], a3, b3, %3, t;\n\t}"
-      ::"r"(tmem_d), "l"(da), "l"(db), "r"(idesc), "r"(accumulate_first) : "memory");
+      "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t"
+      "@q tcgen05.mma.cta_group::1.kind::f16 [%0], a1, b1, %3, t;\n\t"
+      "@q tcgen05.mma.cta_group::1.kind::f16 [%0], a2, b2, %3, t;\n\t"
+      "@q tcgen05.mma.cta_group::1.kind::f16 [%0], a3, b3, %3, t;\n\t}"
+      ::"r"(tmem_d), "l"(da), "l"(db), "r"(idesc), "r"(accumulate_first), "r"(leader) : "memory");
 }
 
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float* v) {
@@ -256,9 +261,7 @@ __device__ __forceinline__ void epilogue_block(const GemmArgs& a, float4* stg4, 
 // One epilogue warp's share of a finished accumulator: TMEM lanes [32 q, 32 q + 32) (= rows m0 + 32 q ..) and the
 // 32-column groups half, half + 2, ... of the BN columns starting at TMEM column `tmem_acc`.  er = epilogue_row of
 // the lane's own row (lane = row while the block comes out of TMEM).
-// CHAINS > 1: the tile's K range was accumulated in that many partial accumulators, BN columns apart (one per MMA
-// issuer); they are added up here, in order, as the block leaves TMEM.
-template <int BN, int EPI, int CHAINS = 1>
+template <int BN, int EPI>
 __device__ __forceinline__ void drain_accumulator(const GemmArgs& a, uint32_t tmem_acc, int q, int half, int lane,
                                                   float4* stg4, int m0, int n0, int M, const EpiRow& er) {
   const int rows_here = min(32, M - (m0 + q * 32));          // rows of this quarter that exist (may be <= 0)
@@ -268,13 +271,6 @@ __device__ __forceinline__ void drain_accumulator(const GemmArgs& a, uint32_t tm
     if (n_chunk >= a.N) break;                               // ragged last tile (N is a multiple of 32)
     float v[32];
     tmem_ld32(tmem_acc + ((uint32_t)(q * 32) << 16) + (uint32_t)(c * 32), v);
-#pragma unroll
-    for (int ch = 1; ch < CHAINS; ++ch) {
-      float w[32];
-      tmem_ld32(tmem_acc + ((uint32_t)(q * 32) << 16) + (uint32_t)(ch * BN + c * 32), w);
-#pragma unroll
-      for (int j = 0; j < 32; ++j) v[j] += w[j];
-    }
     // transpose through shared memory: from lane = row (how TMEM hands the block out) to 8 lanes per row
 #pragma unroll
     for (int j = 0; j < 8; ++j)

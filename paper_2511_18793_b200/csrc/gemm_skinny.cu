@@ -153,49 +153,47 @@ __global__ void __launch_bounds__(kSkinnyThreads, 2)
     // nothing to do for this row tile
   } else if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer
-    if (lane == 0) {
-      bool ok = true;
-      int issued = pre;                          // k-steps whose `full` barrier has been armed
-      for (int s = 0; s < pre; ++s) {
-        if (blockIdx.y != 0) {
-          mbar_expect_tx(full_bar(s), C::kStageBytes);
-          tma_load_2d(base + s * C::kStageBytes, &tmW, (k_begin + s) * BK, n0, full_bar(s));
-        }
-        tma_load_2d(base + s * C::kStageBytes + C::kTileBytesW, &tmX, (k_begin + s) * BK, m0, full_bar(s));
+    const uint32_t leader = elect_one();
+    bool ok = true;
+    int issued = pre;                            // k-steps whose `full` barrier has been armed
+    for (int s = 0; s < pre; ++s) {
+      if (blockIdx.y != 0) {
+        mbar_expect_tx_if(full_bar(s), C::kStageBytes, leader);
+        tma_load_2d_if(base + s * C::kStageBytes, &tmW, (k_begin + s) * BK, n0, full_bar(s), leader);
       }
-      int s = 0;
-      uint32_t round = 1;                        // parity bit of the round that k-step `pre` belongs to (pre = STAGES here)
-      for (int k = pre; k < k_count; ++k, ++issued) {
-        if (!mbar_wait_or_abort(empty_bar(s), round ^ 1u, abort_flag)) { ok = false; break; }
-        const uint32_t fb = full_bar(s), dst = base + s * C::kStageBytes;
-        mbar_expect_tx(fb, C::kStageBytes);
-        tma_load_2d(dst, &tmW, (k_begin + k) * BK, n0, fb);
-        tma_load_2d(dst + C::kTileBytesW, &tmX, (k_begin + k) * BK, m0, fb);
-        if (++s == STAGES) { s = 0; round ^= 1u; }
-      }
-      if (!ok) {                                 // drain: wait (bounded) for the copies still in flight
-        *abort_flag = 1;
-        for (int j = max(0, issued - STAGES); j < issued; ++j) mbar_wait(full_bar(j % STAGES), (j / STAGES) & 1);
-      }
+      tma_load_2d_if(base + s * C::kStageBytes + C::kTileBytesW, &tmX, (k_begin + s) * BK, m0, full_bar(s), leader);
+    }
+    int s = 0;
+    uint32_t round = 1;                          // parity bit of the round that k-step `pre` belongs to (pre = STAGES here)
+    for (int k = pre; k < k_count; ++k, ++issued) {
+      if (!warp_wait_uniform(empty_bar(s), round ^ 1u, abort_flag)) { ok = false; break; }
+      const uint32_t fb = full_bar(s), dst = base + s * C::kStageBytes;
+      mbar_expect_tx_if(fb, C::kStageBytes, leader);
+      tma_load_2d_if(dst, &tmW, (k_begin + k) * BK, n0, fb, leader);
+      tma_load_2d_if(dst + C::kTileBytesW, &tmX, (k_begin + k) * BK, m0, fb, leader);
+      if (++s == STAGES) { s = 0; round ^= 1u; }
+    }
+    if (!ok && lane == 0) {                      // drain: wait (bounded) for the copies still in flight
+      *abort_flag = 1;
+      for (int j = max(0, issued - STAGES); j < issued; ++j) mbar_wait(full_bar(j % STAGES), (j / STAGES) & 1);
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer
-    if (lane == 0) {
-      bool ok = true;
-      const uint64_t dw0 = smem_desc(base), dx0 = smem_desc(base + C::kTileBytesW);
-      int s = 0;
-      uint32_t round = 0;
-      for (int k = 0; k < k_count; ++k) {
-        if (!mbar_wait_or_abort(full_bar(s), round, abort_flag)) { ok = false; break; }
-        tc_fence_after();
-        const uint64_t so = (uint64_t)(s * (C::kStageBytes >> 4));
-        tc_mma_kstep(tmem_base, dw0 + so, dx0 + so, C::kInstrDesc, k > 0 ? 1u : 0u);
-        tc_commit(empty_bar(s));
-        if (++s == STAGES) { s = 0; round ^= 1u; }
-      }
-      if (ok) tc_commit(acc_full);
-      else *abort_flag = 1;
+    const uint32_t leader = elect_one();
+    bool ok = true;
+    const uint64_t dw0 = smem_desc(base), dx0 = smem_desc(base + C::kTileBytesW);
+    int s = 0;
+    uint32_t round = 0;
+    for (int k = 0; k < k_count; ++k) {
+      if (!warp_wait_uniform(full_bar(s), round, abort_flag)) { ok = false; break; }
+      tc_fence_after();
+      const uint64_t so = (uint64_t)(s * (C::kStageBytes >> 4));
+      tc_mma_kstep(tmem_base, dw0 + so, dx0 + so, C::kInstrDesc, k > 0 ? 1u : 0u, leader);
+      tc_commit_if(empty_bar(s), leader);
+      if (++s == STAGES) { s = 0; round ^= 1u; }
     }
+    if (ok) tc_commit_if(acc_full, leader);
+    else if (leader) *abort_flag = 1;
   } else {
     // ------------------------------------------------------------------ epilogue, first half: the accumulator into shared memory
     // (under the main loop: the rows' norm scales, 8 lanes per row, each lane every eighth partial sum)
@@ -336,8 +334,7 @@ int gemm_skinny_splits(int N, int K, int row_class, int n_sm) {
 
 // Up to 128 rows every product is bound by reading W, and this kernel keeps more of it in flight.  With more rows W is
 // shared by several row tiles and the general kernel's wider tiles win again -- except where its k-loop is the bound: one
-// CTA walks all of K at 0.29 us per k-step (0.17 with two issuers, N <= 1024), however few tiles there are, while here K is
-// split.  Measured at 256 / 512 rows, general -> this kernel: 2048 x 8192 41 -> 17 / 41 -> 34 us, 1536 x 8960 45 -> 17 /
+// CTA walks all of K at 0.1 to 0.2 us per k-step, however few tiles there are, while here K is split.  Measured at 256 / 512 rows, general -> this kernel: 2048 x 8192 41 -> 17 / 41 -> 34 us, 1536 x 8960 45 -> 17 /
 // 46 -> 31, 896 x 4864 17 -> 10 / 18 -> 13; but 16384 x 2048 21 -> 37 / 33 -> 66, 6144 x 4096 25 -> 36.
 bool gemm_skinny_applies(const GemmArgs& a, int n_sm) {
   if (!a.skinny || a.M > a.skinny || a.skinny > kSkinnyClassRows) return false;
@@ -346,7 +343,7 @@ bool gemm_skinny_applies(const GemmArgs& a, int n_sm) {
   const int s = gemm_skinny_splits(a.N, a.K, a.skinny, n_sm);
   const int waves = (tiles * s + 2 * n_sm - 1) / (2 * n_sm), k_cta = (k_iters + s - 1) / s;
   const double here = waves * (7.0 + 0.75 * k_cta);
-  const double there = 4.0 + (a.chains == 2 && a.N <= 1024 ? 0.17 : 0.29) * k_iters;      // (its least: one wave of tiles)
+  const double there = 4.0 + 0.16 * k_iters;      // (its least: one wave of tiles)
   return here < 0.9 * there;
 }
 

@@ -34,32 +34,37 @@ __device__ __forceinline__ void cluster_sync_all() {
   asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
-// A copy of this CTA into its own shared memory whose completion is counted by the LEADER's barrier.
-__device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap* tm, int x, int y, uint32_t leader_bar) {
+// A copy of this CTA into its own shared memory whose completion is counted by the LEADER CTA's barrier (`leader`: the
+// elected lane, see elect_one).
+__device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap* tm, int x, int y, uint32_t leader_bar, uint32_t leader) {
   asm volatile(
-      "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
-      ::"r"(dst), "l"(tm), "r"(x), "r"(y), "r"(leader_bar) : "memory");
+      "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %5, 0;\n\t"
+      "@q cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];\n\t}"
+      ::"r"(dst), "l"(tm), "r"(x), "r"(y), "r"(leader_bar), "r"(leader) : "memory");
 }
 // The four MMAs (K = 16 each) of one 64-deep k-step over the pair, in one statement (see tc_mma_kstep).
-__device__ __forceinline__ void tc_mma_pair_kstep(uint32_t tmem_d, uint64_t da, uint64_t db, uint32_t accumulate_first) {
+__device__ __forceinline__ void tc_mma_pair_kstep(uint32_t tmem_d, uint64_t da, uint64_t db, uint32_t accumulate_first, uint32_t leader) {
   asm volatile(
-      "{\n\t.reg .pred p, t;\n\t.reg .b64 a1, b1, a2, b2, a3, b3;\n\t"
+      "{\n\t.reg .pred p, t, q;\n\t.reg .b64 a1, b1, a2, b2, a3, b3;\n\t"
       "setp.ne.b32 p, %4, 0;\n\t"
       "setp.eq.b32 t, %4, %4;\n\t"
+      "setp.ne.b32 q, %5, 0;\n\t"
       "add.s64 a1, %1, 2;\n\tadd.s64 b1, %2, 2;\n\t"
       "add.s64 a2, %1, 4;\n\tadd.s64 b2, %2, 4;\n\t"
       "add.s64 a3, %1, 6;\n\tadd.s64 b3, %2, 6;\n\t"
-      "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t"
-      "tcgen05.mma.cta_group::2.kind::f16 [%0], a1, b1, %3, t;\n\t"
-      "tcgen05.mma.cta_group::2.kind::f16 [%0], a2, b2, %3, t;\n\t"
-      "tcgen05.mma.cta_group::2.kind::f16 [%0], a3, b3, %3, t;\n\t}"
-      ::"r"(tmem_d), "l"(da), "l"(db), "r"(kInstrDesc2), "r"(accumulate_first) : "memory");
+      "@q tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t"
+      "@q tcgen05.mma.cta_group::2.kind::f16 [%0], a1, b1, %3, t;\n\t"
+      "@q tcgen05.mma.cta_group::2.kind::f16 [%0], a2, b2, %3, t;\n\t"
+      "@q tcgen05.mma.cta_group::2.kind::f16 [%0], a3, b3, %3, t;\n\t}"
+      ::"r"(tmem_d), "l"(da), "l"(db), "r"(kInstrDesc2), "r"(accumulate_first), "r"(leader) : "memory");
 }
 // Arrives (once the MMAs issued so far have completed) on the barrier at this offset in BOTH CTAs of the pair.
-__device__ __forceinline__ void tc_commit_pair(uint32_t bar) {
+__device__ __forceinline__ void tc_commit_pair(uint32_t bar, uint32_t leader) {
   const uint16_t both = 3;
-  asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
-               ::"r"(bar), "h"(both) : "memory");
+  asm volatile(
+      "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %2, 0;\n\t"
+      "@q tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;\n\t}"
+      ::"r"(bar), "h"(both), "r"(leader) : "memory");
 }
 __device__ __forceinline__ void mbar_arrive_leader(uint32_t bar) {
   asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar & kLeaderMask) : "memory");
@@ -119,49 +124,49 @@ __global__ void __launch_bounds__(kThreads) gemm_tc_pair_kernel(const __grid_con
 
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer (both CTAs)
-    if (lane == 0) {
-      int s = 0;
-      uint32_t round = 0;
-      bool ok = true;
-      for (int tile = pair; tile < n_tiles && ok; tile += n_pairs) {
-        const TileMN tt = tile_of(tile, tiles_m, tiles_n, band);
-        const int m0 = tt.m * (2 * BM) + rank * BM;                      // this CTA's rows
-        const int nb0 = tt.n * kBN2 + rank * (kBN2 / 2);                 // this CTA's half of the W tile
-        for (int k = 0; k < k_iters; ++k) {
-          // (round 0 never waits: the parity before a fresh barrier's first one counts as complete)
-          if (!mbar_wait_or_abort(empty_bar(s), round ^ 1u, abort_flag)) { ok = false; break; }
-          const uint32_t dst = base + s * kStageBytes2, fb = full_bar(s) & kLeaderMask;
-          if (rank == 0) mbar_expect_tx(full_bar(s), 2 * kStageBytes2);  // the bytes of both CTAs' copies
-          tma_load_2d_pair(dst, &tmA, k * BK, m0, fb);
-          tma_load_2d_pair(dst + kTileBytesA, &tmB, k * BK, nb0, fb);
-          if (++s == STAGES) { s = 0; round ^= 1u; }
-        }
+    const uint32_t leader = elect_one();
+    int s = 0;
+    uint32_t round = 0;
+    bool ok = true;
+    for (int tile = pair; tile < n_tiles && ok; tile += n_pairs) {
+      const TileMN tt = tile_of(tile, tiles_m, tiles_n, band);
+      const int m0 = tt.m * (2 * BM) + rank * BM;                      // this CTA's rows
+      const int nb0 = tt.n * kBN2 + rank * (kBN2 / 2);                 // this CTA's half of the W tile
+      for (int k = 0; k < k_iters; ++k) {
+        // (round 0 never waits: the parity before a fresh barrier's first one counts as complete)
+        if (!warp_wait_uniform(empty_bar(s), round ^ 1u, abort_flag)) { ok = false; break; }
+        const uint32_t dst = base + s * kStageBytes2, fb = full_bar(s) & kLeaderMask;
+        mbar_expect_tx_if(full_bar(s), 2 * kStageBytes2, rank == 0 ? leader : 0u);   // the bytes of both CTAs' copies
+        tma_load_2d_pair(dst, &tmA, k * BK, m0, fb, leader);
+        tma_load_2d_pair(dst + kTileBytesA, &tmB, k * BK, nb0, fb, leader);
+        if (++s == STAGES) { s = 0; round ^= 1u; }
       }
-      if (!ok) *abort_flag = 1;
     }
+    if (!ok && lane == 0) *abort_flag = 1;
   } else if (warp == 1) {
-    // ------------------------------------------------------------------ MMA issuer (leader only)
-    if (lane == 0 && rank == 0) {
+    // ------------------------------------------------------------------ MMA issuer (leader CTA only)
+    if (rank == 0) {
+      const uint32_t leader = elect_one();
       int t_local = 0, s = 0;
       uint32_t round = 0;
       bool ok = true;
       const uint64_t da0 = smem_desc(base), db0 = smem_desc(base + kTileBytesA);   // slot 0; later slots add to the address field
       for (int tile = pair; tile < n_tiles && ok; tile += n_pairs, ++t_local) {
         const int b = t_local & 1;
-        if (t_local >= 2 && !mbar_wait_or_abort(acc_empty(b), ((t_local >> 1) - 1) & 1, abort_flag)) { ok = false; break; }
+        if (t_local >= 2 && !warp_wait_uniform(acc_empty(b), ((t_local >> 1) - 1) & 1, abort_flag)) { ok = false; break; }
         tc_fence_after();
         const uint32_t tmem_acc = tmem_base + (uint32_t)(b * kBN2);
         for (int k = 0; k < k_iters; ++k) {
-          if (!mbar_wait_or_abort(full_bar(s), round, abort_flag)) { ok = false; break; }
+          if (!warp_wait_uniform(full_bar(s), round, abort_flag)) { ok = false; break; }
           tc_fence_after();
           const uint64_t so = (uint64_t)(s * (kStageBytes2 >> 4));
-          tc_mma_pair_kstep(tmem_acc, da0 + so, db0 + so, k > 0 ? 1u : 0u);
-          tc_commit_pair(empty_bar(s));          // slot free in both CTAs once these MMAs have read it
+          tc_mma_pair_kstep(tmem_acc, da0 + so, db0 + so, k > 0 ? 1u : 0u, leader);
+          tc_commit_pair(empty_bar(s), leader);  // slot free in both CTAs once these MMAs have read it
           if (++s == STAGES) { s = 0; round ^= 1u; }
         }
-        if (ok) tc_commit_pair(acc_full(b));     // accumulator complete, in both CTAs
+        if (ok) tc_commit_pair(acc_full(b), leader);     // accumulator complete, in both CTAs
       }
-      if (!ok) *abort_flag = 1;
+      if (!ok && lane == 0) *abort_flag = 1;
     }
   } else {
     // ------------------------------------------------------------------ epilogue (warps 2..9, both CTAs)
@@ -210,10 +215,12 @@ void launch_pair(const GemmArgs& a, int n_sm, cudaStream_t st) {
   const int pairs = (int)(tiles < n_sm / 2 ? tiles : n_sm / 2);
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(2 * pairs); cfg.blockDim = dim3(kThreads); cfg.dynamicSmemBytes = kSmemBytes2; cfg.stream = st;
-  cudaLaunchAttribute at[1];
+  cudaLaunchAttribute at[2];
   at[0].id = cudaLaunchAttributeClusterDimension;
   at[0].val.clusterDim.x = 2; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
-  cfg.attrs = at; cfg.numAttrs = 1;
+  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at; cfg.numAttrs = pdl_enabled() ? 2 : 1;
   cudaLaunchKernelEx(&cfg, gemm_tc_pair_kernel<EPI>, ta, tb, a, a.status);
 }
 

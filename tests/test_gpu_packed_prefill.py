@@ -12,7 +12,7 @@ pytestmark = pytest.mark.gpu
                                                 ("bf16", 100, 50),      # two chunks, the tensor-core kernels
                                                 ("bf16", 3, 300)])      # more than one tile of positions per request
 def test_packed_prefill_equals_one_request_at_a_time(dtype, batch, n_hist):
-    from gpu_helpers import Case
+    from gpu_helpers import Case, hidden_tolerance
     base = synth.WORKLOADS["tiny" if dtype == "fp32" else "small"]
     w = synth.scaled(base, n_layers=2, n_items=5_000, batch=batch, n_hist=n_hist)
     case = Case(w)
@@ -25,6 +25,10 @@ def test_packed_prefill_equals_one_request_at_a_time(dtype, batch, n_hist):
     together = case.eng.get_hidden().clone()
     for b in sorted({0, 1, 2, batch // 2, batch - 2, batch - 1}):
         case.eng.prefill(case.hist_dev[b:b + 1], n[b:b + 1])
-        # the same sums in the same order whatever the other rows of a pass are: the same bits
-        assert torch.equal(together[b], case.eng.get_hidden()[0]), b
+        alone = case.eng.get_hidden()[0]
+        if dtype == "fp32":      # the same sums in the same order whatever the other rows of a pass are: the same bits
+            assert torch.equal(together[b], alone), b
+        else:                    # the attention's kernel goes by the number of requests, and another order of its sums flips bf16
+            # roundings downstream: two results, each within the bf16 rounding model's bound of the exact one
+            assert (together[b] - alone).abs().max().item() < 2 * hidden_tolerance(w), b
     case.eng.close()
