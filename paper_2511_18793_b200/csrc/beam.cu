@@ -103,8 +103,19 @@ __device__ __forceinline__ unsigned probe_extensions(unsigned long long* slots, 
 // mask from the prefix map, cost 1.4 % (16 layers, one request) to 3 % (4 layers, 64 requests) of a whole decode.
 inline bool select_probes(const SelectArgs& a) { return a.filter && a.per_beam >= a.T && !a.prefix_filter && !a.final_mask_from_map; }
 
+// What a fused kernel goes on with: the selection as it stands in shared memory (score, parent slot, code).
+struct Selected { bool active; int n; const float* s; const int* r; const int* t; };
+// 4 bytes of global memory into shared memory without passing through a register.
+__device__ __forceinline__ void cp_async4(int* dst, const int* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_ints(int* dst, const int* src, int n) {
+  for (int i = threadIdx.x; i < n; i += blockDim.x) cp_async4(dst + i, src + i);
+}
+
+// s_codes: the input beams' codes in shared memory ([in_stride][tuple_len], brought by cp.async of all threads), or null.
 template <int VPL, bool PROBE>
-__device__ __forceinline__ void select_body(const SelectArgs& a) {
+__device__ __forceinline__ Selected select_body(const SelectArgs& a, const int* s_codes = nullptr) {
   const int b = blockIdx.x;
   extern __shared__ unsigned char smem_raw[];
   const int nb_cap = a.in_stride;
@@ -136,8 +147,8 @@ __device__ __forceinline__ void select_body(const SelectArgs& a) {
     bias[j] = (a.logit_bias && t < a.T) ? a.logit_bias[(long long)b * a.bias_stride + t] : 0.f;
     z0[j] = (direct0 && t < a.T) ? a.logits[row0 * a.row_stride + a.col_off + t] : 0.f;
   }
-  if (a.gate_mode == 1 && gate_v != a.gate_value) return;
-  if (a.gate_mode == 2 && !(gate_v < a.gate_value)) return;
+  if (a.gate_mode == 1 && gate_v != a.gate_value) return Selected{false, 0, sel_s, sel_r, sel_t};
+  if (a.gate_mode == 2 && !(gate_v < a.gate_value)) return Selected{false, 0, sel_s, sel_r, sel_t};
   const int nb = min(nb_raw, nb_cap);
   const bool all_codes = a.per_beam >= a.T;
   const int want = all_codes ? min(a.K, a.T) : min(a.per_beam, a.K);
@@ -340,6 +351,7 @@ __device__ __forceinline__ void select_body(const SelectArgs& a) {
     }
     if (lane == 0) *s_nout = n_out;
   }
+  if (s_codes) asm volatile("cp.async.wait_all;" ::: "memory");
   __syncthreads();
 
   // ---- stage 3: the output beams, all threads
@@ -356,7 +368,7 @@ __device__ __forceinline__ void select_body(const SelectArgs& a) {
       const int k = i / a.tuple_len, l = i - k * a.tuple_len;
       int c = -1;
       if (k < n_out) {
-        if (l < a.n) c = a.in_codes[((long long)b * a.in_stride + sel_r[k]) * a.tuple_len + l];
+        if (l < a.n) c = s_codes ? s_codes[sel_r[k] * a.tuple_len + l] : a.in_codes[((long long)b * a.in_stride + sel_r[k]) * a.tuple_len + l];
         else if (l == a.n) c = sel_t[k];
       }
       a.out_codes[((long long)b * a.out_stride + k) * a.tuple_len + l] = c;
@@ -367,6 +379,7 @@ __device__ __forceinline__ void select_body(const SelectArgs& a) {
     a.host_status[threadIdx.x] = *(volatile int*)(a.status + threadIdx.x);
     __threadfence_system();
   }
+  return Selected{true, n_out, sel_s, sel_r, sel_t};
 }
 
 // Codes per lane of a codebook of T codes, as a constant.
@@ -388,10 +401,11 @@ __global__ void __launch_bounds__(select_max_threads(VPL)) select_kernel(SelectA
 }  // namespace
 
 cudaError_t select_step_configure(int bytes);
+size_t advance_smem_bytes(int Kmax, int L);
 
 size_t select_smem_bytes(int in_stride, int K) {
-  return (size_t)in_stride * K * (sizeof(float) + sizeof(int)) + (size_t)in_stride * sizeof(int) +
-         (size_t)K * (sizeof(float) + 2 * sizeof(int)) + sizeof(int);
+  return ((size_t)in_stride * K * (sizeof(float) + sizeof(int)) + (size_t)in_stride * sizeof(int) +
+          (size_t)K * (sizeof(float) + 2 * sizeof(int)) + sizeof(int) + 15) / 16 * 16;
 }
 
 // The attribute belongs to the device, and several contexts may share one: it is only ever raised.
@@ -399,7 +413,7 @@ cudaError_t select_configure(int max_beam) {
   static int configured_bytes[64] = {};
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) dev = 0;
-  int bytes = (int)select_smem_bytes(max_beam, max_beam);
+  int bytes = (int)(select_smem_bytes(max_beam, max_beam) + advance_smem_bytes(max_beam, kMaxLevels));
   if (bytes <= configured_bytes[dev]) return cudaSuccess;
   configured_bytes[dev] = bytes;
   cudaError_t e = cudaSuccess;
@@ -669,10 +683,22 @@ __global__ void draft_state_init_kernel(EngineState e, int batch, __nv_bfloat16*
 // Eq. 3 after the product: s_{l+1}[k] = tanh((W_s s_l)[parent] + (W_e E)[code] + b).  G holds [logits | W_s s_l] of
 // every beam slot of level l (W_s s_l from column t_cols on), U = W_e E for every code token.  Which (parent, code) a
 // slot takes is decided exactly as in trans_gather_kernel.
+__device__ __forceinline__ void draft_state(const EngineState& e, int b, int k, int l, int parent, int code, const float* __restrict__ G,
+                                            long long g_stride, int t_cols, const float* __restrict__ U,
+                                            const float* __restrict__ bias, __nv_bfloat16* s_act, int tid, int n_thr) {
+  __nv_bfloat16* dst = s_act + ((long long)b * e.Kmax + k) * e.d;
+  if (parent < 0 || code < 0) {                    // no such beam
+    for (int c = tid; c < e.d; c += n_thr) dst[c] = __float2bfloat16_rn(0.f);
+    return;
+  }
+  const float* z = G + ((long long)b * e.Kmax + parent) * g_stride + t_cols;
+  const float* u = U + (long long)(e.li.off[l - 1] + code) * e.d;
+#pragma unroll 4
+  for (int c = tid; c < e.d; c += n_thr) dst[c] = __float2bfloat16_rn(tanhf(z[c] + u[c] + bias[c]));
+}
 __device__ __forceinline__ void draft_step_slot(const EngineState& e, int b, int k, int l, const float* __restrict__ G,
                                                 long long g_stride, int t_cols, const float* __restrict__ U,
                                                 const float* __restrict__ bias, __nv_bfloat16* s_act, int tid, int n_thr) {
-  __nv_bfloat16* dst = s_act + ((long long)b * e.Kmax + k) * e.d;
   const int dm = e.d_m[b];
   int src_level, parent;
   bool live = dm < e.L || e.row_m[b] < e.L;
@@ -682,14 +708,7 @@ __device__ __forceinline__ void draft_step_slot(const EngineState& e, int b, int
   live = live && k < e.dw_count[src_level * e.Bmax + b];
   if (live && parent == -2) parent = e.dw_parent[s_idx];
   const int code = live ? e.dw_codes[s_idx * e.L + (l - 1)] : -1;
-  live = live && code >= 0 && parent >= 0;
-  if (!live) {
-    for (int c = tid; c < e.d; c += n_thr) dst[c] = __float2bfloat16_rn(0.f);
-    return;
-  }
-  const float* z = G + ((long long)b * e.Kmax + parent) * g_stride + t_cols;
-  const float* u = U + (long long)(e.li.off[l - 1] + code) * e.d;
-  for (int c = tid; c < e.d; c += n_thr) dst[c] = __float2bfloat16_rn(tanhf(z[c] + u[c] + bias[c]));
+  draft_state(e, b, k, l, live ? parent : -1, code, G, g_stride, t_cols, U, bias, s_act, tid, n_thr);
 }
 __global__ void draft_step_kernel(EngineState e, int batch, int l, const float* __restrict__ G, long long g_stride, int t_cols,
                                   const float* __restrict__ U, const float* __restrict__ bias, __nv_bfloat16* s_act) {
@@ -708,10 +727,15 @@ __global__ void __launch_bounds__(select_max_threads(VPL)) select_step_kernel(Se
                                                           const float* __restrict__ bias, __nv_bfloat16* s_act) {
   pdl_wait();
   pdl_launch();
-  select_body<VPL, false>(a);                      // (an earlier level than the last: nothing to probe)
-  __syncthreads();                                 // the block's own selection (global writes) is visible to all its threads
-  for (int k = threadIdx.x >> 5; k < e.Kmax; k += blockDim.x >> 5)          // a warp per beam slot
-    draft_step_slot(e, blockIdx.x, k, l, G, g_stride, t_cols, U, bias, s_act, threadIdx.x & 31, 32);
+  const Selected sel = select_body<VPL, false>(a);   // (an earlier level than the last: nothing to probe)
+  const int warp = threadIdx.x >> 5, n_warps = blockDim.x >> 5, lane = threadIdx.x & 31;    // a warp per beam slot
+  if (sel.active) {                                // (whose selection is still in shared memory: nothing to read back)
+    for (int k = warp; k < e.Kmax; k += n_warps)
+      draft_state(e, blockIdx.x, k, l, k < sel.n ? sel.r[k] : -1, k < sel.n ? sel.t[k] : -1, G, g_stride, t_cols, U, bias, s_act, lane, 32);
+    return;
+  }
+  for (int k = warp; k < e.Kmax; k += n_warps)
+    draft_step_slot(e, blockIdx.x, k, l, G, g_stride, t_cols, U, bias, s_act, lane, 32);
 }
 
 // dst[b, r, :] = src[(b * row_mul + r), 0 : T] + bias[b, :]
@@ -888,79 +912,87 @@ __global__ void nodes_from_prefixes_kernel(EngineState e, int batch, int n_beams
 // ----------------------------------------------------------------------------------------------------
 // accept / roll back (Algorithm 2's rejection and update steps)
 // ----------------------------------------------------------------------------------------------------
-// After B_{n+1} has been selected for a request whose beams B_n had logits in this pass:
+// The fused kernel reads all it may need about its request at its start, under the selection, into shared memory: each
+// dependent read behind the selection would be an L2 round trip of 0.6 us in a kernel of 13 (and there were up to 14).
+struct AdvanceSmem {
+  unsigned long long* key;       // [L][Kmax] keys of the alive nodes of level n + 1 (row 0), then of the beams of levels 1..L
+  int* codes;                    // [Kmax][L] tb_codes of level n
+  int* node;                     // [Kmax][L] dw_codes of level n + 1
+  int *dbeam, *nidx, *self;      // [Kmax]    d_beam and node_index of level n + 1, tb_self of level n
+  int* anc;                      // [Kmax][L] tb_anc of level n
+  int* beams;                    // [L][Kmax][L] tb_codes of levels 1..L (the round's end only)
+};
+__device__ __forceinline__ AdvanceSmem advance_smem(unsigned char* base, int Kmax, int L) {
+  AdvanceSmem m;
+  m.key = reinterpret_cast<unsigned long long*>(base);
+  m.codes = reinterpret_cast<int*>(m.key + (size_t)L * Kmax);
+  m.node = m.codes + Kmax * L; m.anc = m.node + Kmax * L;
+  m.dbeam = m.anc + Kmax * L; m.nidx = m.dbeam + Kmax; m.self = m.nidx + Kmax;
+  m.beams = m.self + Kmax;
+  return m;
+}
+
+// After B_{n+1} has been selected for a request whose beams B_n had logits in this pass (sel.active):
 //   n + 1 == L : the request is finished; B_L is the result.
 //   otherwise  : every beam of B_{n+1} inherits its parent's KV slots (a slot-table rewrite: rejected drafts'
 //                KV rows simply become unreachable) and is matched against the alive nodes of level n+1 of the draft
 //                tree.  If every beam is such a node, its hidden state is already in the pass and selection goes on;
 //                else level n+1 is the rejection level and the request waits for the next round.
-__device__ __forceinline__ void advance_body(const EngineState& e, int n, int K, int* out_codes, float* out_score, int* out_count) {
-  const int b = blockIdx.x;
-  if (e.row_cur[b] != n) return;
-  const int L = e.L, Kmax = e.Kmax;
-  const int n1 = n + 1;
-  const int cnt = e.tb_count[n1 * e.Bmax + b];
+// nd: nodes of level n + 1.
+__device__ __forceinline__ void advance_body(const EngineState& e, const AdvanceSmem& sm, const Selected& sel, int n, int K, int nd,
+                                             int* out_codes, float* out_score, int* out_count) {
+  const int b = blockIdx.x, L = e.L, Kmax = e.Kmax, n1 = n + 1, cnt = sel.n;
   if (n1 == L) {
-    for (int k = threadIdx.x; k < K; k += blockDim.x) {
-      const long long s = lvl_bk(e, L, b, k);
-      out_score[(long long)b * K + k] = k < cnt ? e.tb_score[s] : -INFINITY;
-      for (int l = 0; l < L; ++l) out_codes[((long long)b * K + k) * L + l] = k < cnt ? e.tb_codes[s * L + l] : -1;
+    for (int k = threadIdx.x; k < K; k += blockDim.x) out_score[(long long)b * K + k] = k < cnt ? sel.s[k] : -INFINITY;
+    for (int i = threadIdx.x; i < K * L; i += blockDim.x) {
+      const int k = i / L, l = i - k * L;
+      out_codes[(long long)b * K * L + i] = k >= cnt ? -1 : l < n ? sm.codes[sel.r[k] * L + l] : sel.t[k];
     }
     if (threadIdx.x == 0) { out_count[b] = cnt; e.row_m[b] = L; e.row_cur[b] = -1; }
     return;
   }
   __shared__ int all_matched;
-  __shared__ unsigned long long s_node[128];       // keys of the alive nodes of level n + 1 (a dead one: no key)
   if (threadIdx.x == 0) all_matched = 1;
-  const int nd = min(e.dw_count[(long long)n1 * e.Bmax + b], Kmax);
-  for (int k = threadIdx.x; k < nd; k += blockDim.x) {
-    const long long s = lvl_bk(e, n1, b, k);
-    s_node[k] = e.d_beam[s] < 0 ? kEmptyKey : prefix_key_of(e, e.dw_codes + s * L, n1);
-  }
+  for (int k = threadIdx.x; k < nd; k += blockDim.x)           // (a dead node: no key)
+    sm.key[k] = sm.dbeam[k] < 0 ? kEmptyKey : prefix_key_of(e, sm.node + k * L, n1);
   __syncthreads();
   for (int r = threadIdx.x; r < cnt; r += blockDim.x) {
     const long long bi = lvl_bk(e, n1, b, r);
-    const int parent = e.tb_parent[bi];
-    const long long pi = lvl_bk(e, n, b, parent);
-    for (int i = 0; i + 1 < n; ++i) e.tb_anc[bi * L + i] = e.tb_anc[pi * L + i];
-    if (n >= 1) e.tb_anc[bi * L + (n - 1)] = e.tb_self[pi];
-    const unsigned long long key = prefix_key_of(e, e.tb_codes + bi * L, n1);
+    const int parent = sel.r[r];
+    for (int i = 0; i + 1 < n; ++i) e.tb_anc[bi * L + i] = sm.anc[parent * L + i];
+    if (n >= 1) e.tb_anc[bi * L + (n - 1)] = sm.self[parent];
+    const unsigned long long key = prefix_key_of(e, sm.codes + parent * L, n) + (unsigned long long)sel.t[r] * e.li.mult[n];
     int match = -1;
     for (int k = nd - 1; k >= 0; --k)
-      if (s_node[k] == key) match = k;
-    if (match >= 0) {
-      e.tb_src[bi] = e.node_index[((long long)b * L + n1) * Kmax + match];
-      e.tb_self[bi] = match;
-    } else {
-      e.tb_src[bi] = -1;
-      e.tb_self[bi] = -1;
-      all_matched = 0;
-    }
+      if (sm.key[k] == key) match = k;
+    e.tb_src[bi] = match >= 0 ? sm.nidx[match] : -1;
+    e.tb_self[bi] = match;
+    if (match < 0) all_matched = 0;
   }
   __syncthreads();
   if (threadIdx.x == 0) {
-    e.row_m[b] = n1;
+    e.row_m[b] = cnt == 0 ? L : n1;                // (no beam survived -- possible only with an empty codebook: finish empty)
     e.row_cur[b] = (all_matched && cnt > 0) ? n1 : -1;
-    if (cnt == 0) {               // no beam survived (possible only with an empty codebook): finish empty
-      e.row_m[b] = L;
-      out_count[b] = 0;
-    }
+    if (cnt == 0) out_count[b] = 0;
   }
 }
+
 // End of a round: accepted length of every draft = the largest i <= (level reached) with D[k][0..i) in B_i;
 // trace outputs; counters for the host (unfinished requests, primary tokens, accepted levels), which the last block to get
 // here writes to the host's pinned memory together with the status word (a copy node behind every round costs 10 us).
 // adaptive: a request whose round settled only the one level that the pass settles anyway gained nothing from its drafts
 // and stops drafting (its remaining rounds are plain autoregressive steps).
-__device__ __forceinline__ void round_end_body(const EngineState& e, int K, const RoundEnd& re) {
+// What the block read about its request at the start of the kernel:
+struct RowState { int m, m_start, spec, tokens, nd_last; };    // nd_last: drafted tuples (nodes of level L)
+__device__ __forceinline__ void round_end_body(const EngineState& e, const AdvanceSmem& sm, const Selected& sel, const RowState& rs, int K,
+                                               const RoundEnd& re) {
   const int b = blockIdx.x, batch = gridDim.x, round = re.round;
   const int L = e.L, Kmax = e.Kmax;
   const nezha_trace& tr = re.tr;
   __shared__ int acc_sum;
-  __shared__ unsigned long long s_beam[128];
-  const int took_part = e.row_tok_count[b] > 0;
-  const int m_now = e.row_m[b];
-  const int nd = took_part ? e.dw_count[(long long)L * e.Bmax + b] : 0;
+  const int took_part = rs.tokens > 0;
+  const int m_now = sel.active ? L : rs.m;         // (behind the last level an active request is finished)
+  const int nd = took_part ? rs.nd_last : 0;
   const long long tro = ((long long)(round - 1) * batch + b);
   if (threadIdx.x == 0) acc_sum = 0;
   // thread k answers for drafted tuple k (K <= 128 <= threads)
@@ -968,17 +1000,20 @@ __device__ __forceinline__ void round_end_body(const EngineState& e, int K, cons
   const bool mine = k < K && k < nd;
   int acc = mine ? 0 : -1;
   if (nd > 0) {
-    const int* dc = e.dw_codes + lvl_bk(e, L, b, mine ? k : 0) * L;
+    for (int i = threadIdx.x; i < m_now * Kmax; i += blockDim.x) {
+      const int lv = i / Kmax, r = i - lv * Kmax;  // beams of level lv + 1 (beyond their count -- at most K -- the codes are -1)
+      unsigned long long key;
+      if (sel.active && lv == L - 1)
+        key = r < sel.n ? prefix_key_of(e, sm.codes + sel.r[r] * L, L - 1) + (unsigned long long)sel.t[r] * e.li.mult[L - 1] : kEmptyKey;
+      else key = r < K && sm.beams[(lv * Kmax + r) * L] >= 0 ? prefix_key_of(e, sm.beams + (lv * Kmax + r) * L, lv + 1) : kEmptyKey;
+      sm.key[i] = key;
+    }
+    __syncthreads();
     unsigned long long key = 0;
-    for (int i = 1; i <= m_now; ++i) {
-      const int nbi = e.tb_count[i * e.Bmax + b];
-      __syncthreads();
-      if (k < nbi) s_beam[k] = prefix_key_of(e, e.tb_codes + lvl_bk(e, i, b, k) * L, i);
-      __syncthreads();
-      if (mine) key += (unsigned long long)(unsigned)dc[i - 1] * e.li.mult[i - 1];
+    for (int i = 1; i <= m_now && mine && acc == i - 1; ++i) {
+      key += (unsigned long long)(unsigned)sm.node[k * L + i - 1] * e.li.mult[i - 1];
       bool in = false;
-      if (mine && acc == i - 1)
-        for (int r = 0; r < nbi; ++r) in |= s_beam[r] == key;
+      for (int r = 0; r < K; ++r) in |= sm.key[(i - 1) * Kmax + r] == key;
       if (in) acc = i;
     }
   }
@@ -988,7 +1023,7 @@ __device__ __forceinline__ void round_end_body(const EngineState& e, int K, cons
     if (tr.accepted_len) tr.accepted_len[tro * K + k] = acc;
     if (tr.drafts)
       for (int l = 0; l < L; ++l)
-        tr.drafts[(tro * K + k) * L + l] = (k < nd) ? e.dw_codes[lvl_bk(e, L, b, k) * L + l] : -1;
+        tr.drafts[(tro * K + k) * L + l] = (k < nd) ? sm.node[k * L + l] : -1;
     if (tr.tree_codes)
       for (int j = 1; j <= L; ++j) {
         const int nj = took_part ? min(e.dw_count[(long long)j * e.Bmax + b], Kmax) : 0;
@@ -1003,11 +1038,11 @@ __device__ __forceinline__ void round_end_body(const EngineState& e, int K, cons
   if (threadIdx.x == 0) {
     if (tr.n_draft) tr.n_draft[tro] = took_part ? nd : -1;
     if (tr.level_reached) tr.level_reached[tro] = took_part ? m_now : -1;
-    int spec = e.row_spec[b];
-    if (took_part && re.adaptive) { spec = (m_now - e.row_m_start[b] >= 2) ? 1 : 0; e.row_spec[b] = spec; }
+    int spec = rs.spec;
+    if (took_part && re.adaptive) { spec = (m_now - rs.m_start >= 2) ? 1 : 0; e.row_spec[b] = spec; }
     if (m_now < L && spec) atomicMax(e.draft_rows, batch * Kmax);            // somebody drafts next round
     if (m_now < L) atomicAdd(&e.counters[0], 1);
-    if (took_part) atomicAdd(&e.counters[1], e.row_tok_count[b]);
+    if (took_part) atomicAdd(&e.counters[1], rs.tokens);
     if (acc_sum) atomicAdd(&e.counters[2], acc_sum);
     if (round == 1 && nd) atomicAdd(&e.counters[3], nd);
     __threadfence();
@@ -1026,15 +1061,31 @@ __device__ __forceinline__ void round_end_body(const EngineState& e, int K, cons
 // the end of the round, in one launch.
 template <int VPL, bool PROBE>
 __global__ void __launch_bounds__(select_max_threads(VPL)) select_advance_kernel(SelectArgs a, EngineState e, int n, int K, int* out_codes,
-                                                             float* out_score, int* out_count, RoundEnd re) {
+                                                             float* out_score, int* out_count, RoundEnd re, int select_bytes) {
+  extern __shared__ unsigned char smem_raw[];
+  const int b = blockIdx.x, L = e.L, Kmax = e.Kmax, n1 = n + 1;
+  const AdvanceSmem sm = advance_smem(smem_raw + select_bytes, Kmax, L);
   pdl_wait();
   pdl_launch();
-  select_body<VPL, PROBE>(a);
-  __syncthreads();                                 // the block's own selection (global writes) is visible to all its threads
-  advance_body(e, n, K, out_codes, out_score, out_count);
+  cp_async_ints(sm.codes, e.tb_codes + lvl_bk(e, n, b, 0) * L, Kmax * L);
+  cp_async_ints(sm.node, e.dw_codes + lvl_bk(e, n1, b, 0) * L, Kmax * L);
+  if (n1 < L) {
+    cp_async_ints(sm.dbeam, e.d_beam + lvl_bk(e, n1, b, 0), Kmax);
+    cp_async_ints(sm.nidx, e.node_index + ((long long)b * L + n1) * Kmax, Kmax);
+    cp_async_ints(sm.self, e.tb_self + lvl_bk(e, n, b, 0), Kmax);
+    cp_async_ints(sm.anc, e.tb_anc + lvl_bk(e, n, b, 0) * L, Kmax * L);
+  }
+  if (re.host)
+    for (int lv = 1; lv <= L; ++lv) cp_async_ints(sm.beams + (lv - 1) * Kmax * L, e.tb_codes + lvl_bk(e, lv, b, 0) * L, Kmax * L);
+  const int nd = min(e.dw_count[(long long)n1 * e.Bmax + b], Kmax);
+  RowState rs{0, 0, 0, 0, 0};
+  if (re.host) rs = RowState{e.row_m[b], e.row_m_start[b], e.row_spec[b], e.row_tok_count[b], nd};
+  const Selected sel = select_body<VPL, PROBE>(a, sm.codes);
+  if (sel.active) advance_body(e, sm, sel, n, K, nd, out_codes, out_score, out_count);
+  else asm volatile("cp.async.wait_all;" ::: "memory");
   if (re.host) {
     __syncthreads();
-    round_end_body(e, K, re);
+    round_end_body(e, sm, sel, rs, K, re);
   }
 }
 
@@ -1124,6 +1175,7 @@ void launch_draft_step(const EngineState& e, int batch, int l, const float* G, l
   launch_pdl(draft_step_kernel, dim3(batch * e.Kmax), dim3(128), 0, st, e, batch, l, G, g_stride, t_cols, U, bias,
              (__nv_bfloat16*)s_act);
 }
+size_t advance_smem_bytes(int Kmax, int L) { return (size_t)Kmax * (8 * L + 4 * (3 * L + 3 + L * L)); }
 cudaError_t select_step_configure(int bytes) {
   cudaError_t e = cudaSuccess;
   auto set = [&](auto vpl) {
@@ -1166,14 +1218,14 @@ void launch_nodes_from_prefixes(const EngineState& e, int batch, int n_beams, in
 void launch_select_advance(const SelectArgs& a, const EngineState& e, int n, int K, int* out_codes, float* out_score,
                            int* out_count, const RoundEnd& re, cudaStream_t st) {
   if (a.batch <= 0) return;
-  const size_t smem = select_smem_bytes(a.in_stride, a.K);
+  const size_t select_bytes = select_smem_bytes(a.in_stride, a.K), smem = select_bytes + advance_smem_bytes(e.Kmax, e.L);
   LaunchScope ls(kcSelect, st);
   const int warps = select_warps(a);
   const dim3 block(32 * warps), grid(a.batch);
   with_vpl(a.T, [&](auto vpl) {
     constexpr int V = decltype(vpl)::value;
     launch_pdl(select_probes(a) ? select_advance_kernel<V, true> : select_advance_kernel<V, false>, grid, block, smem, st, a, e, n,
-               K, out_codes, out_score, out_count, re);
+               K, out_codes, out_score, out_count, re, (int)select_bytes);
   });
 }
 void launch_copy_logits(const float* src, long long row_stride, int col_off, const int* row_index, int row_mul,
