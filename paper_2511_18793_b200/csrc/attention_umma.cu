@@ -96,6 +96,30 @@ __device__ __forceinline__ void tmem_st32(uint32_t taddr, const float* v) {
         "f"(v[27]), "f"(v[28]), "f"(v[29]), "f"(v[30]), "f"(v[31]) : "memory");
   asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
 }
+// 64 columns of the warp's TMEM lanes: both loads are on their way before the one wait.
+__device__ __forceinline__ void tmem_ld64(uint32_t taddr, float* v) {
+  uint32_t r[64];
+#pragma unroll
+  for (int h = 0; h < 2; ++h)
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
+        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
+        "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+        : "=r"(r[32 * h + 0]), "=r"(r[32 * h + 1]), "=r"(r[32 * h + 2]), "=r"(r[32 * h + 3]), "=r"(r[32 * h + 4]), "=r"(r[32 * h + 5]),
+          "=r"(r[32 * h + 6]), "=r"(r[32 * h + 7]), "=r"(r[32 * h + 8]), "=r"(r[32 * h + 9]), "=r"(r[32 * h + 10]), "=r"(r[32 * h + 11]),
+          "=r"(r[32 * h + 12]), "=r"(r[32 * h + 13]), "=r"(r[32 * h + 14]), "=r"(r[32 * h + 15]), "=r"(r[32 * h + 16]), "=r"(r[32 * h + 17]),
+          "=r"(r[32 * h + 18]), "=r"(r[32 * h + 19]), "=r"(r[32 * h + 20]), "=r"(r[32 * h + 21]), "=r"(r[32 * h + 22]), "=r"(r[32 * h + 23]),
+          "=r"(r[32 * h + 24]), "=r"(r[32 * h + 25]), "=r"(r[32 * h + 26]), "=r"(r[32 * h + 27]), "=r"(r[32 * h + 28]), "=r"(r[32 * h + 29]),
+          "=r"(r[32 * h + 30]), "=r"(r[32 * h + 31])
+        : "r"(taddr + 32u * h));
+  // (the values pass through the wait, so that nothing that reads them can be moved in front of it)
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+  for (int i = 0; i < 64; ++i) {
+    asm volatile("" : "+r"(r[i]));
+    v[i] = __uint_as_float(r[i]);
+  }
+}
 __device__ __forceinline__ float ex2u(float x) {
   float y;
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
@@ -327,13 +351,13 @@ __global__ void __launch_bounds__(kThreadsU, UmmaCfg<HD, PT>::kCtasPerSm) attn_u
       const int sb = PT ? (j & 1) : 0;               // S / P buffer of this tile
       const uint32_t par = (uint32_t)(PT ? (j >> 1) : j) & 1u;
       const uint32_t col_s = 64u * sb;
-      ok = warp_wait(s_full(sb), par, abort_flag, lane);
+      ok = warp_wait_uniform(s_full(sb), par, abort_flag);
       if (!ok) { if (lane == 0) gave_up(7, j); break; }
       if (warp_dead) {                               // (its P rows stay whatever they are: O rows nobody reads)
         if (!PT) {
           if (lane == 0) mbar_arrive(s_free);
           if (j >= 1) {
-            ok = warp_wait(pv_done(j - 1), pv_parity(j - 1), abort_flag, lane);
+            ok = warp_wait_uniform(pv_done(j - 1), pv_parity(j - 1), abort_flag);
             if (!ok) { if (lane == 0) gave_up(8, j); break; }
           }
         }
@@ -342,8 +366,7 @@ __global__ void __launch_bounds__(kThreadsU, UmmaCfg<HD, PT>::kCtasPerSm) attn_u
       }
       tc_fence_after();
       float sv[kPosU];
-      tmem_ld32(tmem_base + lane_addr + col_s, sv);
-      tmem_ld32(tmem_base + lane_addr + col_s + 32u, sv + 32);
+      tmem_ld64(tmem_base + lane_addr + col_s, sv);
       tc_fence_before();
       __syncwarp();
       if (!PT && lane == 0) mbar_arrive(s_free);     // the scores are in registers: S may take tile j + 1
@@ -362,29 +385,31 @@ __global__ void __launch_bounds__(kThreadsU, UmmaCfg<HD, PT>::kCtasPerSm) attn_u
         for (int c = 0; c < kPosU; ++c)
           if (j * kPosU + c >= ctx) sv[c] = -INFINITY;
       }
-      float mx = -INFINITY;
+      float mq[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};      // four chains: one is 32 dependent steps
 #pragma unroll
-      for (int c = 0; c < kPosU; c += 2) mx = max3(mx, sv[c], sv[c + 1]);
-      mx *= sc;
+      for (int c = 0; c < kPosU; c += 8)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) mq[q] = max3(mq[q], sv[c + 2 * q], sv[c + 2 * q + 1]);
+      const float mx = max3(fmaxf(mq[0], mq[1]), mq[2], mq[3]) * sc;
       // raise the reference only when the true maximum has run away from it: p stays below 2^8 otherwise
       const bool raise = mx > m_ref + kRaise || (m_ref == -INFINITY && mx > -INFINITY);
       const float m_new = raise ? mx : m_ref;
       const float m_safe = m_new == -INFINITY ? 0.f : m_new;
       const float corr = raise ? ex2u(m_ref - m_safe) : 1.f;     // ex2(-inf) = 0 the first time
       const f32x2 sc2 = pack2(sc, sc), neg_m2 = pack2(-m_safe, -m_safe);
-      f32x2 rs2 = pack2(0.f, 0.f);
+      f32x2 rs2[2] = {pack2(0.f, 0.f), pack2(0.f, 0.f)};
       uint32_t pk[kPosU / 2];
 #pragma unroll
       for (int c = 0; c < kPosU; c += 2) {
         float x0, x1;
         unpack2(fma2(pack2(sv[c], sv[c + 1]), sc2, neg_m2), x0, x1);
         const float p0 = ex2u(x0), p1 = ex2u(x1);
-        rs2 = add2(rs2, pack2(p0, p1));
+        rs2[(c >> 1) & 1] = add2(rs2[(c >> 1) & 1], pack2(p0, p1));
         __nv_bfloat162 pb = __floats2bfloat162_rn(p0, p1);
         pk[c >> 1] = *reinterpret_cast<uint32_t*>(&pb);
       }
       float rs_lo, rs_hi;
-      unpack2(rs2, rs_lo, rs_hi);
+      unpack2(add2(rs2[0], rs2[1]), rs_lo, rs_hi);
       const float rs = rs_lo + rs_hi;
       l_run = l_run * corr + rs;
       m_ref = m_new;
@@ -392,7 +417,7 @@ __global__ void __launch_bounds__(kThreadsU, UmmaCfg<HD, PT>::kCtasPerSm) attn_u
       // read by P_{j-2} V_{j-2}, which completed before S_j did); only a rescale of O has to wait for P_{j-1} V_{j-1}.
       const bool rescale = j > 0 && __any_sync(0xffffffffu, raise);
       if (j >= 1 && (!PT || rescale)) {
-        ok = warp_wait(pv_done(j - 1), pv_parity(j - 1), abort_flag, lane);
+        ok = warp_wait_uniform(pv_done(j - 1), pv_parity(j - 1), abort_flag);
         if (!ok) { if (lane == 0) gave_up(9, j); break; }
       }
       if (rescale) {                                 // rescale O
@@ -420,7 +445,7 @@ __global__ void __launch_bounds__(kThreadsU, UmmaCfg<HD, PT>::kCtasPerSm) attn_u
       if (lane == 0) mbar_arrive(p_full(sb));
     }
     if (ok && NT > 0) {
-      ok = warp_wait(pv_done(NT - 1), pv_parity(NT - 1), abort_flag, lane);
+      ok = warp_wait_uniform(pv_done(NT - 1), pv_parity(NT - 1), abort_flag);
       if (!ok && lane == 0) gave_up(10, NT);
       tc_fence_after();
     }
