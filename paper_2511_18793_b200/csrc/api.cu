@@ -295,15 +295,24 @@ void gemm(nezha_ctx* c, const void* A, long long lda, const void* W, long long l
 // RMSNorm scale is applied in the epilogue), or null.  Returns the number of partial sums per row a kEpiAddNorm
 // epilogue of this launch writes (one per 32 columns).
 int gemm_fused(nezha_ctx* c, const void* A, long long lda, const void* W, void* C, long long ldc, long long M,
-               const int* M_dev, int N, int K, int epi, const float* ss_in, int ss_parts, const GemmFuse* extra) {
+               const int* M_dev, int N, int K, int epi, const float* ss_in, int ss_parts, const GemmFuse* extra,
+               const void* next_w = nullptr, long long next_w_bytes = 0) {
   GemmArgs a{A, lda, W, (long long)K, C, ldc, (int)M, M_dev, N, K, epi, nullptr, c->es.status};
   if (extra) a.f = *extra;
   a.f.ss_in = ss_in; a.f.ss_in_parts = ss_parts; a.f.ss_ld = c->Ms; a.f.inv_dim = 1.f / (float)c->d; a.f.eps = c->cfg.rms_eps;
   a.M_expected = c->m_expected;
   a.skinny = c->skinny_now;
+  a.next_w = next_w; a.next_w_bytes = next_w_bytes;
   launch_gemm_tc(a, c->st);
   return N / 32;
 }
+
+// How much of the gate/up weights the output projection's launch asks for ahead, where it streams its weights: HBM is idle
+// while that launch waits for the attention kernel, and its own weights are few.  A call of one request on the 16-layer
+// d = 2048 backbone (64 MB of gate/up weights), drafted / verified: 873 / 2313 us without, 862 / 2272 with 8 MB, 850 / 2246
+// with 16, 845 / 2239 with 24, 849 / 2245 with 40, 874 / 2277 with all of them (they then delay the projection's own).  The
+// QKV launch asking ahead (gate/up weights, beyond the attention) or the gate/up launch (down weights): nothing, or slower.
+constexpr long long kNextWeights = 24LL << 20;
 
 // The layers of the primary model on the fused path.  On entry resid holds the embeddings, xn = embedding * gain of
 // the first attention norm and ss_e the rows' sums of squares (launch_embed_norm).  Five kernels per layer:
@@ -345,7 +354,7 @@ void run_layers_fused(nezha_ctx* c, long long M, const int* M_dev, bool verify, 
     GemmFuse fo{};
     fo.xg = c->xn; fo.gain = w.mlp_norm; fo.ss_out = c->ss_a;
     const int parts_a = gemm_fused(c, c->attn, (long long)c->Hq * c->hd, w.wo, c->resid, c->d, M, M_dev, c->d, c->Hq * c->hd,
-                                   kEpiAddNorm, nullptr, 0, &fo);
+                                   kEpiAddNorm, nullptr, 0, &fo, w.w_gu, std::min(kNextWeights, 4LL * c->F * c->d));
     gemm_fused(c, c->xn, c->d, w.w_gu, c->act, c->F, M, M_dev, 2 * c->F, c->d, kEpiSwiGLU, c->ss_a, parts_a, nullptr);
     GemmFuse fd{};
     fd.xg = c->xn; fd.gain = (i + 1 < c->nl) ? c->layers[i + 1].attn_norm : c->final_norm; fd.ss_out = c->ss_b;

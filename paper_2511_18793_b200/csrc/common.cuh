@@ -280,6 +280,9 @@ struct GemmArgs {
   // other kernels': a caller that needs the same bits from two launches gives both the same class.  W must be constant
   // data (it is read before the launch's dependency on its predecessor is resolved).
   int skinny;
+  // Optional, and only a hint (the weight-streaming kernel heeds it, the others do not): constant data that the launch after
+  // this one starts with, asked for into L2 while this launch waits for its predecessor.  16-byte aligned, a multiple of 16.
+  const void* next_w; long long next_w_bytes;
 };
 
 void launch_gemm_simt(const GemmArgs& a, bool bf16, cudaStream_t st);

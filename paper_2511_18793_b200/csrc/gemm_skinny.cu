@@ -120,6 +120,12 @@ __global__ void __launch_bounds__(kSkinnyThreads, 2)
         mbar_expect_tx(full_bar(s), C::kStageBytes);
         tma_load_2d(base + s * C::kStageBytes, &tmW, (k_begin + s) * BK, n0, full_bar(s));
       }
+    // behind them, in shares of 8 KB, the head of the next launch's weights (see kNextWeights in api.cu)
+    if (blockIdx.y == 0)
+      for (long long o = (long long)blockIdx.x * 8192; o < a.next_w_bytes; o += (long long)gridDim.x * 8192) {
+        const uint32_t bytes = (uint32_t)min(8192LL, a.next_w_bytes - o);
+        asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"((const char*)a.next_w + o), "r"(bytes) : "memory");
+      }
   }
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32((const void*)tmem_slot)),
