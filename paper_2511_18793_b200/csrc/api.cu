@@ -15,8 +15,9 @@
 namespace nz {
 void launch_hs_pack(const LevelInfo& li, const int* codes, unsigned long long n, unsigned long long* keys, int* status,
                     cudaStream_t st);
-void launch_set_build(const LevelInfo& li, HashSetView hs, PrefixMapView pm, const int* codes, unsigned long long n,
-                      unsigned long long* n_unique, int* status, int n_sm, cudaStream_t st);
+void plan_build(const LevelInfo& li, HashSetView hs, PrefixMapView pm, unsigned long long n, BuildScratch* sc);
+void launch_set_build(const LevelInfo& li, HashSetView hs, PrefixMapView pm, const BuildScratch& sc, const int* codes,
+                      unsigned long long n, unsigned long long* n_unique, int* status, int n_sm, cudaStream_t st);
 int sm_count();
 void launch_hs_probe(HashSetView hs, const unsigned long long* keys, unsigned long long n, uint8_t* found,
                      cudaStream_t st);
@@ -80,6 +81,7 @@ struct nezha_ctx {
   void* draft_wcat[kMaxLevels]; float* draft_u; float* draft_hl; void* draft_sact; float* draft_g;
   int* h_rows; unsigned long long* n_unique_dev;
   EngineState es;
+  BuildScratch build;
   int* host_counters;       // pinned
   // CUDA graphs of the decode segments (one per round), keyed by everything that shapes the launch sequence
   struct Segment { int seen; cudaGraphExec_t exec; long long launches[kcCount]; };
@@ -196,6 +198,7 @@ size_t carve(nezha_ctx* c) {
       if (n > 0) prefixes *= (double)g.T[n - 1];
       const double slots = ceil((prefixes < items ? prefixes : items) / c->load_factor) + 1;
       const bool direct = prefixes * e.pm.set_words <= slots * e.pm.stride;
+      total += total & 1;                    // (16-byte boundaries)
       e.pm.level_off[n] = total;
       e.pm.level_slots[n] = direct ? 0 : (unsigned long long)slots;
       total += direct ? (unsigned long long)prefixes * e.pm.set_words : (unsigned long long)slots * e.pm.stride;
@@ -203,6 +206,18 @@ size_t carve(nezha_ctx* c) {
     for (int n = g.L; n < kMaxLevels; ++n) { e.pm.level_off[n] = 0; e.pm.level_slots[n] = 0; }
     e.pm.n_words = total;
     e.pm.slots = cv.take<unsigned long long>(e.pm.n_words);
+  }
+  plan_build(li, e.hs, e.pm, c->n_items, &c->build);
+  if (c->build.on) {
+    BuildDeal &bp = c->build.by_prefix, &bb = c->build.by_bucket;
+    bp.count = cv.take<unsigned>(bp.parts + bb.parts + 2);       // (one piece: cleared by one call)
+    bb.count = bp.count + bp.parts + 1;
+    bp.offset = cv.take<unsigned>((size_t)kBuildBlocks * bp.parts);
+    bb.offset = cv.take<unsigned>((size_t)kBuildBlocks * bb.parts);
+    c->build.keys = cv.take<unsigned>(c->n_items);
+    c->build.n_valid = cv.take<unsigned>(kBuildBlocks);
+    c->build.any = cv.take<unsigned>(((size_t)c->build.by_prefix.parts << c->build.by_prefix.shift) / 32);
+    c->build.n_over = cv.take<unsigned>(c->build.by_bucket.parts);
   }
   // weights
   const size_t esz = c->esz;
@@ -808,7 +823,7 @@ nezha_status nezha_create(const nezha_config* cfg, const nezha_weights* w, const
 
 nezha_status nezha_build_hashset(nezha_ctx* c, uint64_t* n_unique) {
   if (!c) return NEZHA_ERR_ARG;
-  launch_set_build(c->es.li, c->es.hs, c->es.pm, c->catalog, c->n_items, c->n_unique_dev, c->es.status, sm_count(), c->st);
+  launch_set_build(c->es.li, c->es.hs, c->es.pm, c->build, c->catalog, c->n_items, c->n_unique_dev, c->es.status, sm_count(), c->st);
   // (into pinned memory: the copy is queued with the status word's, and one wait serves both)
   NZ_CUDA(c, cudaMemcpyAsync(c->host_counters, c->n_unique_dev, sizeof(unsigned long long), cudaMemcpyDeviceToHost, c->st));
   NZ_CUDA(c, cudaGetLastError());

@@ -221,6 +221,24 @@ __device__ __forceinline__ bool pm_test(const unsigned long long* bits, int t) {
   return bits != nullptr && ((__ldg(bits + (t >> 6)) >> (t & 63)) & 1ull);
 }
 
+// Plan and scratch of a build by parts (launch_set_build).  The items are dealt out twice: by runs of 2^shift prefixes of the
+// prefix map's longest region, and by runs of 2^shift buckets of the hash set.
+constexpr int kBuildBlocks = 148;         // blocks that share the catalogue out (one per SM)
+constexpr int kBuildMaxParts = 8192;
+struct BuildDeal {
+  int parts, shift;
+  unsigned* count;                 // [parts + 1] keys of each part, then their exclusive sums
+  unsigned* offset;                // [kBuildBlocks][parts] where a block's keys of a part start within the part
+};
+struct BuildScratch {
+  int on;                          // 0: no build by parts
+  BuildDeal by_prefix, by_bucket;
+  unsigned* keys;                  // [n] the packed keys, part after part, of one deal after the other
+  unsigned* n_valid;               // [kBuildBlocks] keys a block has packed
+  unsigned* any;                   // [by_prefix.parts << shift] bits: which prefixes some item begins with
+  unsigned* n_over;                // [by_bucket.parts] keys that ran over the end of a part (left at the part's start in keys)
+};
+
 // --------------------------------------------------------------------------------------------------
 // model / engine description shared by the host code and the kernels
 // --------------------------------------------------------------------------------------------------

@@ -64,25 +64,40 @@ __global__ void __launch_bounds__(256) hs_pack_kernel(LevelInfo li, const int* _
 // The bucket is looked at with one plain load.  What it shows may be out of date, but only in one direction -- a slot that
 // looks free may have been taken since -- and the compare-and-swap says by whom.  (A compare-and-swap without a look, at a
 // slot the hash names: slower, 1,004 us against 778 for 10M items, because some lane of a warp always has to go on.)
+template <typename Slot> struct SlotBucket {
+  static constexpr int kSlots = kBucketBytes / sizeof(Slot);
+  static constexpr Slot kFree = ~(Slot)0;
+  union { unsigned w[8]; Slot s[kSlots]; };
+  __device__ __forceinline__ void load(const Slot* bucket) {
+    asm volatile("ld.global.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]), "=r"(w[4]), "=r"(w[5]), "=r"(w[6]), "=r"(w[7])
+                 : "l"(bucket) : "memory");
+  }
+  __device__ __forceinline__ bool has(Slot val) const {
+    bool hit = false;
+#pragma unroll
+    for (int i = 0; i < kSlots; ++i) hit |= s[i] == val;
+    return hit;
+  }
+  __device__ __forceinline__ int first_free() const {
+    int f = kSlots;
+#pragma unroll
+    for (int i = kSlots - 1; i >= 0; --i)
+      if (s[i] == kFree) f = i;
+    return f;
+  }
+};
 template <typename Slot>
 __device__ __forceinline__ int hs_insert_slot(unsigned long long* slots, unsigned long long n_buckets, unsigned long long b, Slot val) {
-  constexpr int kSlots = kBucketBytes / sizeof(Slot);
-  constexpr Slot kFree = ~(Slot)0;
+  using B = SlotBucket<Slot>;
   for (int step = 0; step < kMaxProbeBuckets; ++step) {
-    Slot* bucket = reinterpret_cast<Slot*>(slots) + b * kSlots;
-    union { unsigned w[8]; Slot s[kSlots]; } k;
-    asm volatile("ld.global.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-                 : "=r"(k.w[0]), "=r"(k.w[1]), "=r"(k.w[2]), "=r"(k.w[3]), "=r"(k.w[4]), "=r"(k.w[5]), "=r"(k.w[6]), "=r"(k.w[7])
-                 : "l"(bucket) : "memory");
-    int first_free = kSlots;
-#pragma unroll
-    for (int s = kSlots - 1; s >= 0; --s) {
-      if (k.s[s] == val) return 0;
-      if (k.s[s] == kFree) first_free = s;
-    }
-    for (int s = first_free; s < kSlots; ++s) {
-      const Slot cur = atomicCAS(bucket + s, kFree, val);
-      if (cur == kFree) return 1;
+    Slot* bucket = reinterpret_cast<Slot*>(slots) + b * B::kSlots;
+    B k;
+    k.load(bucket);
+    if (k.has(val)) return 0;
+    for (int s = k.first_free(); s < B::kSlots; ++s) {
+      const Slot cur = atomicCAS(bucket + s, B::kFree, val);
+      if (cur == B::kFree) return 1;
       if (cur == val) return 0;
     }
     if (++b == n_buckets) b = 0;
@@ -117,6 +132,30 @@ __device__ __forceinline__ int pm_add(const PrefixMapView& pm, int n, unsigned l
   return -1;
 }
 
+template <bool NARROW>
+__device__ __forceinline__ int hs_insert(const HashSetView& hs, unsigned long long key) {
+  if constexpr (NARROW) {
+    const unsigned m = hs_mix32((unsigned)key);
+    if (m != ~0u) return hs_insert_slot<unsigned>(hs.slots, hs.n_buckets, __umulhi(m, (unsigned)hs.n_buckets), m);
+    return atomicExch(const_cast<unsigned*>(hs_special(hs)), 1u) == 0u ? 1 : 0;
+  } else {
+    return hs_insert_slot<unsigned long long>(hs.slots, hs.n_buckets, hs_bucket(key, hs.n_buckets), key);
+  }
+}
+
+// Adds a block's inserted items up (every thread of the block calls this once).
+__device__ __forceinline__ void count_inserted(int inserted, unsigned long long* n_unique) {
+  inserted = (int)__reduce_add_sync(0xffffffffu, (unsigned)inserted);
+  __shared__ int part[32];
+  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = inserted;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    int sum = 0;
+    for (int w = 0; w < (int)blockDim.x >> 5; ++w) sum += part[w];
+    if (sum) atomicAdd(n_unique, (unsigned long long)sum);
+  }
+}
+
 // The hash set and the prefix map in one pass over the catalogue.  An item that is in the set already is done.  A new one
 // sets its bit behind its L - 1 codes, and only where that prefix was not there yet does it go on to the next shorter one:
 // whoever brought a prefix has entered it everywhere above, so almost every item ends after two or three random accesses
@@ -133,14 +172,7 @@ __global__ void __launch_bounds__(256) set_build_kernel(LevelInfo li, HashSetVie
     load_codes<VEC>(codes, i, li.L, c);
     const unsigned long long key = pack_checked(li, c);
     if (key == kEmptyKey) { atomicOr(status, kStBadCode); continue; }
-    int r;
-    if constexpr (NARROW) {
-      const unsigned m = hs_mix32((unsigned)key);
-      if (m != ~0u) r = hs_insert_slot<unsigned>(hs.slots, hs.n_buckets, __umulhi(m, (unsigned)hs.n_buckets), m);
-      else r = atomicExch(const_cast<unsigned*>(hs_special(hs)), 1u) == 0u ? 1 : 0;
-    } else {
-      r = hs_insert_slot<unsigned long long>(hs.slots, hs.n_buckets, hs_bucket(key, hs.n_buckets), key);
-    }
+    int r = hs_insert<NARROW>(hs, key);
     if (r > 0) {
       ++inserted;
       unsigned long long p = key;
@@ -155,15 +187,302 @@ __global__ void __launch_bounds__(256) set_build_kernel(LevelInfo li, HashSetVie
     }
     if (r < 0) atomicOr(status, kStHashFull);
   }
-  inserted = (int)__reduce_add_sync(0xffffffffu, (unsigned)inserted);
-  __shared__ int part[8];
-  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = inserted;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    int sum = 0;
-    for (int w = 0; w < 8; ++w) sum += part[w];
-    if (sum) atomicAdd(n_unique, (unsigned long long)sum);
+  count_inserted(inserted, n_unique);
+}
+
+// ---- the same build by parts, for many items ---------------------------------------------------------------------------------
+// Above, an item is a random access to a table that DRAM holds (bits; 10M items: 403 us of atomics on 537 MB) and two to one that
+// the L2 holds (bucket, then slot; 254 us), behind a pass that clears both.  Here the items are dealt out to parts that a block's
+// shared memory holds: by prefix, for the bits, and by bucket, for the hash set.  A block builds a part there and writes it
+// once, which also replaces the clearing.
+// 10M items over 256^4 codes, load factor 0.5, whole calls: 968 us above, 437 here, of which the bits take 122 (537 MB written; 82
+// at the copy bandwidth), the slots 73, counting 65, the two deals 66 and 41, the rest launches.  30M: 2,907 -> 1,248.
+// key / prefixes (the last code, at most 1,023) and the remainder.  Both roundings go down, and by less than 2^-10 of 1,024: the
+// product's integer part is the quotient or one less.  (With the compiler's division the first deal of 10M items took 69 us, not 66.)
+struct KeySplit {
+  unsigned prefixes; float inv;     // inv: below 1 / prefixes
+  __device__ __forceinline__ unsigned operator()(unsigned key, unsigned* prefix) const {
+    unsigned t = __float2uint_rz(__fmul_rz(__uint2float_rz(key), inv));
+    unsigned p = key - t * prefixes;
+    if (p >= prefixes) { p -= prefixes; ++t; }
+    *prefix = p;
+    return t;
   }
+};
+struct DealPrefix {
+  KeySplit split; int shift;
+  __device__ __forceinline__ int operator()(unsigned key) const {
+    unsigned p;
+    split(key, &p);
+    return (int)(p >> shift);
+  }
+};
+struct DealBucket {
+  unsigned n_buckets; int shift;
+  __device__ __forceinline__ int operator()(unsigned key) const { return (int)(__umulhi(hs_mix32(key), n_buckets) >> shift); }
+};
+
+// The items in kBuildBlocks equal runs, one per block: packs a run's keys (left in keys[] at the run's start, without those
+// with a bad code) and counts them by part, for both deals.  The block's place within each part is what the counter held before.
+template <bool VEC>
+__global__ void __launch_bounds__(1024) part_count_kernel(LevelInfo li, HashSetView hs, PrefixMapView pm, BuildScratch sc, DealBucket by_bucket,
+                                                          const int* __restrict__ codes, unsigned n, unsigned run,
+                                                          unsigned* __restrict__ keys, unsigned long long* n_unique, int* status) {
+  extern __shared__ unsigned hist[];                    // [by_prefix.parts], [by_bucket.parts]
+  __shared__ unsigned n_keys;
+  const int parts = sc.by_prefix.parts, both = parts + sc.by_bucket.parts;
+  for (int p = threadIdx.x; p < both; p += 1024) hist[p] = 0;
+  if (threadIdx.x == 0) n_keys = 0;
+  // what the kernels behind this one add to: the regions of the shorter prefixes, the special word, the number of items
+  for (unsigned long long w = blockIdx.x * 1024ull + threadIdx.x; w < pm.level_off[li.L - 1]; w += kBuildBlocks * 1024ull) pm.slots[w] = 0;
+  if (blockIdx.x == 0 && threadIdx.x == 0) { *const_cast<unsigned*>(hs_special(hs)) = 0; *n_unique = 0; }
+  __syncthreads();
+  const unsigned lo = min(n, blockIdx.x * run), hi = min(n, lo + run);
+  const int lane = threadIdx.x & 31;
+  constexpr int kItems = 4;                             // in flight per thread
+  for (unsigned i0 = lo; i0 < hi; i0 += 1024 * kItems) {
+    int c[kItems][kMaxLevels];
+#pragma unroll
+    for (int j = 0; j < kItems; ++j) {
+      const unsigned i = i0 + 1024 * j + threadIdx.x;
+      if (i < hi) load_codes<VEC>(codes, i, li.L, c[j]);
+    }
+#pragma unroll
+    for (int j = 0; j < kItems; ++j) {
+      const unsigned i = i0 + 1024 * j + threadIdx.x;
+      unsigned prefix = 0, last = 0;
+      bool ok = i < hi;
+#pragma unroll
+      for (int l = 0; l < kMaxLevels; ++l)
+        if (l < li.L && i < hi) {
+          ok &= (unsigned)c[j][l] < (unsigned)li.T[l];
+          const unsigned term = (unsigned)c[j][l] * (unsigned)li.mult[l];
+          if (l == li.L - 1) last = term; else prefix += term;
+        }
+      if (i < hi && !ok) atomicOr(status, kStBadCode);
+      const unsigned members = __ballot_sync(0xffffffffu, ok);
+      unsigned at = 0;
+      if (lane == 0 && members) at = atomicAdd(&n_keys, (unsigned)__popc(members));
+      at = __shfl_sync(0xffffffffu, at, 0);
+      if (ok) {
+        keys[lo + at + __popc(members & ((1u << lane) - 1))] = prefix + last;
+        atomicAdd(&hist[prefix >> sc.by_prefix.shift], 1u);
+        atomicAdd(&hist[parts + by_bucket(prefix + last)], 1u);
+      }
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) sc.n_valid[blockIdx.x] = n_keys;
+  for (int p = threadIdx.x; p < both; p += 1024) {
+    const BuildDeal& dl = p < parts ? sc.by_prefix : sc.by_bucket;
+    const int q = p < parts ? p : p - parts;
+    const unsigned h = hist[p];
+    dl.offset[(size_t)blockIdx.x * dl.parts + q] = h ? atomicAdd(&dl.count[q], h) : 0u;
+  }
+}
+
+// v[] of every thread of a block of 1024 (thread t: elements kEach t ..) becomes the exclusive prefix sums; returns what comes after
+// the thread's elements.  tmp: 32 words of shared memory, free again after the next barrier.
+template <int kEach>
+__device__ __forceinline__ unsigned block_exclusive_sums(unsigned (&v)[kEach], unsigned* tmp) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  unsigned sum = 0;
+#pragma unroll
+  for (int j = 0; j < kEach; ++j) sum += v[j];
+  unsigned incl = sum;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned up = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += up;
+  }
+  if (lane == 31) tmp[warp] = incl;
+  __syncthreads();
+  const unsigned before = __reduce_add_sync(0xffffffffu, lane < warp ? tmp[lane] : 0u);
+  unsigned start = before + incl - sum;
+#pragma unroll
+  for (int j = 0; j < kEach; ++j) { const unsigned x = v[j]; v[j] = start; start += x; }
+  return start;
+}
+
+// The counts become the parts' starts (one block of 1024 threads per deal).
+constexpr int kPartsEach = kBuildMaxParts / 1024;
+__global__ void __launch_bounds__(1024) part_scan_kernel(BuildScratch sc) {
+  __shared__ unsigned tmp[32];
+  const BuildDeal& dl = blockIdx.x == 0 ? sc.by_prefix : sc.by_bucket;
+  unsigned v[kPartsEach];
+#pragma unroll
+  for (int j = 0; j < kPartsEach; ++j) {
+    const int p = threadIdx.x * kPartsEach + j;
+    v[j] = p < dl.parts ? dl.count[p] : 0u;
+  }
+  const unsigned total = block_exclusive_sums(v, tmp);
+#pragma unroll
+  for (int j = 0; j < kPartsEach; ++j) {
+    const int p = threadIdx.x * kPartsEach + j;
+    if (p < dl.parts) dl.count[p] = v[j];
+  }
+  if (threadIdx.x == 1023) dl.count[dl.parts] = total;
+}
+
+// Deals a run's keys out to the parts, kDealKeys at a time: sorted by part in shared memory first, so that a part's keys go out
+// as one piece.  (Each key stored by itself: 92 us for 10M keys and 8,192 parts, 110 G stores/s; so: 66, and 41 for 1,221 parts)
+constexpr int kDealKeys = 32 << 10;
+template <typename Deal>
+__global__ void __launch_bounds__(1024) part_deal_kernel(BuildDeal dl, Deal part_of, const unsigned* __restrict__ n_valid, unsigned n,
+                                                         unsigned run, const unsigned* __restrict__ keys, unsigned* __restrict__ out) {
+  extern __shared__ unsigned sorted[];                  // [kDealKeys], then cursor[parts], base[parts]
+  __shared__ unsigned tmp[32];
+  unsigned *cursor = sorted + kDealKeys, *base = cursor + dl.parts;
+  for (int p = threadIdx.x; p < dl.parts; p += 1024) {
+    cursor[p] = 0;
+    base[p] = dl.count[p] + dl.offset[(size_t)blockIdx.x * dl.parts + p];
+  }
+  const unsigned lo = min(n, blockIdx.x * run), hi = lo + n_valid[blockIdx.x];
+  for (unsigned i0 = lo; i0 < hi; i0 += kDealKeys) {
+    const unsigned cnt = min((unsigned)kDealKeys, hi - i0);
+    // base + cursor = where the part's next key goes; the cursor starts again as a count
+    __syncthreads();
+    for (int p = threadIdx.x; p < dl.parts; p += 1024) { base[p] += cursor[p]; cursor[p] = 0; }
+    __syncthreads();
+#pragma unroll 4
+    for (unsigned i = threadIdx.x; i < cnt; i += 1024) atomicAdd(&cursor[part_of(keys[i0 + i])], 1u);
+    __syncthreads();
+    unsigned v[kPartsEach];
+#pragma unroll
+    for (int j = 0; j < kPartsEach; ++j) {
+      const int p = threadIdx.x * kPartsEach + j;
+      v[j] = p < dl.parts ? cursor[p] : 0u;
+    }
+    block_exclusive_sums(v, tmp);
+#pragma unroll
+    for (int j = 0; j < kPartsEach; ++j) {
+      const int p = threadIdx.x * kPartsEach + j;
+      if (p < dl.parts) { cursor[p] = v[j]; base[p] -= v[j]; }
+    }
+    __syncthreads();
+#pragma unroll 4
+    for (unsigned i = threadIdx.x; i < cnt; i += 1024) {
+      const unsigned k = keys[i0 + i];
+      sorted[atomicAdd(&cursor[part_of(k)], 1u)] = k;
+    }
+    __syncthreads();
+#pragma unroll 4
+    for (unsigned i = threadIdx.x; i < cnt; i += 1024) {
+      const unsigned k = sorted[i];
+      out[base[part_of(k)] + i] = k;
+    }
+  }
+}
+
+// One block per part of the prefix map's longest region: its bits, which of its prefixes begin an item, and how many items are
+// distinct.
+__global__ void __launch_bounds__(512, 3) part_bits_kernel(PrefixMapView pm, BuildScratch sc, int last, KeySplit split,
+                                                           unsigned long long* n_unique) {
+  extern __shared__ __align__(16) unsigned bits[];      // [2^shift][2 * set_words], then [2^shift / 32] for sc.any
+  const int shift = sc.by_prefix.shift, row = 2 * pm.set_words, all = row << shift, any_words = 1 << (shift - 5);
+  unsigned* any = bits + all;
+  for (int w = threadIdx.x * 4; w < all; w += 512 * 4) *reinterpret_cast<uint4*>(bits + w) = make_uint4(0, 0, 0, 0);
+  for (int w = threadIdx.x; w < any_words; w += 512) any[w] = 0;
+  const unsigned begin = sc.by_prefix.count[blockIdx.x], end = sc.by_prefix.count[blockIdx.x + 1], p0 = (unsigned)blockIdx.x << shift;
+  __syncthreads();
+  int inserted = 0;
+  for (unsigned i = begin + threadIdx.x; i < end; i += 512) {
+    unsigned p;
+    const unsigned t = split(sc.keys[i], &p), bit = 1u << (t & 31);
+    p -= p0;
+    unsigned* word = bits + p * row + (t >> 5);
+    if (*(volatile unsigned*)word & bit) continue;       // (a repeated item; the popular ones are worth the look)
+    const unsigned was = atomicOr(word, bit);
+    if (was == 0) atomicOr(any + (p >> 5), 1u << (p & 31));
+    inserted += !(was & bit);
+  }
+  __syncthreads();
+  const unsigned words = min(1u << shift, split.prefixes - p0) * pm.set_words;
+  unsigned long long* out = pm.slots + pm.level_off[last] + (unsigned long long)p0 * pm.set_words;
+  for (unsigned w = threadIdx.x; w < words / 2; w += 512)
+    __stcs(reinterpret_cast<uint4*>(out) + w, reinterpret_cast<const uint4*>(bits)[w]);
+  if (threadIdx.x == 0 && (words & 1)) out[words - 1] = reinterpret_cast<const unsigned long long*>(bits)[words - 1];
+  for (int w = threadIdx.x; w < any_words; w += 512) sc.any[(size_t)blockIdx.x * any_words + w] = any[w];
+  count_inserted(inserted, n_unique);
+}
+
+// One block per part of the hash set: its buckets.  A key whose walk runs over the part's end goes back to the start of the
+// part's keys, for part_over_kernel; those read so far are at least as many, hence the barrier between reading and writing.
+__global__ void __launch_bounds__(512, 3) part_slots_kernel(HashSetView hs, BuildScratch sc) {
+  using B = SlotBucket<unsigned>;
+  extern __shared__ __align__(16) unsigned slots[];     // [2^shift][8]
+  __shared__ unsigned n_over;
+  const int shift = sc.by_bucket.shift;
+  const unsigned b0 = (unsigned)blockIdx.x << shift, n_local = min(1u << shift, (unsigned)hs.n_buckets - b0);
+  const unsigned begin = sc.by_bucket.count[blockIdx.x], end = sc.by_bucket.count[blockIdx.x + 1];
+  for (unsigned w = threadIdx.x; w < n_local * 2; w += 512) reinterpret_cast<uint4*>(slots)[w] = make_uint4(~0u, ~0u, ~0u, ~0u);
+  if (threadIdx.x == 0) n_over = 0;
+  constexpr int kItems = 4;
+  for (unsigned i0 = begin; i0 < end; i0 += 512 * kItems) {
+    unsigned key[kItems];
+#pragma unroll
+    for (int j = 0; j < kItems; ++j) {
+      const unsigned i = i0 + 512 * j + threadIdx.x;
+      key[j] = i < end ? sc.keys[i] : 0u;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < kItems; ++j) {
+      if (i0 + 512 * j + threadIdx.x >= end) break;
+      const unsigned m = hs_mix32(key[j]);
+      if (m == B::kFree) { *const_cast<unsigned*>(hs_special(hs)) = 1u; continue; }
+      bool done = false;
+      for (unsigned b = __umulhi(m, (unsigned)hs.n_buckets) - b0; b < n_local && !done; ++b) {
+        B k;
+        const uint32_t at = (uint32_t)__cvta_generic_to_shared(slots + b * B::kSlots);
+        asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(k.w[0]), "=r"(k.w[1]), "=r"(k.w[2]), "=r"(k.w[3]) : "r"(at) : "memory");
+        asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(k.w[4]), "=r"(k.w[5]), "=r"(k.w[6]), "=r"(k.w[7]) : "r"(at + 16) : "memory");
+        done = k.has(m);
+        for (int s = k.first_free(); s < B::kSlots && !done; ++s) {
+          const unsigned cur = atomicCAS(slots + b * B::kSlots + s, B::kFree, m);
+          done = cur == B::kFree || cur == m;
+        }
+      }
+      if (!done) sc.keys[begin + atomicAdd(&n_over, 1u)] = key[j];
+    }
+  }
+  __syncthreads();
+  uint4* out = reinterpret_cast<uint4*>(hs.slots) + (size_t)b0 * 2;
+  for (unsigned w = threadIdx.x; w < n_local * 2; w += 512) out[w] = reinterpret_cast<const uint4*>(slots)[w];
+  if (threadIdx.x == 0) sc.n_over[blockIdx.x] = n_over;
+}
+// (one warp per part)
+__global__ void __launch_bounds__(256) part_over_kernel(HashSetView hs, BuildScratch sc, int* status) {
+  const int part = (int)(blockIdx.x * 8 + (threadIdx.x >> 5));
+  if (part >= sc.by_bucket.parts) return;
+  const unsigned begin = sc.by_bucket.count[part], n = sc.n_over[part];
+  for (unsigned i = threadIdx.x & 31; i < n; i += 32)
+    if (hs_insert<true>(hs, sc.keys[begin + i]) < 0) atomicOr(status, kStHashFull);
+}
+
+// The shorter prefixes, all in direct regions.  A thread gathers one word of the bits behind a prefix of n = L - 2 codes
+// (neighbouring threads: neighbouring prefixes, whose bits in sc.any are neighbours), and enters the prefix further up where it
+// begins an item.
+__global__ void __launch_bounds__(256) part_up_kernel(LevelInfo li, PrefixMapView pm, BuildScratch sc, int n, int* status) {
+  const unsigned q_count = (unsigned)li.mult[n], q = blockIdx.x * 256 + threadIdx.x, t0 = blockIdx.y * 64;
+  if (q >= q_count) return;
+  const int nt = min(64, li.T[n] - (int)t0);
+  unsigned long long word = 0;
+#pragma unroll 16
+  for (int t = 0; t < nt; ++t) {
+    const unsigned p = q + (t0 + t) * q_count;
+    word |= (unsigned long long)((sc.any[p >> 5] >> (p & 31)) & 1u) << t;
+  }
+  pm.slots[pm.level_off[n] + (unsigned long long)q * pm.set_words + blockIdx.y] = word;
+  if (!word) return;
+  unsigned p = q;
+  int r = 1;
+  for (int lv = n - 1; lv >= 0 && r > 0; --lv) {        // (as in set_build_kernel)
+    const unsigned c = p / (unsigned)li.mult[lv];
+    p -= c * (unsigned)li.mult[lv];
+    r = pm_add(pm, lv, p, (int)c, false);
+  }
+  if (r < 0) atomicOr(status, kStHashFull);
 }
 
 // A thread answers kProbeKeysPerThread keys: it loads them (coalesced: thread t of the block takes keys t, t + 256, ...),
@@ -194,9 +513,65 @@ __global__ void __launch_bounds__(256) hs_probe_kernel(HashSetView hs, const uns
   }
 }
 
+// Fills in the sizes of a build by parts, or leaves on = 0 where it does not apply (wide keys, a hashed region, more than
+// kBuildMaxParts parts) or does not pay: its eight launches and its passes over all counters cost some 40 us, so it starts at
+// 1.5M items; a region of less than 16 MB has too few parts for the chip.  One pass -> by parts, us: 0.6M items 68 -> 92, 1M
+// 81 -> 96 (8 MB) and 90 -> 103 (17 MB), 1.2M 104 -> 104 (34 MB), 2M 129 -> 117 (17 MB), 4M 228 -> 176 (34 MB) and 192 -> 179
+// (8 MB), 12M 672 -> 366 (34 MB).
+// (A part is at most 64 KB, so that three blocks of an SM overlap their phases.)
+constexpr unsigned long long kBuildMinItems = 3ull << 19, kBuildMinRegion = 16ull << 20;
+void plan_build(const LevelInfo& li, HashSetView hs, PrefixMapView pm, unsigned long long n, BuildScratch* sc) {
+  *sc = BuildScratch{};
+  if (li.L < 2 || !hs.narrow || n < kBuildMinItems || n >= 1ull << 31) return;
+  for (int l = 0; l < li.L; ++l)
+    if (pm.level_slots[l] != 0) return;                  // (a direct longest region means that the shorter ones are direct too)
+  const unsigned long long prefixes = li.mult[li.L - 1];
+  if (prefixes * pm.set_words * 8 < kBuildMinRegion) return;
+  auto deal = [](unsigned long long things, int bytes_each, BuildDeal* dl) {
+    while ((2ull << dl->shift) * bytes_each <= 64u << 10) ++dl->shift;
+    const unsigned long long parts = (things + (1ull << dl->shift) - 1) >> dl->shift;
+    dl->parts = (int)(parts <= kBuildMaxParts ? parts : 0);
+    return dl->parts != 0;
+  };
+  sc->on = deal(prefixes, pm.set_words * 8, &sc->by_prefix) && deal(hs.n_buckets, kBucketBytes, &sc->by_bucket);
+}
+
 // Clears both tables and enters the n items; *n_unique = how many of them are distinct.
-void launch_set_build(const LevelInfo& li, HashSetView hs, PrefixMapView pm, const int* codes, unsigned long long n,
-                      unsigned long long* n_unique, int* status, int n_sm, cudaStream_t st) {
+void launch_set_build(const LevelInfo& li, HashSetView hs, PrefixMapView pm, const BuildScratch& sc, const int* codes,
+                      unsigned long long n, unsigned long long* n_unique, int* status, int n_sm, cudaStream_t st) {
+  const bool vec = codes_vec(li, codes);
+  if (sc.on) {
+    const int last = li.L - 1;
+    const unsigned prefixes = (unsigned)li.mult[last], run = (unsigned)((n + kBuildBlocks - 1) / kBuildBlocks);
+    const KeySplit split{prefixes, nextafterf((float)(1.0 / (double)prefixes), 0.f)};
+    const DealPrefix by_prefix{split, sc.by_prefix.shift};
+    const DealBucket by_bucket{(unsigned)hs.n_buckets, sc.by_bucket.shift};
+    const int both = sc.by_prefix.parts + sc.by_bucket.parts;
+    const int bits_bytes = (1 << sc.by_prefix.shift) * pm.set_words * 8 + (1 << sc.by_prefix.shift) / 8;
+    const int slots_bytes = kBucketBytes << sc.by_bucket.shift;
+    // the packed keys wait in the hash set's slots, which are at least as many as the items, until they have been dealt out twice
+    unsigned* keys = reinterpret_cast<unsigned*>(hs.slots);
+    auto go = [&](auto kernel, dim3 grid, int threads, int bytes, auto... args) {
+      if (bytes > 48 << 10) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+      LaunchScope ls(kcHash, st);
+      kernel<<<grid, threads, bytes, st>>>(args...);
+    };
+    auto deal = [&](auto kernel, const BuildDeal& dl, auto part_of) {
+      go(kernel, kBuildBlocks, 1024, (kDealKeys + 2 * dl.parts) * 4, dl, part_of, (const unsigned*)sc.n_valid, (unsigned)n, run, (const unsigned*)keys, sc.keys);
+    };
+    // (the longest region is the last, and written whole)
+    cudaMemsetAsync(sc.by_prefix.count, 0, (size_t)(both + 2) * sizeof(unsigned), st);
+    go(vec ? part_count_kernel<true> : part_count_kernel<false>, kBuildBlocks, 1024, both * 4, li, hs, pm, sc, by_bucket, codes,
+       (unsigned)n, run, keys, n_unique, status);
+    go(part_scan_kernel, 2, 1024, 0, sc);
+    deal(part_deal_kernel<DealPrefix>, sc.by_prefix, by_prefix);
+    go(part_bits_kernel, sc.by_prefix.parts, 512, bits_bytes, pm, sc, last, split, n_unique);
+    go(part_up_kernel, dim3((unsigned)((li.mult[last - 1] + 255) / 256), (li.T[last - 1] + 63) / 64), 256, 0, li, pm, sc, last - 1, status);
+    deal(part_deal_kernel<DealBucket>, sc.by_bucket, by_bucket);
+    go(part_slots_kernel, sc.by_bucket.parts, 512, slots_bytes, hs, sc);
+    go(part_over_kernel, (sc.by_bucket.parts + 7) / 8, 256, 0, hs, sc, status);
+    return;
+  }
   cudaMemsetAsync(n_unique, 0, sizeof(unsigned long long), st);
   cudaMemsetAsync(hs.slots, 0xff, (size_t)hs.n_buckets * kBucketBytes, st);
   cudaMemsetAsync(hs.slots + hs.n_buckets * (kBucketBytes / 8), 0, kBucketBytes, st);      // the special word (HashSetView)
@@ -206,7 +581,7 @@ void launch_set_build(const LevelInfo& li, HashSetView hs, PrefixMapView pm, con
   const unsigned long long blocks = (n + 255) / 256;
   const unsigned grid = (unsigned)(blocks < 8ull * n_sm ? blocks : 8ull * n_sm);
   auto go = [&](auto kernel) { kernel<<<grid, 256, 0, st>>>(li, hs, pm, codes, n, n_unique, status); };
-  if (codes_vec(li, codes)) { if (hs.narrow) go(set_build_kernel<true, true>); else go(set_build_kernel<true, false>); }
+  if (vec) { if (hs.narrow) go(set_build_kernel<true, true>); else go(set_build_kernel<true, false>); }
   else { if (hs.narrow) go(set_build_kernel<false, true>); else go(set_build_kernel<false, false>); }
 }
 void launch_hs_pack(const LevelInfo& li, const int* codes, unsigned long long n, unsigned long long* keys, int* status,
