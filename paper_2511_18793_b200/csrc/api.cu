@@ -322,12 +322,13 @@ int gemm_fused(nezha_ctx* c, const void* A, long long lda, const void* W, void* 
   return N / 32;
 }
 
-// How much of the gate/up weights the output projection's launch asks for ahead, where it streams its weights: HBM is idle
-// while that launch waits for the attention kernel, and its own weights are few.  A call of one request on the 16-layer
-// d = 2048 backbone (64 MB of gate/up weights), drafted / verified: 873 / 2313 us without, 862 / 2272 with 8 MB, 850 / 2246
-// with 16, 845 / 2239 with 24, 849 / 2245 with 40, 874 / 2277 with all of them (they then delay the projection's own).  The
-// QKV launch asking ahead (gate/up weights, beyond the attention) or the gate/up launch (down weights): nothing, or slower.
-constexpr long long kNextWeights = 24LL << 20;
+// How far the output projection's launch reads ahead, where it streams its weights: its own and, asked for into L2, the head of
+// the gate/up weights.  HBM is idle while that launch waits for the attention kernel, but only so long.  A call of one request
+// on the 16-layer d = 2048 backbone (8 MB of its own, 64 MB of gate/up weights), drafted / verified: 873 / 2313 us without, 862 /
+// 2272 with 8 MB, 850 / 2246 with 16, 845 / 2239 with 24, 849 / 2245 with 40, 874 / 2277 with all of them.  d = 3584, 28 layers
+// (26 MB of its own): 8.64 ms without or with 6 MB, 8.75 with 24.  The QKV launch asking ahead (gate/up weights, beyond the
+// attention) or the gate/up launch (down weights): nothing, or slower.
+constexpr long long kNextWeights = 32LL << 20;
 
 // The layers of the primary model on the fused path.  On entry resid holds the embeddings, xn = embedding * gain of
 // the first attention norm and ss_e the rows' sums of squares (launch_embed_norm).  Five kernels per layer:
@@ -366,10 +367,12 @@ void run_layers_fused(nezha_ctx* c, long long M, const int* M_dev, bool verify, 
     t.ext_req_stride = t.ext_positions * t.ext_pos_stride; t.ext_rows_total = (long long)c->Bmax * t.ext_positions;
     if (attention_tc_supported(t)) launch_attention_tc(t, c->st);
     else launch_attention_simt(t, true, c->st);
+    const long long own_weights = 2LL * c->d * c->Hq * c->hd, 
+                    ahead = std::max(0LL, std::min(kNextWeights - own_weights, 4LL * c->F * c->d));
     GemmFuse fo{};
     fo.xg = c->xn; fo.gain = w.mlp_norm; fo.ss_out = c->ss_a;
     const int parts_a = gemm_fused(c, c->attn, (long long)c->Hq * c->hd, w.wo, c->resid, c->d, M, M_dev, c->d, c->Hq * c->hd,
-                                   kEpiAddNorm, nullptr, 0, &fo, w.w_gu, std::min(kNextWeights, 4LL * c->F * c->d));
+                                   kEpiAddNorm, nullptr, 0, &fo, w.w_gu, ahead);
     gemm_fused(c, c->xn, c->d, w.w_gu, c->act, c->F, M, M_dev, 2 * c->F, c->d, kEpiSwiGLU, c->ss_a, parts_a, nullptr);
     GemmFuse fd{};
     fd.xg = c->xn; fd.gain = (i + 1 < c->nl) ? c->layers[i + 1].attn_norm : c->final_norm; fd.ss_out = c->ss_b;
