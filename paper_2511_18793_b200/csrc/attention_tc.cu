@@ -85,7 +85,8 @@ struct AttnCfg {
 };
 
 // SPLIT: blockIdx.x = KV head * cluster size + rank, a power of two of at most 8 CTAs per cluster; RW = 1.
-template <int HD, int RW, int KW, bool SPLIT>
+// VERIFY: a verify pass (a.n_ext_max > 0), as opposed to a causal prompt pass.
+template <int HD, int RW, int KW, bool SPLIT, bool VERIFY>
 __global__ void __launch_bounds__(AttnCfg<HD, RW, KW>::kThreads) attn_tc_kernel(const __grid_constant__ CUtensorMap tmK,
                                                                                const __grid_constant__ CUtensorMap tmV,
                                                                                const __grid_constant__ CUtensorMap tmKx,
@@ -98,8 +99,11 @@ __global__ void __launch_bounds__(AttnCfg<HD, RW, KW>::kThreads) attn_tc_kernel(
   constexpr int NB = HD / 8;                        // n-blocks of the output
   constexpr int kRows = 16 * RW;
 
-  pdl_wait();                                       // before the first global read and before any exit
-  pdl_launch();
+  // A verify pass reads nothing of the launch before, the QKV projection, but q and the draft positions' K and V: the tables
+  // and the context cache are older, and complete, because that launch lets this one start only when its own wait is over.
+  // So only those wait here; the barriers, the tables and the first context tiles do not: 5.9 -> 3.6 us per launch at 40 rows of
+  // 37 positions (and 5.1 -> 4.5 for the prompt form, which this takes out of).
+  if constexpr (!VERIFY) { pdl_wait(); pdl_launch(); }
   // the row tile is the slowest grid index: tiles beyond a request's rows (the grid covers the largest row count a
   // call may have) are scheduled after every tile that has work, instead of holding its place in the first wave
   // (a causal prefill has no such tiles to speak of, and its last tiles see the most context: those go first)
@@ -109,13 +113,16 @@ __global__ void __launch_bounds__(AttnCfg<HD, RW, KW>::kThreads) attn_tc_kernel(
     asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
   }
   const int req_local = blockIdx.y, kvh = SPLIT ? (int)(blockIdx.x / n_split) : (int)blockIdx.x;
-  const int tile = a.n_ext_max > 0 ? (int)blockIdx.z : (int)(gridDim.z - 1 - blockIdx.z);
+  const int tile = VERIFY ? (int)blockIdx.z : (int)(gridDim.z - 1 - blockIdx.z);
   const int G = a.Hq / a.Hkv;
-  const int4 info = a.req_info[req_local];          // {first token, token count, cache row, context length or -1}
+  const int4 info = VERIFY ? __ldcg(a.req_info + req_local) : a.req_info[req_local];   // {first token, token count, cache row, context length or -1}
   const int tok0 = info.x, n_tok = info.y, request = info.z;
   const int R = n_tok * G;                          // query rows of this (request, kv head)
   const int r0 = tile * kRows;
-  if (r0 >= R) return;                              // (all CTAs of a cluster alike)
+  if (r0 >= R) {                                    // (all CTAs of a cluster alike)
+    if constexpr (VERIFY) { pdl_wait(); pdl_launch(); }
+    return;
+  }
   // context positions this tile needs: all of them, or (causal prefill) up to its last token's own position
   const int max_ctx = info.w >= 0 ? info.w : min((r0 + kRows - 1) / G, n_tok - 1) + 1;
   const int n_tiles = (max_ctx + kPos - 1) / kPos;
@@ -123,7 +130,7 @@ __global__ void __launch_bounds__(AttnCfg<HD, RW, KW>::kThreads) attn_tc_kernel(
   // head) follow the context as n_xt more tiles of the same loop; a query row sees only its own ancestors and itself
   // among them, through a per-row bit mask.  Rows nobody sees are finite (the cache is zeroed when the engine is made),
   // so their P = 0 contributes exactly nothing.
-  const int n_xt = a.n_ext_max > 0 ? (a.ext_positions + kPos - 1) / kPos : 0;
+  const int n_xt = VERIFY ? (a.ext_positions + kPos - 1) / kPos : 0;
   // this CTA's share of the tiles: all, or the cluster's in order of rank
   const int t0 = SPLIT ? (int)((n_tiles + n_xt) * rank / n_split) : 0;
   const int NT = (SPLIT ? (int)((n_tiles + n_xt) * (rank + 1) / n_split) : n_tiles + n_xt) - t0;
@@ -158,9 +165,10 @@ __global__ void __launch_bounds__(AttnCfg<HD, RW, KW>::kThreads) attn_tc_kernel(
     // ------------------------------------------------------------------ TMA producer
     const uint32_t leader = elect_one();
     int t = 0;
-    bool ok = true;
+    bool ok = true, waited = !VERIFY;
     for (; t < NT; ++t) {
       const int s = t % S;
+      if (!waited && (t >= S || t0 + t >= n_tiles)) { pdl_wait(); waited = true; }
       if (t >= S && !warp_wait_uniform(empty_bar(s), ((t / S) - 1) & 1, abort_flag)) { ok = false; break; }
       mbar_expect_tx_if(full_bar(s), C::kStageBytes, leader);
       // a context tile, or 64 draft positions of [positions, kv heads * hd]: this head's columns
@@ -190,6 +198,16 @@ __global__ void __launch_bounds__(AttnCfg<HD, RW, KW>::kThreads) attn_tc_kernel(
       head[i] = kvh * G + rr % G;
       ctx[i] = !live[i] ? 0 : (info.w >= 0 ? info.w : rr / G + 1);
     }
+    int xpos[2][kMaxLevels];                        // the rows' visible draft positions inside the request's block, or -1
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+      for (int e = 0; e < kMaxLevels; ++e) {
+        long long off = -1;
+        if (VERIFY && live[i] && e < a.n_ext_max) off = __ldcg(a.tok_ext + (long long)tok[i] * a.n_ext_max + e);
+        xpos[i][e] = off >= 0 ? (int)((off - (long long)request * a.ext_req_stride) / a.ext_pos_stride) : -1;
+      }
+    if constexpr (VERIFY) { pdl_wait(); pdl_launch(); }
     // Q fragments (A operand): a0 = (qr, k0..1), a1 = (qr+8, k0..1), a2 = (qr, k8..9), a3 = (qr+8, k8..9)
     uint32_t qf[KS][4];
     {
@@ -207,16 +225,6 @@ __global__ void __launch_bounds__(AttnCfg<HD, RW, KW>::kThreads) attn_tc_kernel(
 #pragma unroll
     for (int j = 0; j < NB; ++j) { o[j][0] = o[j][1] = o[j][2] = o[j][3] = 0.f; }
     const int ctx_min = __reduce_min_sync(0xffffffffu, min(ctx[0], ctx[1]));   // tiles below it need no masking
-    int xpos[2][kMaxLevels];                        // the rows' visible draft positions inside the request's block, or -1
-#pragma unroll
-    for (int i = 0; i < 2; ++i)
-#pragma unroll
-      for (int e = 0; e < kMaxLevels; ++e) {
-        long long off = -1;
-        if (live[i] && e < a.n_ext_max) off = a.tok_ext[(long long)tok[i] * a.n_ext_max + e];
-        xpos[i][e] = off >= 0 ? (int)((off - (long long)request * a.ext_req_stride) / a.ext_pos_stride) : -1;
-      }
-
     for (int tl = g; tl < NT; tl += KW) {
       const int s = tl % S, t = t0 + tl;
       const bool got = mbar_wait_or_abort(full_bar(s), (tl / S) & 1, abort_flag);
@@ -242,7 +250,7 @@ __global__ void __launch_bounds__(AttnCfg<HD, RW, KW>::kThreads) attn_tc_kernel(
       }
       // ---- mask (only tiles that reach past some row's context), online softmax in base 2
       // rows qr and qr+8; columns j*8 + qc*2 + {0,1}
-      if (t >= n_tiles) {                            // a tile of draft positions: each row's own mask
+      if (VERIFY && t >= n_tiles) {                  // a tile of draft positions: each row's own mask
         unsigned long long mk[2] = {0ull, 0ull};
 #pragma unroll
         for (int i = 0; i < 2; ++i)
@@ -427,12 +435,12 @@ __global__ void __launch_bounds__(AttnCfg<HD, RW, KW>::kThreads) attn_tc_kernel(
 }
 
 // splits > 1: the SPLIT form in clusters of that many CTAs.
-template <int HD, int RW, int KW, bool SPLIT = false>
-void launch(const CUtensorMap* tk, const CUtensorMap* tv, const AttnArgs& a, cudaStream_t st, int splits = 1) {
+template <int HD, int RW, int KW, bool SPLIT, bool VERIFY>
+void launch_form(const CUtensorMap* tk, const CUtensorMap* tv, const AttnArgs& a, cudaStream_t st, int splits) {
   using C = AttnCfg<HD, RW, KW>;
   static PerDeviceOnce configured;
   configured.run([] {
-    cudaFuncSetAttribute(attn_tc_kernel<HD, RW, KW, SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes);
+    cudaFuncSetAttribute(attn_tc_kernel<HD, RW, KW, SPLIT, VERIFY>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes);
   });
   const int G = a.Hq / a.Hkv;
   dim3 grid(a.Hkv * splits, a.n_rows, (a.max_tokens_per_row * G + 16 * RW - 1) / (16 * RW));
@@ -461,7 +469,12 @@ void launch(const CUtensorMap* tk, const CUtensorMap* tv, const AttnArgs& a, cud
     ++n;
   }
   cfg.attrs = at; cfg.numAttrs = n;
-  cudaLaunchKernelEx(&cfg, attn_tc_kernel<HD, RW, KW, SPLIT>, *tk, *tv, tkx, tvx, a, a.status);
+  cudaLaunchKernelEx(&cfg, attn_tc_kernel<HD, RW, KW, SPLIT, VERIFY>, *tk, *tv, tkx, tvx, a, a.status);
+}
+template <int HD, int RW, int KW, bool SPLIT = false>
+void launch(const CUtensorMap* tk, const CUtensorMap* tv, const AttnArgs& a, cudaStream_t st, int splits = 1) {
+  if (a.n_ext_max > 0) launch_form<HD, RW, KW, SPLIT, true>(tk, tv, a, st, splits);
+  else launch_form<HD, RW, KW, SPLIT, false>(tk, tv, a, st, splits);
 }
 
 }  // namespace
