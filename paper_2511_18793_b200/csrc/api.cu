@@ -317,7 +317,7 @@ int gemm_fused(nezha_ctx* c, const void* A, long long lda, const void* W, void* 
   a.f.ss_in = ss_in; a.f.ss_in_parts = ss_parts; a.f.ss_ld = c->Ms; a.f.inv_dim = 1.f / (float)c->d; a.f.eps = c->cfg.rms_eps;
   a.M_expected = c->m_expected;
   a.skinny = c->skinny_now;
-  a.next_w = next_w; a.next_w_bytes = next_w_bytes;
+  a.next_w = next_w; a.next_w_bytes = next_w_bytes; a.early = 1;
   launch_gemm_tc(a, c->st);
   return N / 32;
 }
@@ -367,7 +367,7 @@ void run_layers_fused(nezha_ctx* c, long long M, const int* M_dev, bool verify, 
     t.ext_req_stride = t.ext_positions * t.ext_pos_stride; t.ext_rows_total = (long long)c->Bmax * t.ext_positions;
     if (attention_tc_supported(t)) launch_attention_tc(t, c->st);
     else launch_attention_simt(t, true, c->st);
-    const long long own_weights = 2LL * c->d * c->Hq * c->hd, 
+    const long long own_weights = 2LL * c->d * c->Hq * c->hd,
                     ahead = std::max(0LL, std::min(kNextWeights - own_weights, 4LL * c->F * c->d));
     GemmFuse fo{};
     fo.xg = c->xn; fo.gain = w.mlp_norm; fo.ss_out = c->ss_a;

@@ -35,9 +35,11 @@ struct LaunchScope {
 // programmatic dependent launch: the kernels of the decode path are launched so that a kernel may be scheduled, and
 // run the part of its prologue that touches no global memory, while its predecessor in the stream is still finishing
 // --------------------------------------------------------------------------------------------------
-// EVERY thread block of a kernel launched with launch_pdl must execute pdl_wait() before its first global memory
-// access and before it exits (a block that exits without waiting lets the grid "complete" while its predecessor is
-// still running, and the grid after it would then start too early).  pdl_wait() returns once the preceding grid has
+// EVERY thread block of a kernel launched with launch_pdl must execute pdl_wait() before it touches anything that the
+// preceding grid writes (or writes what that one reads), and before it exits (a block that exits without waiting lets the
+// grid "complete" while its predecessor is still running, and the grid after it would then start too early).  What is older
+// than the preceding grid may be read before, past the L1 (__ldcg, TMA): pdl_launch() always comes behind pdl_wait(), so when
+// a block starts, all grids but that one are complete.  pdl_wait() returns once the preceding grid has
 // completed and its writes are visible; pdl_launch() lets the following grid start being scheduled.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
@@ -301,6 +303,7 @@ struct GemmArgs {
   // Optional, and only a hint (the weight-streaming kernel heeds it, the others do not): constant data that the launch after
   // this one starts with, asked for into L2 while this launch waits for its predecessor.  16-byte aligned, a multiple of 16.
   const void* next_w; long long next_w_bytes;
+  int early;             // W is constant and M_dev older than the launch before this one: both may be read while that one still runs
 };
 
 void launch_gemm_simt(const GemmArgs& a, bool bf16, cudaStream_t st);
