@@ -6,8 +6,8 @@
 // A producer warp brings K/V tiles of 64 positions into a shared-memory ring with TMA (128-byte swizzle); RW x KW
 // consumer warps run S = Q K^T and O += P V on mma.sync m16n8k16 (fp32 accumulation) with an online softmax in
 // registers.  Two shapes of the same kernel:
-//   RW = 4, KW = 1   64 rows per CTA, every warp walks all tiles                       (many query rows per request)
-//   RW = 1, KW = 4   16 rows per CTA, the four warps take every fourth tile and their   (few rows: one beam set of a
+//   KW = 1           16 RW rows per CTA (RW 2 to 8), every warp walks all tiles        (many query rows per request)
+//   RW = 1, KW = 2   16 rows per CTA, the two warps take every second tile and their   (few rows: one beam set of a
 //                    softmax states are merged through shared memory at the end          small model, plain decode)
 // Where that leaves SMs idle -- few requests, whatever their context -- the tiles are also split over the CTAs of a cluster,
 // which merge their softmax states through distributed shared memory (SPLIT, see launch_attention_tc).
