@@ -31,7 +31,7 @@ sys.path.insert(0, os.path.join(ROOT, "tests"))
 METRIC, UNIT = "items_per_s_decoded", "items/s"
 # bumped whenever a kernel of the family changes in a way that can change its DRAM traffic: a traffic figure taken
 # from an older revision is reported as null
-KERNEL_REV = {"gemm": 7, "gemm_skinny": 2, "attention_tc": 3, "attention_umma": 5, "probe": 3}
+KERNEL_REV = {"gemm": 8, "gemm_skinny": 3, "attention_tc": 4, "attention_umma": 6, "probe": 4}
 # dram__bytes_read.sum + dram__bytes_write.sum per launch, averaged over the launches of the class in one decode step
 # (ncu, eager launches, L2 flushed before the step); key = class @ workload
 NCU_TRAFFIC = {
@@ -176,12 +176,13 @@ def probe_bench(args, w, eng, cat_dev, config, dev):
     gbs = n * 41.0 / (ms / 1e3) / 1e9
     rec = ncu_traffic(f"probe@{w.name}@{n}")
     traffic = rec["dram_bytes_per_launch"] if rec else None
-    slots = 4 * max(2, math.ceil(math.ceil(max(1, w.n_items) / w.load_factor) / 4))      # buckets of four 8-byte slots
+    slot_bytes = 4 if math.prod(w.T[: w.L]) <= 1 << 32 else 8                             # buckets of 32 bytes
+    slots = 32 // slot_bytes * max(2, math.ceil(math.ceil(max(1, w.n_items) / w.load_factor) / (32 // slot_bytes)))
     print(json.dumps({"metric": "hash_probes_per_s", "value": n / (ms / 1e3), "unit": "probes/s", "n_gpus": 1,
                       "steps": args.steps, "warmup": max(args.warmup, 3), "ms_per_step": ms, "higher_is_better": True,
                       "dtype": "u64", "data": "synthetic",
                       "config": {"workload": config["workload"], "keys": n, "hit_fraction": float(found.float().mean()),
-                                 "table_bytes": slots * 8, "l2": "keys alone (8 bytes each) exceed L2"},
+                                 "table_bytes": slots * slot_bytes, "l2": "keys alone (8 bytes each) exceed L2"},
                       "clocks": clocks, "gpu_launches": args.steps,
                       "roofline": {"kernel": "hs_probe_kernel", "bound": "hbm", "achieved": gbs, "peak": peaks["hbm_gbs"],
                                    "unit": "GB/s", "frac": gbs / peaks["hbm_gbs"], "traffic": traffic,

@@ -123,6 +123,12 @@ __global__ void __launch_bounds__(kSkinnyThreads, 2)
         mbar_expect_tx(full_bar(s), C::kStageBytes);
         tma_load_2d(base + s * C::kStageBytes, &tmW, (k_begin + s) * BK, n0, full_bar(s));
       }
+    // The down projection's next few k-steps into L2: the widest product by K behind the one that takes longest.  (4 steps, one
+    // request drafted / verified: 821 -> 816 / 2148 -> 2134 us; 16 steps: nothing; the gate/up and QKV launches asking too: slower.)
+    constexpr int kAhead = EPI == kEpiAddNorm ? 4 : 0;
+    if (kAhead > 0 && w_ahead)
+      for (int s = pre; s < min(k_count, pre + kAhead); ++s)
+        asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global.tile [%0, {%1, %2}];" ::"l"(&tmW), "r"((k_begin + s) * BK), "r"(n0) : "memory");
     // behind them, in shares of 8 KB, the head of the next launch's weights (see kNextWeights in api.cu)
     if (blockIdx.y == 0)
       for (long long o = (long long)blockIdx.x * 8192; o < a.next_w_bytes; o += (long long)gridDim.x * 8192) {
