@@ -213,13 +213,19 @@ class Engine:
         assert codes.dtype == torch.int32 and codes.dim() == 2 and codes.shape[1] == self.L
         assert codes.device == self.arena.device
         codes = codes.contiguous()
-        keys = torch.empty(codes.shape[0], dtype=torch.int64, device=codes.device)   # bit pattern of uint64
-        self._check(lib.nezha_pack(self._h, _ptr(codes), codes.shape[0], _ptr(keys)))
+        n = codes.shape[0]
+        keys = codes.new_empty(n, dtype=torch.int64)     # bit pattern of uint64 (new_empty: no device to look up and parse)
+        st = lib.nezha_pack(self._h, codes.data_ptr(), n, keys.data_ptr())
+        if st:
+            self._check(st)
         return keys
 
     def probe(self, keys: torch.Tensor, out: Optional[torch.Tensor] = None) -> torch.Tensor:
-        found = out if out is not None else torch.empty(keys.shape[0], dtype=torch.uint8, device=keys.device)
-        self._check(lib.nezha_probe(self._h, _ptr(keys), keys.shape[0], _ptr(found)))
+        n = keys.shape[0]
+        found = keys.new_empty(n, dtype=torch.uint8) if out is None else out
+        st = lib.nezha_probe(self._h, _ptr(keys), n, found.data_ptr() if out is None else _ptr(out))
+        if st:
+            self._check(st)
         return found
 
     def contains_noalloc(self, codes: torch.Tensor, found: torch.Tensor) -> torch.Tensor:
