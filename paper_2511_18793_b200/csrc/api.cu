@@ -16,7 +16,7 @@ namespace nz {
 void launch_hs_pack(const LevelInfo& li, const int* codes, unsigned long long n, unsigned long long* keys, int* status,
                     cudaStream_t st);
 void plan_build(const LevelInfo& li, HashSetView hs, PrefixMapView pm, unsigned long long n, BuildScratch* sc);
-void launch_set_build(const LevelInfo& li, HashSetView hs, PrefixMapView pm, const BuildScratch& sc, const int* codes,
+cudaError_t launch_set_build(const LevelInfo& li, HashSetView hs, PrefixMapView pm, const BuildScratch& sc, const int* codes,
                       unsigned long long n, unsigned long long* n_unique, int* status, int n_sm, cudaStream_t st);
 int sm_count();
 void launch_hs_probe(HashSetView hs, const unsigned long long* keys, unsigned long long n, uint8_t* found,
@@ -826,7 +826,8 @@ nezha_status nezha_create(const nezha_config* cfg, const nezha_weights* w, const
 
 nezha_status nezha_build_hashset(nezha_ctx* c, uint64_t* n_unique) {
   if (!c) return NEZHA_ERR_ARG;
-  launch_set_build(c->es.li, c->es.hs, c->es.pm, c->build, c->catalog, c->n_items, c->n_unique_dev, c->es.status, sm_count(), c->st);
+  NZ_CUDA(c, launch_set_build(c->es.li, c->es.hs, c->es.pm, c->build, c->catalog, c->n_items, c->n_unique_dev, c->es.status,
+                              sm_count(), c->st));
   // (into pinned memory: the copy is queued with the status word's, and one wait serves both)
   NZ_CUDA(c, cudaMemcpyAsync(c->host_counters, c->n_unique_dev, sizeof(unsigned long long), cudaMemcpyDeviceToHost, c->st));
   NZ_CUDA(c, cudaGetLastError());

@@ -537,7 +537,7 @@ void plan_build(const LevelInfo& li, HashSetView hs, PrefixMapView pm, unsigned 
 }
 
 // Clears both tables and enters the n items; *n_unique = how many of them are distinct.
-void launch_set_build(const LevelInfo& li, HashSetView hs, PrefixMapView pm, const BuildScratch& sc, const int* codes,
+cudaError_t launch_set_build(const LevelInfo& li, HashSetView hs, PrefixMapView pm, const BuildScratch& sc, const int* codes,
                       unsigned long long n, unsigned long long* n_unique, int* status, int n_sm, cudaStream_t st) {
   const bool vec = codes_vec(li, codes);
   if (sc.on) {
@@ -551,10 +551,14 @@ void launch_set_build(const LevelInfo& li, HashSetView hs, PrefixMapView pm, con
     const int slots_bytes = kBucketBytes << sc.by_bucket.shift;
     // the packed keys wait in the hash set's slots, which are at least as many as the items, until they have been dealt out twice
     unsigned* keys = reinterpret_cast<unsigned*>(hs.slots);
+    cudaError_t failed = cudaSuccess;
     auto go = [&](auto kernel, dim3 grid, int threads, int bytes, auto... args) {
-      if (bytes > 48 << 10) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+      // (the limit that needs no attribute, 48 KB, counts the kernel's static shared memory too)
+      if (bytes > 32 << 10) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
       LaunchScope ls(kcHash, st);
       kernel<<<grid, threads, bytes, st>>>(args...);
+      const cudaError_t e = cudaPeekAtLastError();
+      if (failed == cudaSuccess) failed = e;
     };
     auto deal = [&](auto kernel, const BuildDeal& dl, auto part_of) {
       go(kernel, kBuildBlocks, 1024, (kDealKeys + 2 * dl.parts) * 4, dl, part_of, (const unsigned*)sc.n_valid, (unsigned)n, run, (const unsigned*)keys, sc.keys);
@@ -570,19 +574,20 @@ void launch_set_build(const LevelInfo& li, HashSetView hs, PrefixMapView pm, con
     deal(part_deal_kernel<DealBucket>, sc.by_bucket, by_bucket);
     go(part_slots_kernel, sc.by_bucket.parts, 512, slots_bytes, hs, sc);
     go(part_over_kernel, (sc.by_bucket.parts + 7) / 8, 256, 0, hs, sc, status);
-    return;
+    return failed;
   }
   cudaMemsetAsync(n_unique, 0, sizeof(unsigned long long), st);
   cudaMemsetAsync(hs.slots, 0xff, (size_t)hs.n_buckets * kBucketBytes, st);
   cudaMemsetAsync(hs.slots + hs.n_buckets * (kBucketBytes / 8), 0, kBucketBytes, st);      // the special word (HashSetView)
   cudaMemsetAsync(pm.slots, 0, (size_t)pm.n_words * sizeof(unsigned long long), st);
-  if (!n) return;
+  if (!n) return cudaSuccess;
   LaunchScope ls(kcHash, st);
   const unsigned long long blocks = (n + 255) / 256;
   const unsigned grid = (unsigned)(blocks < 8ull * n_sm ? blocks : 8ull * n_sm);
   auto go = [&](auto kernel) { kernel<<<grid, 256, 0, st>>>(li, hs, pm, codes, n, n_unique, status); };
   if (vec) { if (hs.narrow) go(set_build_kernel<true, true>); else go(set_build_kernel<true, false>); }
   else { if (hs.narrow) go(set_build_kernel<false, true>); else go(set_build_kernel<false, false>); }
+  return cudaPeekAtLastError();
 }
 void launch_hs_pack(const LevelInfo& li, const int* codes, unsigned long long n, unsigned long long* keys, int* status,
                     cudaStream_t st) {

@@ -14,7 +14,9 @@ pytestmark = pytest.mark.gpu
 # (63, 61, 59, 37): 8,389,269 prefixes of one word in 1,025 parts, the last of 661 prefixes.  256^3: the most parts, 8,192.
 # (128, 128, 64): the smallest region, 16 MB in 256 parts.  1,572,864: the fewest items.
 @pytest.mark.parametrize("T,n,load_factor", [((63, 61, 59, 37, 50), 1_600_000, 0.25), ((63, 61, 59, 37, 50), 4_100_000, 0.95),
-                                             ((256,) * 4, 1_600_000, 0.1), ((240, 256, 256, 250), 1_572_864, 0.1),
+                                             ((256,) * 4, 1_600_000, 0.1),
+                                             ((256,) * 4, 2_013_000, 0.03),   # 8,192 + 4,096 counters: 48 KB to the byte
+                                             ((240, 256, 256, 250), 1_572_864, 0.1),
                                              ((128, 128, 64, 16), 1_572_864, 0.5), ((128, 128, 64, 16), 1_572_863, 0.5)])
 def test_build_by_parts(T, n, load_factor):
     from gpu_helpers import Case
