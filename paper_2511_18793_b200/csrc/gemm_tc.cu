@@ -241,6 +241,10 @@ void launch_bn(const GemmArgs& a, cudaStream_t st) {
 // 4096 rows, N 512 to 22016, K 512 to 11008): the plan it picks is 0.6 % behind the best of each on average, the table of
 // relative wave costs it replaces was 6 % (4096 rows x 896 x 896 14.4 -> 10.8 us, 2048 x 8192 at 200 rows 28 -> 23).  The tiling
 // never changes the order in which a product's K range is summed, so it may depend on the row count.
+// Beyond the fitted rows the pairs are taken unless the model has them 30 % behind: there launches are long and run back to back
+// at the power cap, where a pair's lighter shared-memory traffic is clock.  Whole prompt passes of the 24-layer d = 896
+// backbone, by the model alone / with pairs at 10 % / at 30 %: 6.5 k rows 6.37 / 6.08 / 6.05 ms, 7.7 k 7.41 / 7.03 / 7.02,
+// 9.6 k 9.46 / 9.40 / 8.83, 23 k 21.1 / 20.9 / 20.9.  From 1,024 rows on: decodes of 2.6 k rows 2 % faster or 1 % slower.
 constexpr int kPlanPairs = 512;
 int gemm_tc_plan(int M, int N, int K) {
   static const bool no_pairs = getenv("NEZHA_NO_CTA_PAIRS") != nullptr;
@@ -263,7 +267,7 @@ int gemm_tc_plan(int M, int N, int K) {
     const long long pairs = sm_count() / 2;
     const long long tiles = ((M + 2 * BM - 1) / (2 * BM)) * (long long)((N + 255) / 256);
     const long long cost = kPairFixedNs + (tiles + pairs - 1) / pairs * (k_iters * kPairStepNs + kTailNs);
-    if (cost < best) { best = cost; plan = kPlanPairs; }
+    if (M > 4096 ? 10 * cost < 13 * best : cost < best) { best = cost; plan = kPlanPairs; }
   }
   return plan;
 }
