@@ -700,7 +700,11 @@ nezha_status decode_impl(nezha_ctx* c, int batch, int K, int mode, const int* dr
     rs = run_segment(c, key_of(queued, queued), [&] { run_round(queued); });
   }
   if (mode != NEZHA_MODE_DRAFT) c->rounds_seen[mode] = sd.rounds;
-  if (tr.beams || tr.beam_scores) launch_trace_beams(e, batch, K, tr, c->st);
+  if (tr.beams || tr.beam_scores) {                // (the call promises that its outputs are there when it returns)
+    launch_trace_beams(e, batch, K, tr, c->st);
+    NZ_CUDA(c, cudaStreamSynchronize(c->st));
+    NZ_CUDA(c, cudaGetLastError());
+  }
   if (stats) *stats = sd;
   return device_error(c, queued > 0 ? c->host_counters + 16 + 8 * queued + 4 : c->host_counters + 8);
 }

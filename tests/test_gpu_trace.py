@@ -1,0 +1,28 @@
+"""What a traced decode call leaves in the trace's beam sets, and when."""
+import pytest
+import torch
+
+from paper_2511_18793_b200 import binding, synth
+from gpu_helpers import Case
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("mode", [binding.MODE_VERIFIED, binding.MODE_AR])
+def test_trace_is_complete_when_the_call_returns(mode):
+    """The call synchronises: nothing of it is left on the engine's stream, and another stream may read the trace at once."""
+    w = synth.scaled(synth.WORKLOADS["tiny"], n_layers=1, L=8, T=(16,) * 8, batch=512, beam=128, n_hist=1)   # 17 MB of beam sets
+    st, other = torch.cuda.Stream(), torch.cuda.Stream()
+    case = Case(w, stream=st).prefill()
+    out = case.eng.alloc_outputs(w.batch, w.beam, trace=True)
+    beams = out["trace"]["beams"]
+    for _ in range(4):                       # eager, captured, replayed
+        beams.fill_(-7)
+        torch.cuda.synchronize()
+        case.eng.decode(w.beam, mode=mode, out=out)
+        assert st.query()
+        with torch.cuda.stream(other):
+            seen = beams.clone()
+        torch.cuda.synchronize()
+        assert torch.equal(seen, beams) and (beams >= -1).all().item()
+    case.eng.close()
