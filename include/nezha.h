@@ -97,6 +97,7 @@ typedef struct {
   int32_t* accepted_len;         /* device [R, batch, beam]     largest i with D[k][1..i] in B_i            */
   int32_t* level_reached;        /* device [R, batch]           level m the row had settled after the round */
   int32_t* beams;                /* device [L, batch, beam, L]  the true beam sets B_1..B_L, -1 padded      */
+                                 /*                             (beams, beam_scores: left alone in mode 0)  */
   float*   beam_scores;          /* device [L, batch, beam]                                                 */
   int32_t* tree_codes;           /* device [R, L, batch, beam, L]  the round's draft tree: nodes of level j  */
                                  /*                             (j codes each) at index j - 1, -1 padded      */

@@ -700,9 +700,10 @@ nezha_status decode_impl(nezha_ctx* c, int batch, int K, int mode, const int* dr
     rs = run_segment(c, key_of(queued, queued), [&] { run_round(queued); });
   }
   if (mode != NEZHA_MODE_DRAFT) c->rounds_seen[mode] = sd.rounds;
-  if (tr.beams || tr.beam_scores) {                // (the call promises that its outputs are there when it returns)
+  // (mode 0 has no true beam sets: what the tables hold is an earlier call's)
+  if (mode != NEZHA_MODE_DRAFT && (tr.beams || tr.beam_scores)) {
     launch_trace_beams(e, batch, K, tr, c->st);
-    NZ_CUDA(c, cudaStreamSynchronize(c->st));
+    NZ_CUDA(c, cudaStreamSynchronize(c->st));      // (the call promises that its outputs are there when it returns)
     NZ_CUDA(c, cudaGetLastError());
   }
   if (stats) *stats = sd;

@@ -26,3 +26,18 @@ def test_trace_is_complete_when_the_call_returns(mode):
         torch.cuda.synchronize()
         assert torch.equal(seen, beams) and (beams >= -1).all().item()
     case.eng.close()
+
+
+def test_draft_mode_leaves_the_true_beam_sets_alone():
+    """Mode 0 has no true beam sets: an earlier call's are not handed out as its own."""
+    w = synth.scaled(synth.WORKLOADS["small"], n_layers=1, n_items=20_000, batch=3, n_hist=5)
+    case = Case(w).prefill()
+    case.eng.decode(w.beam, mode=binding.MODE_VERIFIED)
+    out = case.eng.alloc_outputs(w.batch, w.beam, trace=True)
+    for t in out["trace"].values():
+        t.fill_(-7)
+    torch.cuda.synchronize()
+    case.eng.decode(w.beam, mode=binding.MODE_DRAFT, out=out)
+    for name, t in out["trace"].items():
+        assert (t == (-7 if name in ("beams", "beam_scores") else -1)).all().item(), name
+    case.eng.close()
