@@ -201,9 +201,10 @@ size_t carve(nezha_ctx* c) {
       total += total & 1;                    // (16-byte boundaries)
       e.pm.level_off[n] = total;
       e.pm.level_slots[n] = direct ? 0 : (unsigned long long)slots;
+      e.pm.level_keys[n] = direct ? (unsigned long long)prefixes : 0;
       total += direct ? (unsigned long long)prefixes * e.pm.set_words : (unsigned long long)slots * e.pm.stride;
     }
-    for (int n = g.L; n < kMaxLevels; ++n) { e.pm.level_off[n] = 0; e.pm.level_slots[n] = 0; }
+    for (int n = g.L; n < kMaxLevels; ++n) { e.pm.level_off[n] = 0; e.pm.level_slots[n] = 0; e.pm.level_keys[n] = 0; }
     e.pm.n_words = total;
     e.pm.slots = cv.take<unsigned long long>(e.pm.n_words);
   }

@@ -202,13 +202,15 @@ struct PrefixMapView {
   int stride, set_words;           // words per slot (a power of two >= 1 + set_words); words per bit set, ceil(max T / 64)
   unsigned long long level_off[kMaxLevels];     // first word of the region of prefixes with n codes
   unsigned long long level_slots[kMaxLevels];   // its slot count; 0 = direct
+  unsigned long long level_keys[kMaxLevels];    // direct: the prefixes it has bit sets for
 };
 // The bit set of a prefix of n codes, or null (an empty set counts as none) if no valid ID begins with it.  Every lane of a
 // warp may call this with the same key (the loads are then broadcasts).
 __device__ __forceinline__ const unsigned long long* pm_find(const PrefixMapView& pm, int n, unsigned long long prefix_key) {
   const unsigned long long ns = pm.level_slots[n];
   const unsigned long long* region = pm.slots + pm.level_off[n];
-  if (ns == 0) return region + prefix_key * pm.set_words;
+  // (nezha_select takes a caller's codes as they are: a key beyond the code space begins no valid ID)
+  if (ns == 0) return prefix_key < pm.level_keys[n] ? region + prefix_key * pm.set_words : nullptr;
   unsigned long long s = __umul64hi(hs_mix(prefix_key), ns);
   for (int step = 0; step < kMaxProbeBuckets; ++step) {
     const unsigned long long* slot = region + s * pm.stride;
