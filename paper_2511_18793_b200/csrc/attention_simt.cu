@@ -40,6 +40,7 @@ __global__ void __launch_bounds__(128) attn_simt_kernel(AttnArgs a) {
         vv[u][j] = kp[u] ? to_f32(vp[u][j]) : 0.f;
       }
     float m_new = m_run;
+    bool any = false;
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       s[u] = 0.f;
@@ -48,9 +49,9 @@ __global__ void __launch_bounds__(128) attn_simt_kernel(AttnArgs a) {
       s[u] += __shfl_xor_sync(0xffffffffu, s[u], 1);
       s[u] += __shfl_xor_sync(0xffffffffu, s[u], 2);
       s[u] += __shfl_xor_sync(0xffffffffu, s[u], 4);
-      if (kp[u]) m_new = fmaxf(m_new, s[u]);
+      if (kp[u]) { m_new = fmaxf(m_new, s[u]); any = true; }
     }
-    if (m_new == -INFINITY) return;                // (nothing seen yet; the same in the group's 8 lanes)
+    if (!any) return;                              // (the same in the group's 8 lanes; scores that are not numbers, or -inf, go on)
     const float corr = (m_run == -INFINITY) ? 0.f : expf(m_run - m_new);
     l_run *= corr;
 #pragma unroll
