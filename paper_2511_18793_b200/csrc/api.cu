@@ -336,7 +336,7 @@ constexpr long long kNextWeights = 32LL << 20;
 // QKV projection (+ norm scale, rotary embedding, KV append) -> attention -> output projection (+ residual, next
 // norm input) -> gate/up projection (+ norm scale, SwiGLU) -> down projection (+ residual, next norm input).
 // On exit xn = resid * final-norm gain and *ss_out / *parts_out describe its row scale.
-void run_layers_fused(nezha_ctx* c, long long M, const int* M_dev, bool verify, int n_rows, int max_tok_per_row,
+void run_layers_fused(nezha_ctx* c, long long M, const int* M_dev, bool verify, int n_rows, int max_tok_per_row, int rule_tok,
                       const float** ss_out, int* parts_out) {
   const EngineState& e = c->es;
   const size_t esz = c->esz;
@@ -360,7 +360,8 @@ void run_layers_fused(nezha_ctx* c, long long M, const int* M_dev, bool verify, 
     t.M = (int)M; t.M_dev = M_dev; t.Hq = c->Hq; t.Hkv = c->Hkv; t.hd = c->hd; t.scale = 1.f / sqrtf((float)c->hd);
     t.row_start = verify ? e.row_tok_start : e.pf_row_start; t.row_count = verify ? e.row_tok_count : e.pf_row_count;
     t.req_info = verify ? e.req_info : e.pf_req_info;
-    t.n_rows = n_rows; t.max_tokens_per_row = max_tok_per_row;
+    t.n_rows = n_rows; t.max_tokens_per_row = max_tok_per_row; t.rule_rows = rule_tok * (c->Hq / c->Hkv);
+    t.rule_rows_most = verify ? t.rule_rows * (c->L - 1) : t.rule_rows;
     t.ctx_bound = verify ? c->ctx_bound : max_tok_per_row;
     t.rows_expected = (c->m_expected > 0 && n_rows > 0) ? (c->m_expected + n_rows - 1) / n_rows * (c->Hq / c->Hkv) : 0;
     t.ctx_rows_total = (long long)c->Bmax * c->Hkv * c->S; t.status = e.status;
@@ -386,7 +387,7 @@ void run_layers_fused(nezha_ctx* c, long long M, const int* M_dev, bool verify, 
 // One pass of the primary model's layers over the tokens described by es.tok_* (resid already holds the
 // embeddings).  verify = false: prefill (KV goes to the context cache, tokens see a causal prefix of it);
 // verify = true: drafted codes (KV goes to the draft region, tokens see the whole context + their own tuple).
-void run_layers(nezha_ctx* c, long long M, const int* M_dev, bool verify, int n_rows, int max_tok_per_row) {
+void run_layers(nezha_ctx* c, long long M, const int* M_dev, bool verify, int n_rows, int max_tok_per_row, int rule_tok) {
   const EngineState& e = c->es;
   const size_t esz = c->esz;
   for (int i = 0; i < c->nl; ++i) {
@@ -413,7 +414,8 @@ void run_layers(nezha_ctx* c, long long M, const int* M_dev, bool verify, int n_
     t.M = (int)M; t.M_dev = M_dev; t.Hq = c->Hq; t.Hkv = c->Hkv; t.hd = c->hd; t.scale = 1.f / sqrtf((float)c->hd);
     t.row_start = verify ? e.row_tok_start : e.pf_row_start; t.row_count = verify ? e.row_tok_count : e.pf_row_count;
     t.req_info = verify ? e.req_info : e.pf_req_info;
-    t.n_rows = n_rows; t.max_tokens_per_row = max_tok_per_row;
+    t.n_rows = n_rows; t.max_tokens_per_row = max_tok_per_row; t.rule_rows = rule_tok * (c->Hq / c->Hkv);
+    t.rule_rows_most = verify ? t.rule_rows * (c->L - 1) : t.rule_rows;
     t.ctx_bound = verify ? c->ctx_bound : max_tok_per_row;
     t.ctx_rows_total = (long long)c->Bmax * c->Hkv * c->S; t.status = e.status;
     t.ext_positions = (c->L > 1 ? c->L - 1 : 1) * c->Kmax; t.ext_pos_stride = (long long)c->Hkv * c->hd;
@@ -431,20 +433,22 @@ void run_layers(nezha_ctx* c, long long M, const int* M_dev, bool verify, int n_
 }
 
 // The verify pass proper: embeddings of the node tokens, all layers, final norm, LM head of levels 2..L.
-void verify_pass(nezha_ctx* c, long long M_bound, int n_rows, int max_tok_per_row) {
+// n_rows requests of at most max_tok_per_row tokens, `beams` of them on each of their levels.
+void verify_pass(nezha_ctx* c, int n_rows, int max_tok_per_row, int beams) {
   const EngineState& e = c->es;
+  const long long M_bound = (long long)n_rows * max_tok_per_row;
   if (M_bound <= 0 || c->L < 2) return;
   const char* w = (const char*)c->lm_head + (size_t)e.li.off[1] * c->d * c->esz;
   if (c->fused) {
     launch_embed_norm(c->embed, e.tok_id, (int)M_bound, e.n_tokens, c->d, c->resid, c->layers[0].attn_norm, c->xn, c->ss_e,
                       c->st);
     const float* ss; int parts;
-    run_layers_fused(c, M_bound, e.n_tokens, true, n_rows, max_tok_per_row, &ss, &parts);
+    run_layers_fused(c, M_bound, e.n_tokens, true, n_rows, max_tok_per_row, beams, &ss, &parts);
     gemm_fused(c, c->xn, c->d, w, c->logits_v, c->Nv, M_bound, e.n_tokens, c->Nv, c->d, kEpiStoreF32, ss, parts, nullptr);
     return;
   }
   launch_embed(c->embed, c->bf16, e.tok_id, (int)M_bound, e.n_tokens, c->d, c->resid, c->st);
-  run_layers(c, M_bound, e.n_tokens, true, n_rows, max_tok_per_row);
+  run_layers(c, M_bound, e.n_tokens, true, n_rows, max_tok_per_row, beams);
   launch_rmsnorm(c->resid, c->d, nullptr, c->final_norm, c->bf16, c->xn, nullptr, (int)M_bound, e.n_tokens, c->d,
                  c->cfg.rms_eps, c->st);
   gemm(c, c->xn, c->d, w, c->d, c->logits_v, c->Nv, M_bound, e.n_tokens, c->Nv, c->d, kEpiStoreF32);
@@ -652,7 +656,7 @@ nezha_status decode_impl(nezha_ctx* c, int batch, int K, int mode, const int* dr
     else if (round == 1 && drafts) launch_draft_set(e, batch, K, drafts, n_draft, c->st);
     else draft_phase(c, batch, K, round == 1, round == 1 ? 1 : round + 1, c->opt_filter != 0);
     launch_build_nodes(e, batch, c->st);
-    verify_pass(c, (long long)batch * K * (L - round), batch, K * (L - round));
+    verify_pass(c, batch, K * (L - round), K);
     for (int n = round; n < L; ++n) {
       SelectArgs s = select_base(c, batch, K);
       const size_t lv_in = (size_t)n * c->Bmax * c->Kmax, lv_out = (size_t)(n + 1) * c->Bmax * c->Kmax;
@@ -876,10 +880,10 @@ nezha_status nezha_prefill(nezha_ctx* c, const int32_t* hist_codes, const int32_
     if (c->fused) {
       launch_embed_norm(c->embed, e.tok_id, (int)M, e.pf_n_tokens, c->d, c->resid, c->layers[0].attn_norm, c->xn, c->ss_e, c->st);
       const float* ss; int parts;
-      run_layers_fused(c, M, e.pf_n_tokens, false, rows, S_call, &ss, &parts);
+      run_layers_fused(c, M, e.pf_n_tokens, false, rows, S_call, S_call, &ss, &parts);
     } else {
       launch_embed(c->embed, c->bf16, e.tok_id, (int)M, e.pf_n_tokens, c->d, c->resid, c->st);
-      run_layers(c, M, e.pf_n_tokens, false, rows, S_call);
+      run_layers(c, M, e.pf_n_tokens, false, rows, S_call, S_call);
     }
     const size_t ho = (size_t)b0 * (c->L + 1) * c->d;
     launch_rmsnorm(c->resid, c->d, c->h_rows, c->final_norm, c->bf16, (char*)c->h_act + ho * c->esz, c->h_f32 + ho,
@@ -967,7 +971,7 @@ nezha_status nezha_primary_logits(nezha_ctx* c, int32_t batch, int32_t n_beams, 
     launch_copy_logits(c->logits0, c->cfg.T[0], 0, nullptr, 1, 0, batch, n_beams, 0, c->cfg.T[0], logits, c->st);
   } else {
     launch_nodes_from_prefixes(e, batch, n_beams, level, prefixes, c->st);
-    verify_pass(c, (long long)batch * n_beams * level, batch, n_beams * level);
+    verify_pass(c, batch, n_beams * level, n_beams);
     launch_copy_logits(c->logits_v, c->Nv, e.li.off[level] - e.li.off[1], e.node_index + (size_t)level * c->Kmax, 0, 0, batch,
                        n_beams, c->L * c->Kmax, c->cfg.T[level], logits, c->st);
   }

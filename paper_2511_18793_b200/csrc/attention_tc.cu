@@ -499,7 +499,8 @@ void launch_attention_tc(const AttnArgs& a, cudaStream_t st) {
   }
   const CUtensorMap *tk = &tk_map, *tv = &tv_map;
   LaunchScope ls(kcAttention, st);
-  // Query rows per (request, KV head): the bound the grid must cover, and what the caller expects (shapes the tile only).
+  // Query rows per (request, KV head): the bound the grid must cover, and what the caller expects (shapes the tile only; the
+  // forms that sum in different orders are chosen by rule_rows and rule_rows_most).
   const int G = a.Hq / a.Hkv;
   const long long r_bound = (long long)a.max_tokens_per_row * G;
   const long long r = a.rows_expected > 0 && a.rows_expected < r_bound ? a.rows_expected : r_bound;
@@ -509,28 +510,34 @@ void launch_attention_tc(const AttnArgs& a, cudaStream_t st) {
   // without / with the split: 7B shape, one request of 1,853 positions 10.3 -> 9.9 / 8.5 ms; 1.5B shape, two of 601 9.5 -> 9.1
   // / 8.9; 0.5B shape, five of 361 3.94 -> 3.56 / 3.62; 1B-sized backbone, one of 37 2.50 -> 2.38 ms (no split: a cluster
   // costs 2 us a launch).
-  const long long ctas = (long long)a.Hkv * a.n_rows * ((r + 15) / 16);
+  const long long ctas = (long long)a.Hkv * a.n_rows * ((a.rule_rows + 15) / 16);
   const int tiles = (a.ctx_bound + kPos - 1) / kPos + (a.n_ext_max > 0 ? (a.ext_positions + kPos - 1) / kPos : 0);
+  // (by the rows of a whole draft tree: going by one level's, a tree of two requests on the 7B shape was split in two, 4.15 -> 4.65 ms)
+  const long long ctas_most = (long long)a.Hkv * a.n_rows * ((a.rule_rows_most + 15) / 16);
   int splits = tiles >= 24 ? 8 : tiles >= 10 ? 4 : 1;
-  while (splits > 1 && splits * ctas > 296) splits /= 2;
+  while (splits > 1 && splits * ctas_most > 296) splits /= 2;
   if (splits > 1) {
     if (a.hd == 64) launch<64, 1, 2, true>(tk, tv, a, st, splits); else launch<128, 1, 2, true>(tk, tv, a, st, splits);
     return;
   }
-  if (r <= 32 || (ctas <= 296 && a.ctx_bound > 0)) {  // 16-row CTAs whose two consumer warps split the KV tiles
+  // 16-row CTAs whose two consumer warps split the KV tiles: also where one level's beams are one such CTA.  From 64 rows on the
+  // tcgen05 kernel, 128 rows per CTA; in between the CTAs below.  64 requests, plain / natural drafts / a whole tree, us: small
+  // shape, 20 rows 737 / 1,115 / 477 (here: 791 / 1,174 / 528); 1B-sized backbone, 32 rows, natural / tree 3,578 / 2,403 (here:
+  // 3,628 / 2,503); 0.5B shape, 56 rows 3,934 / 4,433 / 2,187 (on tcgen05: 4,039 / 4,516 / 2,098).
+  if (a.rule_rows <= 16 || (ctas <= 296 && a.ctx_bound > 0)) {
     if (a.hd == 64) launch<64, 1, 2>(tk, tv, a, st); else launch<128, 1, 2>(tk, tv, a, st);
     return;
   }
   static const bool umma = getenv("NEZHA_NO_UMMA_ATTENTION") == nullptr;
-  if (umma && r >= 64) { launch_attention_umma(a, tk, tv, st); return; }   // many rows: the tcgen05 kernel, 128 rows per CTA
+  if (umma && a.rule_rows >= 64) { launch_attention_umma(a, tk, tv, st); return; }
   // otherwise the fewest CTAs of at most 128 rows, each as short as covers the rows: little padding, K/V streamed
   // as few times as possible
   const int groups = (int)((r + 15) / 16), n_ctas = (groups + 7) / 8;
-  const int rw = (groups + n_ctas - 1) / n_ctas;     // 3 .. 8 warps of 16 rows
+  const int rw = (groups + n_ctas - 1) / n_ctas;     // 1 .. 8 warps of 16 rows
 #define NZ_ATTN_CASE(RW_) \
   case RW_: if (a.hd == 64) launch<64, RW_, 1>(tk, tv, a, st); else launch<128, RW_, 1>(tk, tv, a, st); break;
   switch (rw) {
-    NZ_ATTN_CASE(3) NZ_ATTN_CASE(4) NZ_ATTN_CASE(5) NZ_ATTN_CASE(6) NZ_ATTN_CASE(7)
+    NZ_ATTN_CASE(1) NZ_ATTN_CASE(2) NZ_ATTN_CASE(3) NZ_ATTN_CASE(4) NZ_ATTN_CASE(5) NZ_ATTN_CASE(6) NZ_ATTN_CASE(7)
     default: if (a.hd == 64) launch<64, 8, 1>(tk, tv, a, st); else launch<128, 8, 1>(tk, tv, a, st); break;
   }
 #undef NZ_ATTN_CASE

@@ -360,6 +360,11 @@ struct AttnArgs {
   int n_rows, max_tokens_per_row;
   int ctx_bound;                                // most context positions any token sees (0 = unknown): tiling only
   int rows_expected;                            // 0, or the query rows per (request, kv head) the caller expects: tiling only
+  // What the choice among kernels of different summation orders goes by: the query rows per (request, kv head) of one level's
+  // beams, and of a whole draft tree (a prompt pass: both the longest prompt's).  Functions of the call's arguments alone, the
+  // same in every round and mode, unlike rows_expected, which earlier calls leave behind: a repeated call returns the same
+  // bits, and what one mode selects another verifies on the same sums.
+  int rule_rows, rule_rows_most;
   long long ctx_rows_total;                     // requests * kv heads * positions of the layer's context cache
   // the draft-token cache seen as positions: a request owns ext_positions consecutive positions (level-major, then beam
   // slot), ext_pos_stride elements apart (all KV heads of a position are adjacent), ext_req_stride elements per request
