@@ -33,6 +33,7 @@ bool gemm_tc_supported(const GemmArgs& a);
 void launch_gemm_tc(const GemmArgs& a, cudaStream_t st);
 bool attention_tc_supported(const AttnArgs& a);
 void launch_attention_tc(const AttnArgs& a, cudaStream_t st);
+int attention_split_max(int ctx_positions, int draft_positions);
 }  // namespace nz
 
 using namespace nz;
@@ -102,7 +103,7 @@ struct nezha_ctx {
   int device;               // the GPU that was current at nezha_create
   int state;                // 0 created, 1 hash set built, 2 prefilled
   int batch;                // prefilled batch
-  int ctx_bound;            // most context positions of a prefilled request
+  int split_max;            // attention_split_max of the prefilled requests' verify passes
   std::string err;
 };
 
@@ -362,7 +363,7 @@ void run_layers_fused(nezha_ctx* c, long long M, const int* M_dev, bool verify, 
     t.req_info = verify ? e.req_info : e.pf_req_info;
     t.n_rows = n_rows; t.max_tokens_per_row = max_tok_per_row; t.rule_rows = rule_tok * (c->Hq / c->Hkv);
     t.rule_rows_most = verify ? t.rule_rows * (c->L - 1) : t.rule_rows;
-    t.ctx_bound = verify ? c->ctx_bound : max_tok_per_row;
+    t.split_max = verify ? c->split_max : attention_split_max(max_tok_per_row, 0);
     t.rows_expected = (c->m_expected > 0 && n_rows > 0) ? (c->m_expected + n_rows - 1) / n_rows * (c->Hq / c->Hkv) : 0;
     t.ctx_rows_total = (long long)c->Bmax * c->Hkv * c->S; t.status = e.status;
     t.ext_positions = (c->L > 1 ? c->L - 1 : 1) * c->Kmax; t.ext_pos_stride = (long long)c->Hkv * c->hd;
@@ -416,7 +417,7 @@ void run_layers(nezha_ctx* c, long long M, const int* M_dev, bool verify, int n_
     t.req_info = verify ? e.req_info : e.pf_req_info;
     t.n_rows = n_rows; t.max_tokens_per_row = max_tok_per_row; t.rule_rows = rule_tok * (c->Hq / c->Hkv);
     t.rule_rows_most = verify ? t.rule_rows * (c->L - 1) : t.rule_rows;
-    t.ctx_bound = verify ? c->ctx_bound : max_tok_per_row;
+    t.split_max = verify ? c->split_max : attention_split_max(max_tok_per_row, 0);
     t.ctx_rows_total = (long long)c->Bmax * c->Hkv * c->S; t.status = e.status;
     t.ext_positions = (c->L > 1 ? c->L - 1 : 1) * c->Kmax; t.ext_pos_stride = (long long)c->Hkv * c->hd;
     t.ext_req_stride = t.ext_positions * t.ext_pos_stride; t.ext_rows_total = (long long)c->Bmax * t.ext_positions;
@@ -616,7 +617,7 @@ nezha_status decode_impl(nezha_ctx* c, int batch, int K, int mode, const int* dr
   if (trace) tr = *trace;
   nezha_decode_stats sd{};
   const int R = L - 1;
-  const uintptr_t opts = (uintptr_t)c->ctx_bound << 32 | (uintptr_t)(mode | c->opt_transition << 8 | c->opt_inputs << 12 | c->opt_filter << 16 | c->opt_mask << 20 |
+  const uintptr_t opts = (uintptr_t)c->split_max << 32 | (uintptr_t)(mode | c->opt_transition << 8 | c->opt_inputs << 12 | c->opt_filter << 16 | c->opt_mask << 20 |
                                      (is_tree ? 1 : 0) << 24 | c->opt_level_filter << 25 | c->opt_adaptive << 26);
   // A segment covers rounds first .. last (0 = the part before the rounds).
   auto key_of = [&](int first, int last) {
@@ -740,7 +741,7 @@ nezha_status nezha_create(const nezha_config* cfg, const nezha_weights* w, const
     return NEZHA_ERR_ARG;
   nezha_ctx* c = new nezha_ctx();
   c->cfg = *cfg; c->n_items = n_items; c->load_factor = load_factor; c->catalog = catalog_codes;
-  c->st = (cudaStream_t)cuda_stream; c->arena = nullptr; c->state = 0; c->batch = 0; c->ctx_bound = 0;
+  c->st = (cudaStream_t)cuda_stream; c->arena = nullptr; c->state = 0; c->batch = 0; c->split_max = 1;
   c->device = 0;
   if (cudaGetDevice(&c->device) != cudaSuccess) { delete c; return NEZHA_ERR_CUDA; }
   // the legacy default stream cannot be captured; NEZHA_NO_GRAPHS=1 keeps every launch eager
@@ -896,7 +897,7 @@ nezha_status nezha_prefill(nezha_ctx* c, const int32_t* hist_codes, const int32_
   c->skinny_now = 0;
   NZ_CUDA(c, cudaGetLastError());
   c->batch = batch;
-  c->ctx_bound = 1 + max_n * c->L;
+  c->split_max = attention_split_max(1 + max_n * c->L, (c->L - 1) * c->Kmax);
   c->state = 2;
   return NEZHA_OK;
 }

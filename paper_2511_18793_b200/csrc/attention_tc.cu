@@ -489,6 +489,13 @@ bool attention_tc_supported(const AttnArgs& a) {
   return true;
 }
 
+// How many CTAs may share a request's tiles, were there SMs enough.  All that the launches of a pass take from the length of the
+// histories, and coarse: a decode call's graph is kept for every value.
+int attention_split_max(int ctx_positions, int draft_positions) {
+  const int tiles = (ctx_positions + kPos - 1) / kPos + (draft_positions + kPos - 1) / kPos;
+  return tiles >= 24 ? 8 : tiles >= 10 ? 4 : 1;
+}
+
 void launch_attention_tc(const AttnArgs& a, cudaStream_t st) {
   // the whole context cache of the layer as one [requests * kv_heads * positions, hd] matrix
   const long long rows = (long long)a.ctx_rows_total;
@@ -511,10 +518,9 @@ void launch_attention_tc(const AttnArgs& a, cudaStream_t st) {
   // / 8.9; 0.5B shape, five of 361 3.94 -> 3.56 / 3.62; 1B-sized backbone, one of 37 2.50 -> 2.38 ms (no split: a cluster
   // costs 2 us a launch).
   const long long ctas = (long long)a.Hkv * a.n_rows * ((a.rule_rows + 15) / 16);
-  const int tiles = (a.ctx_bound + kPos - 1) / kPos + (a.n_ext_max > 0 ? (a.ext_positions + kPos - 1) / kPos : 0);
   // (by the rows of a whole draft tree: going by one level's, a tree of two requests on the 7B shape was split in two, 4.15 -> 4.65 ms)
   const long long ctas_most = (long long)a.Hkv * a.n_rows * ((a.rule_rows_most + 15) / 16);
-  int splits = tiles >= 24 ? 8 : tiles >= 10 ? 4 : 1;
+  int splits = a.split_max;
   while (splits > 1 && splits * ctas_most > 296) splits /= 2;
   if (splits > 1) {
     if (a.hd == 64) launch<64, 1, 2, true>(tk, tv, a, st, splits); else launch<128, 1, 2, true>(tk, tv, a, st, splits);
@@ -524,7 +530,7 @@ void launch_attention_tc(const AttnArgs& a, cudaStream_t st) {
   // tcgen05 kernel, 128 rows per CTA; in between the CTAs below.  64 requests, plain / natural drafts / a whole tree, us: small
   // shape, 20 rows 737 / 1,115 / 477 (here: 791 / 1,174 / 528); 1B-sized backbone, 32 rows, natural / tree 3,578 / 2,403 (here:
   // 3,628 / 2,503); 0.5B shape, 56 rows 3,934 / 4,433 / 2,187 (on tcgen05: 4,039 / 4,516 / 2,098).
-  if (a.rule_rows <= 16 || (ctas <= 296 && a.ctx_bound > 0)) {
+  if (a.rule_rows <= 16 || ctas <= 296) {
     if (a.hd == 64) launch<64, 1, 2>(tk, tv, a, st); else launch<128, 1, 2>(tk, tv, a, st);
     return;
   }

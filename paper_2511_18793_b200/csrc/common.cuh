@@ -358,7 +358,7 @@ struct AttnArgs {
   const int4* req_info;                         // [n_rows] {first token, token count, cache row, context length visible to
                                                 //  every token of the request, or -1: token j of the request sees j + 1}
   int n_rows, max_tokens_per_row;
-  int ctx_bound;                                // most context positions any token sees (0 = unknown): tiling only
+  int split_max;                                // attention_split_max of the positions that a token may see
   int rows_expected;                            // 0, or the query rows per (request, kv head) the caller expects: tiling only
   // What the choice among kernels of different summation orders goes by: the query rows per (request, kv head) of one level's
   // beams, and of a whole draft tree (a prompt pass: both the longest prompt's).  Functions of the call's arguments alone, the

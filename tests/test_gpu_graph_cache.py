@@ -1,0 +1,50 @@
+"""Which decode calls replay a captured graph, read off the CUDA runtime calls that they make."""
+import collections
+
+import pytest
+import torch
+from torch.profiler import ProfilerActivity, profile
+
+from paper_2511_18793_b200 import binding, synth
+from gpu_helpers import Case
+
+pytestmark = pytest.mark.gpu
+
+
+def _runtime_calls(call):
+    with profile(activities=[ProfilerActivity.CPU, ProfilerActivity.CUDA]) as p:
+        call()
+        torch.cuda.synchronize()
+    calls = collections.Counter(e.name for e in p.events() if e.name.startswith("cuda"))
+    if not calls:
+        pytest.skip("no activity records: another profiler holds the process")
+    return calls
+
+
+def _replayed(calls):
+    return calls["cudaGraphLaunch"] == 1 and calls["cudaGraphInstantiate"] == 0 and calls["cudaLaunchKernelExC"] == 0
+
+
+def _engines(**kw):
+    """The same engine twice: on a stream of its own, and on the default stream, which replays nothing."""
+    w = synth.scaled(synth.WORKLOADS["small"], n_layers=2, T=(16,) * 4, n_items=20_000, batch=2, beam=5, n_hist=100, **kw)
+    case = Case(w, stream=torch.cuda.Stream())
+    return case, Case(w, weights=case.weights, catalog=case.catalog, hist=case.hist)
+
+
+def test_histories_of_other_lengths_replay_the_same_graph():
+    case, eager = _engines()
+    out = case.eng.alloc_outputs(2, 5)
+    torch.cuda.synchronize()
+    for i, n in enumerate((100, 100, 100, 100, 99, 57, 100, 3)):
+        for c in (case, eager):
+            c.eng.prefill(c.hist_dev[:, :n], torch.full((2,), n, dtype=torch.int32, device="cuda"))
+        torch.cuda.synchronize()
+        calls = _runtime_calls(lambda: case.eng.decode(5, mode=binding.MODE_AR, out=out))
+        assert i < 3 or _replayed(calls), (n, calls)
+        want = eager.eng.decode(5, mode=binding.MODE_AR)
+        for k in ("codes", "scores", "count"):
+            assert torch.equal(out[k], want[k]), (n, k)
+        assert (out["count"] > 0).all().item()
+    case.eng.close()
+    eager.eng.close()
