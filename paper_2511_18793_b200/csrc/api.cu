@@ -85,8 +85,9 @@ struct nezha_ctx {
   BuildScratch build;
   int* host_counters;       // pinned
   // CUDA graphs of the decode segments (one per round), keyed by everything that shapes the launch sequence
-  struct Segment { int seen; cudaGraphExec_t exec; long long launches[kcCount]; };
-  std::map<std::vector<uintptr_t>, Segment> segments;
+  struct Segment { int seen; cudaGraphExec_t exec; long long launches[kcCount]; unsigned long long used; };
+  std::map<std::vector<uintptr_t>, Segment> segments;       // at most kMaxSegments, the least recently used go
+  unsigned long long segment_clock;
   bool use_graphs;
   int opt_transition, opt_inputs, opt_filter;   // nezha_set_option (ablations of the draft head)
   int opt_mask;             // nezha_set_option: 0 = the primary model's last-level mask probes the hash set, 1 (default) = it reads the prefix map
@@ -562,6 +563,9 @@ nezha_status pending_device_error(nezha_ctx* c) {
 }
 
 using SegmentKey = std::vector<uintptr_t>;
+// A program that keeps its result buffers needs a graph per request count, beam, mode and step of the token counts; one that does
+// not makes a new one with every buffer.
+constexpr size_t kMaxSegments = 256;
 // Runs one segment of a decode call (the part before the rounds and the rounds expected, or one round).  The launch sequence of a segment
 // is fixed by its key, so after one eager run it is captured into a CUDA graph and replayed from then on: one
 // launch per call instead of dozens, and no launch gaps between its kernels.  Eager when the stream cannot be
@@ -570,6 +574,14 @@ template <typename F>
 nezha_status run_segment(nezha_ctx* c, const SegmentKey& key, F&& body) {
   if (!c->use_graphs || profile_is_on()) { body(); return NEZHA_OK; }
   nezha_ctx::Segment& sg = c->segments[key];
+  sg.used = ++c->segment_clock;
+  if (c->segments.size() > kMaxSegments) {         // (its graph is not running: every decode call waits for its own)
+    auto oldest = c->segments.begin();
+    for (auto it = c->segments.begin(); it != c->segments.end(); ++it)
+      if (it->second.used < oldest->second.used) oldest = it;
+    if (oldest->second.exec) cudaGraphExecDestroy(oldest->second.exec);
+    c->segments.erase(oldest);
+  }
   if (sg.exec) {
     NZ_CUDA(c, cudaGraphLaunch(sg.exec, c->st));
     profile_add(sg.launches);

@@ -48,3 +48,30 @@ def test_histories_of_other_lengths_replay_the_same_graph():
         assert (out["count"] > 0).all().item()
     case.eng.close()
     eager.eng.close()
+
+
+def test_the_graphs_that_are_kept_are_bounded():
+    """A program that brings other result buffers to every call: the oldest graphs are given back."""
+    case, eager = _engines()
+    for c in (case, eager):
+        c.prefill()
+    counts = torch.zeros(300, 2, dtype=torch.int32, device="cuda")
+    out = case.eng.alloc_outputs(2, 5)
+    torch.cuda.synchronize()
+
+    def decode(i):
+        case.eng.decode(5, mode=binding.MODE_AR, out={**out, "count": counts[i]})
+
+    for i in range(300):
+        for _ in range(3 if i % 50 == 0 else 1):
+            decode(i)
+    want = eager.eng.decode(5, mode=binding.MODE_AR)
+    assert torch.equal(out["codes"], want["codes"]) and torch.equal(out["scores"], want["scores"])
+    assert torch.equal(counts, want["count"].expand(300, 2))
+    assert _replayed(_runtime_calls(lambda: decode(250)))                  # captured 50 buffers ago
+    assert not _replayed(_runtime_calls(lambda: decode(0)))                # 300 ago
+    decode(0)
+    assert _replayed(_runtime_calls(lambda: decode(0)))
+    assert torch.equal(counts[0], want["count"])
+    case.eng.close()
+    eager.eng.close()
