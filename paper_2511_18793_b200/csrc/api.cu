@@ -636,7 +636,7 @@ nezha_status decode_impl(nezha_ctx* c, int batch, int K, int mode, const int* dr
     SegmentKey k{(uintptr_t)first, (uintptr_t)last, (uintptr_t)batch, (uintptr_t)K, opts,
                  (uintptr_t)drafts, (uintptr_t)n_draft, (uintptr_t)out_codes, (uintptr_t)out_scores, (uintptr_t)out_count,
                  (uintptr_t)tr.drafts, (uintptr_t)tr.n_draft, (uintptr_t)tr.accepted_len, (uintptr_t)tr.level_reached,
-                 (uintptr_t)tr.beams ^ ((uintptr_t)tr.tree_codes << 1), (uintptr_t)tr.beam_scores ^ ((uintptr_t)tr.tree_count << 1)};
+                 (uintptr_t)tr.tree_codes, (uintptr_t)tr.tree_count};      // (the trace's beam sets are written behind the graphs)
     for (int r = first > 1 ? first : 1; r <= last; ++r) k.push_back((uintptr_t)c->m_seen[r]);   // shapes the round's tiling
     return k;
   };

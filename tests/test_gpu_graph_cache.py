@@ -75,3 +75,26 @@ def test_the_graphs_that_are_kept_are_bounded():
     assert torch.equal(counts[0], want["count"])
     case.eng.close()
     eager.eng.close()
+
+
+def test_calls_with_other_trace_buffers_are_told_apart():
+    """Trace buffers whose addresses differ in ways that cancel out in beams ^ 2 tree_codes."""
+    case, eager = _engines()
+    case.prefill()
+    R, L, S = 3, 4, 1 << 12                                                # a buffer is less than 4 KB
+    block = torch.empty(16 * S, dtype=torch.uint8, device="cuda")
+    base = -block.data_ptr() % (8 * S)
+    out = case.eng.alloc_outputs(2, 5, trace=True)
+
+    def at(offset, like):
+        return block[base + offset:base + offset + like.numel() * 4].view(torch.int32).view(like.shape)
+
+    for i in range(2):
+        trace = {**out["trace"], "beams": at(2 * S * i, out["trace"]["beams"]), "tree_codes": at(4 * S + S * i, out["trace"]["tree_codes"])}
+        for _ in range(4):
+            trace["tree_codes"].fill_(-7)
+            torch.cuda.synchronize()
+            case.eng.decode(5, mode=binding.MODE_VERIFIED, out={**out, "trace": trace})
+            assert (trace["tree_codes"] >= -1).all().item() and trace["tree_codes"].shape == (R, L, 2, 5, L)
+    case.eng.close()
+    eager.eng.close()
