@@ -557,7 +557,7 @@ cudaError_t launch_set_build(const LevelInfo& li, HashSetView hs, PrefixMapView 
       if (bytes > 32 << 10) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
       LaunchScope ls(kcHash, st);
       kernel<<<grid, threads, bytes, st>>>(args...);
-      const cudaError_t e = cudaPeekAtLastError();
+      const cudaError_t e = cudaGetLastError();      // (taken, so that the call after this one does not report it again)
       if (failed == cudaSuccess) failed = e;
     };
     auto deal = [&](auto kernel, const BuildDeal& dl, auto part_of) {
@@ -587,7 +587,7 @@ cudaError_t launch_set_build(const LevelInfo& li, HashSetView hs, PrefixMapView 
   auto go = [&](auto kernel) { kernel<<<grid, 256, 0, st>>>(li, hs, pm, codes, n, n_unique, status); };
   if (vec) { if (hs.narrow) go(set_build_kernel<true, true>); else go(set_build_kernel<true, false>); }
   else { if (hs.narrow) go(set_build_kernel<false, true>); else go(set_build_kernel<false, false>); }
-  return cudaPeekAtLastError();
+  return cudaGetLastError();
 }
 void launch_hs_pack(const LevelInfo& li, const int* codes, unsigned long long n, unsigned long long* keys, int* status,
                     cudaStream_t st) {
