@@ -129,7 +129,8 @@ nezha_status nezha_create(const nezha_config* cfg, const nezha_weights* weights,
 /* Eq. 4 + Eq. 5: pack every catalogue tuple into a 64-bit key (level 1 least significant) and insert it
  * into the open-addressing hash set.  Duplicated tuples are legal and counted once.
  *   n_unique  host out (may be NULL): number of distinct keys inserted.
- * Synchronises.  Errors: NEZHA_ERR_CATALOG (code out of range), NEZHA_ERR_HASH_FULL. */
+ * Synchronises.  Errors: NEZHA_ERR_CATALOG (code out of range), NEZHA_ERR_HASH_FULL, NEZHA_ERR_CUDA.  After a
+ * CUDA call of the build has failed there are no tables and no prefilled batch: calls that need them return NEZHA_ERR_STATE. */
 nezha_status nezha_build_hashset(nezha_ctx* ctx, uint64_t* n_unique);
 
 /* Eq. 4: pack code tuples (device int32 [n, L]) into keys (device uint64 [n]).  Asynchronous. */

@@ -849,16 +849,21 @@ nezha_status nezha_create(const nezha_config* cfg, const nezha_weights* w, const
 
 nezha_status nezha_build_hashset(nezha_ctx* c, uint64_t* n_unique) {
   if (!c) return NEZHA_ERR_ARG;
+  // Until every kernel is known to have run there are no tables: a build by parts keeps packed keys where the hash set's slots will be.
+  const int state = c->state;
+  c->state = 0;
   NZ_CUDA(c, launch_set_build(c->es.li, c->es.hs, c->es.pm, c->build, c->catalog, c->n_items, c->n_unique_dev, c->es.status,
                               sm_count(), c->st));
-  // (into pinned memory: the copy is queued with the status word's, and one wait serves both)
+  // (into pinned memory: the two copies wait once)
   NZ_CUDA(c, cudaMemcpyAsync(c->host_counters, c->n_unique_dev, sizeof(unsigned long long), cudaMemcpyDeviceToHost, c->st));
+  NZ_CUDA(c, cudaMemcpyAsync(c->host_counters + 8, c->es.status, 4 * sizeof(int), cudaMemcpyDeviceToHost, c->st));
+  NZ_CUDA(c, cudaStreamSynchronize(c->st));
   NZ_CUDA(c, cudaGetLastError());
-  nezha_status ps = pending_device_error(c);
+  c->state = state;
   if (n_unique) memcpy(n_unique, c->host_counters, sizeof(unsigned long long));
-  if (ps != NEZHA_OK) return ps;
-  if (c->state < 1) c->state = 1;
-  return NEZHA_OK;
+  const nezha_status ps = device_error(c, c->host_counters + 8);
+  if (ps == NEZHA_OK && c->state < 1) c->state = 1;
+  return ps;
 }
 
 nezha_status nezha_pack(nezha_ctx* c, const int32_t* codes, size_t n, uint64_t* keys) {

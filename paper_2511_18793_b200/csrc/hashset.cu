@@ -553,12 +553,12 @@ cudaError_t launch_set_build(const LevelInfo& li, HashSetView hs, PrefixMapView 
     unsigned* keys = reinterpret_cast<unsigned*>(hs.slots);
     cudaError_t failed = cudaSuccess;
     auto go = [&](auto kernel, dim3 grid, int threads, int bytes, auto... args) {
+      if (failed != cudaSuccess) return;
       // (the limit that needs no attribute, 48 KB, counts the kernel's static shared memory too)
       if (bytes > 32 << 10) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
       LaunchScope ls(kcHash, st);
       kernel<<<grid, threads, bytes, st>>>(args...);
-      const cudaError_t e = cudaGetLastError();      // (taken, so that the call after this one does not report it again)
-      if (failed == cudaSuccess) failed = e;
+      failed = cudaGetLastError();                   // (taken, so that the call after this one does not report it again)
     };
     auto deal = [&](auto kernel, const BuildDeal& dl, auto part_of) {
       go(kernel, kBuildBlocks, 1024, (kDealKeys + 2 * dl.parts) * 4, dl, part_of, (const unsigned*)sc.n_valid, (unsigned)n, run, (const unsigned*)keys, sc.keys);

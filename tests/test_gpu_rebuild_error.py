@@ -38,3 +38,23 @@ def test_the_next_calls_are_not_refused_too(n):
     assert case.eng.build_hashset() == case.n_unique
     assert case.eng.probe(keys).all().item()
     case.eng.close()
+
+
+@pytest.mark.parametrize("n", [5_000, 1_600_000])
+def test_no_call_reads_tables_whose_rebuild_failed(n):
+    T = (128, 128, 64, 16)
+    rng = np.random.default_rng(n)
+    cat = np.stack([rng.integers(0, t, size=n) for t in T], axis=1).astype(np.int32)
+    w = synth.scaled(synth.WORKLOADS["tiny"], L=4, T=T, n_items=n, batch=1, beam=2, n_hist=1)
+    case = Case(w, catalog=cat, hist=cat[:1, None]).prefill()
+    keys = case.eng.pack(case.cat_dev)
+    _refused_rebuild(case.eng)
+    for call in (lambda: case.eng.probe(keys), lambda: case.eng.decode(2), lambda: case.prefill()):
+        with pytest.raises(binding.NezhaError) as e:
+            call()
+        assert binding.STATUS_NAMES[e.value.status] == "ERR_STATE"
+    case.eng.build_hashset()
+    assert case.eng.probe(keys).all().item()
+    case.prefill()
+    case.eng.decode(2)
+    case.eng.close()
