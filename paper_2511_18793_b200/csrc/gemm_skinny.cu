@@ -106,10 +106,11 @@ __global__ void __launch_bounds__(kSkinnyThreads, 2)
   const int k_begin = split * k_base + min(split, k_rem), k_count = k_base + (split < k_rem ? 1 : 0);
   const int pre = min(STAGES, k_count);          // ring slots filled in the first round
   const int M_early = !a.early ? 0 : a.M_dev ? min(a.M, __ldcg(a.M_dev)) : a.M;
+  const bool idle = a.early && M_early <= 0;      // a round queued for nothing: no row, and nothing is read (see k_run)
   // (a.early: one L2 latency less behind the wait, four times a layer; decode of one request, d = 2048: 2169 -> 2149 us)
   // the weight tiles of the first round are constant data, so they may be fetched while the predecessor still runs: for the first
   // row tile, which always goes through with its copies, and for the others where the rows are known already
-  const bool w_ahead = blockIdx.y == 0 || m0 < M_early;
+  const bool w_ahead = (blockIdx.y == 0 && !idle) || m0 < M_early;
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) { mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), 1); }
@@ -130,7 +131,7 @@ __global__ void __launch_bounds__(kSkinnyThreads, 2)
       for (int s = pre; s < min(k_count, pre + kAhead); ++s)
         asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global.tile [%0, {%1, %2}];" ::"l"(&tmW), "r"((k_begin + s) * BK), "r"(n0) : "memory");
     // behind them, in shares of 8 KB, the head of the next launch's weights (see kNextWeights in api.cu)
-    if (blockIdx.y == 0)
+    if (blockIdx.y == 0 && !idle)
       for (long long o = (long long)blockIdx.x * 8192; o < a.next_w_bytes; o += (long long)gridDim.x * 8192) {
         const uint32_t bytes = (uint32_t)min(8192LL, a.next_w_bytes - o);
         asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"((const char*)a.next_w + o), "r"(bytes) : "memory");
@@ -148,7 +149,10 @@ __global__ void __launch_bounds__(kSkinnyThreads, 2)
   pdl_wait();
   pdl_launch();
   const int M = a.early ? M_early : a.M_dev ? min(a.M, *a.M_dev) : a.M;
-  const bool live = blockIdx.y == 0 || m0 < M;    // the same in all CTAs of a cluster
+  const bool live = (blockIdx.y == 0 && !idle) || m0 < M;     // the same in all CTAs of a cluster
+  // Without rows only the copies that are on their way are waited for (a surplus round of one request, 8 layers of d = 2048: 291 ->
+  // 132 us).
+  const int k_run = M > 0 ? k_count : pre;
   const int rows = max(0, min(MT, M - m0));       // rows of this tile that exist
   // units of the epilogue: unit u = columns n0 + 32 (u / quads) .., rows m0 + 4 (u % quads) ..
   const int ew = warp - 2, quads = (rows + 3) >> 2, col_groups = min(4, (a.N - n0) >> 5), units = col_groups * quads;
@@ -180,7 +184,7 @@ __global__ void __launch_bounds__(kSkinnyThreads, 2)
     }
     int s = 0;
     uint32_t round = 1;                          // parity bit of the round that k-step `pre` belongs to (pre = STAGES here)
-    for (int k = pre; k < k_count; ++k, ++issued) {
+    for (int k = pre; k < k_run; ++k, ++issued) {
       if (!warp_wait_uniform(empty_bar(s), round ^ 1u, abort_flag)) { ok = false; break; }
       const uint32_t fb = full_bar(s), dst = base + s * C::kStageBytes;
       mbar_expect_tx_if(fb, C::kStageBytes, leader);
@@ -199,7 +203,7 @@ __global__ void __launch_bounds__(kSkinnyThreads, 2)
     const uint64_t dw0 = smem_desc(base), dx0 = smem_desc(base + C::kTileBytesW);
     int s = 0;
     uint32_t round = 0;
-    for (int k = 0; k < k_count; ++k) {
+    for (int k = 0; k < k_run; ++k) {
       if (!warp_wait_uniform(full_bar(s), round, abort_flag)) { ok = false; break; }
       tc_fence_after();
       const uint64_t so = (uint64_t)(s * (C::kStageBytes >> 4));
