@@ -1,5 +1,6 @@
 """The catalogue's build by parts of the prefix map's longest region: both code loads, whole and partial last parts, repeated
-items, walks over the ends of parts, a rebuild, and a code outside its codebook."""
+items, walks over the ends of parts, a rebuild, and a code outside its codebook.
+The launch count tells which build ran."""
 import numpy as np
 import pytest
 import torch
@@ -35,6 +36,10 @@ def test_build_by_parts(T, n, load_factor):
     probes = np.concatenate([cat, near, np.stack([rng.integers(0, t, size=300_000) for t in T], axis=1).astype(np.int32)])
     want = V.contains(probes)
     keys = case.eng.pack(torch.from_numpy(probes).cuda())
+    case.eng.profile_read()
+    case.eng.build_hashset()
+    # eight launches by parts; one, for the whole catalogue, just below the least number of items
+    assert case.eng.profile_read()["hash"]["launches"] == (1 if n == 1_572_863 else 8)
     case.eng.set_option(4, 1)                                             # the filter at every level reads every region
     for _ in range(2):
         assert case.n_unique == len(np.unique(keys_cat))
