@@ -290,7 +290,7 @@ def time_decode(ctx, mode, drafts, steps, warmup, flush, dist, world, dev, barri
     # null when no capture matches the current kernel revision
     rec = ncu_traffic(f"{dom}@{w.name}")
     if rec and rec["family"] == "gemm_skinny" and w.batch * w.beam * max(1, w.L - 1) > 128:
-        rec = None                     # that capture is of the weight-streaming kernel: engines of at most 128 rows per pass
+        rec = None                     # that capture has every product in the weight-streaming kernel: at most 128 rows per pass
     if rec:
         roof["traffic"] = rec["dram_bytes_per_launch"]
         roof["traffic_source"] = rec["source"]

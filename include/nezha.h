@@ -156,7 +156,10 @@ nezha_status nezha_prefill(nezha_ctx* ctx, const int32_t* hist_codes, const int3
  *   stats       host out, may be NULL
  *   trace       optional per-round device outputs, may be NULL
  * batch must equal the prefilled batch; 1 <= beam_width <= cfg.max_beam.  Synchronises (modes 1 and 2 read a
- * "rows unfinished" counter once per round). */
+ * "rows unfinished" counter once per round).
+ * The same call on the same prefilled batch returns the same bits.  With bf16 storage a request's scores and hidden states
+ * also depend, within the roundings of that type, on the requests that share its calls: their number and the longest
+ * history choose among kernels that sum in different orders (fp32: they do not). */
 nezha_status nezha_decode(nezha_ctx* ctx, int32_t batch, int32_t beam_width, int32_t mode,
                           int32_t* out_codes, float* out_scores, int32_t* out_count,
                           nezha_decode_stats* stats, const nezha_trace* trace);
@@ -255,11 +258,11 @@ nezha_status nezha_select(nezha_ctx* ctx, int32_t batch, int32_t n_beams, int32_
  * storage type (device pointers, row-major, leading dimensions = K for A and W, N for C).
  *   epilogue 0: C (storage type) = acc;  1: C (float) = acc;  2: C (float) += acc;  3: C (float) = tanh(acc + bias[n])
  *   path     0: the engine's own choice; 1: CUDA-core kernel; 2: tcgen05 kernel (NEZHA_ERR_UNSUPPORTED if the shape
- *               is not covered: bf16 storage, K % 64 == 0, N % 32 == 0); 3: the tcgen05 kernel as the decode calls use
- *               it (the same as path 2); 4: the weight-streaming tcgen05 kernel that the
- *               decode calls of an engine with at most 128 rows per pass use (M <= 128; W is the 128-row MMA operand,
- *               the K range is split over CTAs and the parts are added in a fixed order that depends on N, K and
- *               the device only; W must not be written by work still in flight on the stream)
+ *               is not covered: bf16 storage, K % 64 == 0, N % 32 == 0); 3: the same as path 2; 4: the weight-streaming tcgen05
+ *               kernel as the decode calls of an engine use it whose passes have at most 128 rows (M <= 128 here; such
+ *               engines use it for every product, those of up to 640 rows where it pays.  W is the 128-row MMA operand,
+ *               the K range is split over CTAs and the parts are added in a fixed order that depends on N, K, the
+ *               engine's row class and the device; W must not be written by work still in flight on the stream)
  * Used by every projection of the primary model (Algorithm 1's model call), the LM head and the draft head
  * (Eq. 2-3).  Asynchronous. */
 nezha_status nezha_gemm(nezha_ctx* ctx, const void* A, const void* W, void* C, int32_t M, int32_t N, int32_t K,
@@ -298,7 +301,7 @@ nezha_status nezha_contains_noalloc(nezha_ctx* ctx, const int32_t* codes, size_t
 
 #define NEZHA_PROFILE_CLASSES 16
 /* Kernel classes, in index order: gemm, attention, select, norm, rope_append, embed, swiglu, draft_glue, nodes,
- * accept, hash, misc. */
+ * accept (no launch of its own: select does that step), hash, misc. */
 typedef struct {
   int64_t launches[NEZHA_PROFILE_CLASSES];   /* kernels launched per class since the last read                 */
   double  ms[NEZHA_PROFILE_CLASSES];         /* summed CUDA-event time per class (0 unless timing was enabled) */

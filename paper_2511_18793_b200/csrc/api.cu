@@ -97,7 +97,7 @@ struct nezha_ctx {
   int m_seen[kMaxLevels + 1];   // tokens each round of the last decode call processed, rounded up to a row tile
   // Weight-streaming products: the most rows a pass of this engine's decode calls may have where that is at most
   // kSkinnyClassRows, else 0.  Every product of a decode call is given this class (the choice of its kernel is per engine and
-  // product, so both decode modes compute the same bits).
+  // product, so both decode modes compute the same bits of a product).
   int skinny_class;
   int skinny_now;           // GemmArgs::skinny of the products being queued
   int rounds_seen[3];       // rounds the last decode call of each mode needed: that many are launched without waiting
@@ -619,7 +619,7 @@ nezha_status decode_impl(nezha_ctx* c, int batch, int K, int mode, const int* dr
   const EngineState& e = c->es;
   const int L = c->L;
   // Every product of a decode call is given the engine's row class: the choice of its kernel is per engine and product, never
-  // per launch, so that the speculative and the autoregressive mode, whose passes differ in size, compute the same bits.
+  // per launch, so that a product's bits are the same in the speculative and the autoregressive mode, whose passes differ in size.
   struct ClassScope {
     nezha_ctx* c;
     explicit ClassScope(nezha_ctx* c_) : c(c_) { c->skinny_now = c->skinny_class; }

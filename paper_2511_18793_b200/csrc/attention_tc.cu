@@ -6,7 +6,7 @@
 // A producer warp brings K/V tiles of 64 positions into a shared-memory ring with TMA (128-byte swizzle); RW x KW
 // consumer warps run S = Q K^T and O += P V on mma.sync m16n8k16 (fp32 accumulation) with an online softmax in
 // registers.  Two shapes of the same kernel:
-//   KW = 1           16 RW rows per CTA (RW 2 to 8), every warp walks all tiles        (many query rows per request)
+//   KW = 1           16 RW rows per CTA (RW 1 to 8), every warp walks all tiles        (many query rows per request)
 //   RW = 1, KW = 2   16 rows per CTA, the two warps take every second tile and their   (few rows: one beam set of a
 //                    softmax states are merged through shared memory at the end          small model, plain decode)
 // Where that leaves SMs idle -- few requests, whatever their context -- the tiles are also split over the CTAs of a cluster,
@@ -479,6 +479,7 @@ void launch(const CUtensorMap* tk, const CUtensorMap* tv, const AttnArgs& a, cud
 
 }  // namespace
 
+int sm_count();
 void launch_attention_umma(const AttnArgs& a, const CUtensorMap* tk, const CUtensorMap* tv, cudaStream_t st);
 
 bool attention_tc_supported(const AttnArgs& a) {
@@ -521,7 +522,7 @@ void launch_attention_tc(const AttnArgs& a, cudaStream_t st) {
   // (by the rows of a whole draft tree: going by one level's, a tree of two requests on the 7B shape was split in two, 4.15 -> 4.65 ms)
   const long long ctas_most = (long long)a.Hkv * a.n_rows * ((a.rule_rows_most + 15) / 16);
   int splits = a.split_max;
-  while (splits > 1 && splits * ctas_most > 296) splits /= 2;
+  while (splits > 1 && splits * ctas_most > 2 * sm_count()) splits /= 2;
   if (splits > 1) {
     if (a.hd == 64) launch<64, 1, 2, true>(tk, tv, a, st, splits); else launch<128, 1, 2, true>(tk, tv, a, st, splits);
     return;
@@ -530,7 +531,7 @@ void launch_attention_tc(const AttnArgs& a, cudaStream_t st) {
   // tcgen05 kernel, 128 rows per CTA; in between the CTAs below.  64 requests, plain / natural drafts / a whole tree, us: small
   // shape, 20 rows 737 / 1,115 / 477 (here: 791 / 1,174 / 528); 1B-sized backbone, 32 rows, natural / tree 3,578 / 2,403 (here:
   // 3,628 / 2,503); 0.5B shape, 56 rows 3,934 / 4,433 / 2,187 (on tcgen05: 4,039 / 4,516 / 2,098).
-  if (a.rule_rows <= 16 || ctas <= 296) {
+  if (a.rule_rows <= 16 || ctas <= 2 * sm_count()) {
     if (a.hd == 64) launch<64, 1, 2>(tk, tv, a, st); else launch<128, 1, 2>(tk, tv, a, st);
     return;
   }

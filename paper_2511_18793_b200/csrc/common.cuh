@@ -227,7 +227,7 @@ __device__ __forceinline__ bool pm_test(const unsigned long long* bits, int t) {
 
 // Plan and scratch of a build by parts (launch_set_build).  The items are dealt out twice: by runs of 2^shift prefixes of the
 // prefix map's longest region, and by runs of 2^shift buckets of the hash set.
-constexpr int kBuildBlocks = 148;         // blocks that share the catalogue out (one per SM)
+constexpr int kBuildBlocks = 148;         // blocks that share the catalogue out (one per SM of a B200; the scratch is laid out for them)
 constexpr int kBuildMaxParts = 8192;
 struct BuildDeal {
   int parts, shift;

@@ -353,8 +353,11 @@ int gemm_skinny_splits(int N, int K, int row_class, int n_sm) {
 
 // Up to 128 rows every product is bound by reading W, and this kernel keeps more of it in flight.  With more rows W is
 // shared by several row tiles and the general kernel's wider tiles win again -- except where its k-loop is the bound: one
-// CTA walks all of K at 0.1 to 0.2 us per k-step, however few tiles there are, while here K is split.  Measured at 256 / 512 rows, general -> this kernel: 2048 x 8192 41 -> 17 / 41 -> 34 us, 1536 x 8960 45 -> 17 /
-// 46 -> 31, 896 x 4864 17 -> 10 / 18 -> 13; but 16384 x 2048 21 -> 37 / 33 -> 66, 6144 x 4096 25 -> 36.
+// CTA walks all of K at 0.1 to 0.2 us per k-step, however few tiles there are, while here K is split.  One after another on cold
+// weights, 256 / 384 / 512 / 640 rows, general -> this kernel, us: 2048 x 8192 24 -> 17 / 25 -> 27 / 25 -> 21 / 30 -> 25; 1536 x
+// 8960 26 -> 17 / 25 -> 26 / 27 -> 28 / 27 -> 22; 896 x 4864 15 -> 9 / 16 -> 13 / 16 -> 13 / 16 -> 20; 2048 x 2048 9 -> 11 / 9 ->
+// 17 / ..; 16384 x 2048 20 -> 21 / 27 -> 36 / ..; 6144 x 4096 19 -> 28 / 19 -> 22 / ..  The rule takes the first at 256 rows, the
+// second to 384, the third at all four: the model of one class, not the best of each.
 bool gemm_skinny_applies(const GemmArgs& a, int n_sm) {
   if (!a.skinny || a.M > a.skinny || a.skinny > kSkinnyClassRows) return false;
   if (a.skinny <= kSkinnyRows) return true;
