@@ -58,13 +58,14 @@ struct LayerW { void *attn_norm, *wqkv, *wo, *mlp_norm, *w_gu, *w_down; };
 struct nezha_ctx {
   nezha_config cfg;
   bool bf16; size_t esz;
-  int d, hd, Hq, Hkv, F, nl, L, Bmax, Kmax, S, vocab, Tmax, Nv, qkv_dim;
+  int d, hd, Hq, Hkv, F, nl, L, Bmax, Kmax, S, vocab, Tmax, Nv, Nv_ld, qkv_dim;
   long long Ms, Mv_max; int chunk_rows;
   size_t n_items; double load_factor;
   const int32_t* catalog;
   cudaStream_t st;
   char* arena; size_t arena_bytes;
   // weights (arena copies)
+  int lm_head_rows;
   void *embed, *lm_head, *final_norm, *draft_logit[kMaxLevels], *draft_wse, *draft_b_f32;
   std::vector<LayerW> layers;
   // caches
@@ -169,6 +170,8 @@ size_t carve(nezha_ctx* c) {
   }
   c->vocab = li.vocab_codes + g.L + 1;
   c->Nv = li.vocab_codes - g.T[0];
+  c->fused = c->bf16 && (c->hd == 64 || c->hd == 128) && c->d % 64 == 0 && c->F % 64 == 0;
+  c->Nv_ld = c->fused ? (c->Nv + 31) / 32 * 32 : c->Nv;     // columns of the LM head's product: its epilogue writes 32 at a time
   c->Mv_max = (long long)c->Bmax * c->Kmax * (g.L > 1 ? g.L - 1 : 1);
   c->chunk_rows = (int)(16384 / c->S); if (c->chunk_rows < 1) c->chunk_rows = 1;
   if (c->chunk_rows > c->Bmax) c->chunk_rows = c->Bmax;
@@ -225,7 +228,8 @@ size_t carve(nezha_ctx* c) {
   // weights
   const size_t esz = c->esz;
   c->embed = cv.take_bytes((size_t)c->vocab * c->d * esz);
-  c->lm_head = cv.take_bytes((size_t)c->vocab * c->d * esz);
+  c->lm_head_rows = std::max(c->vocab, li.off[g.L > 1 ? 1 : 0] + c->Nv_ld);      // (the last columns' weights: the placeholders' and zeros)
+  c->lm_head = cv.take_bytes((size_t)c->lm_head_rows * c->d * esz);
   c->final_norm = cv.take_bytes((size_t)c->d * esz);
   c->layers.resize(c->nl);
   for (int i = 0; i < c->nl; ++i) {
@@ -260,11 +264,10 @@ size_t carve(nezha_ctx* c) {
   c->a_se = cv.take_bytes((size_t)c->Bmax * c->Kmax * 2 * c->d * esz);
   c->h_act = cv.take_bytes((size_t)c->Bmax * (c->L + 1) * c->d * esz);
   c->h_f32 = cv.take<float>((size_t)c->Bmax * (c->L + 1) * c->d);
-  c->logits_v = cv.take<float>((size_t)c->Mv_max * (c->Nv > 0 ? c->Nv : 1));
+  c->logits_v = cv.take<float>((size_t)c->Mv_max * (c->Nv_ld > 0 ? c->Nv_ld : 1));
   c->logits0 = cv.take<float>((size_t)c->Bmax * g.T[0]);
   c->logits_d = cv.take<float>((size_t)c->Bmax * c->Kmax * c->Tmax);
   c->h_rows = cv.take<int>((size_t)c->Bmax * (c->L + 1));
-  c->fused = c->bf16 && (c->hd == 64 || c->hd == 128) && c->d % 64 == 0 && c->F % 64 == 0;
   c->ss_a = c->ss_b = c->ss_e = nullptr;
   c->draft_u = c->draft_hl = c->draft_g = nullptr; c->draft_sact = nullptr;
   for (int l = 0; l < kMaxLevels; ++l) c->draft_wcat[l] = nullptr;
@@ -446,14 +449,14 @@ void verify_pass(nezha_ctx* c, int n_rows, int max_tok_per_row, int beams) {
                       c->st);
     const float* ss; int parts;
     run_layers_fused(c, M_bound, e.n_tokens, true, n_rows, max_tok_per_row, beams, &ss, &parts);
-    gemm_fused(c, c->xn, c->d, w, c->logits_v, c->Nv, M_bound, e.n_tokens, c->Nv, c->d, kEpiStoreF32, ss, parts, nullptr);
+    gemm_fused(c, c->xn, c->d, w, c->logits_v, c->Nv_ld, M_bound, e.n_tokens, c->Nv_ld, c->d, kEpiStoreF32, ss, parts, nullptr);
     return;
   }
   launch_embed(c->embed, c->bf16, e.tok_id, (int)M_bound, e.n_tokens, c->d, c->resid, c->st);
   run_layers(c, M_bound, e.n_tokens, true, n_rows, max_tok_per_row, beams);
   launch_rmsnorm(c->resid, c->d, nullptr, c->final_norm, c->bf16, c->xn, nullptr, (int)M_bound, e.n_tokens, c->d,
                  c->cfg.rms_eps, c->st);
-  gemm(c, c->xn, c->d, w, c->d, c->logits_v, c->Nv, M_bound, e.n_tokens, c->Nv, c->d, kEpiStoreF32);
+  gemm(c, c->xn, c->d, w, c->d, c->logits_v, c->Nv_ld, M_bound, e.n_tokens, c->Nv, c->d, kEpiStoreF32);
 }
 
 // Draft-head logits of level l (1-based) for every (request, beam slot): Eq. 2.
@@ -673,7 +676,7 @@ nezha_status decode_impl(nezha_ctx* c, int batch, int K, int mode, const int* dr
     for (int n = round; n < L; ++n) {
       SelectArgs s = select_base(c, batch, K);
       const size_t lv_in = (size_t)n * c->Bmax * c->Kmax, lv_out = (size_t)(n + 1) * c->Bmax * c->Kmax;
-      s.logits = c->logits_v; s.row_stride = c->Nv; s.col_off = e.li.off[n] - e.li.off[1];
+      s.logits = c->logits_v; s.row_stride = c->Nv_ld; s.col_off = e.li.off[n] - e.li.off[1];
       s.src_row = e.tb_src + lv_in; s.src_mul = 0;
       s.in_codes = e.tb_codes + lv_in * L; s.in_score = e.tb_score + lv_in; s.in_count = e.tb_count + (size_t)n * c->Bmax;
       s.n = n; s.T = c->cfg.T[n]; s.per_beam = s.T; s.filter = (n + 1 == L) ? 1 : 0;
@@ -793,6 +796,7 @@ nezha_status nezha_create(const nezha_config* cfg, const nezha_weights* w, const
        cudaMemsetAsync(c->v_ext, 0, (size_t)c->nl * c->ext_layer_elems * c->esz, st) == cudaSuccess;
   ok = ok && cp(c->embed, w->embed, (size_t)c->vocab * c->d * esz) && cp(c->lm_head, w->lm_head, (size_t)c->vocab * c->d * esz) &&
        cp(c->final_norm, w->final_norm, (size_t)c->d * esz);
+  ok = ok && cudaMemsetAsync((char*)c->lm_head + (size_t)c->vocab * c->d * esz, 0, (size_t)(c->lm_head_rows - c->vocab) * c->d * esz, st) == cudaSuccess;
   const size_t q_b = (size_t)c->Hq * c->hd * c->d * esz, kv_b = (size_t)c->Hkv * c->hd * c->d * esz, f_b = (size_t)c->F * c->d * esz;
   for (int i = 0; ok && i < c->nl; ++i) {
     LayerW& lw = c->layers[i];
@@ -990,7 +994,7 @@ nezha_status nezha_primary_logits(nezha_ctx* c, int32_t batch, int32_t n_beams, 
   } else {
     launch_nodes_from_prefixes(e, batch, n_beams, level, prefixes, c->st);
     verify_pass(c, batch, n_beams * level, n_beams);
-    launch_copy_logits(c->logits_v, c->Nv, e.li.off[level] - e.li.off[1], e.node_index + (size_t)level * c->Kmax, 0, 0, batch,
+    launch_copy_logits(c->logits_v, c->Nv_ld, e.li.off[level] - e.li.off[1], e.node_index + (size_t)level * c->Kmax, 0, 0, batch,
                        n_beams, c->L * c->Kmax, c->cfg.T[level], logits, c->st);
   }
   NZ_CUDA(c, cudaGetLastError());
