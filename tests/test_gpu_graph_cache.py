@@ -28,7 +28,10 @@ def _replayed(calls):
 def _engines(**kw):
     """The same engine twice: on a stream of its own, and on the default stream, which replays nothing."""
     w = synth.scaled(synth.WORKLOADS["small"], n_layers=2, T=(16,) * 4, n_items=20_000, batch=2, beam=5, n_hist=100, **kw)
-    case = Case(w, stream=torch.cuda.Stream())
+    st = torch.cuda.Stream()
+    with torch.cuda.stream(st):              # (the engine reads the weights on its stream)
+        case = Case(w, stream=st)
+    torch.cuda.synchronize()
     return case, Case(w, weights=case.weights, catalog=case.catalog, hist=case.hist)
 
 
@@ -37,8 +40,10 @@ def test_histories_of_other_lengths_replay_the_same_graph():
     out = case.eng.alloc_outputs(2, 5)
     torch.cuda.synchronize()
     for i, n in enumerate((100, 100, 100, 100, 99, 57, 100, 3)):
+        hist, lens = case.hist_dev[:, :n].contiguous(), torch.full((2,), n, dtype=torch.int32, device="cuda")
+        torch.cuda.synchronize()
         for c in (case, eager):
-            c.eng.prefill(c.hist_dev[:, :n], torch.full((2,), n, dtype=torch.int32, device="cuda"))
+            c.eng.prefill(hist, lens)
         torch.cuda.synchronize()
         calls = _runtime_calls(lambda: case.eng.decode(5, mode=binding.MODE_AR, out=out))
         assert i < 3 or _replayed(calls), (n, calls)
@@ -53,6 +58,7 @@ def test_histories_of_other_lengths_replay_the_same_graph():
 def test_the_graphs_that_are_kept_are_bounded():
     """A program that brings other result buffers to every call: the oldest graphs are given back."""
     case, eager = _engines()
+    torch.cuda.synchronize()
     for c in (case, eager):
         c.prefill()
     counts = torch.zeros(300, 2, dtype=torch.int32, device="cuda")
@@ -80,6 +86,7 @@ def test_the_graphs_that_are_kept_are_bounded():
 def test_calls_with_other_trace_buffers_are_told_apart():
     """Trace buffers whose addresses differ in ways that cancel out in beams ^ 2 tree_codes."""
     case, eager = _engines()
+    torch.cuda.synchronize()
     case.prefill()
     R, L, S = 3, 4, 1 << 12                                                # a buffer is less than 4 KB
     block = torch.empty(16 * S, dtype=torch.uint8, device="cuda")

@@ -18,7 +18,8 @@ def test_repeated_calls_return_the_same_bits(hd, heads, kv_heads, batch, beam, n
     w = synth.scaled(synth.WORKLOADS["small"], n_layers=2, d_model=hd * heads, n_q_heads=heads, n_kv_heads=kv_heads, n_items=50_000,
                      batch=batch, beam=beam, n_hist=n_hist)
     st = torch.cuda.Stream()
-    case = Case(w, stream=st).prefill()
+    with torch.cuda.stream(st):                          # (the engine reads the weights and histories on its stream)
+        case = Case(w, stream=st).prefill()
     first, outs = {}, {m: case.eng.alloc_outputs(w.batch, w.beam, trace=True) for m in (binding.MODE_AR, binding.MODE_VERIFIED)}
     for mode in (binding.MODE_AR, binding.MODE_AR, binding.MODE_AR, binding.MODE_VERIFIED, binding.MODE_AR, binding.MODE_VERIFIED,
                  binding.MODE_VERIFIED, binding.MODE_VERIFIED):

@@ -13,9 +13,10 @@ pytestmark = pytest.mark.gpu
 def test_a_surplus_round_does_not_stream_the_weights():
     w = synth.scaled(synth.WORKLOADS["paper"], n_layers=8, n_items=50_000, batch=1)
     st = torch.cuda.Stream()
-    case = Case(w, stream=st).prefill()
-    beams = case.eng.decode(w.beam, mode=binding.MODE_AR, trace=True)["trace"]["beams"].clone()
-    tree = beams, (beams[:, :, :, 0] >= 0).sum(dim=2).to(torch.int32).contiguous()
+    with torch.cuda.stream(st):                          # (the engine reads the weights and histories on its stream)
+        case = Case(w, stream=st).prefill()
+        beams = case.eng.decode(w.beam, mode=binding.MODE_AR, trace=True)["trace"]["beams"].clone()
+        tree = beams, (beams[:, :, :, 0] >= 0).sum(dim=2).to(torch.int32).contiguous()
     out = case.eng.alloc_outputs(1, w.beam)
     torch.cuda.synchronize()
 

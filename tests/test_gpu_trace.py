@@ -13,7 +13,8 @@ def test_trace_is_complete_when_the_call_returns(mode):
     """The call synchronises: nothing of it is left on the engine's stream, and another stream may read the trace at once."""
     w = synth.scaled(synth.WORKLOADS["tiny"], n_layers=1, L=8, T=(16,) * 8, batch=512, beam=128, n_hist=1)   # 17 MB of beam sets
     st, other = torch.cuda.Stream(), torch.cuda.Stream()
-    case = Case(w, stream=st).prefill()
+    with torch.cuda.stream(st):              # (the engine reads the weights and histories on its stream)
+        case = Case(w, stream=st).prefill()
     out = case.eng.alloc_outputs(w.batch, w.beam, trace=True)
     beams = out["trace"]["beams"]
     for _ in range(4):                       # eager, captured, replayed
