@@ -5,9 +5,12 @@
 // 128 x 64 tile of W (16 KB per copy, the unit that has to be kept in flight), the rows of A are the MMA's N (MT = 32, 64
 // or 128), and the accumulator in TMEM is a 128 x MT block of C^T.  An output tile is 128 columns of C; the K range of a
 // tile is split over the CTAs of a thread-block cluster (up to 8) so that every SM streams a share of W, whatever N.
-// Each CTA leaves its partial block in its own shared memory; after a cluster barrier pieces of the tile are dealt out to
-// the cluster's warps, which add the parts in rank order, reading their peers' shared memory -- the bits never depend on
-// timing -- and run the same fused epilogue as the other tensor-core kernels.
+// Pieces of the tile are dealt out to the cluster's warps, which add the parts in rank order -- the bits never depend on
+// timing -- and run the same fused epilogue as the other tensor-core kernels.  Up to 48 rows every CTA sends its parts straight from
+// its accumulator to the shared memory of the warps that add them (st.async on their mbarriers); beyond, where there is no room for
+// them beside the ring, it leaves its block in its own, and the warps read their peers' behind a cluster barrier.  The barrier, the
+// round trip of the reads and a second barrier before a CTA may leave are a launch's last 1.3 us: one request on the 16-layer d = 2048
+// backbone, prompt of 40 rows / verified decode (20 rows a pass) 676 -> 635 / 1,344 -> 1,278 us without them.
 // A CTA issues the weight copies of its first ring round BEFORE the launch's dependency on the preceding kernel is
 // resolved (W is constant data), and the kernel is sized for two CTAs per SM, so the weight stream of a launch starts
 // while its predecessor is still draining.
@@ -22,19 +25,25 @@ namespace {
 
 using namespace gemm_detail;
 
-template <int MT> struct SkinnyCfg {
+template <int MT, bool PUSH> struct SkinnyCfg {
   static constexpr int kTileBytesW = 128 * BK * 2;
   static constexpr int kTileBytesX = MT * BK * 2;
   static constexpr int kStageBytes = kTileBytesW + kTileBytesX;
-  static constexpr int kStages = MT == 32 ? 5 : MT == 64 ? 4 : 3;
-  static constexpr int kBarBytes = 128;
-  // (the accumulator's image reuses the ring: a CTA has one tile, and the ring is idle once it is accumulated)
-  static constexpr int kSmemBytes = kStages * kStageBytes + 1024 /*alignment slack*/ + kBarBytes + MT * 4 /*row scales*/;
-  static constexpr int kTmemCols = MT;
+  // The parts of a split tile are sent to the shared memory of the CTAs that add them up (PUSH: up to 48 rows, where the room for
+  // them leaves a ring of four), or left in the CTA's own for its peers to read.
+  static constexpr int kStages = MT == 128 ? 3 : 4;
+  static constexpr int kRecvParts = PUSH ? (MT == 32 ? 36 : 48) : 0;         // of 512 bytes
+  static constexpr int kRecvBytes = kRecvParts * 512;
+  static constexpr int kBarBytes = 192;
+  // (the array is declared 1024-byte aligned; the kernel checks the slack that it really needs)
+  static constexpr int kSlack = 512;
+  // (an image of the accumulator reuses the ring: a CTA has one tile, and the ring is idle once it is accumulated)
+  static constexpr int kSmemBytes = kStages * kStageBytes + kRecvBytes + kSlack + kBarBytes + MT * 4 /*row scales*/;
+  static constexpr int kTmemCols = MT <= 32 ? 32 : MT <= 64 ? 64 : 128;
   // kind::f16 instruction descriptor: D = f32, A = B = bf16, both K-major, N = MT, M = 128.
   static constexpr uint32_t kInstrDesc =
       (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(MT >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
-  static_assert(MT * 512 <= kStages * kStageBytes, "the accumulator's image does not fit in the ring");
+  static_assert((MT + 31) / 32 * 32 * 512 <= kStages * kStageBytes, "the accumulator's image does not fit in the ring");
   static_assert(2 * (kSmemBytes + 1024) <= 228 * 1024, "two CTAs per SM");
 };
 
@@ -43,10 +52,19 @@ __device__ __forceinline__ uint32_t cluster_rank() {
   asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
   return r;
 }
-// Every thread of every CTA of the cluster executes both halves, on every path.
-__device__ __forceinline__ void cluster_sync_all() {
-  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+// Every thread of every CTA of the cluster executes both halves in turn, on every path.  The relaxed arrival orders nothing: it
+// says that the CTA has come so far.
+__device__ __forceinline__ void cluster_arrive_relaxed() { asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+// 16 bytes to the shared memory of CTA `rank` of the cluster, at the address that `local` has in this CTA; they count towards the
+// bytes that the mbarrier at `bar` (an address of this CTA's as well) of that CTA waits for.
+__device__ __forceinline__ void st_peer_f4(uint32_t local, uint32_t bar, uint32_t rank, float x, float y, float z, float w) {
+  uint32_t ra, rb;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(local), "r"(rank));
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(rb) : "r"(bar), "r"(rank));
+  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1, %2, %3, %4}, [%5];"
+               ::"r"(ra), "f"(x), "f"(y), "f"(z), "f"(w), "r"(rb) : "memory");
 }
 // 16 bytes of the shared memory of CTA `rank` of the cluster, at the address that `local` has in this CTA.
 __device__ __forceinline__ float4 ld_peer_f4(uint32_t local, uint32_t rank) {
@@ -56,7 +74,36 @@ __device__ __forceinline__ float4 ld_peer_f4(uint32_t local, uint32_t rank) {
   asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(ra) : "memory");
   return v;
 }
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {
+// The first phase of a barrier that peers signal, waited for by a whole warp; bounded, and given up early when the CTA's abort flag
+// (if given) is raised.  (All lanes ask, here and for the accumulator: with one lane asking for the others, what follows was compiled
+// for a warp that may be split there, and the same prompt and decode took 730 / 1,393 us.)
+__device__ __forceinline__ bool recv_wait(uint32_t bar, volatile uint32_t* abort_flag) {
+  auto here = [&] {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], 0;\n\t"
+        "selp.b32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok) : "r"(bar) : "memory");
+    return __all_sync(0xffffffffu, ok != 0u);
+  };
+  if (here()) return true;
+  const long long t0 = clock64();
+  for (;;) {
+    if (here()) return true;
+    if (__any_sync(0xffffffffu, (abort_flag && *abort_flag) || clock64() - t0 > kWaitCycles)) return false;
+  }
+}
+__device__ __forceinline__ void tmem_ld(uint32_t taddr, float (&v)[8]) {
+  uint32_t r[8];
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+               : "r"(taddr));
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+  for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
+}
+__device__ __forceinline__ void tmem_ld(uint32_t taddr, float (&v)[16]) {
   uint32_t r[16];
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
@@ -79,23 +126,32 @@ constexpr int kSkinnyThreads = 64 + 32 * kSkinnyEpiWarps;
 // one round of peer loads, and what it needs from memory is fetched before the accumulator is ready.  (One warp per 32 x 32
 // block, the blocks dealt out to the CTAs, each row's norm scale added up by one lane: per launch at 20 rows 11.8 instead of 9.1 us for
 // the output and down projections of the d = 2048 backbone, 7.8 instead of 5.4 for QKV.)
-template <int MT, int EPI>
+template <int MT, bool PUSH, int EPI>
 __global__ void __launch_bounds__(kSkinnyThreads, 2)
     gemm_skinny_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmX, GemmArgs a,
                        int splits, int* status) {
-  using C = SkinnyCfg<MT>;
+  using C = SkinnyCfg<MT, PUSH>;
   constexpr int STAGES = C::kStages;
-  extern __shared__ uint8_t smem_raw[];
+  extern __shared__ __align__(1024) uint8_t smem_raw[];
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
+  if (base - smem_u32(smem_raw) > (uint32_t)C::kSlack) {      // (of every CTA alike) less aligned than declared: report, touch nothing
+    pdl_wait();
+    if (threadIdx.x == 0) atomicOr(status, kStInternal);
+    return;
+  }
   uint8_t* gen_base = smem_raw + (base - smem_u32(smem_raw));
-  const uint32_t bar_base = base + STAGES * C::kStageBytes;
-  // barriers: full[STAGES], empty[STAGES], acc_full; then the TMEM slot and the abort flag; then the rows' norm scales
+  constexpr int kRecvAt = STAGES * C::kStageBytes, kBarAt = kRecvAt + C::kRecvBytes;
+  const uint32_t recv_base = base + kRecvAt, bar_base = base + kBarAt;
+  // barriers: full[STAGES], empty[STAGES], acc_full, recv[epilogue warps]; then the TMEM slot and the abort flag; then the rows' norm scales
   auto full_bar = [&](int s) { return bar_base + 8u * s; };
   auto empty_bar = [&](int s) { return bar_base + 8u * (STAGES + s); };
   const uint32_t acc_full = bar_base + 8u * (2 * STAGES);
-  volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(gen_base + STAGES * C::kStageBytes + 8 * (2 * STAGES + 1));
+  auto recv_bar = [&](int w) { return bar_base + 8u * (2 * STAGES + 1 + w); };      // the parts of epilogue warp w's units are here
+  constexpr int kSlotAt = 8 * (2 * STAGES + 1 + kSkinnyEpiWarps);
+  static_assert(kSlotAt + 8 <= C::kBarBytes, "barrier area");
+  volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(gen_base + kBarAt + kSlotAt);
   volatile uint32_t* abort_flag = tmem_slot + 1;
-  float* row_scale = reinterpret_cast<float*>(gen_base + STAGES * C::kStageBytes + C::kBarBytes);
+  float* row_scale = reinterpret_cast<float*>(gen_base + kBarAt + C::kBarBytes);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int tile = blockIdx.x / splits, split = (int)cluster_rank();
@@ -115,6 +171,7 @@ __global__ void __launch_bounds__(kSkinnyThreads, 2)
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) { mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), 1); }
     mbar_init(acc_full, 1);
+    for (int w = 0; w < kSkinnyEpiWarps; ++w) mbar_init(recv_bar(w), 1);
     *abort_flag = 0;
     mbar_fence_init();
     tma_prefetch_map(&tmW);
@@ -146,6 +203,7 @@ __global__ void __launch_bounds__(kSkinnyThreads, 2)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  if (PUSH) cluster_arrive_relaxed();             // this CTA's barriers may be signalled (waited for before the first signal)
   pdl_wait();
   pdl_launch();
   const int M = a.early ? M_early : a.M_dev ? min(a.M, *a.M_dev) : a.M;
@@ -160,12 +218,14 @@ __global__ void __launch_bounds__(kSkinnyThreads, 2)
   const int k8 = lane & 7, rsub = lane >> 3;
   const bool mine = live && warp >= 2 && u_first < units;
   EpiAux aux;                                     // what the warp's next unit needs from memory
+  ChunkCtx cc;
   int pos = 0;
   long long kvd = -1;
   auto fetch = [&](int u) {
     const int n_chunk = n0 + 32 * (u / quads), r = 4 * (u % quads) + rsub;
     if (EPI == kEpiRopeKV && r < rows) { pos = a.f.tok_pos[m0 + r]; kvd = a.f.kv_dst[m0 + r]; }
-    if (r < rows) aux = epi_prefetch<EPI>(a, chunk_ctx<EPI>(a, n_chunk, k8), m0 + r, n_chunk + 4 * k8, pos);
+    cc = chunk_ctx<EPI>(a, n_chunk, k8);
+    if (r < rows) aux = epi_prefetch<EPI>(a, cc, m0 + r, n_chunk + 4 * k8, pos);
   };
 
   if (!live) {
@@ -225,50 +285,97 @@ __global__ void __launch_bounds__(kSkinnyThreads, 2)
       if (k8 == 0) row_scale[r] = a.f.ss_in ? rsqrtf(ss * a.f.inv_dim + a.f.eps) : 1.f;
     }
     if (mine) fetch(u_first);
-    const bool ok = warp_wait(acc_full, 0, abort_flag, lane);
+    if constexpr (PUSH) {
+      // what this warp's units will be sent (nobody signals the barrier before the peers' barriers are known to exist)
+      if (mine && lane == 0) mbar_expect_tx(recv_bar(ew), (uint32_t)((units - u_first + u_step - 1) / u_step * splits * 512));
+      __syncwarp();
+      cluster_wait();
+    }
+    const bool ok = warp_wait_uniform(acc_full, 0, abort_flag);
     tc_fence_after();
-    if (ok) {
-      // TMEM lane = column n0 + 32 q + lane, TMEM column = row; each warp takes a half of the rows of its lane quarter.  The image
-      // of a 32 x 32 block is 32 lines of one row each, their 16-byte chunks swizzled by the row.
-      const int q = warp & 3, half = ew >> 2;
+    if (!ok && lane == 0) *abort_flag = 1;
+    // TMEM lane = column n0 + 32 q + lane, TMEM column = row; the two warps of a lane quarter take turns at the rows.
+    constexpr int kLd = MT >= 64 ? 16 : 8;
+    const int q = warp & 3, half = ew >> 2;
+    if constexpr (PUSH) {
+      // A lane's four rows of a unit are 16 bytes, a unit's part is 512.  (Also after a wait that expired: the peers count on it.)
+      if (q < col_groups) {
+#pragma unroll 1
+        for (int r0 = half * kLd; r0 < rows; r0 += 2 * kLd) {
+          float v[kLd];
+          tmem_ld(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)r0, v);
+#pragma unroll
+          for (int j = 0; j < kLd; j += 4) {
+            const int u = q * quads + ((r0 + j) >> 2);
+            if (r0 + j < rows) {
+              const int slot = u / splits, owner = u - slot * splits;
+              st_peer_f4(recv_base + (uint32_t)((slot * splits + split) * 512 + lane * 16), recv_bar(slot & (kSkinnyEpiWarps - 1)), (uint32_t)owner,
+                         v[j], v[j + 1], v[j + 2], v[j + 3]);
+            }
+          }
+        }
+      }
+    } else if (ok) {
+      // The image of a 32 x 32 block is 32 lines of one row each, their 16-byte chunks swizzled by the row.
       float* img = reinterpret_cast<float*>(gen_base) + q * 1024;
 #pragma unroll 1
-      for (int r0 = half * (MT / 2); r0 < (half + 1) * (MT / 2) && r0 < rows; r0 += 16) {
-        float v[16];
-        tmem_ld16(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)r0, v);
+      for (int r0 = half * kLd; r0 < rows; r0 += 2 * kLd) {
+        float v[kLd];
+        tmem_ld(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)r0, v);
         float* blk = img + (r0 >> 5) * 4096;
 #pragma unroll
-        for (int j = 0; j < 16; ++j) {
+        for (int j = 0; j < kLd; ++j) {
           const int r = (r0 & 31) + j;
           blk[(r * 8 + ((lane >> 2) ^ (r & 7))) * 4 + (lane & 3)] = v[j];
         }
       }
-    } else if (lane == 0) {
-      *abort_flag = 1;
     }
   }
-  // All parts are in place behind this barrier (or their CTA has raised its abort flag).
-  if (splits > 1) cluster_sync_all();
-  else __syncthreads();
+  if constexpr (PUSH) {
+    __syncwarp();
+    if (!live || warp < 2) cluster_wait();       // (the epilogue warps of a live tile have)
+    cluster_arrive_relaxed();                    // this CTA's parts are on their way
+    if (mine && !recv_wait(recv_bar(ew), abort_flag)) *abort_flag = 1;
+  } else {
+    // All parts are in place behind this barrier (or their CTA has raised its abort flag).
+    if (splits > 1) { __syncwarp(); cluster_arrive(); cluster_wait(); }
+    else __syncthreads();
+  }
   if (mine && !*abort_flag) {
     // ------------------------------------------------------------------ epilogue, second half: the parts of a unit, added in rank order
 #pragma unroll 1
     for (int u = u_first; u < units; u += u_step) {
       const int g = u / quads, r = 4 * (u - g * quads) + rsub, n_chunk = n0 + 32 * g, row = m0 + r;
-      const ChunkCtx cc = chunk_ctx<EPI>(a, n_chunk, k8);
-      const uint32_t at = base + (uint32_t)(((r >> 5) * 4 + g) * 4096 + ((r & 31) * 8 + (k8 ^ (r & 7))) * 16);
       float4 x;
-      if (splits > 1) {
-        float4 part[8];
-#pragma unroll
-        for (int sp = 0; sp < 8; ++sp)
-          if (sp < splits) part[sp] = ld_peer_f4(at, (uint32_t)sp);
+      if constexpr (PUSH) {
+        // added as they came (lane = column, four rows), then turned in the room of the first part: lane = row, four columns
+        float4* part = reinterpret_cast<float4*>(gen_base + kRecvAt) + u / splits * splits * 32 + lane;
         x = part[0];
 #pragma unroll
         for (int sp = 1; sp < 8; ++sp)
-          if (sp < splits) { x.x += part[sp].x; x.y += part[sp].y; x.z += part[sp].z; x.w += part[sp].w; }
+          if (sp < splits) {
+            const float4 y = part[sp * 32];
+            x.x += y.x; x.y += y.y; x.z += y.z; x.w += y.w;
+          }
+        __syncwarp();
+        float* turn = reinterpret_cast<float*>(part - lane);
+        turn[lane] = x.x; turn[32 + lane] = x.y; turn[64 + lane] = x.z; turn[96 + lane] = x.w;
+        __syncwarp();
+        x = reinterpret_cast<const float4*>(turn)[lane];
       } else {
-        x = *reinterpret_cast<const float4*>(gen_base + (at - base));
+        const uint32_t at = base + (uint32_t)(((r >> 5) * 4 + g) * 4096 + ((r & 31) * 8 + (k8 ^ (r & 7))) * 16);
+        if (splits > 1) {
+          float4 part[8];
+#pragma unroll
+          for (int sp = 0; sp < 8; ++sp)
+            if (sp < splits) part[sp] = ld_peer_f4(at, (uint32_t)sp);
+          x = part[0];
+#pragma unroll
+          for (int sp = 1; sp < 8; ++sp)
+            if (sp < splits) { x.x += part[sp].x; x.y += part[sp].y; x.z += part[sp].z; x.w += part[sp].w; }
+        } else {
+          x = *reinterpret_cast<const float4*>(gen_base + (at - base));
+        }
       }
       const float rs = row_scale[r];
       x = make_float4(x.x * rs, x.y * rs, x.z * rs, x.w * rs);
@@ -283,8 +390,13 @@ __global__ void __launch_bounds__(kSkinnyThreads, 2)
     }
   }
   tc_fence_before();
-  if (splits > 1) cluster_sync_all();            // no CTA leaves while a peer may still read its part
-  else __syncthreads();
+  __syncwarp();
+  if (PUSH || splits > 1) {                      // no CTA leaves while a peer may still send to it, or read its part
+    if (!PUSH) cluster_arrive_relaxed();         // (what it has read has been used)
+    cluster_wait();
+    if (PUSH && mine && *abort_flag) recv_wait(recv_bar(ew), nullptr);      // given up before: everything sent has to land first
+  }
+  __syncthreads();
   if (warp == 1) {
     __syncwarp();
     tc_fence_after();
@@ -293,9 +405,9 @@ __global__ void __launch_bounds__(kSkinnyThreads, 2)
   if (threadIdx.x == 0 && *abort_flag) atomicOr(status, kStInternal);
 }
 
-template <int MT, int EPI>
+template <int MT, bool PUSH, int EPI>
 void launch(const GemmArgs& a, int tiles, int splits, cudaStream_t st) {
-  using C = SkinnyCfg<MT>;
+  using C = SkinnyCfg<MT, PUSH>;
   CUtensorMap tw, tx;
   if (!tma_map_bf16(a.W, a.N, a.K, a.ldw, 128, &tw) || !tma_map_bf16(a.A, a.M, a.K, a.lda, MT, &tx)) {
     static const int flag = kStInternal;       // cannot happen for shapes gemm_tc_supported accepted; report, do not guess
@@ -304,7 +416,7 @@ void launch(const GemmArgs& a, int tiles, int splits, cudaStream_t st) {
   }
   static PerDeviceOnce configured;
   configured.run([] {
-    cudaFuncSetAttribute(gemm_skinny_kernel<MT, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes);
+    cudaFuncSetAttribute(gemm_skinny_kernel<MT, PUSH, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes);
   });
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(tiles * splits, (a.M + MT - 1) / MT); cfg.blockDim = dim3(kSkinnyThreads); cfg.dynamicSmemBytes = C::kSmemBytes; cfg.stream = st;
@@ -314,21 +426,33 @@ void launch(const GemmArgs& a, int tiles, int splits, cudaStream_t st) {
   at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at; cfg.numAttrs = pdl_enabled() ? 2 : 1;
-  cudaLaunchKernelEx(&cfg, gemm_skinny_kernel<MT, EPI>, tw, tx, a, splits, a.status);
+  cudaLaunchKernelEx(&cfg, gemm_skinny_kernel<MT, PUSH, EPI>, tw, tx, a, splits, a.status);
+}
+
+template <int MT, bool PUSH>
+void launch_epi(const GemmArgs& a, int tiles, int splits, cudaStream_t st) {
+  switch (a.epilogue) {
+    case kEpiStoreAct: launch<MT, PUSH, kEpiStoreAct>(a, tiles, splits, st); break;
+    case kEpiStoreF32: launch<MT, PUSH, kEpiStoreF32>(a, tiles, splits, st); break;
+    case kEpiAddF32: launch<MT, PUSH, kEpiAddF32>(a, tiles, splits, st); break;
+    case kEpiBiasTanhF32: launch<MT, PUSH, kEpiBiasTanhF32>(a, tiles, splits, st); break;
+    case kEpiSwiGLU: launch<MT, PUSH, kEpiSwiGLU>(a, tiles, splits, st); break;
+    case kEpiAddNorm: launch<MT, PUSH, kEpiAddNorm>(a, tiles, splits, st); break;
+    case kEpiRopeKV: launch<MT, PUSH, kEpiRopeKV>(a, tiles, splits, st); break;
+    default: break;
+  }
 }
 
 template <int MT>
 void launch_mt(const GemmArgs& a, int tiles, int splits, cudaStream_t st) {
-  switch (a.epilogue) {
-    case kEpiStoreAct: launch<MT, kEpiStoreAct>(a, tiles, splits, st); break;
-    case kEpiStoreF32: launch<MT, kEpiStoreF32>(a, tiles, splits, st); break;
-    case kEpiAddF32: launch<MT, kEpiAddF32>(a, tiles, splits, st); break;
-    case kEpiBiasTanhF32: launch<MT, kEpiBiasTanhF32>(a, tiles, splits, st); break;
-    case kEpiSwiGLU: launch<MT, kEpiSwiGLU>(a, tiles, splits, st); break;
-    case kEpiAddNorm: launch<MT, kEpiAddNorm>(a, tiles, splits, st); break;
-    case kEpiRopeKV: launch<MT, kEpiRopeKV>(a, tiles, splits, st); break;
-    default: break;
+  if constexpr (MT <= 48) {
+    // a CTA's share of at most MT units, each in `splits` parts, has to fit
+    if (splits > 1 && (MT + splits - 1) / splits * splits <= SkinnyCfg<MT, true>::kRecvParts) {
+      launch_epi<MT, true>(a, tiles, splits, st);
+      return;
+    }
   }
+  launch_epi<MT, false>(a, tiles, splits, st);
 }
 
 }  // namespace
@@ -372,6 +496,7 @@ bool gemm_skinny_applies(const GemmArgs& a, int n_sm) {
 void launch_gemm_skinny(const GemmArgs& a, int n_sm, cudaStream_t st) {
   const int tiles = (a.N + 127) / 128, splits = gemm_skinny_splits(a.N, a.K, a.skinny, n_sm);
   if (a.M <= 32) launch_mt<32>(a, tiles, splits, st);      // (the bound, not the expected count: no row may be dropped)
+  else if (a.M <= 48) launch_mt<48>(a, tiles, splits, st);
   else if (a.M <= 64) launch_mt<64>(a, tiles, splits, st);
   else launch_mt<128>(a, tiles, splits, st);
 }

@@ -130,6 +130,24 @@ def test_weight_streaming_gemm(ctx, N, K):
     ctx.eng.sync()
 
 
+@pytest.mark.parametrize("N,K", [(12544, 768), (7552, 1280), (6272, 1536), (5376, 1792), (1024, 1024)])
+def test_weight_streaming_gemm_parts_of_every_split(ctx, N, K):
+    """A tile's K range over 3, 5, 6, 7 and 4 CTAs of a B200: the sent parts' places for full, partial and single units of four rows, on
+    both sides of the row counts where the parts are sent (32, 48), against the fp64 product and bit for bit the read parts' sum."""
+    g = torch.Generator(device="cuda"); g.manual_seed(N + K)
+    A = (torch.randn(64, K, generator=g, device="cuda") * 0.5).bfloat16()
+    W = (torch.randn(N, K, generator=g, device="cuda") * 0.05).bfloat16()
+    ref = _ref(A, W)
+    full = torch.empty(64, N, dtype=torch.float32, device="cuda")
+    ctx.eng.gemm(A, W, full, epilogue=1, path=4)
+    assert np.abs(full.cpu().numpy() - ref).max() < 2e-5 * np.abs(ref).max() * np.sqrt(K / 64) + 1e-6
+    for M in (1, 4, 5, 31, 32, 33, 47, 48, 49):
+        out = torch.full((M, N), float("nan"), dtype=torch.float32, device="cuda")
+        ctx.eng.gemm(A[:M].contiguous(), W, out, epilogue=1, path=4)
+        assert torch.equal(out, full[:M]), (N, K, M)
+    ctx.eng.sync()
+
+
 def test_weight_streaming_gemm_takes_at_most_128_rows(ctx):
     A = torch.zeros(129, 64, dtype=torch.bfloat16, device="cuda")
     W = torch.zeros(128, 64, dtype=torch.bfloat16, device="cuda")
