@@ -80,7 +80,7 @@ struct nezha_ctx {
   bool fused; float *ss_a, *ss_b, *ss_e;
   // draft head with merged products (fused path, default options): [W_logit_l ; W_s] per level, U = E W_e^T for every
   // code token, H_l = W_logit_l h_l per request, the level's states as a bf16 A operand, the level's product
-  void* draft_wcat[kMaxLevels]; float* draft_u; float* draft_hl; void* draft_sact; float* draft_g;
+  void* draft_wcat[kMaxLevels]; float* draft_u; float* draft_hl; void* draft_sact; float *draft_g, *draft_g1;
   int* h_rows; unsigned long long* n_unique_dev;
   EngineState es;
   BuildScratch build;
@@ -269,7 +269,7 @@ size_t carve(nezha_ctx* c) {
   c->logits_d = cv.take<float>((size_t)c->Bmax * c->Kmax * c->Tmax);
   c->h_rows = cv.take<int>((size_t)c->Bmax * (c->L + 1));
   c->ss_a = c->ss_b = c->ss_e = nullptr;
-  c->draft_u = c->draft_hl = c->draft_g = nullptr; c->draft_sact = nullptr;
+  c->draft_u = c->draft_hl = c->draft_g = c->draft_g1 = nullptr; c->draft_sact = nullptr;
   for (int l = 0; l < kMaxLevels; ++l) c->draft_wcat[l] = nullptr;
   if (c->fused) {
     for (int l = 0; l < c->L; ++l) c->draft_wcat[l] = cv.take_bytes((size_t)(g.T[l] + c->d) * c->d * esz);
@@ -277,6 +277,7 @@ size_t carve(nezha_ctx* c) {
     c->draft_hl = cv.take<float>((size_t)c->L * c->Bmax * c->Tmax);
     c->draft_sact = cv.take_bytes((size_t)c->Bmax * c->Kmax * c->d * esz);
     c->draft_g = cv.take<float>((size_t)c->Bmax * c->Kmax * (c->Tmax + c->d));
+    c->draft_g1 = cv.take<float>((size_t)c->Bmax * (c->Tmax + c->d));
     c->ss_a = cv.take<float>((size_t)(c->d / 32) * c->Ms);      // one partial sum per 32 columns
     c->ss_b = cv.take<float>((size_t)(c->d / 32) * c->Ms);
     c->ss_e = cv.take<float>((size_t)c->Ms);
@@ -500,28 +501,38 @@ void draft_level_product(nezha_ctx* c, int batch, int l, bool with_state, bool i
   gemm(c, c->draft_sact, c->d, c->draft_wcat[l - 1], c->d, c->draft_g, c->Tmax + c->d, (long long)batch * c->Kmax,
        in_round ? c->es.draft_rows : nullptr, T + (with_state ? c->d : 0), c->d, kEpiStoreF32);
 }
-void draft_level_step(nezha_ctx* c, int batch, int l) {
-  launch_draft_step(c->es, batch, l, c->draft_g, c->Tmax + c->d, c->cfg.T[l - 1], c->draft_u, (const float*)c->draft_b_f32, c->draft_sact,
+// Level 1 of a decode call: every beam slot's state is s_1 = h_0, so the product has one row per request, and every round's is the same.
+void draft_first_product(nezha_ctx* c, int batch) {
+  const int T = c->cfg.T[0];
+  gemm(c, c->h_act, (long long)(c->L + 1) * c->d, c->draft_wcat[0], c->d, c->draft_g1, c->Tmax + c->d, batch, c->es.draft_rows,
+       T + (c->L > 1 ? c->d : 0), c->d, kEpiStoreF32);
+}
+void draft_level_step(nezha_ctx* c, int batch, int l, bool first_product = false) {
+  launch_draft_step(c->es, batch, l, first_product ? c->draft_g1 : c->draft_g, first_product ? 1 : c->Kmax, c->Tmax + c->d, c->cfg.T[l - 1], c->draft_u, (const float*)c->draft_b_f32, c->draft_sact,
                     c->st);
 }
 
 // Algorithm 3's inference loop (from the empty beam), or its continuation from the true beams (Algorithm 2's drafting step).
-// `first_level` = smallest level any request can still need drafting at (levels below are teacher-forced only).
+// `first_level` = smallest level any request can still need drafting at (levels below are teacher-forced only).  Where it starts from is
+// in place: the beginning of the call and the end of each round see to that (EngineState::d_m).
+// first_product: level 1's product has not been made in this call.  with_nodes: the round's token list as well.
 // out_*: the last level's beams go straight to these buffers (mode 0), with the status words to the host.
-void draft_phase(nezha_ctx* c, int batch, int K, bool from_scratch, int first_level, bool filter, int* out_codes = nullptr,
+void draft_phase(nezha_ctx* c, int batch, int K, int first_level, bool filter, bool first_product, bool with_nodes, int* out_codes = nullptr,
                  float* out_scores = nullptr, int* out_count = nullptr) {
   const EngineState& e = c->es;
   const bool fast = draft_fast(c);
-  launch_draft_init(e, batch, from_scratch ? 1 : 0, fast ? c->draft_sact : nullptr, c->st);
   for (int l = 1; l <= c->L; ++l) {
-    if (fast && (l >= first_level || l < c->L)) draft_level_product(c, batch, l, l < c->L, true);
+    float* const g = l == 1 ? c->draft_g1 : c->draft_g;
+    const int per_req = l == 1 ? 1 : c->Kmax;
+    if (fast && l == 1 && first_product) draft_first_product(c, batch);
+    if (fast && l > 1 && (l >= first_level || l < c->L)) draft_level_product(c, batch, l, l < c->L, true);
     if (l >= first_level) {
       if (!fast) draft_logits_level(c, batch, l);
       SelectArgs s = select_base(c, batch, K);
       const size_t lv_in = (size_t)(l - 1) * c->Bmax * c->Kmax, lv_out = (size_t)l * c->Bmax * c->Kmax;
       s.logits = c->logits_d; s.row_stride = c->cfg.T[l - 1]; s.col_off = 0; s.src_row = nullptr; s.src_mul = c->Kmax;
       if (fast) {
-        s.logits = c->draft_g; s.row_stride = c->Tmax + c->d;
+        s.logits = g; s.row_stride = c->Tmax + c->d; s.src_mul = per_req;
         s.logit_bias = c->draft_hl + (size_t)(l - 1) * c->Bmax * c->Tmax; s.bias_stride = c->Tmax;
       }
       s.in_codes = e.dw_codes + lv_in * c->L; s.in_score = e.dw_score + lv_in; s.in_count = e.dw_count + (size_t)(l - 1) * c->Bmax;
@@ -538,13 +549,14 @@ void draft_phase(nezha_ctx* c, int batch, int K, bool from_scratch, int first_le
       // fused kernel is one CTA per request; at d = 4096 its 20 x 4096 state elements per request take 64 us on 32 SMs
       // against 14 us for the update spread over (request, beam) CTAs.
       if (fast && l < c->L && c->d <= 1024) {
-        launch_select_step(s, e, l, c->draft_g, c->Tmax + c->d, c->cfg.T[l - 1], c->draft_u, (const float*)c->draft_b_f32,
+        launch_select_step(s, e, l, g, per_req, c->Tmax + c->d, c->cfg.T[l - 1], c->draft_u, (const float*)c->draft_b_f32,
                            c->draft_sact, c->st);
         continue;
       }
-      launch_select(s, c->st);
+      if (with_nodes && l == c->L) launch_select_nodes(s, e, c->st);
+      else launch_select(s, c->st);
     }
-    if (l < c->L) { if (fast) draft_level_step(c, batch, l); else draft_transition_level(c, batch, l); }
+    if (l < c->L) { if (fast) draft_level_step(c, batch, l, l == 1); else draft_transition_level(c, batch, l); }
   }
 }
 
@@ -644,9 +656,10 @@ nezha_status decode_impl(nezha_ctx* c, int batch, int K, int mode, const int* dr
     return k;
   };
   auto begin = [&] {
-    launch_decode_begin(e, batch, K, out_codes, out_scores, out_count, tr, c->st);
+    launch_decode_begin(e, batch, K, mode == NEZHA_MODE_DRAFT || (mode == NEZHA_MODE_VERIFIED && !drafts) ? 1 : 0, out_codes, out_scores, out_count, tr,
+                        c->st);
     if (mode == NEZHA_MODE_DRAFT) {
-      draft_phase(c, batch, K, true, 1, c->opt_filter != 0, out_codes, out_scores, out_count);
+      draft_phase(c, batch, K, 1, c->opt_filter != 0, true, false, out_codes, out_scores, out_count);
       return;
     }
     // B_1 from the prefill hidden state h_0 (Algorithm 1's LM head, top-K and pruning at l = 1), settled at once
@@ -662,7 +675,7 @@ nezha_status decode_impl(nezha_ctx* c, int batch, int K, int mode, const int* dr
     s.out_codes = e.tb_codes + lv_out * L; s.out_score = e.tb_score + lv_out; s.out_parent = e.tb_parent + lv_out;
     s.out_count = e.tb_count + (size_t)1 * c->Bmax;
     s.status = e.status; s.host_status = c->host_counters + 8;
-    launch_select_advance(s, e, 0, K, out_codes, out_scores, out_count, RoundEnd{}, c->st);
+    launch_select_advance(s, e, 1, K, out_codes, out_scores, out_count, RoundEnd{}, c->st);
   };
   auto run_round = [&](int round) {
     // drafts are mostly rejected or mostly accepted in a steady workload, so the round's token count repeats: tile for it
@@ -670,27 +683,26 @@ nezha_status decode_impl(nezha_ctx* c, int batch, int K, int mode, const int* dr
     if (mode == NEZHA_MODE_AR) launch_draft_set(e, batch, K, nullptr, nullptr, c->st);
     else if (round == 1 && drafts && is_tree) launch_draft_tree_set(e, batch, K, drafts, n_draft, c->st);
     else if (round == 1 && drafts) launch_draft_set(e, batch, K, drafts, n_draft, c->st);
-    else draft_phase(c, batch, K, round == 1, round == 1 ? 1 : round + 1, c->opt_filter != 0);
-    launch_build_nodes(e, batch, c->st);
+    const bool drafting = mode == NEZHA_MODE_VERIFIED && !(round == 1 && drafts);
+    if (drafting) draft_phase(c, batch, K, round == 1 ? 1 : round + 1, c->opt_filter != 0, round == (drafts ? 2 : 1), true);
+    else launch_build_nodes(e, batch, c->st);
     // Plain decoding has no draft tree: its passes hold one level's beams.  (With the tree's bound five requests of beam 9 on the
     // d = 2048 backbone ran on the 128-row accumulator instead of the 48-row one, 1,424 -> 1,328 us.)
     verify_pass(c, batch, mode == NEZHA_MODE_AR ? K : K * (L - round), K);
-    for (int n = round; n < L; ++n) {
-      SelectArgs s = select_base(c, batch, K);
-      const size_t lv_in = (size_t)n * c->Bmax * c->Kmax, lv_out = (size_t)(n + 1) * c->Bmax * c->Kmax;
-      s.logits = c->logits_v; s.row_stride = c->Nv_ld; s.col_off = e.li.off[n] - e.li.off[1];
-      s.src_row = e.tb_src + lv_in; s.src_mul = 0;
-      s.in_codes = e.tb_codes + lv_in * L; s.in_score = e.tb_score + lv_in; s.in_count = e.tb_count + (size_t)n * c->Bmax;
-      s.n = n; s.T = c->cfg.T[n]; s.per_beam = s.T; s.filter = (n + 1 == L) ? 1 : 0;
-      s.prefix_filter = (c->opt_level_filter && n + 1 < L) ? 1 : 0;
-      s.gate = e.row_cur; s.gate_mode = 1; s.gate_value = n;
-      s.out_codes = e.tb_codes + lv_out * L; s.out_score = e.tb_score + lv_out; s.out_parent = e.tb_parent + lv_out;
-      s.out_count = e.tb_count + (size_t)(n + 1) * c->Bmax;
-      RoundEnd re{};
-      if (n + 1 == L)
-        re = RoundEnd{c->host_counters + 16 + 8 * round, round, mode == NEZHA_MODE_VERIFIED ? c->opt_adaptive : 0, tr};
-      launch_select_advance(s, e, n, K, out_codes, out_scores, out_count, re, c->st);
-    }
+    // (a request in this pass has at least `round` levels settled)
+    const int n = round;
+    SelectArgs s = select_base(c, batch, K);
+    const size_t lv_in = (size_t)n * c->Bmax * c->Kmax, lv_out = (size_t)(n + 1) * c->Bmax * c->Kmax;
+    s.logits = c->logits_v; s.row_stride = c->Nv_ld; s.col_off = e.li.off[n] - e.li.off[1];
+    s.src_row = e.tb_src + lv_in; s.src_mul = 0;
+    s.in_codes = e.tb_codes + lv_in * L; s.in_score = e.tb_score + lv_in; s.in_count = e.tb_count + (size_t)n * c->Bmax;
+    s.n = n; s.T = c->cfg.T[n]; s.per_beam = s.T; s.filter = (n + 1 == L) ? 1 : 0;
+    s.prefix_filter = (c->opt_level_filter && n + 1 < L) ? 1 : 0;
+    s.gate = e.row_cur; s.gate_mode = 1; s.gate_value = n;
+    s.out_codes = e.tb_codes + lv_out * L; s.out_score = e.tb_score + lv_out; s.out_parent = e.tb_parent + lv_out;
+    s.out_count = e.tb_count + (size_t)(n + 1) * c->Bmax;
+    const RoundEnd re{c->host_counters + 16 + 8 * round, round, mode == NEZHA_MODE_VERIFIED ? c->opt_adaptive : 0, mode == NEZHA_MODE_VERIFIED ? 1 : 0, tr};
+    launch_select_advance(s, e, L, K, out_codes, out_scores, out_count, re, c->st);
     c->m_expected = 0;
   };
   // Whether another round is needed is known only from a round's counters.  A steady workload needs the same number of rounds
@@ -1011,7 +1023,7 @@ nezha_status nezha_draft_logits(nezha_ctx* c, int32_t batch, int32_t n_beams, in
     return fail(c, NEZHA_ERR_ARG, "nezha_draft_logits: bad argument");
   const EngineState& e = c->es;
   // start set = the given prefixes at level `level`; teacher-force the transitions, then Eq. 2 for the next level
-  launch_decode_begin(e, batch, 0, nullptr, nullptr, nullptr, nezha_trace{}, c->st);
+  launch_decode_begin(e, batch, 0, 0, nullptr, nullptr, nullptr, nezha_trace{}, c->st);
   launch_fill_i32(e.d_m, batch, level, c->st);
   launch_fill_i32(e.dw_count + (size_t)level * c->Bmax, batch, n_beams, c->st);
   if (level > 0) {

@@ -108,7 +108,7 @@ __device__ __forceinline__ unsigned probe_extensions(unsigned long long* slots, 
 inline bool select_probes(const SelectArgs& a) { return a.filter && a.per_beam >= a.T && !a.prefix_filter && !a.final_mask_from_map; }
 
 // What a fused kernel goes on with: the selection as it stands in shared memory (score, parent slot, code).
-struct Selected { bool active; int n; const float* s; const int* r; const int* t; };
+struct Selected { bool active; int gate, n; const float* s; const int* r; const int* t; };      // gate: the value that decided it
 // 4 bytes of global memory into shared memory without passing through a register.
 __device__ __forceinline__ void cp_async4(int* dst, const int* src) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
@@ -117,9 +117,20 @@ __device__ __forceinline__ void cp_async_ints(int* dst, const int* src, int n) {
   for (int i = threadIdx.x; i < n; i += blockDim.x) cp_async4(dst + i, src + i);
 }
 
+// What differs from level to level.  (Apart from the kernel's parameters: a copy of those that a loop changes lives in local memory.)
+struct SelectLevel {
+  int n, T, per_beam, filter, prefix_filter, col_off, gate_value;
+  const int* src_row; const int* in_codes; const float* in_score; const int* in_count;
+  int* out_codes; float* out_score; int* out_parent; int* out_count;
+};
+__device__ __forceinline__ SelectLevel level_of(const SelectArgs& a) {
+  return SelectLevel{a.n, a.T, a.per_beam, a.filter, a.prefix_filter, a.col_off, a.gate_value, a.src_row, a.in_codes, a.in_score, a.in_count,
+                     a.out_codes, a.out_score, a.out_parent, a.out_count};
+}
+
 // s_codes: the input beams' codes in shared memory ([in_stride][tuple_len], brought by cp.async of all threads), or null.
 template <int VPL, bool PROBE>
-__device__ __forceinline__ Selected select_body(const SelectArgs& a, const int* s_codes = nullptr) {
+__device__ __forceinline__ Selected select_body(const SelectArgs& a, const SelectLevel& v, const int* s_codes = nullptr) {
   const int b = blockIdx.x;
   extern __shared__ unsigned char smem_raw[];
   const int nb_cap = a.in_stride;
@@ -135,80 +146,80 @@ __device__ __forceinline__ Selected select_body(const SelectArgs& a, const int* 
 
   // ---- first wave of loads (none of these addresses depends on a loaded value)
   const int gate_v = a.gate_mode ? a.gate[b] : 0;
-  const int nb_raw = a.in_count[b];
+  const int nb_raw = v.in_count[b];
   const bool has0 = warp < nb_cap;                                   // this warp's first beam slot exists in the arrays
   const long long slot0 = (long long)b * a.in_stride + warp;
-  const bool direct0 = has0 && !a.src_row && warp < a.src_mul;       // its logits row is known without a look-up
+  const bool direct0 = has0 && !v.src_row && warp < a.src_mul;       // its logits row is known without a look-up
   long long row0 = 0;
-  if (has0) row0 = a.src_row ? (long long)a.src_row[slot0] : (long long)b * a.src_mul + warp;
-  const float base0 = has0 ? a.in_score[slot0] : 0.f;
+  if (has0) row0 = v.src_row ? (long long)v.src_row[slot0] : (long long)b * a.src_mul + warp;
+  const float base0 = has0 ? v.in_score[slot0] : 0.f;
   unsigned long long pk0 = 0;
   if (has0)
-    for (int l = 0; l < a.n; ++l) pk0 += (unsigned long long)a.in_codes[slot0 * a.tuple_len + l] * a.li.mult[l];
+    for (int l = 0; l < v.n; ++l) pk0 += (unsigned long long)v.in_codes[slot0 * a.tuple_len + l] * a.li.mult[l];
   float bias[VPL], z0[VPL];
 #pragma unroll
   for (int j = 0; j < VPL; ++j) {
     const int t = lane + 32 * j;
-    bias[j] = (a.logit_bias && t < a.T) ? a.logit_bias[(long long)b * a.bias_stride + t] : 0.f;
-    z0[j] = (direct0 && t < a.T) ? a.logits[row0 * a.row_stride + a.col_off + t] : 0.f;
+    bias[j] = (a.logit_bias && t < v.T) ? a.logit_bias[(long long)b * a.bias_stride + t] : 0.f;
+    z0[j] = (direct0 && t < v.T) ? a.logits[row0 * a.row_stride + v.col_off + t] : 0.f;
   }
-  if (a.gate_mode == 1 && gate_v != a.gate_value) return Selected{false, 0, sel_s, sel_r, sel_t};
-  if (a.gate_mode == 2 && !(gate_v < a.gate_value)) return Selected{false, 0, sel_s, sel_r, sel_t};
+  if (a.gate_mode == 1 && gate_v != v.gate_value) return Selected{false, gate_v, 0, sel_s, sel_r, sel_t};
+  if (a.gate_mode == 2 && !(gate_v < v.gate_value)) return Selected{false, gate_v, 0, sel_s, sel_r, sel_t};
   const int nb = min(nb_raw, nb_cap);
   if (threadIdx.x == 0) *s_running = 0;
-  const bool all_codes = a.per_beam >= a.T;
-  const int want = all_codes ? min(a.K, a.T) : min(a.per_beam, a.K);
-  const unsigned long long mult_n = a.li.mult[a.n];
+  const bool all_codes = v.per_beam >= v.T;
+  const int want = all_codes ? min(a.K, v.T) : min(v.per_beam, a.K);
+  const unsigned long long mult_n = a.li.mult[v.n];
 
   for (int r = warp; r < nb; r += n_warps) {
     const bool first = r == warp;
     const long long slot = (long long)b * a.in_stride + r;
-    const long long row = first ? row0 : (a.src_row ? (long long)a.src_row[slot] : (long long)b * a.src_mul + r);
-    const float* z = a.logits + row * a.row_stride + a.col_off;
+    const long long row = first ? row0 : (v.src_row ? (long long)v.src_row[slot] : (long long)b * a.src_mul + r);
+    const float* z = a.logits + row * a.row_stride + v.col_off;
     float key[VPL];
     float mx = -INFINITY;
     if (!(first && direct0)) {       // (all under way before the first is used: one by one they took 2 to 4 us)
 #pragma unroll
-      for (int j = 0; j < VPL; ++j) z0[j] = lane + 32 * j < a.T ? z[lane + 32 * j] : 0.f;
+      for (int j = 0; j < VPL; ++j) z0[j] = lane + 32 * j < v.T ? z[lane + 32 * j] : 0.f;
     }
 #pragma unroll
     for (int j = 0; j < VPL; ++j) {
       const int t = lane + 32 * j;
-      key[j] = (t < a.T) ? z0[j] + bias[j] : -INFINITY;
+      key[j] = (t < v.T) ? z0[j] + bias[j] : -INFINITY;
       mx = fmaxf(mx, key[j]);
     }
-    const float base = first ? base0 : a.in_score[slot];
+    const float base = first ? base0 : v.in_score[slot];
     unsigned long long prefix_key = pk0;
     if (!first) {
       prefix_key = 0;
-      for (int l = 0; l < a.n; ++l) prefix_key += (unsigned long long)a.in_codes[slot * a.tuple_len + l] * a.li.mult[l];
+      for (int l = 0; l < v.n; ++l) prefix_key += (unsigned long long)v.in_codes[slot * a.tuple_len + l] * a.li.mult[l];
     }
     mx = warp_max(mx);
     float sum = 0.f;
 #pragma unroll
-    for (int j = 0; j < VPL; ++j) sum += (lane + 32 * j < a.T) ? expf(key[j] - mx) : 0.f;
+    for (int j = 0; j < VPL; ++j) sum += (lane + 32 * j < v.T) ? expf(key[j] - mx) : 0.f;
     sum = warp_sum(sum);
     const float lse = mx + logf(sum);
 #pragma unroll
     for (int j = 0; j < VPL; ++j) {
-      if (lane + 32 * j < a.T) {
+      if (lane + 32 * j < v.T) {
         key[j] -= lse;                                   // log-probability
         if (all_codes) key[j] += base;                   // rank by cumulative log-probability
       }
     }
     // The bit set of the codes that may follow this beam: Eq. 5 for all T_L extensions at the last level, "some valid ID
     // begins with it" at an earlier level.
-    const bool use_bits = a.prefix_filter || (all_codes && a.filter && a.final_mask_from_map);
-    const unsigned long long* bits = use_bits ? pm_find(a.pm, a.n, prefix_key) : nullptr;
+    const bool use_bits = v.prefix_filter || (all_codes && v.filter && a.final_mask_from_map);
+    const unsigned long long* bits = use_bits ? pm_find(a.pm, v.n, prefix_key) : nullptr;
     if (all_codes && use_bits) {
 #pragma unroll
       for (int j = 0; j < VPL; ++j) {
         const int t = lane + 32 * j;
-        if (t < a.T && !pm_test(bits, t)) key[j] = -INFINITY;
+        if (t < v.T && !pm_test(bits, t)) key[j] = -INFINITY;
       }
-    } else if (PROBE && all_codes && a.filter) {
-      const unsigned ok = a.hs.narrow ? probe_extensions<true, VPL>(a.hs.slots, a.hs.n_buckets, prefix_key, mult_n, a.T)
-                                      : probe_extensions<false, VPL>(a.hs.slots, a.hs.n_buckets, prefix_key, mult_n, a.T);
+    } else if (PROBE && all_codes && v.filter) {
+      const unsigned ok = a.hs.narrow ? probe_extensions<true, VPL>(a.hs.slots, a.hs.n_buckets, prefix_key, mult_n, v.T)
+                                      : probe_extensions<false, VPL>(a.hs.slots, a.hs.n_buckets, prefix_key, mult_n, v.T);
 #pragma unroll
       for (int j = 0; j < VPL; ++j)
         if (!((ok >> j) & 1u)) key[j] = -INFINITY;
@@ -280,14 +291,14 @@ __device__ __forceinline__ Selected select_body(const SelectArgs& a, const int* 
       }
     }
     __syncwarp();
-    if (!all_codes && (a.filter || a.prefix_filter)) {   // filter the chosen codes, keep their order
+    if (!all_codes && (v.filter || v.prefix_filter)) {   // filter the chosen codes, keep their order
       int kept = 0;
       for (int c0 = 0; c0 < cnt; c0 += 32) {
         const int c = c0 + lane;
         bool ok = false; float sv = 0.f; int t = 0;
         if (c < cnt) {
           sv = l_score[(size_t)r * a.K + c]; t = l_tok[(size_t)r * a.K + c];
-          ok = a.prefix_filter ? pm_test(bits, t) : hs_contains_thread(a.hs, prefix_key + (unsigned long long)t * mult_n);
+          ok = v.prefix_filter ? pm_test(bits, t) : hs_contains_thread(a.hs, prefix_key + (unsigned long long)t * mult_n);
         }
         const unsigned m = __ballot_sync(0xffffffffu, ok);
         __syncwarp();
@@ -388,25 +399,25 @@ __device__ __forceinline__ Selected select_body(const SelectArgs& a, const int* 
   for (int k = threadIdx.x; k < a.K; k += blockDim.x) {
     const long long o = (long long)b * a.out_stride + k;
     const bool live = k < n_out;
-    a.out_score[o] = live ? sel_s[k] : -INFINITY;
-    if (a.out_parent) a.out_parent[o] = live ? sel_r[k] : -1;
+    v.out_score[o] = live ? sel_s[k] : -INFINITY;
+    if (v.out_parent) v.out_parent[o] = live ? sel_r[k] : -1;
     if (a.out_token) a.out_token[o] = live ? sel_t[k] : -1;
   }
-  if (a.out_codes) {
+  if (v.out_codes) {
     for (int i = threadIdx.x; i < a.K * a.tuple_len; i += blockDim.x) {
       const int k = i / a.tuple_len, l = i - k * a.tuple_len;
       int c = -1;
       if (k < n_out) {
-        if (l < a.n) c = s_codes ? s_codes[sel_r[k] * a.tuple_len + l] : a.in_codes[((long long)b * a.in_stride + sel_r[k]) * a.tuple_len + l];
-        else if (l == a.n) c = sel_t[k];
+        if (l < v.n) c = s_codes ? s_codes[sel_r[k] * a.tuple_len + l] : v.in_codes[((long long)b * a.in_stride + sel_r[k]) * a.tuple_len + l];
+        else if (l == v.n) c = sel_t[k];
       }
-      a.out_codes[((long long)b * a.out_stride + k) * a.tuple_len + l] = c;
+      v.out_codes[((long long)b * a.out_stride + k) * a.tuple_len + l] = c;
     }
   }
-  if (threadIdx.x == 0) a.out_count[b] = n_out;
+  if (threadIdx.x == 0) v.out_count[b] = n_out;
   // (what the kernels before this one reported; the host looks when the stream is idle, so nothing waits for the bus here: 1.5 us)
   if (a.host_status && b == 0 && threadIdx.x < 4) a.host_status[threadIdx.x] = *(volatile int*)(a.status + threadIdx.x);
-  return Selected{true, n_out, sel_s, sel_r, sel_t};
+  return Selected{true, gate_v, n_out, sel_s, sel_r, sel_t};
 }
 
 // Codes per lane of a codebook of T codes, as a constant.
@@ -422,7 +433,7 @@ template <int VPL, bool PROBE>
 __global__ void __launch_bounds__(select_max_threads(VPL)) select_kernel(SelectArgs a) {
   pdl_wait();
   pdl_launch();
-  select_body<VPL, PROBE>(a);
+  select_body<VPL, PROBE>(a, level_of(a));
 }
 
 }  // namespace
@@ -480,8 +491,9 @@ __global__ void fill_i32_kernel(int* p, long long n, int v) {
 
 // Start of a decode call, one block per request: B_0 = { empty beam, score 0 }, nothing settled, and the fill values of the
 // call's outputs (out_* and the trace's pointers may be null; their slots of rounds that do not run keep these values).
-__global__ void __launch_bounds__(128) decode_begin_kernel(EngineState e, int batch, int K, int* out_codes, float* out_scores,
-                                                           int* out_count, nezha_trace tr) {
+// from_scratch: round 1 drafts, from the empty beam (Algorithm 3's initialisation).
+__global__ void __launch_bounds__(128) decode_begin_kernel(EngineState e, int batch, int K, int from_scratch, int* out_codes,
+                                                           float* out_scores, int* out_count, nezha_trace tr) {
   pdl_wait();
   pdl_launch();
   const int b = blockIdx.x, L = e.L, R = e.L - 1;
@@ -496,10 +508,17 @@ __global__ void __launch_bounds__(128) decode_begin_kernel(EngineState e, int ba
     e.row_cur[b] = 0;
     e.row_spec[b] = 1;
     e.row_m_start[b] = 0;
-    e.d_m[b] = L;
+    e.d_m[b] = from_scratch ? 0 : L;
     if (out_count) out_count[b] = 0;
   }
-  for (int l = threadIdx.x; l <= L; l += blockDim.x) e.dw_count[(long long)l * e.Bmax + b] = 0;     // no draft tree yet
+  for (int l = threadIdx.x; l <= L; l += blockDim.x) e.dw_count[(long long)l * e.Bmax + b] = l == 0 && from_scratch ? 1 : 0;
+  if (from_scratch)
+    for (int k = threadIdx.x; k < e.Kmax; k += blockDim.x) {
+      const long long s = lvl_bk(e, 0, b, k);
+      e.dw_score[s] = k == 0 ? 0.f : -INFINITY;
+      e.dw_parent[s] = k == 0 ? 0 : -1;
+      for (int l = 0; l < L; ++l) e.dw_codes[s * L + l] = -1;
+    }
   if (out_scores) for (int i = threadIdx.x; i < K; i += blockDim.x) out_scores[(long long)b * K + i] = -INFINITY;
   auto fill = [&](int* p, int slices, int per) {       // [slices][batch][per]
     if (!p) return;
@@ -509,41 +528,6 @@ __global__ void __launch_bounds__(128) decode_begin_kernel(EngineState e, int ba
   fill(out_codes, 1, K * L);
   fill(tr.drafts, R, K * L); fill(tr.n_draft, R, 1); fill(tr.accepted_len, R, K); fill(tr.level_reached, R, 1);
   fill(tr.tree_codes, R * L, K * L); fill(tr.tree_count, R * L, 1);
-}
-
-// Start of a round's drafting (Algorithm 2's drafting step): the draft head continues from the true beams B_m, or from
-// the empty beam in the first round (Algorithm 3's initialisation).
-// Also clears the round's counters (this is the first kernel of a drafting round) and, when s_act is given, starts
-// every beam slot's draft state at s_1 = h_0 (Eq. 1).  Grid = (requests, beam slots); slot 0's block does the bookkeeping.
-// (One block per request for all of its slots took 9 us at one request of d = 2048 and 30 us at d = 4096, beam 20.)
-__global__ void __launch_bounds__(128) draft_init_kernel(EngineState e, int batch, int from_scratch, __nv_bfloat16* s_act) {
-  pdl_wait();
-  pdl_launch();
-  const int b = blockIdx.x;
-  if (s_act) {
-    const float* h0 = e.h_f32 + (long long)b * (e.L + 1) * e.d;
-    __nv_bfloat16* dst = s_act + ((long long)b * e.Kmax + blockIdx.y) * e.d;
-    for (int c = threadIdx.x; c < e.d; c += blockDim.x) dst[c] = __float2bfloat16_rn(h0[c]);
-  }
-  if (blockIdx.y != 0) return;
-  if (b == 0 && threadIdx.x < 8) e.counters[threadIdx.x] = 0;
-  if (b == 0 && threadIdx.x == 0) *e.n_tokens = 0;
-  const int m = e.row_m[b];
-  if (m >= e.L || !e.row_spec[b]) {              // finished, or its drafting is switched off: an empty tree this round
-    if (threadIdx.x == 0) e.d_m[b] = e.L;
-    if ((int)threadIdx.x <= e.L) e.dw_count[(long long)threadIdx.x * e.Bmax + b] = 0;
-    return;
-  }
-  const int mm = from_scratch ? 0 : m;
-  const int cnt = e.tb_count[mm * e.Bmax + b];
-  for (int k = threadIdx.x; k < e.Kmax; k += blockDim.x) {
-    const long long s = lvl_bk(e, mm, b, k);
-    const bool live = k < cnt;
-    e.dw_score[s] = live ? e.tb_score[s] : -INFINITY;
-    e.dw_parent[s] = live ? k : -1;
-    for (int l = 0; l < e.L; ++l) e.dw_codes[s * e.L + l] = live ? e.tb_codes[s * e.L + l] : -1;
-  }
-  if (threadIdx.x == 0) { e.dw_count[mm * e.Bmax + b] = cnt; e.d_m[b] = mm; }
 }
 
 // Caller-supplied drafted tuples for the round (or none: n_draft == nullptr and drafts == nullptr -> an empty tree).
@@ -709,22 +693,23 @@ __global__ void draft_state_init_kernel(EngineState e, int batch, __nv_bfloat16*
 
 // Eq. 3 after the product: s_{l+1}[k] = tanh((W_s s_l)[parent] + (W_e E)[code] + b).  G holds [logits | W_s s_l] of
 // every beam slot of level l (W_s s_l from column t_cols on), U = W_e E for every code token.  Which (parent, code) a
-// slot takes is decided exactly as in trans_gather_kernel.
+// slot takes is decided exactly as in trans_gather_kernel.  per_req: rows of G per request, Kmax (row = the parent's slot), or 1: at
+// level 1 every slot's state is s_1 = h_0 (Eq. 1).
 __device__ __forceinline__ void draft_state(const EngineState& e, int b, int k, int l, int parent, int code, const float* __restrict__ G,
-                                            long long g_stride, int t_cols, const float* __restrict__ U,
+                                            int per_req, long long g_stride, int t_cols, const float* __restrict__ U,
                                             const float* __restrict__ bias, __nv_bfloat16* s_act, int tid, int n_thr) {
   __nv_bfloat16* dst = s_act + ((long long)b * e.Kmax + k) * e.d;
   if (parent < 0 || code < 0) {                    // no such beam
     for (int c = tid; c < e.d; c += n_thr) dst[c] = __float2bfloat16_rn(0.f);
     return;
   }
-  const float* z = G + ((long long)b * e.Kmax + parent) * g_stride + t_cols;
+  const float* z = G + ((long long)b * per_req + (per_req > 1 ? parent : 0)) * g_stride + t_cols;
   const float* u = U + (long long)(e.li.off[l - 1] + code) * e.d;
 #pragma unroll 4
   for (int c = tid; c < e.d; c += n_thr) dst[c] = __float2bfloat16_rn(tanhf(z[c] + u[c] + bias[c]));
 }
 __device__ __forceinline__ void draft_step_slot(const EngineState& e, int b, int k, int l, const float* __restrict__ G,
-                                                long long g_stride, int t_cols, const float* __restrict__ U,
+                                                int per_req, long long g_stride, int t_cols, const float* __restrict__ U,
                                                 const float* __restrict__ bias, __nv_bfloat16* s_act, int tid, int n_thr) {
   const int dm = e.d_m[b];
   int src_level, parent;
@@ -735,34 +720,34 @@ __device__ __forceinline__ void draft_step_slot(const EngineState& e, int b, int
   live = live && k < e.dw_count[src_level * e.Bmax + b];
   if (live && parent == -2) parent = e.dw_parent[s_idx];
   const int code = live ? e.dw_codes[s_idx * e.L + (l - 1)] : -1;
-  draft_state(e, b, k, l, live ? parent : -1, code, G, g_stride, t_cols, U, bias, s_act, tid, n_thr);
+  draft_state(e, b, k, l, live ? parent : -1, code, G, per_req, g_stride, t_cols, U, bias, s_act, tid, n_thr);
 }
-__global__ void draft_step_kernel(EngineState e, int batch, int l, const float* __restrict__ G, long long g_stride, int t_cols,
+__global__ void draft_step_kernel(EngineState e, int batch, int l, const float* __restrict__ G, int per_req, long long g_stride, int t_cols,
                                   const float* __restrict__ U, const float* __restrict__ bias, __nv_bfloat16* s_act) {
   pdl_wait();
   pdl_launch();
   const int bk = blockIdx.x;
   const int b = bk / e.Kmax, k = bk - b * e.Kmax;
   if (b >= batch) return;
-  draft_step_slot(e, b, k, l, G, g_stride, t_cols, U, bias, s_act, threadIdx.x, blockDim.x);
+  draft_step_slot(e, b, k, l, G, per_req, g_stride, t_cols, U, bias, s_act, threadIdx.x, blockDim.x);
 }
 // The selection of draft level l and the state update that follows it, in one launch: a block selects its request's
 // beams (or skips that when the request's level is already settled) and then advances the states of its own slots.
 template <int VPL>
 __global__ void __launch_bounds__(select_max_threads(VPL)) select_step_kernel(SelectArgs a, EngineState e, int l, const float* __restrict__ G,
-                                                          long long g_stride, int t_cols, const float* __restrict__ U,
+                                                          int per_req, long long g_stride, int t_cols, const float* __restrict__ U,
                                                           const float* __restrict__ bias, __nv_bfloat16* s_act) {
   pdl_wait();
   pdl_launch();
-  const Selected sel = select_body<VPL, false>(a);   // (an earlier level than the last: nothing to probe)
+  const Selected sel = select_body<VPL, false>(a, level_of(a));   // (an earlier level than the last: nothing to probe)
   const int warp = threadIdx.x >> 5, n_warps = blockDim.x >> 5, lane = threadIdx.x & 31;    // a warp per beam slot
   if (sel.active) {                                // (whose selection is still in shared memory: nothing to read back)
     for (int k = warp; k < e.Kmax; k += n_warps)
-      draft_state(e, blockIdx.x, k, l, k < sel.n ? sel.r[k] : -1, k < sel.n ? sel.t[k] : -1, G, g_stride, t_cols, U, bias, s_act, lane, 32);
+      draft_state(e, blockIdx.x, k, l, k < sel.n ? sel.r[k] : -1, k < sel.n ? sel.t[k] : -1, G, per_req, g_stride, t_cols, U, bias, s_act, lane, 32);
     return;
   }
   for (int k = warp; k < e.Kmax; k += n_warps)
-    draft_step_slot(e, blockIdx.x, k, l, G, g_stride, t_cols, U, bias, s_act, lane, 32);
+    draft_step_slot(e, blockIdx.x, k, l, G, per_req, g_stride, t_cols, U, bias, s_act, lane, 32);
 }
 
 // dst[b, r, :] = src[(b * row_mul + r), 0 : T] + bias[b, :]
@@ -790,9 +775,7 @@ __device__ __forceinline__ unsigned long long prefix_key_of(const EngineState& e
 // per distinct drafted prefix.  A level-m node of the tree is alive if its codes are a beam of B_m; a higher node if its
 // parent is alive.  Tokens of a request are contiguous; the requests take their place in the list in the order in which
 // their blocks get there (no row of a pass depends on where it stands).
-__global__ void __launch_bounds__(128) nodes_kernel(EngineState e, int batch) {
-  pdl_wait();
-  pdl_launch();
+__device__ __forceinline__ void nodes_body(const EngineState& e) {
   const int b = blockIdx.x;
   const int L = e.L, Kmax = e.Kmax;
   __shared__ int s_off, n_alive, s_rank[kMaxLevels][128], s_level_start[kMaxLevels + 1];
@@ -903,6 +886,21 @@ __global__ void __launch_bounds__(128) nodes_kernel(EngineState e, int batch) {
   }
 }
 
+__global__ void __launch_bounds__(128) nodes_kernel(EngineState e) {
+  pdl_wait();
+  pdl_launch();
+  nodes_body(e);
+}
+// The draft head's last selection, whose tuples nothing asks for before the round's end, and beside it (blockIdx.y = 1) the token
+// list, which goes by the levels before.
+template <int VPL, bool PROBE>
+__global__ void __launch_bounds__(select_max_threads(VPL)) select_nodes_kernel(SelectArgs a, EngineState e) {
+  pdl_wait();
+  pdl_launch();
+  if (blockIdx.y == 0) select_body<VPL, PROBE>(a, level_of(a));
+  else nodes_body(e);
+}
+
 // Teacher-forced nodes: beams given by the caller, every beam processes all of its `level` codes.
 __global__ void nodes_from_prefixes_kernel(EngineState e, int batch, int n_beams, int level, const int* prefixes) {
   pdl_wait();
@@ -947,7 +945,8 @@ struct AdvanceSmem {
   int* node;                     // [Kmax][L] dw_codes of level n + 1
   int *dbeam, *nidx, *self;      // [Kmax]    d_beam and node_index of level n + 1, tb_self of level n
   int* anc;                      // [Kmax][L] tb_anc of level n
-  int* beams;                    // [L][Kmax][L] tb_codes of levels 1..L (the round's end only)
+  int* drafted;                  // [Kmax][L] dw_codes of level L (the round's end only, like what follows)
+  int* beams;                    // [L][Kmax][L] tb_codes of levels 1..L
 };
 __device__ __forceinline__ AdvanceSmem advance_smem(unsigned char* base, int Kmax, int L) {
   AdvanceSmem m;
@@ -955,7 +954,7 @@ __device__ __forceinline__ AdvanceSmem advance_smem(unsigned char* base, int Kma
   m.codes = reinterpret_cast<int*>(m.key + (size_t)L * Kmax);
   m.node = m.codes + Kmax * L; m.anc = m.node + Kmax * L;
   m.dbeam = m.anc + Kmax * L; m.nidx = m.dbeam + Kmax; m.self = m.nidx + Kmax;
-  m.beams = m.self + Kmax;
+  m.drafted = m.self + Kmax; m.beams = m.drafted + Kmax * L;
   return m;
 }
 
@@ -965,10 +964,11 @@ __device__ __forceinline__ AdvanceSmem advance_smem(unsigned char* base, int Kma
 //                KV rows simply become unreachable) and is matched against the alive nodes of level n+1 of the draft
 //                tree.  If every beam is such a node, its hidden state is already in the pass and selection goes on;
 //                else level n+1 is the rejection level and the request waits for the next round.
-// nd: nodes of level n + 1.
-__device__ __forceinline__ void advance_body(const EngineState& e, const AdvanceSmem& sm, const Selected& sel, int n, int K, int nd,
+// nd: nodes of level n + 1.  Returns where the request stands: levels settled, and the level whose beams have logits in this pass (or -1).
+struct Advanced { int m, cur; };
+__device__ __forceinline__ Advanced advance_body(const EngineState& e, const AdvanceSmem& sm, const Selected& sel, int n, int K, int nd,
                                              int* out_codes, float* out_score, int* out_count) {
-  const int b = blockIdx.x, L = e.L, Kmax = e.Kmax, n1 = n + 1, cnt = sel.n;
+  const int b = blockIdx.x, L = e.L, n1 = n + 1, cnt = sel.n;
   if (n1 == L) {
     for (int k = threadIdx.x; k < K; k += blockDim.x) out_score[(long long)b * K + k] = k < cnt ? sel.s[k] : -INFINITY;
     for (int i = threadIdx.x; i < K * L; i += blockDim.x) {
@@ -976,7 +976,7 @@ __device__ __forceinline__ void advance_body(const EngineState& e, const Advance
       out_codes[(long long)b * K * L + i] = k >= cnt ? -1 : l < n ? sm.codes[sel.r[k] * L + l] : sel.t[k];
     }
     if (threadIdx.x == 0) { out_count[b] = cnt; e.row_m[b] = L; e.row_cur[b] = -1; }
-    return;
+    return Advanced{L, -1};
   }
   __shared__ int all_matched;
   if (threadIdx.x == 0) all_matched = 1;
@@ -997,11 +997,13 @@ __device__ __forceinline__ void advance_body(const EngineState& e, const Advance
     if (match < 0) all_matched = 0;
   }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    e.row_m[b] = cnt == 0 ? L : n1;                // (no beam survived -- possible only with an empty codebook: finish empty)
-    e.row_cur[b] = (all_matched && cnt > 0) ? n1 : -1;
+  const Advanced ad{cnt == 0 ? L : n1, (all_matched && cnt > 0) ? n1 : -1};   // (no beam survived -- possible only with an empty codebook:
+  if (threadIdx.x == 0) {                                                       //  finish empty)
+    e.row_m[b] = ad.m;
+    e.row_cur[b] = ad.cur;
     if (cnt == 0) out_count[b] = 0;
   }
+  return ad;
 }
 
 // End of a round: accepted length of every draft = the largest i <= (level reached) with D[k][0..i) in B_i;
@@ -1009,16 +1011,16 @@ __device__ __forceinline__ void advance_body(const EngineState& e, const Advance
 // here writes to the host's pinned memory together with the status word (a copy node behind every round costs 10 us).
 // adaptive: a request whose round settled only the one level that the pass settles anyway gained nothing from its drafts
 // and stops drafting (its remaining rounds are plain autoregressive steps).
+// re.draft_next: the start of the next round's drafting (Algorithm 2's drafting step): the draft head continues from the true beams B_m.
 // What the block read about its request at the start of the kernel:
 struct RowState { int m, m_start, spec, tokens, nd_last; };    // nd_last: drafted tuples (nodes of level L)
-__device__ __forceinline__ void round_end_body(const EngineState& e, const AdvanceSmem& sm, const Selected& sel, const RowState& rs, int K,
+__device__ __forceinline__ void round_end_body(const EngineState& e, const AdvanceSmem& sm, int m_now, const RowState& rs, int K,
                                                const RoundEnd& re) {
   const int b = blockIdx.x, batch = gridDim.x, round = re.round;
   const int L = e.L, Kmax = e.Kmax;
   const nezha_trace& tr = re.tr;
   __shared__ int acc_sum;
   const int took_part = rs.tokens > 0;
-  const int m_now = sel.active ? L : rs.m;         // (behind the last level an active request is finished)
   const int nd = took_part ? rs.nd_last : 0;
   const long long tro = ((long long)(round - 1) * batch + b);
   if (threadIdx.x == 0) acc_sum = 0;
@@ -1029,16 +1031,12 @@ __device__ __forceinline__ void round_end_body(const EngineState& e, const Advan
   if (nd > 0) {
     for (int i = threadIdx.x; i < m_now * Kmax; i += blockDim.x) {
       const int lv = i / Kmax, r = i - lv * Kmax;  // beams of level lv + 1 (beyond their count -- at most K -- the codes are -1)
-      unsigned long long key;
-      if (sel.active && lv == L - 1)
-        key = r < sel.n ? prefix_key_of(e, sm.codes + sel.r[r] * L, L - 1) + (unsigned long long)sel.t[r] * e.li.mult[L - 1] : kEmptyKey;
-      else key = r < K && sm.beams[(lv * Kmax + r) * L] >= 0 ? prefix_key_of(e, sm.beams + (lv * Kmax + r) * L, lv + 1) : kEmptyKey;
-      sm.key[i] = key;
+      sm.key[i] = r < K && sm.beams[(lv * Kmax + r) * L] >= 0 ? prefix_key_of(e, sm.beams + (lv * Kmax + r) * L, lv + 1) : kEmptyKey;
     }
     __syncthreads();
     unsigned long long key = 0;
     for (int i = 1; i <= m_now && mine && acc == i - 1; ++i) {
-      key += (unsigned long long)(unsigned)sm.node[k * L + i - 1] * e.li.mult[i - 1];
+      key += (unsigned long long)(unsigned)sm.drafted[k * L + i - 1] * e.li.mult[i - 1];
       bool in = false;
       for (int r = 0; r < K; ++r) in |= sm.key[(i - 1) * Kmax + r] == key;
       if (in) acc = i;
@@ -1050,7 +1048,7 @@ __device__ __forceinline__ void round_end_body(const EngineState& e, const Advan
     if (tr.accepted_len) tr.accepted_len[tro * K + k] = acc;
     if (tr.drafts)
       for (int l = 0; l < L; ++l)
-        tr.drafts[(tro * K + k) * L + l] = (k < nd) ? sm.node[k * L + l] : -1;
+        tr.drafts[(tro * K + k) * L + l] = (k < nd) ? sm.drafted[k * L + l] : -1;
     if (tr.tree_codes)
       for (int j = 1; j <= L; ++j) {
         const int nj = took_part ? min(e.dw_count[(long long)j * e.Bmax + b], Kmax) : 0;
@@ -1061,13 +1059,30 @@ __device__ __forceinline__ void round_end_body(const EngineState& e, const Advan
   if (tr.tree_count && threadIdx.x < L)
     tr.tree_count[((long long)(round - 1) * L + threadIdx.x) * batch + b] =
         took_part ? min(min(e.dw_count[(long long)(threadIdx.x + 1) * e.Bmax + b], Kmax), K) : -1;
-  __syncthreads();
+  __syncthreads();                                 // (the round's draft tree has been read)
+  const int spec = took_part && re.adaptive ? (m_now - rs.m_start >= 2 ? 1 : 0) : rs.spec;
+  if (re.draft_next) {
+    const bool drafts = m_now < L && spec;         // (not finished, and its drafting not switched off; otherwise an empty tree)
+    if (drafts) {
+      const int cnt = e.tb_count[(long long)m_now * e.Bmax + b];
+      for (int i = threadIdx.x; i < Kmax * (L + 1); i += blockDim.x) {
+        const int s = i / (L + 1), l = i - s * (L + 1);
+        const long long o = lvl_bk(e, m_now, b, s);
+        const bool live = s < cnt;
+        if (l < L) e.dw_codes[o * L + l] = live ? sm.beams[((m_now - 1) * Kmax + s) * L + l] : -1;
+        else { e.dw_score[o] = live ? e.tb_score[o] : -INFINITY; e.dw_parent[o] = live ? s : -1; }
+      }
+      if (threadIdx.x == 0) { e.dw_count[(long long)m_now * e.Bmax + b] = cnt; e.d_m[b] = m_now; }
+    } else {
+      if (threadIdx.x == 0) e.d_m[b] = L;
+      if ((int)threadIdx.x <= L) e.dw_count[(long long)threadIdx.x * e.Bmax + b] = 0;
+    }
+  }
   int last = 0;
   if (threadIdx.x == 0) {
     if (tr.n_draft) tr.n_draft[tro] = took_part ? nd : -1;
     if (tr.level_reached) tr.level_reached[tro] = took_part ? m_now : -1;
-    int spec = rs.spec;
-    if (took_part && re.adaptive) { spec = (m_now - rs.m_start >= 2) ? 1 : 0; e.row_spec[b] = spec; }
+    if (took_part && re.adaptive) e.row_spec[b] = spec;
     if (m_now < L && spec) atomicMax(e.draft_rows, batch * Kmax);            // somebody drafts next round
     if (m_now < L) atomicAdd(&e.counters[0], 1);
     if (took_part) atomicAdd(&e.counters[1], rs.tokens);
@@ -1081,38 +1096,68 @@ __device__ __forceinline__ void round_end_body(const EngineState& e, const Advan
     __threadfence();
     const int i = threadIdx.x;
     re.host[i] = i < 4 ? *(volatile int*)(e.counters + i) : *(volatile int*)(e.status + i - 4);
+    e.counters[i] = 0;                             // for the next round
+    if (i == 0) *e.n_tokens = 0;
   }
 }
 
-// The selection of B_{n+1}, the step above (both act on the requests whose current level is n) and, behind the last level,
-// the end of the round, in one launch.
+// A pass's selections of a request, one level after the other for as long as its beams are nodes of the pass: B_{n+1} from the logits
+// of B_n, the step above, and on with n + 1 -- and, behind the last, the end of the round.  One launch: with a launch per level the
+// levels that a rejection leaves over were launches for nothing (64 requests, small shape, natural drafts: three of seven).
+// a: the arguments of the first level; levels: the levels from there on up to (not including) `last`.
 template <int VPL, bool PROBE>
-__global__ void __launch_bounds__(select_max_threads(VPL)) select_advance_kernel(SelectArgs a, EngineState e, int n, int K, int* out_codes,
+__global__ void __launch_bounds__(select_max_threads(VPL)) select_advance_kernel(SelectArgs a, EngineState e, int last, int K, int* out_codes,
                                                              float* out_score, int* out_count, RoundEnd re, int select_bytes) {
   extern __shared__ unsigned char smem_raw[];
-  const int b = blockIdx.x, L = e.L, Kmax = e.Kmax, n1 = n + 1;
+  const int b = blockIdx.x, L = e.L, Kmax = e.Kmax;
   const AdvanceSmem sm = advance_smem(smem_raw + select_bytes, Kmax, L);
   pdl_wait();
   pdl_launch();
-  cp_async_ints(sm.codes, e.tb_codes + lvl_bk(e, n, b, 0) * L, Kmax * L);
-  cp_async_ints(sm.node, e.dw_codes + lvl_bk(e, n1, b, 0) * L, Kmax * L);
-  if (n1 < L) {
-    cp_async_ints(sm.dbeam, e.d_beam + lvl_bk(e, n1, b, 0), Kmax);
-    cp_async_ints(sm.nidx, e.node_index + ((long long)b * L + n1) * Kmax, Kmax);
-    cp_async_ints(sm.self, e.tb_self + lvl_bk(e, n, b, 0), Kmax);
-    cp_async_ints(sm.anc, e.tb_anc + lvl_bk(e, n, b, 0) * L, Kmax * L);
-  }
-  if (re.host)
-    for (int lv = 1; lv <= L; ++lv) cp_async_ints(sm.beams + (lv - 1) * Kmax * L, e.tb_codes + lvl_bk(e, lv, b, 0) * L, Kmax * L);
-  const int nd = min(e.dw_count[(long long)n1 * e.Bmax + b], Kmax);
+  auto fetch_beams = [&](int lv) { cp_async_ints(sm.beams + (lv - 1) * Kmax * L, e.tb_codes + lvl_bk(e, lv, b, 0) * L, Kmax * L); };
   RowState rs{0, 0, 0, 0, 0};
-  if (re.host) rs = RowState{e.row_m[b], e.row_m_start[b], e.row_spec[b], e.row_tok_count[b], nd};
-  const Selected sel = select_body<VPL, PROBE>(a, sm.codes);
-  if (sel.active) advance_body(e, sm, sel, n, K, nd, out_codes, out_score, out_count);
-  else asm volatile("cp.async.wait_all;" ::: "memory");
   if (re.host) {
+    cp_async_ints(sm.drafted, e.dw_codes + lvl_bk(e, L, b, 0) * L, Kmax * L);
+    for (int lv = 1; lv <= L; ++lv) fetch_beams(lv);
+    rs = RowState{e.row_m[b], e.row_m_start[b], e.row_spec[b], e.row_tok_count[b], min(e.dw_count[(long long)L * e.Bmax + b], Kmax)};
+  }
+  int m_now = rs.m;
+  SelectLevel v = level_of(a);
+#pragma unroll 1
+  for (;;) {
+    const int n = v.n, n1 = n + 1;
+    cp_async_ints(sm.codes, e.tb_codes + lvl_bk(e, n, b, 0) * L, Kmax * L);
+    cp_async_ints(sm.node, e.dw_codes + lvl_bk(e, n1, b, 0) * L, Kmax * L);
+    if (n1 < L) {
+      cp_async_ints(sm.dbeam, e.d_beam + lvl_bk(e, n1, b, 0), Kmax);
+      cp_async_ints(sm.nidx, e.node_index + ((long long)b * L + n1) * Kmax, Kmax);
+      cp_async_ints(sm.self, e.tb_self + lvl_bk(e, n, b, 0), Kmax);
+      cp_async_ints(sm.anc, e.tb_anc + lvl_bk(e, n, b, 0) * L, Kmax * L);
+    }
+    const int nd = min(e.dw_count[(long long)n1 * e.Bmax + b], Kmax);
+    const Selected sel = select_body<VPL, PROBE>(a, v, sm.codes);
+    int cur = sel.gate;                            // where an inactive request stands: not here, or further on
+    if (sel.active) {
+      const Advanced ad = advance_body(e, sm, sel, n, K, nd, out_codes, out_score, out_count);
+      m_now = ad.m; cur = ad.cur;
+    } else {
+      asm volatile("cp.async.wait_all;" ::: "memory");
+    }
+    __syncthreads();                               // the tables that this level has written and the next reads, and shared memory
+    if (re.host && sel.active) fetch_beams(n1);    // (as they are now)
+    if (cur < n1 || n1 >= last) break;
+    // on to level n1
+    const long long lv = (long long)e.Bmax * Kmax;
+    v.col_off += v.T;
+    v.n = n1; v.T = e.li.T[n1]; v.per_beam = v.T; v.gate_value = n1;
+    v.filter = n1 + 1 == L ? 1 : 0;
+    if (v.filter) v.prefix_filter = 0;
+    v.src_row += lv; v.in_codes += lv * L; v.in_score += lv; v.in_count += e.Bmax;
+    v.out_codes += lv * L; v.out_score += lv; v.out_parent += lv; v.out_count += e.Bmax;
+  }
+  if (re.host) {
+    asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
-    round_end_body(e, sm, sel, rs, K, re);
+    round_end_body(e, sm, m_now, rs, K, re);
   }
 }
 
@@ -1153,14 +1198,10 @@ void launch_fill_i32(int* p, long long n, int v, cudaStream_t st) {
   LaunchScope ls(kcMisc, st);
   launch_pdl(fill_i32_kernel, dim3((unsigned)((n + 255) / 256 < 1184 ? (n + 255) / 256 : 1184)), dim3(256), 0, st, p, n, v);
 }
-void launch_decode_begin(const EngineState& e, int batch, int K, int* out_codes, float* out_scores, int* out_count,
+void launch_decode_begin(const EngineState& e, int batch, int K, int from_scratch, int* out_codes, float* out_scores, int* out_count,
                          const nezha_trace& tr, cudaStream_t st) {
   LaunchScope ls(kcMisc, st);
-  launch_pdl(decode_begin_kernel, dim3(batch), dim3(128), 0, st, e, batch, K, out_codes, out_scores, out_count, tr);
-}
-void launch_draft_init(const EngineState& e, int batch, int from_scratch, void* s_act, cudaStream_t st) {
-  LaunchScope ls(kcDraftGlue, st);
-  launch_pdl(draft_init_kernel, dim3(batch, s_act ? e.Kmax : 1), dim3(128), 0, st, e, batch, from_scratch, (__nv_bfloat16*)s_act);
+  launch_pdl(decode_begin_kernel, dim3(batch), dim3(128), 0, st, e, batch, K, from_scratch, out_codes, out_scores, out_count, tr);
 }
 void launch_draft_set(const EngineState& e, int batch, int K, const int* drafts, const int* n_draft, cudaStream_t st) {
   LaunchScope ls(kcDraftGlue, st);
@@ -1196,13 +1237,13 @@ void launch_draft_state_init(const EngineState& e, int batch, void* s_act, cudaS
   LaunchScope ls(kcDraftGlue, st);
   launch_pdl(draft_state_init_kernel, dim3(batch * e.Kmax), dim3(128), 0, st, e, batch, (__nv_bfloat16*)s_act);
 }
-void launch_draft_step(const EngineState& e, int batch, int l, const float* G, long long g_stride, int t_cols, const float* U,
+void launch_draft_step(const EngineState& e, int batch, int l, const float* G, int per_req, long long g_stride, int t_cols, const float* U,
                        const float* bias, void* s_act, cudaStream_t st) {
   LaunchScope ls(kcDraftGlue, st);
-  launch_pdl(draft_step_kernel, dim3(batch * e.Kmax), dim3(128), 0, st, e, batch, l, G, g_stride, t_cols, U, bias,
+  launch_pdl(draft_step_kernel, dim3(batch * e.Kmax), dim3(128), 0, st, e, batch, l, G, per_req, g_stride, t_cols, U, bias,
              (__nv_bfloat16*)s_act);
 }
-size_t advance_smem_bytes(int Kmax, int L) { return (size_t)Kmax * (8 * L + 4 * (3 * L + 3 + L * L)); }
+size_t advance_smem_bytes(int Kmax, int L) { return (size_t)Kmax * (8 * L + 4 * (4 * L + 3 + L * L)); }
 cudaError_t select_step_configure(int bytes) {
   cudaError_t e = cudaSuccess;
   auto set = [&](auto vpl) {
@@ -1211,11 +1252,13 @@ cudaError_t select_step_configure(int bytes) {
     if (e == cudaSuccess) e = cudaFuncSetAttribute(select_advance_kernel<V, false>, attr, bytes);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(select_advance_kernel<V, true>, attr, bytes);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(select_step_kernel<V>, attr, bytes);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(select_nodes_kernel<V, false>, attr, bytes);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(select_nodes_kernel<V, true>, attr, bytes);
   };
   set(Vpl<1>{}); set(Vpl<8>{}); set(Vpl<16>{}); set(Vpl<32>{});
   return e;
 }
-void launch_select_step(const SelectArgs& a, const EngineState& e, int l, const float* G, long long g_stride, int t_cols,
+void launch_select_step(const SelectArgs& a, const EngineState& e, int l, const float* G, int per_req, long long g_stride, int t_cols,
                         const float* U, const float* bias, void* s_act, cudaStream_t st) {
   if (a.batch <= 0) return;
   const size_t smem = select_smem_bytes(a.in_stride, a.K);
@@ -1224,7 +1267,7 @@ void launch_select_step(const SelectArgs& a, const EngineState& e, int l, const 
   const dim3 block(32 * warps), grid(a.batch);
   __nv_bfloat16* s = (__nv_bfloat16*)s_act;
   with_vpl(a.T, [&](auto vpl) {
-    launch_pdl(select_step_kernel<decltype(vpl)::value>, grid, block, smem, st, a, e, l, G, g_stride, t_cols, U, bias, s);
+    launch_pdl(select_step_kernel<decltype(vpl)::value>, grid, block, smem, st, a, e, l, G, per_req, g_stride, t_cols, U, bias, s);
   });
 }
 void launch_copy_logits_bias(const float* src, long long row_stride, int row_mul, int batch, int n_beams, int T,
@@ -1235,24 +1278,38 @@ void launch_copy_logits_bias(const float* src, long long row_stride, int row_mul
 }
 void launch_build_nodes(const EngineState& e, int batch, cudaStream_t st) {
   LaunchScope ls(kcNodes, st);
-  launch_pdl(nodes_kernel, dim3(batch), dim3(128), 0, st, e, batch);
+  launch_pdl(nodes_kernel, dim3(batch), dim3(128), 0, st, e);
+}
+void launch_select_nodes(const SelectArgs& a, const EngineState& e, cudaStream_t st) {
+  if (a.batch <= 0) return;
+  const size_t smem = select_smem_bytes(a.in_stride, a.K);
+  LaunchScope ls(kcSelect, st);
+  const dim3 block(32 * select_warps(a)), grid(a.batch, 2);
+  with_vpl(a.T, [&](auto vpl) {
+    constexpr int V = decltype(vpl)::value;
+    launch_pdl(select_probes(a) ? select_nodes_kernel<V, true> : select_nodes_kernel<V, false>, grid, block, smem, st, a, e);
+  });
 }
 void launch_nodes_from_prefixes(const EngineState& e, int batch, int n_beams, int level, const int* prefixes,
                                 cudaStream_t st) {
   LaunchScope ls(kcNodes, st);
   launch_pdl(nodes_from_prefixes_kernel, dim3(batch), dim3(128), 0, st, e, batch, n_beams, level, prefixes);
 }
-void launch_select_advance(const SelectArgs& a, const EngineState& e, int n, int K, int* out_codes, float* out_score,
+void launch_select_advance(const SelectArgs& a, const EngineState& e, int last, int K, int* out_codes, float* out_score,
                            int* out_count, const RoundEnd& re, cudaStream_t st) {
   if (a.batch <= 0) return;
   const size_t select_bytes = select_smem_bytes(a.in_stride, a.K), smem = select_bytes + advance_smem_bytes(e.Kmax, e.L);
   LaunchScope ls(kcSelect, st);
-  const int warps = select_warps(a);
-  const dim3 block(32 * warps), grid(a.batch);
-  with_vpl(a.T, [&](auto vpl) {
+  SelectArgs widest = a;                           // (of the levels: the codes per lane and the warps)
+  for (int n = a.n + 1; n < last; ++n) widest.T = a.li.T[n] > widest.T ? a.li.T[n] : widest.T;
+  SelectArgs final_level = a;
+  final_level.filter = last == e.L ? 1 : 0; final_level.per_beam = final_level.T;
+  if (final_level.filter) final_level.prefix_filter = 0;
+  const dim3 block(32 * select_warps(widest)), grid(a.batch);
+  with_vpl(widest.T, [&](auto vpl) {
     constexpr int V = decltype(vpl)::value;
-    launch_pdl(select_probes(a) ? select_advance_kernel<V, true> : select_advance_kernel<V, false>, grid, block, smem, st, a, e, n,
-               K, out_codes, out_score, out_count, re, (int)select_bytes);
+    launch_pdl(select_probes(final_level) ? select_advance_kernel<V, true> : select_advance_kernel<V, false>, grid, block, smem, st, a, e,
+               last, K, out_codes, out_score, out_count, re, (int)select_bytes);
   });
 }
 void launch_copy_logits(const float* src, long long row_stride, int col_off, const int* row_index, int row_mul,

@@ -79,21 +79,23 @@ struct SelectArgs {
 void launch_select(const SelectArgs& a, cudaStream_t st);
 // What closes a round, behind its last selection (host == null: not this one): the trace's outputs and, in pinned host memory,
 // the counters (words 0-3) and the status words (4-7).
-struct RoundEnd { int* host; int round, adaptive; nezha_trace tr; };
-// launch_select (gated on row_cur == n) followed, in the same launch, by the accept / roll-back step of level n and, behind
-// the last level, the end of the round
-void launch_select_advance(const SelectArgs& a, const EngineState& e, int n, int K, int* out_codes, float* out_score,
+struct RoundEnd { int* host; int round, adaptive, draft_next; nezha_trace tr; };
+// launch_select of level a.n (gated on row_cur == a.n) followed, in the same launch, by the accept / roll-back step of that level, the
+// same for the levels up to (not including) `last` as long as the request's beams are nodes of the pass and, where re.host is
+// given, the end of the round.  Levels behind the first: logits next to each other, tables tb_* of the next level.
+void launch_select_advance(const SelectArgs& a, const EngineState& e, int last, int K, int* out_codes, float* out_score,
                            int* out_count, const RoundEnd& re, cudaStream_t st);
 // launch_select followed, in the same launch, by launch_draft_step of level l (same arguments as there)
-void launch_select_step(const SelectArgs& a, const EngineState& e, int l, const float* G, long long g_stride, int t_cols,
+void launch_select_step(const SelectArgs& a, const EngineState& e, int l, const float* G, int per_req, long long g_stride, int t_cols,
                         const float* U, const float* bias, void* s_act, cudaStream_t st);
+// launch_select and, beside it in the same launch, launch_build_nodes
+void launch_select_nodes(const SelectArgs& a, const EngineState& e, cudaStream_t st);
 size_t select_smem_bytes(int in_stride, int K);
 cudaError_t select_configure(int max_beam);
 
 // out_* and every pointer of tr may be null
-void launch_decode_begin(const EngineState& e, int batch, int K, int* out_codes, float* out_scores, int* out_count,
+void launch_decode_begin(const EngineState& e, int batch, int K, int from_scratch, int* out_codes, float* out_scores, int* out_count,
                          const nezha_trace& tr, cudaStream_t st);
-void launch_draft_init(const EngineState& e, int batch, int from_scratch, void* s_act, cudaStream_t st);   // s_act may be null
 void launch_draft_set(const EngineState& e, int batch, int K, const int* drafts, const int* n_draft, cudaStream_t st);
 // the whole tree given by the caller: tree_codes [L][batch][K][L], tree_count [L][batch]
 void launch_draft_tree_set(const EngineState& e, int batch, int K, const int* tree_codes, const int* tree_count, cudaStream_t st);
@@ -103,7 +105,7 @@ void launch_trans_gather(const EngineState& e, int batch, int l, const void* emb
 void launch_trans_add(const EngineState& e, int batch, int l, const void* embed, bool bf16, cudaStream_t st);
 // The draft head with its two per-level products merged (see DraftFast in api.cu)
 void launch_draft_state_init(const EngineState& e, int batch, void* s_act, cudaStream_t st);
-void launch_draft_step(const EngineState& e, int batch, int l, const float* G, long long g_stride, int t_cols, const float* U,
+void launch_draft_step(const EngineState& e, int batch, int l, const float* G, int per_req, long long g_stride, int t_cols, const float* U,
                        const float* bias, void* s_act, cudaStream_t st);
 void launch_copy_logits_bias(const float* src, long long row_stride, int row_mul, int batch, int n_beams, int T,
                              const float* bias, long long bias_stride, float* dst, cudaStream_t st);
