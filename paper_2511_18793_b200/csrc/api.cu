@@ -306,9 +306,9 @@ size_t carve(nezha_ctx* c) {
 }
 
 void gemm(nezha_ctx* c, const void* A, long long lda, const void* W, long long ldw, void* C, long long ldc, long long M,
-          const int* M_dev, int N, int K, int epi, const float* bias = nullptr) {
+          const int* M_dev, int N, int K, int epi, const float* bias = nullptr, bool early = false) {
   GemmArgs a{A, lda, W, ldw, C, ldc, (int)M, M_dev, N, K, epi, bias, c->es.status};
-  a.skinny = c->skinny_now;
+  a.skinny = c->skinny_now; a.early = early ? 1 : 0;
   if (c->bf16 && gemm_tc_supported(a)) launch_gemm_tc(a, c->st);
   else launch_gemm_simt(a, c->bf16, c->st);
 }
@@ -398,9 +398,6 @@ void run_layers(nezha_ctx* c, long long M, const int* M_dev, bool verify, int n_
   const size_t esz = c->esz;
   for (int i = 0; i < c->nl; ++i) {
     const LayerW& w = c->layers[i];
-    launch_rmsnorm(c->resid, c->d, nullptr, w.attn_norm, c->bf16, c->xn, nullptr, (int)M, M_dev, c->d, c->cfg.rms_eps,
-                   c->st);
-    gemm(c, c->xn, c->d, w.wqkv, c->d, c->qkv, c->qkv_dim, M, M_dev, c->qkv_dim, c->d, kEpiStoreAct);
     char* kc = (char*)c->k_ctx + (size_t)i * c->ctx_layer_elems * esz;
     char* vc = (char*)c->v_ctx + (size_t)i * c->ctx_layer_elems * esz;
     char* ke = (char*)c->k_ext + (size_t)i * c->ext_layer_elems * esz;
@@ -411,7 +408,20 @@ void run_layers(nezha_ctx* c, long long M, const int* M_dev, bool verify, int n_
     r.k_cache = verify ? ke : kc; r.v_cache = verify ? ve : vc;
     r.cos_tab = c->rope_cos; r.sin_tab = c->rope_sin;
     r.M = (int)M; r.M_dev = M_dev; r.Hq = c->Hq; r.Hkv = c->Hkv; r.hd = c->hd;
-    launch_rope_append(r, c->bf16, c->st);
+    // fp32 rows that are few and narrow: the norms, the rotary embedding and SwiGLU inside the products
+    auto rows = [&](const void* W, int N, const void* gain) {
+      return !c->bf16 && norm_gemm_rows_applies((int)M, N, c->d, c->resid, c->d, W, gain);
+    };
+    const bool rows_qkv = rows(w.wqkv, c->qkv_dim, w.attn_norm);
+    if (rows_qkv) {
+      const GemmArgs a{c->resid, c->d, w.wqkv, c->d, c->qkv, c->qkv_dim, (int)M, M_dev, c->qkv_dim, c->d, kEpiStoreF32, nullptr, e.status};
+      launch_norm_gemm_rows(a, w.attn_norm, c->cfg.rms_eps, &r, false, c->st);
+    } else {
+      launch_rmsnorm(c->resid, c->d, nullptr, w.attn_norm, c->bf16, c->xn, nullptr, (int)M, M_dev, c->d, c->cfg.rms_eps,
+                     c->st);
+      gemm(c, c->xn, c->d, w.wqkv, c->d, c->qkv, c->qkv_dim, M, M_dev, c->qkv_dim, c->d, kEpiStoreAct);
+      launch_rope_append(r, c->bf16, c->st);
+    }
     AttnArgs t{};
     t.q = c->qkv; t.q_stride = c->qkv_dim; t.out = c->attn; t.out_stride = (long long)c->Hq * c->hd;
     t.k_ctx = kc; t.v_ctx = vc; t.ctx_row_stride = (long long)c->Hkv * c->S * c->hd; t.ctx_head_stride = (long long)c->S * c->hd;
@@ -429,12 +439,17 @@ void run_layers(nezha_ctx* c, long long M, const int* M_dev, bool verify, int n_
     if (c->bf16 && attention_tc_supported(t)) launch_attention_tc(t, c->st);
     else launch_attention_simt(t, c->bf16, c->st);
     gemm(c, c->attn, (long long)c->Hq * c->hd, w.wo, (long long)c->Hq * c->hd, c->resid, c->d, M, M_dev, c->d,
-         c->Hq * c->hd, kEpiAddF32);
-    launch_rmsnorm(c->resid, c->d, nullptr, w.mlp_norm, c->bf16, c->xn, nullptr, (int)M, M_dev, c->d, c->cfg.rms_eps,
-                   c->st);
-    gemm(c, c->xn, c->d, w.w_gu, c->d, c->gu, 2 * c->F, M, M_dev, 2 * c->F, c->d, kEpiStoreAct);
-    launch_swiglu(c->gu, c->act, (int)M, M_dev, c->F, c->bf16, c->st);
-    gemm(c, c->act, c->F, w.w_down, c->F, c->resid, c->d, M, M_dev, c->d, c->F, kEpiAddF32);
+         c->Hq * c->hd, kEpiAddF32, nullptr, true);
+    if (rows(w.w_gu, 2 * c->F, w.mlp_norm)) {
+      const GemmArgs a{c->resid, c->d, w.w_gu, c->d, c->act, c->F, (int)M, M_dev, 2 * c->F, c->d, kEpiStoreF32, nullptr, e.status};
+      launch_norm_gemm_rows(a, w.mlp_norm, c->cfg.rms_eps, nullptr, true, c->st);
+    } else {
+      launch_rmsnorm(c->resid, c->d, nullptr, w.mlp_norm, c->bf16, c->xn, nullptr, (int)M, M_dev, c->d, c->cfg.rms_eps,
+                     c->st);
+      gemm(c, c->xn, c->d, w.w_gu, c->d, c->gu, 2 * c->F, M, M_dev, 2 * c->F, c->d, kEpiStoreAct);
+      launch_swiglu(c->gu, c->act, (int)M, M_dev, c->F, c->bf16, c->st);
+    }
+    gemm(c, c->act, c->F, w.w_down, c->F, c->resid, c->d, M, M_dev, c->d, c->F, kEpiAddF32, nullptr, true);
   }
 }
 
@@ -455,6 +470,11 @@ void verify_pass(nezha_ctx* c, int n_rows, int max_tok_per_row, int beams) {
   }
   launch_embed(c->embed, c->bf16, e.tok_id, (int)M_bound, e.n_tokens, c->d, c->resid, c->st);
   run_layers(c, M_bound, e.n_tokens, true, n_rows, max_tok_per_row, beams);
+  if (!c->bf16 && norm_gemm_rows_applies((int)M_bound, c->Nv, c->d, c->resid, c->d, w, c->final_norm)) {
+    const GemmArgs a{c->resid, c->d, w, c->d, c->logits_v, c->Nv_ld, (int)M_bound, e.n_tokens, c->Nv, c->d, kEpiStoreF32, nullptr, e.status};
+    launch_norm_gemm_rows(a, c->final_norm, c->cfg.rms_eps, nullptr, false, c->st);
+    return;
+  }
   launch_rmsnorm(c->resid, c->d, nullptr, c->final_norm, c->bf16, c->xn, nullptr, (int)M_bound, e.n_tokens, c->d,
                  c->cfg.rms_eps, c->st);
   gemm(c, c->xn, c->d, w, c->d, c->logits_v, c->Nv_ld, M_bound, e.n_tokens, c->Nv, c->d, kEpiStoreF32);
@@ -462,8 +482,13 @@ void verify_pass(nezha_ctx* c, int n_rows, int max_tok_per_row, int beams) {
 
 // Draft-head logits of level l (1-based) for every (request, beam slot): Eq. 2.
 void draft_logits_level(nezha_ctx* c, int batch, int l) {
+  const int T = c->cfg.T[l - 1], rows = batch * c->Kmax;
+  if (!c->bf16 && draft_gemm_rows_applies(rows, T, c->es, c->draft_logit[l - 1])) {
+    const GemmArgs a{nullptr, 0, c->draft_logit[l - 1], c->d, c->logits_d, T, rows, nullptr, T, c->d, kEpiStoreF32, nullptr, c->es.status};
+    launch_draft_gemm_rows(a, c->es, l, c->embed, false, c->st);
+    return;
+  }
   launch_draft_x(c->es, batch, l, c->xd, c->bf16, c->st);
-  const int T = c->cfg.T[l - 1];
   gemm(c, c->xd, c->d, c->draft_logit[l - 1], c->d, c->logits_d, T, (long long)batch * c->Kmax, nullptr, T, c->d,
        kEpiStoreF32);
 }
@@ -473,8 +498,14 @@ void draft_logits_level(nezha_ctx* c, int batch, int l) {
 void draft_transition_level(nezha_ctx* c, int batch, int l) {
   if (!c->es.draft_use_s) return;
   if (c->es.draft_additive) { launch_trans_add(c->es, batch, l, c->embed, c->bf16, c->st); return; }
-  launch_trans_gather(c->es, batch, l, c->embed, c->a_se, c->bf16, c->st);
   float* out = c->es.state_lv + (size_t)(l + 1) * c->Bmax * c->Kmax * c->d;
+  if (!c->bf16 && draft_gemm_rows_applies(batch * c->Kmax, c->d, c->es, c->draft_wse)) {
+    const GemmArgs a{nullptr, 0, c->draft_wse, 2 * c->d, out, c->d, batch * c->Kmax, nullptr, c->d, 2 * c->d, kEpiBiasTanhF32,
+                     (const float*)c->draft_b_f32, c->es.status};
+    launch_draft_gemm_rows(a, c->es, l, c->embed, true, c->st);
+    return;
+  }
+  launch_trans_gather(c->es, batch, l, c->embed, c->a_se, c->bf16, c->st);
   gemm(c, c->a_se, 2 * c->d, c->draft_wse, 2 * c->d, out, c->d, (long long)batch * c->Kmax, nullptr, c->d, 2 * c->d,
        kEpiBiasTanhF32, (const float*)c->draft_b_f32);
 }

@@ -644,8 +644,6 @@ __global__ void draft_x_kernel(EngineState e, int batch, int l, T* x) {
 }
 
 // Eq. 3 input rows [s_l ; e_l] for the step s_l -> s_{l+1}.
-//   requests still teacher-forcing (d_m >= l): beam k of the start set, its own state, its l-th code;
-//   requests drafting (d_m < l): survivor k of level l, its parent's state, the code just chosen.
 //   ADD = true (ablation: Transition replaced by addition): writes s_{l+1} = s_l + e_l (fp32) itself, no GEMM follows.
 template <typename T, bool ADD>
 __global__ void trans_gather_kernel(EngineState e, int batch, int l, const T* embed, T* A) {
@@ -656,16 +654,8 @@ __global__ void trans_gather_kernel(EngineState e, int batch, int l, const T* em
   if (b >= batch) return;
   T* dst = A + (long long)bk * 2 * e.d;
   float* nxt = e.state_lv + ((long long)(l + 1) * e.Bmax * e.Kmax + bk) * e.d;
-  const int dm = e.d_m[b];
-  int src_level, parent;
-  bool live = dm < e.L || e.row_m[b] < e.L;
-  if (dm >= l) { src_level = min(dm, e.L); parent = k; }
-  else { src_level = l; parent = -2; }
-  const long long s_idx = lvl_bk(e, src_level, b, k);
-  live = live && k < e.dw_count[src_level * e.Bmax + b];
-  if (live && parent == -2) parent = e.dw_parent[s_idx];
-  const int code = live ? e.dw_codes[s_idx * e.L + (l - 1)] : -1;
-  live = live && code >= 0 && parent >= 0;
+  const auto [parent, code] = draft_source(e, b, k, l);
+  const bool live = code >= 0 && parent >= 0;
   if (!live) {
     if (ADD) { for (int c = threadIdx.x; c < e.d; c += blockDim.x) nxt[c] = 0.f; }
     else { for (int c = threadIdx.x; c < 2 * e.d; c += blockDim.x) dst[c] = from_f32<T>(0.f); }
@@ -711,16 +701,8 @@ __device__ __forceinline__ void draft_state(const EngineState& e, int b, int k, 
 __device__ __forceinline__ void draft_step_slot(const EngineState& e, int b, int k, int l, const float* __restrict__ G,
                                                 int per_req, long long g_stride, int t_cols, const float* __restrict__ U,
                                                 const float* __restrict__ bias, __nv_bfloat16* s_act, int tid, int n_thr) {
-  const int dm = e.d_m[b];
-  int src_level, parent;
-  bool live = dm < e.L || e.row_m[b] < e.L;
-  if (dm >= l) { src_level = min(dm, e.L); parent = k; }
-  else { src_level = l; parent = -2; }
-  const long long s_idx = lvl_bk(e, src_level, b, k);
-  live = live && k < e.dw_count[src_level * e.Bmax + b];
-  if (live && parent == -2) parent = e.dw_parent[s_idx];
-  const int code = live ? e.dw_codes[s_idx * e.L + (l - 1)] : -1;
-  draft_state(e, b, k, l, live ? parent : -1, code, G, per_req, g_stride, t_cols, U, bias, s_act, tid, n_thr);
+  const auto [parent, code] = draft_source(e, b, k, l);
+  draft_state(e, b, k, l, parent, code, G, per_req, g_stride, t_cols, U, bias, s_act, tid, n_thr);
 }
 __global__ void draft_step_kernel(EngineState e, int batch, int l, const float* __restrict__ G, int per_req, long long g_stride, int t_cols,
                                   const float* __restrict__ U, const float* __restrict__ bias, __nv_bfloat16* s_act) {

@@ -334,6 +334,10 @@ struct RopeAppendArgs {
   int Hq, Hkv, hd;
 };
 void launch_rope_append(const RopeAppendArgs& a, bool bf16, cudaStream_t st);
+// fp32: C = RMSNorm(A, gain) W^T with, where `rope` is given, what launch_rope_append does (C = its qkv, of which only q is written) or,
+// `swiglu`, C [M, N / 2] = what launch_swiglu makes of the product; else the product as it is.  Where norm_gemm_rows_applies.
+bool norm_gemm_rows_applies(int M, int N, int K, const void* A, long long lda, const void* W, const void* gain);
+void launch_norm_gemm_rows(const GemmArgs& a, const void* gain, float eps, const RopeAppendArgs* rope, bool swiglu, cudaStream_t st);
 void launch_swiglu(const void* gu, void* act, int M, const int* M_dev, int F, bool bf16, cudaStream_t st);
 
 // --------------------------------------------------------------------------------------------------

@@ -59,6 +59,25 @@ inline __host__ __device__ long long lvl_bk(const EngineState& e, int n, int b, 
   return ((long long)n * e.Bmax + b) * e.Kmax + k;
 }
 
+#ifdef __CUDACC__
+// Where slot k of request b gets its state s_{l+1} from (Eq. 3's step from level l): the slot of the state s_l and the code, -1 = none.
+//   requests still teacher-forcing (d_m >= l): beam k of the start set, its own state, its l-th code;
+//   requests drafting (d_m < l): survivor k of level l, its parent's state, the code just chosen.
+// What a drafting request asks for is asked for at once (one after the other these were four round trips to the L2).
+struct DraftSource { int parent, code; };
+__device__ __forceinline__ DraftSource draft_source(const EngineState& e, int b, int k, int l) {
+  const int dm = e.d_m[b], m = e.row_m[b];
+  const long long s_l = lvl_bk(e, l, b, k);
+  int count = e.dw_count[l * e.Bmax + b], parent = e.dw_parent[s_l], code = e.dw_codes[s_l * e.L + (l - 1)];
+  if (dm >= l) {
+    const int src = min(dm, e.L);
+    count = e.dw_count[src * e.Bmax + b]; parent = k; code = e.dw_codes[lvl_bk(e, src, b, k) * e.L + (l - 1)];
+  }
+  const bool live = (dm < e.L || m < e.L) && k < count;
+  return DraftSource{live ? parent : -1, live ? code : -1};
+}
+#endif
+
 struct SelectArgs {
   const float* logits; long long row_stride; int col_off;
   const int* src_row; int src_mul;      // logits row of beam r of request b: src_row ? src_row[b*in_stride+r] : b*src_mul+r
@@ -107,6 +126,9 @@ void launch_trans_add(const EngineState& e, int batch, int l, const void* embed,
 void launch_draft_state_init(const EngineState& e, int batch, void* s_act, cudaStream_t st);
 void launch_draft_step(const EngineState& e, int batch, int l, const float* G, int per_req, long long g_stride, int t_cols, const float* U,
                        const float* bias, void* s_act, cudaStream_t st);
+// fp32: launch_draft_x, or launch_trans_gather (`state`), with the product behind it in one launch
+bool draft_gemm_rows_applies(int M, int N, const EngineState& e, const void* W);
+void launch_draft_gemm_rows(const GemmArgs& a, const EngineState& e, int l, const void* embed, bool state, cudaStream_t st);
 void launch_copy_logits_bias(const float* src, long long row_stride, int row_mul, int batch, int n_beams, int T,
                              const float* bias, long long bias_stride, float* dst, cudaStream_t st);
 void launch_build_nodes(const EngineState& e, int batch, cudaStream_t st);
