@@ -81,6 +81,7 @@ struct nezha_ctx {
   // draft head with merged products (fused path, default options): [W_logit_l ; W_s] per level, U = E W_e^T for every
   // code token, H_l = W_logit_l h_l per request, the level's states as a bf16 A operand, the level's product
   void* draft_wcat[kMaxLevels]; float* draft_u; float* draft_hl; void* draft_sact; float *draft_g, *draft_g1;
+  int hl_ld;                // row length of draft_hl: the levels' codes, rounded up to 32
   int* h_rows; unsigned long long* n_unique_dev;
   EngineState es;
   BuildScratch build;
@@ -241,7 +242,13 @@ size_t carve(nezha_ctx* c) {
     w.w_gu = cv.take_bytes((size_t)2 * c->F * c->d * esz);
     w.w_down = cv.take_bytes((size_t)c->d * c->F * esz);
   }
-  for (int l = 0; l < c->L; ++l) c->draft_logit[l] = cv.take_bytes((size_t)g.T[l] * c->d * esz);
+  c->hl_ld = (li.vocab_codes + 31) / 32 * 32;
+  if (c->fused) {                // one matrix of all levels' rows (the prompt pass multiplies with all of it), zeros behind them
+    char* all = (char*)cv.take_bytes((size_t)c->hl_ld * c->d * esz);
+    for (int l = 0; l < c->L; ++l) c->draft_logit[l] = all ? all + (size_t)li.off[l] * c->d * esz : nullptr;
+  } else {
+    for (int l = 0; l < c->L; ++l) c->draft_logit[l] = cv.take_bytes((size_t)g.T[l] * c->d * esz);
+  }
   c->draft_wse = cv.take_bytes((size_t)c->d * 2 * c->d * esz);
   c->draft_b_f32 = cv.take<float>(c->d);
   // KV caches
@@ -274,7 +281,7 @@ size_t carve(nezha_ctx* c) {
   if (c->fused) {
     for (int l = 0; l < c->L; ++l) c->draft_wcat[l] = cv.take_bytes((size_t)(g.T[l] + c->d) * c->d * esz);
     c->draft_u = cv.take<float>((size_t)li.vocab_codes * c->d);
-    c->draft_hl = cv.take<float>((size_t)c->L * c->Bmax * c->Tmax);
+    c->draft_hl = cv.take<float>((size_t)c->Bmax * (c->L + 1) * c->hl_ld);
     c->draft_sact = cv.take_bytes((size_t)c->Bmax * c->Kmax * c->d * esz);
     c->draft_g = cv.take<float>((size_t)c->Bmax * c->Kmax * (c->Tmax + c->d));
     c->draft_g1 = cv.take<float>((size_t)c->Bmax * (c->Tmax + c->d));
@@ -564,7 +571,7 @@ void draft_phase(nezha_ctx* c, int batch, int K, int first_level, bool filter, b
       s.logits = c->logits_d; s.row_stride = c->cfg.T[l - 1]; s.col_off = 0; s.src_row = nullptr; s.src_mul = c->Kmax;
       if (fast) {
         s.logits = g; s.row_stride = c->Tmax + c->d; s.src_mul = per_req;
-        s.logit_bias = c->draft_hl + (size_t)(l - 1) * c->Bmax * c->Tmax; s.bias_stride = c->Tmax;
+        s.logit_bias = c->draft_hl + (size_t)l * c->hl_ld + e.li.off[l - 1]; s.bias_stride = (long long)(c->L + 1) * c->hl_ld;
       }
       s.in_codes = e.dw_codes + lv_in * c->L; s.in_score = e.dw_score + lv_in; s.in_count = e.dw_count + (size_t)(l - 1) * c->Bmax;
       s.n = l - 1; s.T = c->cfg.T[l - 1]; s.per_beam = K < s.T ? K : s.T; s.filter = (filter && l == c->L) ? 1 : 0;
@@ -871,6 +878,8 @@ nezha_status nezha_create(const nezha_config* cfg, const nezha_weights* w, const
     launch_embed(w->draft_b, c->bf16, c->es.n_tokens, 1, nullptr, c->d, (float*)c->draft_b_f32, st);
   }
   if (ok && c->fused) {
+    ok = cudaMemsetAsync((char*)c->draft_logit[0] + (size_t)c->es.li.vocab_codes * c->d * esz, 0, (size_t)(c->hl_ld - c->es.li.vocab_codes) * c->d * esz, st) ==
+         cudaSuccess;
     // [W_logit_l ; W_s] per level, and U = E W_e^T (fp32) for every code token: Eq. 3's input term of a chosen code
     for (int l = 0; ok && l < c->L; ++l)
       ok = cp(c->draft_wcat[l], w->draft_logit[l], (size_t)cfg->T[l] * c->d * esz) &&
@@ -955,10 +964,11 @@ nezha_status nezha_prefill(nezha_ctx* c, const int32_t* hist_codes, const int32_
     const size_t ho = (size_t)b0 * (c->L + 1) * c->d;
     launch_rmsnorm(c->resid, c->d, c->h_rows, c->final_norm, c->bf16, (char*)c->h_act + ho * c->esz, c->h_f32 + ho,
                    rows * (c->L + 1), nullptr, c->d, c->cfg.rms_eps, c->st);
-    if (c->fused)                  // the request-constant half of Eq. 2: W_logit_l h_l for every level
-      for (int l = 1; l <= c->L; ++l)
-        gemm(c, (char*)c->h_act + (ho + (size_t)l * c->d) * c->esz, (long long)(c->L + 1) * c->d, c->draft_logit[l - 1], c->d,
-             c->draft_hl + ((size_t)(l - 1) * c->Bmax + b0) * c->Tmax, c->Tmax, rows, nullptr, c->cfg.T[l - 1], c->d, kEpiStoreF32);
+    // The request-constant half of Eq. 2, W_logit_l h_l for every level: one product of all hidden states with all levels' rows, of
+    // which each level's own block is used (a product per level: two more launches of 5 us for the weights of one).
+    if (c->fused)
+      gemm(c, (char*)c->h_act + ho * c->esz, c->d, c->draft_logit[0], c->d, c->draft_hl + (size_t)b0 * (c->L + 1) * c->hl_ld, c->hl_ld,
+           (long long)rows * (c->L + 1), nullptr, c->hl_ld, c->d, kEpiStoreF32);
   }
   c->skinny_now = 0;
   NZ_CUDA(c, cudaGetLastError());
@@ -1070,7 +1080,7 @@ nezha_status nezha_draft_logits(nezha_ctx* c, int32_t batch, int32_t n_beams, in
     for (int l = 1; l <= level; ++l) { draft_level_product(c, batch, l, true); draft_level_step(c, batch, l); }
     draft_level_product(c, batch, level + 1, false);
     launch_copy_logits_bias(c->draft_g, c->Tmax + c->d, c->Kmax, batch, n_beams, c->cfg.T[level],
-                            c->draft_hl + (size_t)level * c->Bmax * c->Tmax, c->Tmax, logits, c->st);
+                            c->draft_hl + (size_t)(level + 1) * c->hl_ld + e.li.off[level], (long long)(c->L + 1) * c->hl_ld, logits, c->st);
   } else {
     for (int l = 1; l <= level; ++l) draft_transition_level(c, batch, l);
     draft_logits_level(c, batch, level + 1);
