@@ -288,7 +288,8 @@ __global__ void __launch_bounds__(kSkinnyThreads, 2)
     if constexpr (PUSH) {
       // what this warp's units will be sent (nobody signals the barrier before the peers' barriers are known to exist)
       if (mine && lane == 0) mbar_expect_tx(recv_bar(ew), (uint32_t)((units - u_first + u_step - 1) / u_step * splits * 512));
-      __syncwarp();
+      // the row scales are in place: a unit's are another warp's work, and no barrier of the whole block comes before they are read
+      asm volatile("barrier.sync.aligned 1, %0;" ::"n"(32 * kSkinnyEpiWarps) : "memory");
       cluster_wait();
     }
     const bool ok = warp_wait_uniform(acc_full, 0, abort_flag);
