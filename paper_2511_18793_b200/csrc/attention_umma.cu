@@ -345,7 +345,7 @@ __global__ void __launch_bounds__(kThreadsU, UmmaCfg<HD, PT>::kCtasPerSm) attn_u
     for (int e = 0; e < kMaxLevels; ++e) {
       long long off = -1;
       if (live && e < a.n_ext_max) off = a.tok_ext[(long long)tok * a.n_ext_max + e];
-      xpos[e] = off >= 0 ? (int)((off - (long long)request * a.ext_req_stride) / a.ext_pos_stride) : -1;
+      xpos[e] = off >= 0 ? (int)((unsigned)(off - (long long)request * a.ext_req_stride) / (unsigned)a.ext_pos_stride) : -1;
     }
     for (int j = 0; j < NT; ++j) {
       const int sb = PT ? (j & 1) : 0;               // S / P buffer of this tile
