@@ -85,7 +85,8 @@ struct nezha_ctx {
   int* h_rows; unsigned long long* n_unique_dev;
   EngineState es;
   BuildScratch build;
-  int* host_counters;       // pinned
+  int* host_counters;       // pinned: [0..1] items, [8..11] status, [16 + 4 r ..] status at the end of round r
+  int4* host_rows;          // [L - 1][Bmax], pinned: a request's counters of a round (RoundEnd)
   // CUDA graphs of the decode segments (one per round), keyed by everything that shapes the launch sequence
   struct Segment { int seen; cudaGraphExec_t exec; long long launches[kcCount]; unsigned long long used; };
   std::map<std::vector<uintptr_t>, Segment> segments;       // at most kMaxSegments, the least recently used go
@@ -185,7 +186,6 @@ size_t carve(nezha_ctx* c) {
   e.Bmax = c->Bmax; e.Kmax = c->Kmax; e.L = c->L; e.d = c->d; e.Hkv = c->Hkv; e.hd = c->hd;
   e.draft_use_h = 1; e.draft_use_s = 1; e.draft_additive = 0;
   e.status = cv.take<int>(8);
-  e.counters = cv.take<int>(8);
   c->n_unique_dev = cv.take<unsigned long long>(1);
   // 32-bit slots where every packed key fits them (mult has become prod T here; see HashSetView)
   e.hs.n_buckets = bucket_count(c->n_items, c->load_factor, 8);
@@ -739,7 +739,7 @@ nezha_status decode_impl(nezha_ctx* c, int batch, int K, int mode, const int* dr
     s.gate = e.row_cur; s.gate_mode = 1; s.gate_value = n;
     s.out_codes = e.tb_codes + lv_out * L; s.out_score = e.tb_score + lv_out; s.out_parent = e.tb_parent + lv_out;
     s.out_count = e.tb_count + (size_t)(n + 1) * c->Bmax;
-    const RoundEnd re{c->host_counters + 16 + 8 * round, round, mode == NEZHA_MODE_VERIFIED ? c->opt_adaptive : 0, mode == NEZHA_MODE_VERIFIED ? 1 : 0, tr};
+    const RoundEnd re{c->host_counters + 16 + 4 * round, c->host_rows + (size_t)(round - 1) * c->Bmax, round, mode == NEZHA_MODE_VERIFIED ? c->opt_adaptive : 0, mode == NEZHA_MODE_VERIFIED ? 1 : 0, tr};
     launch_select_advance(s, e, L, K, out_codes, out_scores, out_count, re, c->st);
     c->m_expected = 0;
   };
@@ -758,7 +758,11 @@ nezha_status decode_impl(nezha_ctx* c, int batch, int K, int mode, const int* dr
     NZ_CUDA(c, cudaStreamSynchronize(c->st));
     NZ_CUDA(c, cudaGetLastError());
     for (int r = sd.rounds + 1; r <= queued && !finished; ++r) {
-      const int* hc = c->host_counters + 16 + 8 * r;
+      int hc[4] = {0, 0, 0, 0};                      // unfinished requests, primary tokens, accepted levels, drafted tuples
+      for (int b = 0; b < batch; ++b) {
+        const int4 row = c->host_rows[(size_t)(r - 1) * c->Bmax + b];
+        hc[0] += row.x; hc[1] += row.y; hc[2] += row.z; hc[3] += row.w;
+      }
       // (the tiling hint keeps still while the count stays within a quarter of it: every value is a graph of its own)
       const int m = (hc[1] + 127) / 128 * 128;
       if (m > c->m_seen[r] || 4 * m < 3 * c->m_seen[r]) c->m_seen[r] = m;
@@ -780,7 +784,7 @@ nezha_status decode_impl(nezha_ctx* c, int batch, int K, int mode, const int* dr
     NZ_CUDA(c, cudaGetLastError());
   }
   if (stats) *stats = sd;
-  return device_error(c, queued > 0 ? c->host_counters + 16 + 8 * queued + 4 : c->host_counters + 8);
+  return device_error(c, queued > 0 ? c->host_counters + 16 + 4 * queued : c->host_counters + 8);
 }
 
 }  // namespace
@@ -824,7 +828,11 @@ nezha_status nezha_create(const nezha_config* cfg, const nezha_weights* w, const
   carve(c);
   auto bail = [&](nezha_status s) { if (c->host_counters) cudaFreeHost(c->host_counters); delete c; return s; };
   c->host_counters = nullptr;
-  if (cudaMallocHost((void**)&c->host_counters, (16 + 8 * (kMaxLevels + 1)) * sizeof(int)) != cudaSuccess) return bail(NEZHA_ERR_CUDA);
+  constexpr size_t kHostWords = 16 + 4 * (kMaxLevels + 1) + 12;      // (a multiple of 16 bytes: the rows follow)
+  static_assert(kHostWords % 4 == 0, "alignment");
+  if (cudaMallocHost((void**)&c->host_counters, kHostWords * sizeof(int) + (size_t)std::max(1, c->L - 1) * c->Bmax * sizeof(int4)) != cudaSuccess)
+    return bail(NEZHA_ERR_CUDA);
+  c->host_rows = reinterpret_cast<int4*>(c->host_counters + kHostWords);
   if (select_configure(c->Kmax) != cudaSuccess) return bail(NEZHA_ERR_CUDA);
   if (c->fused) {                  // needs the tensor-core GEMM (TMA descriptors) for every projection
     GemmArgs probe{c->xn, c->d, c->layers[0].wqkv, c->d, c->qkv, c->qkv_dim, 128, nullptr, c->qkv_dim, c->d, kEpiStoreAct, nullptr,

@@ -11,10 +11,16 @@ namespace nz {
 
 namespace {
 
+template <int V> struct Int { static constexpr int value = V; };
+
 template <typename T, int HD>
 __global__ void __launch_bounds__(128) attn_simt_kernel(AttnArgs a) {
   constexpr int DPL = HD / 8;
-  constexpr int U = HD <= 32 ? 4 : 2;              // positions of a group in flight: their K and V rows are all asked for at once
+  // Positions of a group in flight: their K and V rows are all asked for at once, 64 registers of them.  (With 16 floats a position and a
+  // group's four in flight, a context of 61 took four round trips to the L2 in a row, 5.2 us a launch.)
+  constexpr int U = HD >= 128 ? 2 : 256 / HD;
+  constexpr int UX = 2;                            // draft rows: at most kMaxLevels, over four groups
+  static_assert(4 * UX >= kMaxLevels, "draft rows");
   pdl_wait();
   pdl_launch();
   const int m = a.M_dev ? min(a.M, *a.M_dev) : a.M;
@@ -29,11 +35,12 @@ __global__ void __launch_bounds__(128) attn_simt_kernel(AttnArgs a) {
   for (int j = 0; j < DPL; ++j) { qv[j] = to_f32(qp[j]) * a.scale; acc[j] = 0.f; }
   float m_run = -INFINITY, l_run = 0.f;
 
-  // U positions (k / v: their rows, null = none) into the running softmax of the lane's group
-  auto visit = [&](const T* const* kp, const T* const* vp) {
-    float kv[U][DPL], vv[U][DPL], s[U];
+  // N positions (k / v: their rows, null = none) into the running softmax of the lane's group
+  auto visit = [&](auto count, const T* const* kp, const T* const* vp) {
+    constexpr int N = decltype(count)::value;
+    float kv[N][DPL], vv[N][DPL], s[N];
 #pragma unroll
-    for (int u = 0; u < U; ++u)
+    for (int u = 0; u < N; ++u)
 #pragma unroll
       for (int j = 0; j < DPL; ++j) {
         kv[u][j] = kp[u] ? to_f32(kp[u][j]) : 0.f;
@@ -42,7 +49,7 @@ __global__ void __launch_bounds__(128) attn_simt_kernel(AttnArgs a) {
     float m_new = m_run;
     bool any = false;
 #pragma unroll
-    for (int u = 0; u < U; ++u) {
+    for (int u = 0; u < N; ++u) {
       s[u] = 0.f;
 #pragma unroll
       for (int j = 0; j < DPL; ++j) s[u] = fmaf(qv[j], kv[u][j], s[u]);
@@ -57,7 +64,7 @@ __global__ void __launch_bounds__(128) attn_simt_kernel(AttnArgs a) {
 #pragma unroll
     for (int j = 0; j < DPL; ++j) acc[j] *= corr;
 #pragma unroll
-    for (int u = 0; u < U; ++u) {
+    for (int u = 0; u < N; ++u) {
       const float pw = kp[u] ? expf(s[u] - m_new) : 0.f;
       l_run += pw;
 #pragma unroll
@@ -78,19 +85,19 @@ __global__ void __launch_bounds__(128) attn_simt_kernel(AttnArgs a) {
       kp[u] = p < ctx_len ? kc + (long long)p * HD : nullptr;
       vp[u] = vc + (long long)p * HD;
     }
-    visit(kp, vp);
+    visit(Int<U>{}, kp, vp);
   }
-  for (int e0 = 0; e0 < a.n_ext_max; e0 += 4 * U) {
-    const T *kp[U], *vp[U];
+  if (a.n_ext_max > 0) {
+    const T *kp[UX], *vp[UX];
 #pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int e = e0 + 4 * u + pg;
+    for (int u = 0; u < UX; ++u) {
+      const int e = 4 * u + pg;
       const long long off = (e < a.n_ext_max) ? a.tok_ext[(long long)i * a.n_ext_max + e] : -1;
       const long long eo = off + (long long)kvh * a.ext_head_stride + sub * DPL;
       kp[u] = off >= 0 ? reinterpret_cast<const T*>(a.k_ext) + eo : nullptr;
       vp[u] = reinterpret_cast<const T*>(a.v_ext) + eo;
     }
-    visit(kp, vp);
+    visit(Int<UX>{}, kp, vp);
   }
   // merge the 4 position groups
 #pragma unroll

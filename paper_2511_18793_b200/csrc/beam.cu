@@ -497,7 +497,6 @@ __global__ void __launch_bounds__(128) decode_begin_kernel(EngineState e, int ba
   pdl_wait();
   pdl_launch();
   const int b = blockIdx.x, L = e.L, R = e.L - 1;
-  if (b == 0 && threadIdx.x < 8) e.counters[threadIdx.x] = 0;
   if (b == 0 && threadIdx.x == 0) { *e.draft_rows = batch * e.Kmax; *e.n_tokens = 0; }
   if (threadIdx.x == 0) {
     e.tb_count[0 * e.Bmax + b] = 1;
@@ -537,7 +536,6 @@ __global__ void draft_set_kernel(EngineState e, int batch, int K, const int* dra
   pdl_wait();
   pdl_launch();
   const int b = blockIdx.x;
-  if (b == 0 && threadIdx.x < 8) e.counters[threadIdx.x] = 0;      // first kernel of the round: clear its counters
   if (b == 0 && threadIdx.x == 0) *e.n_tokens = 0;
   if (b >= batch) return;
   const int L = e.L, k = threadIdx.x;
@@ -594,7 +592,6 @@ __global__ void draft_tree_set_kernel(EngineState e, int batch, int K, const int
   pdl_wait();
   pdl_launch();
   const int b = blockIdx.x;
-  if (b == 0 && threadIdx.x < 8) e.counters[threadIdx.x] = 0;
   if (b == 0 && threadIdx.x == 0) *e.n_tokens = 0;
   if (b >= batch) return;
   const int L = e.L, k = threadIdx.x;
@@ -989,8 +986,9 @@ __device__ __forceinline__ Advanced advance_body(const EngineState& e, const Adv
 }
 
 // End of a round: accepted length of every draft = the largest i <= (level reached) with D[k][0..i) in B_i;
-// trace outputs; counters for the host (unfinished requests, primary tokens, accepted levels), which the last block to get
-// here writes to the host's pinned memory together with the status word (a copy node behind every round costs 10 us).
+// trace outputs; the request's own counters (unfinished, primary tokens, accepted levels, drafted tuples) and, once, the status word
+// straight to the host's pinned memory: no block waits for another or for the bus.  (Added up on the device, with the last block copying
+// the sums from one thread behind a system-wide fence, this took 11 us of a round.)
 // adaptive: a request whose round settled only the one level that the pass settles anyway gained nothing from its drafts
 // and stops drafting (its remaining rounds are plain autoregressive steps).
 // re.draft_next: the start of the next round's drafting (Algorithm 2's drafting step): the draft head continues from the true beams B_m.
@@ -1060,27 +1058,15 @@ __device__ __forceinline__ void round_end_body(const EngineState& e, const Advan
       if ((int)threadIdx.x <= L) e.dw_count[(long long)threadIdx.x * e.Bmax + b] = 0;
     }
   }
-  int last = 0;
   if (threadIdx.x == 0) {
     if (tr.n_draft) tr.n_draft[tro] = took_part ? nd : -1;
     if (tr.level_reached) tr.level_reached[tro] = took_part ? m_now : -1;
     if (took_part && re.adaptive) e.row_spec[b] = spec;
     if (m_now < L && spec) atomicMax(e.draft_rows, batch * Kmax);            // somebody drafts next round
-    if (m_now < L) atomicAdd(&e.counters[0], 1);
-    if (took_part) atomicAdd(&e.counters[1], rs.tokens);
-    if (acc_sum) atomicAdd(&e.counters[2], acc_sum);
-    if (round == 1 && nd) atomicAdd(&e.counters[3], nd);
-    __threadfence();
-    last = atomicAdd(&e.counters[7], 1) == batch - 1;
+    if (b == 0) *e.n_tokens = 0;                   // for the next round's token list
+    re.rows[b] = make_int4(m_now < L ? 1 : 0, took_part ? rs.tokens : 0, acc_sum, nd);
   }
-  // (eight lanes, and no wait for the bus: one thread and a system-wide fence took 11 us of a round)
-  if (threadIdx.x < 32 && __shfl_sync(0xffffffffu, last, 0) && threadIdx.x < 8) {
-    __threadfence();
-    const int i = threadIdx.x;
-    re.host[i] = i < 4 ? *(volatile int*)(e.counters + i) : *(volatile int*)(e.status + i - 4);
-    e.counters[i] = 0;                             // for the next round
-    if (i == 0) *e.n_tokens = 0;
-  }
+  if (b == 0 && threadIdx.x < 4) re.host[threadIdx.x] = *(volatile int*)(e.status + threadIdx.x);
 }
 
 // A pass's selections of a request, one level after the other for as long as its beams are nodes of the pass: B_{n+1} from the logits

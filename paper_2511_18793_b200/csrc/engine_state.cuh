@@ -49,8 +49,6 @@ struct EngineState {
                                           //        all the attention kernel needs to know about a request, in one load
   int* n_tokens;        // [1] tokens of the verify pass
   int* pf_n_tokens;     // [1] tokens of the prefill chunk
-  int* counters;        // [8]: 0 unfinished rows, 1 primary tokens (round), 2 accepted levels (round), 3 drafted (round),
-                        //      7 blocks that have closed the round
 
   const float* h_f32;   // [Bmax][L+1][d]
 };
@@ -96,9 +94,9 @@ struct SelectArgs {
   const int* status; int* host_status;  // optional: the status words are copied to pinned host memory
 };
 void launch_select(const SelectArgs& a, cudaStream_t st);
-// What closes a round, behind its last selection (host == null: not this one): the trace's outputs and, in pinned host memory,
-// the counters (words 0-3) and the status words (4-7).
-struct RoundEnd { int* host; int round, adaptive, draft_next; nezha_trace tr; };
+// What closes a round, behind its last selection (host == null: not this one): the trace's outputs and, in pinned host memory, the status
+// words (host) and each request's counters (rows).
+struct RoundEnd { int* host; int4* rows; int round, adaptive, draft_next; nezha_trace tr; };
 // launch_select of level a.n (gated on row_cur == a.n) followed, in the same launch, by the accept / roll-back step of that level, the
 // same for the levels up to (not including) `last` as long as the request's beams are nodes of the pass and, where re.host is
 // given, the end of the round.  Levels behind the first: logits next to each other, tables tb_* of the next level.
