@@ -102,8 +102,8 @@ __global__ void __launch_bounds__(AttnCfg<HD, RW, KW>::kThreads) attn_tc_kernel(
   // A verify pass reads nothing of the launch before, the QKV projection, but q and the draft positions' K and V: the tables
   // and the context cache are older, and complete, because that launch lets this one start only when its own wait is over.
   // So only those wait here; the barriers, the tables and the first context tiles do not: 5.9 -> 3.6 us per launch at 40 rows of
-  // 37 positions (and 5.1 -> 4.5 for the prompt form, which this takes out of).
-  if constexpr (!VERIFY) { pdl_wait(); pdl_launch(); }
+  // 37 positions (and 5.1 -> 4.5 for the prompt form, which this takes out of).  A prompt pass reads its K and V from that launch: there only
+  // the request's entry and the barriers come before the wait.
   // the row tile is the slowest grid index: tiles beyond a request's rows (the grid covers the largest row count a
   // call may have) are scheduled after every tile that has work, instead of holding its place in the first wave
   // (a causal prefill has no such tiles to speak of, and its last tiles see the most context: those go first)
@@ -115,12 +115,13 @@ __global__ void __launch_bounds__(AttnCfg<HD, RW, KW>::kThreads) attn_tc_kernel(
   const int req_local = blockIdx.y, kvh = SPLIT ? (int)(blockIdx.x / n_split) : (int)blockIdx.x;
   const int tile = VERIFY ? (int)blockIdx.z : (int)(gridDim.z - 1 - blockIdx.z);
   const int G = a.Hq / a.Hkv;
-  const int4 info = VERIFY ? __ldcg(a.req_info + req_local) : a.req_info[req_local];   // {first token, token count, cache row, context length or -1}
+  const int4 info = __ldcg(a.req_info + req_local);   // {first token, token count, cache row, context length or -1}
   const int tok0 = info.x, n_tok = info.y, request = info.z;
   const int R = n_tok * G;                          // query rows of this (request, kv head)
   const int r0 = tile * kRows;
   if (r0 >= R) {                                    // (all CTAs of a cluster alike)
-    if constexpr (VERIFY) { pdl_wait(); pdl_launch(); }
+    pdl_wait();
+    pdl_launch();
     return;
   }
   // context positions this tile needs: all of them, or (causal prefill) up to its last token's own position
@@ -152,6 +153,7 @@ __global__ void __launch_bounds__(AttnCfg<HD, RW, KW>::kThreads) attn_tc_kernel(
     mbar_fence_init();
   }
   __syncthreads();
+  if constexpr (!VERIFY) { pdl_wait(); pdl_launch(); }
 
   float o[NB][4];
   float m_run[2] = {-INFINITY, -INFINITY}, l_run[2] = {0.f, 0.f};   // m in the scaled log2 domain
