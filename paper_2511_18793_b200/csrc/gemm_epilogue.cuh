@@ -216,25 +216,32 @@ __device__ __forceinline__ EpiRow epilogue_row(const GemmArgs& a, int row, int M
   return r;
 }
 
+// Rows 4 it0 .. 4 it0 + 15 of a 32 x 32 block: what their lanes need from memory.
+template <int EPI>
+__device__ __forceinline__ void epilogue_fetch(const GemmArgs& a, const ChunkCtx& cc, int lane, int row0, int rows_here, int n, const EpiRow& er,
+                                               int it0, EpiAux (&aux)[4]) {
+  const int rsub = lane >> 3;
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    const int r = (it0 + u) * 4 + rsub;
+    const int p_r = (EPI == kEpiRopeKV) ? __shfl_sync(0xffffffffu, er.pos, r) : 0;
+    if (r < rows_here) aux[u] = epi_prefetch<EPI>(a, cc, row0 + r, n, p_r);
+  }
+}
+
 // The epilogue proper on one staged 32 x 32 block (rows row0 .. row0 + 31, columns n_chunk .. n_chunk + 31) that sits in
 // the warp's transpose tile in the swizzled "8 lanes per row" image described above.  er = epilogue_row of row
 // row0 + lane; rows_here = how many of the 32 rows exist (> 0).  The caller has made the tile visible to the warp.
+// The block's row quads from it_lo on up to it_hi (0, 4 or 8); aux: epilogue_fetch of it_lo where `fetched`.
 template <int EPI>
 __device__ __forceinline__ void epilogue_block(const GemmArgs& a, float4* stg4, int lane, int row0, int rows_here, int n_chunk,
-                                               const EpiRow& er) {
+                                               const EpiRow& er, const ChunkCtx& cc, int it_lo, int it_hi, bool fetched, EpiAux (&aux)[4]) {
   const int k = lane & 7, rsub = lane >> 3;
-  const ChunkCtx cc = chunk_ctx<EPI>(a, n_chunk, k);
   const int n = n_chunk + 4 * k;
 #pragma unroll
   for (int it0 = 0; it0 < 8; it0 += 4) {
-    if (it0 * 4 >= rows_here) break;                           // warp-uniform
-    EpiAux aux[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int r = (it0 + u) * 4 + rsub;
-      const int p_r = (EPI == kEpiRopeKV) ? __shfl_sync(0xffffffffu, er.pos, r) : 0;
-      if (r < rows_here) aux[u] = epi_prefetch<EPI>(a, cc, row0 + r, n, p_r);
-    }
+    if (it0 < it_lo || it0 >= it_hi || it0 * 4 >= rows_here) continue;      // warp-uniform
+    if (!fetched || it0 > it_lo) epilogue_fetch<EPI>(a, cc, lane, row0, rows_here, n, er, it0, aux);
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
       const int r = (it0 + u) * 4 + rsub;
@@ -245,7 +252,7 @@ __device__ __forceinline__ void epilogue_block(const GemmArgs& a, float4* stg4, 
     }
   }
   __syncwarp();
-  if (EPI == kEpiAddNorm && lane < rows_here) {
+  if (EPI == kEpiAddNorm && lane < min(rows_here, 4 * it_hi) && lane >= 4 * it_lo) {
     // one partial sum of squares per 32-column group, added up in column order: the same bits whatever the tile width
     float ssq = 0.f;
 #pragma unroll
@@ -258,15 +265,33 @@ __device__ __forceinline__ void epilogue_block(const GemmArgs& a, float4* stg4, 
   __syncwarp();
 }
 
+// What an epilogue warp asks for while its tile is still being multiplied: the memory operands of the first rows that it will finish.  Behind
+// the accumulator they are a round trip to the L2 in every launch of one tile a CTA, and so was the second half of a 32-column tile's rows,
+// which one warp finished alone while its neighbour had none: small shape, 64 requests 732 -> 711 us; prompt of five on the d = 2048
+// backbone 1,416 -> 1,364; the large shapes, whose tiles follow one another, as before.
+struct EpiFirst { ChunkCtx cc; EpiAux aux[4]; };
+// Which part of a tile a warp finishes: 32-column groups half, half + 2, ... of all of its quarter's rows or, of a tile of one group, that
+// group's row quads 4 half .. 4 half + 3.
+template <int BN> __device__ __forceinline__ int first_group(int half) { return BN == 32 ? 0 : half; }
+template <int BN> __device__ __forceinline__ int first_quad(int half) { return BN == 32 ? 4 * half : 0; }
+template <int BN, int EPI>
+__device__ __forceinline__ void epilogue_first(const GemmArgs& a, int q, int half, int lane, int m0, int n0, int M, const EpiRow& er, EpiFirst& first) {
+  const int n_chunk = n0 + 32 * first_group<BN>(half), rows_here = min(32, M - (m0 + q * 32));
+  if (n_chunk >= a.N || rows_here <= 0) return;
+  first.cc = chunk_ctx<EPI>(a, n_chunk, lane & 7);
+  epilogue_fetch<EPI>(a, first.cc, lane, m0 + q * 32, rows_here, n_chunk + 4 * (lane & 7), er, first_quad<BN>(half), first.aux);
+}
+
 // One epilogue warp's share of a finished accumulator: TMEM lanes [32 q, 32 q + 32) (= rows m0 + 32 q ..) and the
-// 32-column groups half, half + 2, ... of the BN columns starting at TMEM column `tmem_acc`.  er = epilogue_row of
-// the lane's own row (lane = row while the block comes out of TMEM).
+// part of the BN columns starting at TMEM column `tmem_acc` that first_group / first_quad name.  er = epilogue_row of
+// the lane's own row (lane = row while the block comes out of TMEM); first = epilogue_first of the tile.
 template <int BN, int EPI>
 __device__ __forceinline__ void drain_accumulator(const GemmArgs& a, uint32_t tmem_acc, int q, int half, int lane,
-                                                  float4* stg4, int m0, int n0, int M, const EpiRow& er) {
+                                                  float4* stg4, int m0, int n0, int M, const EpiRow& er, EpiFirst& first) {
   const int rows_here = min(32, M - (m0 + q * 32));          // rows of this quarter that exist (may be <= 0)
+  const int it_lo = first_quad<BN>(half), it_hi = BN == 32 ? it_lo + 4 : 8;
 #pragma unroll 1
-  for (int c = half; c < BN / 32; c += 2) {
+  for (int c = first_group<BN>(half); c < BN / 32; c += 2) {
     const int n_chunk = n0 + c * 32;
     if (n_chunk >= a.N) break;                               // ragged last tile (N is a multiple of 32)
     float v[32];
@@ -277,7 +302,11 @@ __device__ __forceinline__ void drain_accumulator(const GemmArgs& a, uint32_t tm
       stg4[lane * 8 + (j ^ (lane & 7))] =
           make_float4(v[4 * j] * er.rs, v[4 * j + 1] * er.rs, v[4 * j + 2] * er.rs, v[4 * j + 3] * er.rs);
     __syncwarp();
-    if (rows_here > 0) epilogue_block<EPI>(a, stg4, lane, m0 + q * 32, rows_here, n_chunk, er);
+    if (rows_here > 0) {
+      const bool fetched = c == first_group<BN>(half);
+      if (!fetched) first.cc = chunk_ctx<EPI>(a, n_chunk, lane & 7);
+      epilogue_block<EPI>(a, stg4, lane, m0 + q * 32, rows_here, n_chunk, er, first.cc, it_lo, it_hi, fetched, first.aux);
+    }
     __syncwarp();
   }
 }

@@ -178,10 +178,12 @@ __global__ void __launch_bounds__(kThreads) gemm_tc_kernel(const __grid_constant
       const int m0 = (tile % tiles_m) * BM, n0 = tn * BN;
       const int b = t_local & 1;
       const EpiRow er = epilogue_row<EPI>(a, m0 + q * 32 + lane, M);   // overlaps the main loop
+      EpiFirst first;
+      epilogue_first<BN, EPI>(a, q, half, lane, m0, n0, M, er, first);
       ok = warp_wait_uniform(acc_full(b), (t_local >> 1) & 1, abort_flag);
       if (!ok) break;
       tc_fence_after();
-      drain_accumulator<BN, EPI>(a, tmem_base + (uint32_t)(b * BN), q, half, lane, stg4, m0, n0, M, er);
+      drain_accumulator<BN, EPI>(a, tmem_base + (uint32_t)(b * BN), q, half, lane, stg4, m0, n0, M, er, first);
       // this warp is done reading the accumulator: hand it back to the MMA warp
       tc_fence_before();
       __syncwarp();

@@ -180,10 +180,12 @@ __global__ void __launch_bounds__(kThreads) gemm_tc_pair_kernel(const __grid_con
       const int m0 = tt.m * (2 * BM) + rank * BM, n0 = tt.n * kBN2;
       const int b = t_local & 1;
       const EpiRow er = epilogue_row<EPI>(a, m0 + q * 32 + lane, M);
+      EpiFirst first;
+      epilogue_first<kBN2, EPI>(a, q, half, lane, m0, n0, M, er, first);
       ok = warp_wait_uniform(acc_full(b), (t_local >> 1) & 1, abort_flag);
       if (!ok) break;
       tc_fence_after();
-      drain_accumulator<kBN2, EPI>(a, tmem_base + (uint32_t)(b * kBN2), q, half, lane, stg4, m0, n0, M, er);
+      drain_accumulator<kBN2, EPI>(a, tmem_base + (uint32_t)(b * kBN2), q, half, lane, stg4, m0, n0, M, er, first);
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive_leader(acc_empty(b));   // hand the accumulator (of this CTA) back to the leader's MMA warp
