@@ -195,8 +195,9 @@ __global__ void __launch_bounds__(256) set_build_kernel(LevelInfo li, HashSetVie
 // the L2 holds (bucket, then slot; 254 us), behind a pass that clears both.  Here the items are dealt out to parts that a block's
 // shared memory holds: by prefix, for the bits, and by bucket, for the hash set.  A block builds a part there and writes it
 // once, which also replaces the clearing.
-// 10M items over 256^4 codes, load factor 0.5, whole calls: 968 us above, 437 here, of which the bits take 122 (537 MB written; 82
-// at the copy bandwidth), the slots 73, counting 65, the two deals 66 and 41, the rest launches.  30M: 2,907 -> 1,248.
+// 10M items over 256^4 codes, load factor 0.5, whole calls: 968 us above, 445 here, of which the bits take 113 (537 MB written; 82
+// at the copy bandwidth), the slots 73, counting 58, the two deals 67 and 41, the rest launches.  30M: 2,907 -> 1,248 (before the ring and the
+// bulk copies).
 // key / prefixes (the last code, at most 1,023) and the remainder.  Both roundings go down, and by less than 2^-10 of 1,024: the
 // product's integer part is the quotient or one less.  (With the compiler's division the first deal of 10M items took 69 us, not 66.)
 struct KeySplit {
