@@ -2,7 +2,7 @@
 // swapped on the tensor core.
 //
 // With a handful of rows the product is bound by reading W once from HBM.  The 128-row MMA operand is therefore a
-// 128 x 64 tile of W (16 KB per copy, the unit that has to be kept in flight), the rows of A are the MMA's N (MT = 32, 64
+// 128 x 64 tile of W (16 KB per copy, the unit that has to be kept in flight), the rows of A are the MMA's N (MT = 32, 48, 64
 // or 128), and the accumulator in TMEM is a 128 x MT block of C^T.  An output tile is 128 columns of C; the K range of a
 // tile is split over the CTAs of a thread-block cluster (up to 8) so that every SM streams a share of W, whatever N.
 // Pieces of the tile are dealt out to the cluster's warps, which add the parts in rank order -- the bits never depend on
