@@ -15,8 +15,9 @@ namespace nz {
 // candidates in order (repeated warp arg-max; ties to the smaller code):
 //   per_beam <  T : the per_beam most probable codes, THEN the hash-set filter on those       (Algorithm 3: top-K, then verification)
 //   per_beam >= T : the filter on all T codes, THEN the K best by cumulative log-probability  (top-k restricted to V)
-// The sorted per-beam lists go to shared memory and warp 0 merges them into the K best of the request
-// (ties to the smaller parent rank, then the smaller code).
+// The sorted per-beam lists go to shared memory.  The K best of the request (ties to the smaller parent rank, then the smaller code) are
+// ranked all with all among the candidates that the lists' order leaves in the running; more than kSelectKeys of those are merged
+// list by list by warp 0.
 namespace {
 
 struct Cand { float s; int r; int t; };
@@ -320,29 +321,26 @@ __device__ __forceinline__ Selected select_body(const SelectArgs& a, const Selec
   auto cand_key = [&](int r, int c) {
     return (unsigned long long)ordered_bits(l_score[(size_t)r * a.K + c]) << 32 | (0xffffffffu - ((unsigned)r << 16 | (unsigned)l_tok[(size_t)r * a.K + c]));
   };
-  // The lists are sorted: if all have m = ceil(K / nb) entries, K candidates are at least as good as the worst of their m-th, and
-  // what is worse than that is out.  (Each warp finds that bound for itself.)
+  // A list's scores do not rise: if all lists have m = ceil(K / nb) entries, K candidates score no less than the worst of their m-th, and
+  // what scores less is out.  (By the score alone: where per_beam < T a list is in the order of the beam's own log-probabilities, and
+  // two of them whose sums with the beam's score are rounded to the same number may stand there with the larger code first.  Each warp
+  // finds the bound for itself.)
   const int m = nb > 0 ? (a.K + nb - 1) / nb : 1;
   int n_cand = 0;
-  unsigned long long bound = ~0ull;
+  unsigned bound = ~0u;
   for (int r = lane; r < nb; r += 32) {
     const int c = l_cnt[r];
     n_cand += c;
-    const unsigned long long k = c >= m ? cand_key(r, m - 1) : 0ull;
-    if (k < bound) bound = k;
+    bound = min(bound, c >= m ? ordered_bits(l_score[(size_t)r * a.K + m - 1]) : 0u);
   }
   n_cand = (int)__reduce_add_sync(0xffffffffu, (unsigned)n_cand);
-  {
-    const unsigned hi = __reduce_min_sync(0xffffffffu, (unsigned)(bound >> 32));
-    const unsigned lo = __reduce_min_sync(0xffffffffu, (unsigned)(bound >> 32) == hi ? (unsigned)bound : 0xffffffffu);
-    bound = (unsigned long long)hi << 32 | lo;
-  }
+  bound = __reduce_min_sync(0xffffffffu, bound);
   const int n_out = min(n_cand, a.K), key_cap = select_keys(nb_cap, a.K);
   for (int i0 = warp * 32; i0 < nb * a.K; i0 += blockDim.x) {
     const int i = i0 + lane, r = i / a.K, c = i - r * a.K;
     unsigned long long k = 0;
     if (r < nb && c < l_cnt[r]) k = cand_key(r, c);
-    const bool in = k != 0ull && k >= bound;
+    const bool in = k != 0ull && (unsigned)(k >> 32) >= bound;
     const unsigned ins = __ballot_sync(0xffffffffu, in);
     int at = 0;
     if (lane == 0 && ins) at = atomicAdd(s_running, __popc(ins));
@@ -369,6 +367,14 @@ __device__ __forceinline__ Selected select_body(const SelectArgs& a, const Selec
     int ptr[RPL];
 #pragma unroll
     for (int q = 0; q < RPL; ++q) ptr[q] = 0;
+    if (!all_codes) {                                      // the equal sums of a list by their codes (see the bound)
+      for (int r = lane; r < nb; r += 32)
+        for (int c = 1; c < l_cnt[r]; ++c)
+          for (size_t i = (size_t)r * a.K + c; i > (size_t)r * a.K && l_score[i - 1] == l_score[i] && l_tok[i - 1] > l_tok[i]; --i) {
+            const int t = l_tok[i]; l_tok[i] = l_tok[i - 1]; l_tok[i - 1] = t;
+          }
+      __syncwarp();
+    }
     for (int k = 0; k < a.K; ++k) {
       float bs = -INFINITY; int br = 0x7fffffff, bt = 0x7fffffff;
 #pragma unroll
