@@ -60,10 +60,6 @@ __device__ __forceinline__ uint32_t kv_addr(uint32_t tile, int pos, int chunk) {
   return tile + sub * (kPos * 128) + pos * 128 + ((c ^ (pos & 7)) << 4);
 }
 
-__device__ __forceinline__ void cluster_sync_all() {       // every thread of every CTA of the cluster, on every path
-  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
 __device__ __forceinline__ float ld_peer(uint32_t local, uint32_t rank) {
   uint32_t ra;
   float v;

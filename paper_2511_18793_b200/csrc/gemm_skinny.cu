@@ -52,11 +52,6 @@ __device__ __forceinline__ uint32_t cluster_rank() {
   asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
   return r;
 }
-// Every thread of every CTA of the cluster executes both halves in turn, on every path.  The relaxed arrival orders nothing: it
-// says that the CTA has come so far.
-__device__ __forceinline__ void cluster_arrive_relaxed() { asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory"); }
-__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
-__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 // 16 bytes to the shared memory of CTA `rank` of the cluster, at the address that `local` has in this CTA; they count towards the
 // bytes that the mbarrier at `bar` (an address of this CTA's as well) of that CTA waits for.
 __device__ __forceinline__ void st_peer_f4(uint32_t local, uint32_t bar, uint32_t rank, float x, float y, float z, float w) {
@@ -292,7 +287,6 @@ __global__ void __launch_bounds__(kSkinnyThreads, 2)
     }
     const bool ok = warp_wait_uniform(acc_full, 0, abort_flag);
     tc_fence_after();
-    if (!ok && lane == 0) *abort_flag = 1;
     // TMEM lane = column n0 + 32 q + lane, TMEM column = row; the two warps of a lane quarter take turns at the rows.
     constexpr int kLd = MT >= 64 ? 16 : 8;
     const int q = warp & 3, half = ew >> 2;
@@ -329,9 +323,9 @@ __global__ void __launch_bounds__(kSkinnyThreads, 2)
         }
       }
     }
+    if (!ok && lane == 0) *abort_flag = 1;       // (behind the collective loads, which want the warp's lanes together)
   }
   if constexpr (PUSH) {
-    __syncwarp();
     if (!live || warp < 2) cluster_wait();       // (the epilogue warps of a live tile have)
     cluster_arrive_relaxed();                    // this CTA's parts are on their way
     // The row scales are in place: a unit's are another warp's work, and no barrier of the whole block comes before they are read.
@@ -340,7 +334,7 @@ __global__ void __launch_bounds__(kSkinnyThreads, 2)
     if (mine && !recv_wait(recv_bar(ew), abort_flag)) *abort_flag = 1;
   } else {
     // All parts are in place behind this barrier (or their CTA has raised its abort flag).
-    if (splits > 1) { __syncwarp(); cluster_arrive(); cluster_wait(); }
+    if (splits > 1) cluster_sync_all();
     else __syncthreads();
   }
   if (mine && !*abort_flag) {
@@ -392,7 +386,6 @@ __global__ void __launch_bounds__(kSkinnyThreads, 2)
     }
   }
   tc_fence_before();
-  __syncwarp();
   if (PUSH || splits > 1) {                      // no CTA leaves while a peer may still send to it, or read its part
     if (!PUSH) cluster_arrive_relaxed();         // (what it has read has been used)
     cluster_wait();

@@ -55,6 +55,25 @@ __device__ __forceinline__ bool mbar_wait_or_abort(uint32_t bar, uint32_t parity
     if (*abort_flag || clock64() - t0 > kWaitCycles) return false;
   }
 }
+// Barriers of the CTAs of a cluster: every thread of every CTA executes both halves in turn, on every path.  The .aligned forms want all
+// lanes of a warp together, and the code in front of a barrier may have split them (a branch for one lane, a row that does not
+// exist), so each form brings the warp together first.  The relaxed arrival orders nothing: it says that the CTA has come so far.
+__device__ __forceinline__ void cluster_arrive_relaxed() {
+  __syncwarp();
+  asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_arrive() {
+  __syncwarp();
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait() {
+  __syncwarp();
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_sync_all() {
+  cluster_arrive();
+  cluster_wait();
+}
 // Fetches a tensor map into the descriptor cache ahead of its first copy (the map is a kernel parameter: this reads
 // nothing an earlier kernel wrote, so it may run before the dependency wait).
 __device__ __forceinline__ void tma_prefetch_map(const CUtensorMap* tm) {
