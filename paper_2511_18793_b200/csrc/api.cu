@@ -5,6 +5,7 @@
 #include <stdlib.h>
 #include <string.h>
 
+#include <algorithm>
 #include <map>
 #include <string>
 #include <vector>
@@ -39,6 +40,14 @@ int attention_split_max(int ctx_positions, int draft_positions);
 using namespace nz;
 
 namespace {
+
+// H_l = W_logit_l h_l of a prefilled batch (draft_hl): up to this many requests one product of all hidden states with all levels' rows
+// ([batch][L + 1][hl_ld], of which each level's own block is used), beyond a product per level ([L][Bmax][Tmax]).  The one product does
+// L + 1 times the arithmetic and saves L - 1 launches: 256 / 512 / 1,024 requests, per level -> at once, us: four levels of 256 codes, d = 512
+// 14.3 -> 5.2 / 14.4 -> 6.0 / 14.7 -> 9.0, d = 4096 46 -> 15 / 46 -> 17 / 47 -> 45; three of 512, d = 2048 21 -> 10 / 21 -> 12 / 21 -> 24; six of
+// 1,024, d = 512 22 -> 16 / 22 -> 29 / 24 -> 56.  And its results take L + 1 times the room, or more.
+constexpr int kJointConstants = 256;
+bool joint_constants(int batch) { return batch <= kJointConstants; }
 
 struct Carver {
   char* base; size_t off;
@@ -81,7 +90,7 @@ struct nezha_ctx {
   // draft head with merged products (fused path, default options): [W_logit_l ; W_s] per level, U = E W_e^T for every
   // code token, H_l = W_logit_l h_l per request, the level's states as a bf16 A operand, the level's product
   void* draft_wcat[kMaxLevels]; float* draft_u; float* draft_hl; void* draft_sact; float *draft_g, *draft_g1;
-  int hl_ld;                // row length of draft_hl: the levels' codes, rounded up to 32
+  int hl_ld;                // row length of draft_hl where one product makes it (joint_constants): the levels' codes, rounded up to 32
   int* h_rows; unsigned long long* n_unique_dev;
   EngineState es;
   BuildScratch build;
@@ -281,7 +290,8 @@ size_t carve(nezha_ctx* c) {
   if (c->fused) {
     for (int l = 0; l < c->L; ++l) c->draft_wcat[l] = cv.take_bytes((size_t)(g.T[l] + c->d) * c->d * esz);
     c->draft_u = cv.take<float>((size_t)li.vocab_codes * c->d);
-    c->draft_hl = cv.take<float>((size_t)c->Bmax * (c->L + 1) * c->hl_ld);
+    const size_t at_once = (size_t)std::min(c->Bmax, kJointConstants) * (c->L + 1) * c->hl_ld, per_level = (size_t)c->L * c->Bmax * c->Tmax;
+    c->draft_hl = cv.take<float>(joint_constants(c->Bmax) ? at_once : std::max(at_once, per_level));
     c->draft_sact = cv.take_bytes((size_t)c->Bmax * c->Kmax * c->d * esz);
     c->draft_g = cv.take<float>((size_t)c->Bmax * c->Kmax * (c->Tmax + c->d));
     c->draft_g1 = cv.take<float>((size_t)c->Bmax * (c->Tmax + c->d));
@@ -532,6 +542,11 @@ SelectArgs select_base(nezha_ctx* c, int batch, int K) {
 bool draft_fast(const nezha_ctx* c) {
   return c->fused && c->opt_transition == 0 && c->opt_inputs == 0;
 }
+// Level l's constants of the requests: of the first, and from one to the next.
+const float* level_constants(const nezha_ctx* c, int l) {
+  return joint_constants(c->batch) ? c->draft_hl + (size_t)l * c->hl_ld + c->es.li.off[l - 1] : c->draft_hl + (size_t)(l - 1) * c->Bmax * c->Tmax;
+}
+long long level_constants_stride(const nezha_ctx* c) { return joint_constants(c->batch) ? (long long)(c->L + 1) * c->hl_ld : c->Tmax; }
 // in_round: inside a decode round, where the device knows whether any request still drafts (a round queued for nothing, or
 // one in which the adaptive policy has switched every request's drafting off, runs its products over zero rows)
 void draft_level_product(nezha_ctx* c, int batch, int l, bool with_state, bool in_round = false) {
@@ -571,7 +586,7 @@ void draft_phase(nezha_ctx* c, int batch, int K, int first_level, bool filter, b
       s.logits = c->logits_d; s.row_stride = c->cfg.T[l - 1]; s.col_off = 0; s.src_row = nullptr; s.src_mul = c->Kmax;
       if (fast) {
         s.logits = g; s.row_stride = c->Tmax + c->d; s.src_mul = per_req;
-        s.logit_bias = c->draft_hl + (size_t)l * c->hl_ld + e.li.off[l - 1]; s.bias_stride = (long long)(c->L + 1) * c->hl_ld;
+        s.logit_bias = level_constants(c, l); s.bias_stride = level_constants_stride(c);
       }
       s.in_codes = e.dw_codes + lv_in * c->L; s.in_score = e.dw_score + lv_in; s.in_count = e.dw_count + (size_t)(l - 1) * c->Bmax;
       s.n = l - 1; s.T = c->cfg.T[l - 1]; s.per_beam = K < s.T ? K : s.T; s.filter = (filter && l == c->L) ? 1 : 0;
@@ -972,11 +987,14 @@ nezha_status nezha_prefill(nezha_ctx* c, const int32_t* hist_codes, const int32_
     const size_t ho = (size_t)b0 * (c->L + 1) * c->d;
     launch_rmsnorm(c->resid, c->d, c->h_rows, c->final_norm, c->bf16, (char*)c->h_act + ho * c->esz, c->h_f32 + ho,
                    rows * (c->L + 1), nullptr, c->d, c->cfg.rms_eps, c->st);
-    // The request-constant half of Eq. 2, W_logit_l h_l for every level: one product of all hidden states with all levels' rows, of
-    // which each level's own block is used (a product per level: two more launches of 5 us for the weights of one).
-    if (c->fused)
+    // the request-constant half of Eq. 2, W_logit_l h_l for every level
+    if (c->fused && joint_constants(batch))
       gemm(c, (char*)c->h_act + ho * c->esz, c->d, c->draft_logit[0], c->d, c->draft_hl + (size_t)b0 * (c->L + 1) * c->hl_ld, c->hl_ld,
            (long long)rows * (c->L + 1), nullptr, c->hl_ld, c->d, kEpiStoreF32);
+    else if (c->fused)
+      for (int l = 1; l <= c->L; ++l)
+        gemm(c, (char*)c->h_act + (ho + (size_t)l * c->d) * c->esz, (long long)(c->L + 1) * c->d, c->draft_logit[l - 1], c->d,
+             c->draft_hl + ((size_t)(l - 1) * c->Bmax + b0) * c->Tmax, c->Tmax, rows, nullptr, c->cfg.T[l - 1], c->d, kEpiStoreF32);
   }
   c->skinny_now = 0;
   NZ_CUDA(c, cudaGetLastError());
@@ -1088,7 +1106,7 @@ nezha_status nezha_draft_logits(nezha_ctx* c, int32_t batch, int32_t n_beams, in
     for (int l = 1; l <= level; ++l) { draft_level_product(c, batch, l, true); draft_level_step(c, batch, l); }
     draft_level_product(c, batch, level + 1, false);
     launch_copy_logits_bias(c->draft_g, c->Tmax + c->d, c->Kmax, batch, n_beams, c->cfg.T[level],
-                            c->draft_hl + (size_t)(level + 1) * c->hl_ld + e.li.off[level], (long long)(c->L + 1) * c->hl_ld, logits, c->st);
+                            level_constants(c, level + 1), level_constants_stride(c), logits, c->st);
   } else {
     for (int l = 1; l <= level; ++l) draft_transition_level(c, batch, l);
     draft_logits_level(c, batch, level + 1);
