@@ -29,3 +29,25 @@ def test_repeated_calls_return_the_same_bits(hd, heads, kv_heads, batch, beam, n
         for a, b in zip(first.setdefault(mode, got), got):
             assert torch.equal(a, b), mode
     case.eng.close()
+
+
+# A product of at most 48 rows: its row scales are one warp's work and another's operand, its parts come from other CTAs.
+@pytest.mark.parametrize("n_hist", [1, 6, 10])           # 9, 29 and 45 rows a prompt pass
+def test_passes_of_few_rows_return_the_same_bits_many_times(n_hist):
+    w = synth.scaled(synth.WORKLOADS["paper"], n_layers=2, L=4, T=(64,) * 4, n_items=50_000, batch=1, beam=10, n_hist=n_hist)
+    st = torch.cuda.Stream()
+    with torch.cuda.stream(st):
+        case = Case(w, stream=st)
+    out = {m: case.eng.alloc_outputs(1, w.beam) for m in (binding.MODE_AR, binding.MODE_VERIFIED)}
+    first = None
+    for _ in range(150):
+        case.prefill()
+        got = [case.eng.get_hidden()]
+        for mode, o in out.items():
+            got += [case.eng.decode(w.beam, mode=mode, out=o)[k].clone() for k in ("codes", "scores")]
+        torch.cuda.synchronize()
+        first = first or [t.clone() for t in got]
+        for a, b in zip(first, got):
+            assert torch.equal(a, b)
+    assert torch.isfinite(first[0]).all()
+    case.eng.close()
