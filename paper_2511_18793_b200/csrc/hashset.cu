@@ -405,9 +405,18 @@ __global__ void __launch_bounds__(1024) part_deal_kernel(BuildDeal dl, Deal part
 
 // A copy from shared to global memory by the copy engine; one thread's, 16-byte aligned, a multiple of 16.  Every thread that has written
 // the source fences before the barrier in front of it, and the source has to outlive it.
+// STREAM: what is written is the first to leave the L2 again.
 __device__ __forceinline__ void bulk_fence() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+template <bool STREAM>
 __device__ __forceinline__ void bulk_store(void* dst, const void* src, unsigned bytes) {
-  asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(dst), "r"((uint32_t)__cvta_generic_to_shared(src)), "r"(bytes) : "memory");
+  const uint32_t at = (uint32_t)__cvta_generic_to_shared(src);
+  if constexpr (STREAM) {
+    unsigned long long policy;
+    asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(policy));
+    asm volatile("cp.async.bulk.global.shared::cta.bulk_group.L2::cache_hint [%0], [%1], %2, %3;" ::"l"(dst), "r"(at), "r"(bytes), "l"(policy) : "memory");
+  } else {
+    asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(dst), "r"(at), "r"(bytes) : "memory");
+  }
   asm volatile("cp.async.bulk.commit_group;" ::: "memory");
 }
 __device__ __forceinline__ void bulk_wait() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
@@ -438,8 +447,10 @@ __global__ void __launch_bounds__(512, 3) part_bits_kernel(PrefixMapView pm, Bui
   __syncthreads();
   const unsigned words = min(1u << shift, split.prefixes - p0) * pm.set_words;
   unsigned long long* out = pm.slots + pm.level_off[last] + (unsigned long long)p0 * pm.set_words;
-  // (one bulk copy out of shared memory, none of it through the threads' registers: 10M items 122 -> 113 us, 4.8 TB/s)
-  if (threadIdx.x == 0 && words >= 2) bulk_store(out, bits, words / 2 * 16);
+  // One bulk copy out of shared memory, none of it through the threads' registers.  The region is larger than the L2, and what the next
+  // kernels read -- the packed keys -- is in there: 10M items of 256^4 / 1,024^3 codes by the threads' streaming stores 122 / 91 us (and the
+  // second deal 41 / 41), by a plain bulk copy 111 / 115 (51 / 49), by this one 86 / 83 (41 / 41).
+  if (threadIdx.x == 0 && words >= 2) bulk_store<true>(out, bits, words / 2 * 16);
   if (threadIdx.x == 0 && (words & 1)) out[words - 1] = reinterpret_cast<const unsigned long long*>(bits)[words - 1];
   for (int w = threadIdx.x; w < any_words; w += 512) sc.any[(size_t)blockIdx.x * any_words + w] = any[w];
   count_inserted(inserted, n_unique);
@@ -489,7 +500,7 @@ __global__ void __launch_bounds__(512, 3) part_slots_kernel(HashSetView hs, Buil
   bulk_fence();
   __syncthreads();
   if (threadIdx.x == 0) {
-    bulk_store(reinterpret_cast<uint4*>(hs.slots) + (size_t)b0 * 2, slots, n_local * kBucketBytes);
+    bulk_store<false>(reinterpret_cast<uint4*>(hs.slots) + (size_t)b0 * 2, slots, n_local * kBucketBytes);
     sc.n_over[blockIdx.x] = n_over;
     bulk_wait();
   }
