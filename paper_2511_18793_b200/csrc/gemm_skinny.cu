@@ -10,7 +10,8 @@
 // its accumulator to the shared memory of the warps that add them (st.async on their mbarriers); beyond, where there is no room for
 // them beside the ring, it leaves its block in its own, and the warps read their peers' behind a cluster barrier.  The barrier, the
 // round trip of the reads and a second barrier before a CTA may leave are a launch's last 1.3 us: one request on the 16-layer d = 2048
-// backbone, prompt of 40 rows / verified decode (20 rows a pass) 676 -> 635 / 1,344 -> 1,278 us without them.
+// backbone, prompt of 40 rows / verified decode (20 rows a pass) 676 -> 635 / 1,344 -> 1,278 us without them.  (The 48-row accumulator
+// alone, read / sent: prompt of 41 rows and drafts 779 / 702 us, prompt of five and passes of 45 rows 2,636 / 2,526.)
 // A CTA issues the weight copies of its first ring round BEFORE the launch's dependency on the preceding kernel is
 // resolved (W is constant data), and the kernel is sized for two CTAs per SM, so the weight stream of a launch starts
 // while its predecessor is still draining.
@@ -441,7 +442,7 @@ void launch_epi(const GemmArgs& a, int tiles, int splits, cudaStream_t st) {
 template <int MT>
 void launch_mt(const GemmArgs& a, int tiles, int splits, cudaStream_t st) {
   if constexpr (MT <= 48) {
-    // a CTA's share of at most MT units, each in `splits` parts, has to fit
+    // a CTA's share of at most MT units, each in `splits` parts, has to fit (at 48 rows that of 5 and of 7 CTAs does not)
     if (splits > 1 && (MT + splits - 1) / splits * splits <= SkinnyCfg<MT, true>::kRecvParts) {
       launch_epi<MT, true>(a, tiles, splits, st);
       return;

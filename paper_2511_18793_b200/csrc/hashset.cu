@@ -195,9 +195,8 @@ __global__ void __launch_bounds__(256) set_build_kernel(LevelInfo li, HashSetVie
 // the L2 holds (bucket, then slot; 254 us), behind a pass that clears both.  Here the items are dealt out to parts that a block's
 // shared memory holds: by prefix, for the bits, and by bucket, for the hash set.  A block builds a part there and writes it
 // once, which also replaces the clearing.
-// 10M items over 256^4 codes, load factor 0.5, whole calls: 968 us above, 445 here, of which the bits take 113 (537 MB written; 82
-// at the copy bandwidth), the slots 73, counting 58, the two deals 67 and 41, the rest launches.  30M: 2,907 -> 1,248 (before the ring and the
-// bulk copies).
+// 10M items over 256^4 codes, load factor 0.5, whole calls: 968 us above, 390 here, of which the bits take 86 (537 MB written; 82
+// at the copy bandwidth), the slots 67, counting 58, the two deals 70 and 41, the rest launches.  30M: 2,907 -> 1,157.
 // key / prefixes (the last code, at most 1,023) and the remainder.  Both roundings go down, and by less than 2^-10 of 1,024: the
 // product's integer part is the quotient or one less.  (With the compiler's division the first deal of 10M items took 69 us, not 66.)
 struct KeySplit {
@@ -243,7 +242,9 @@ __global__ void __launch_bounds__(1024) part_count_kernel(LevelInfo li, HashSetV
   const unsigned lo = min(n, blockIdx.x * run), hi = min(n, lo + run);
   const int lane = threadIdx.x & 31;
   constexpr int kItems = kCountItems;                   // per thread and step
-  // RING: a thread's items of the next steps are on their way into shared memory, read by nobody else (10M items: 66 -> 58 us)
+  // RING: a thread's items of the next steps are on their way into shared memory, read by nobody else (10M items: 66 -> 58 us, and as much
+  // of the whole call as its runs differ by; 30M: the call 1,198 -> 1,152).  Rows of three codes are not copied so: their 12 bytes lie on no
+  // 16-byte boundaries.
   auto ask = [&](unsigned i0, int slot) {
 #pragma unroll
     for (int j = 0; j < kItems; ++j) {
@@ -619,8 +620,8 @@ cudaError_t launch_set_build(const LevelInfo& li, HashSetView hs, PrefixMapView 
     };
     // (the longest region is the last, and written whole)
     cudaMemsetAsync(sc.by_prefix.count, 0, (size_t)(both + 2) * sizeof(unsigned), st);
-    // (131 KB of ring beside at most 64 KB of counters)
-    const bool ring = vec && li.L == 4 && both * 4 + 16 + kCountRingBytes <= (227 << 10) - 1024;
+    static_assert(2 * kBuildMaxParts * 4 + 16 + kCountRingBytes <= (227 << 10) - 1024, "the ring beside both deals' counters");
+    const bool ring = vec && li.L == 4;
     go(ring ? part_count_kernel<true, true> : vec ? part_count_kernel<true, false> : part_count_kernel<false, false>, kBuildBlocks, 1024,
        both * 4 + (ring ? 16 + kCountRingBytes : 0), li, hs, pm, sc, by_bucket, codes, (unsigned)n, run, keys, n_unique, status);
     go(part_scan_kernel, 2, 1024, 0, sc);

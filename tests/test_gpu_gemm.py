@@ -98,7 +98,8 @@ def test_gemm_odd_number_of_k_steps_many_tiles_per_cta(ctx, N, K, path):
 @pytest.mark.parametrize("N,K", [(512, 512), (3072, 2048), (2048, 8192), (2080, 2048), (16384, 2048), (32, 64), (256, 192)])
 def test_weight_streaming_gemm(ctx, N, K):
     """The kernel for launches of at most 128 rows (weights as the 128-row MMA operand, K split over CTAs): every epilogue
-    against the fp64 product, for row counts in each of its three accumulator widths (32, 64, 128); a row's bits depend neither on the
+    against the fp64 product, for row counts in each of its four accumulator widths (32, 48, 64, 128), the first two with the
+    parts of a split tile sent and (one CTA a tile, or no room for the parts) with them read; a row's bits depend neither on the
     number of rows nor on the order in which the CTAs of a tile arrive (run twice)."""
     g = torch.Generator(device="cuda"); g.manual_seed(N * 11 + K)
     A64 = (torch.randn(128, K, generator=g, device="cuda") * 0.5).bfloat16()
