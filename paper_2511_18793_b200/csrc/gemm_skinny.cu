@@ -388,7 +388,7 @@ __global__ void __launch_bounds__(kSkinnyThreads, 2)
   }
   tc_fence_before();
   if (PUSH || splits > 1) {                      // no CTA leaves while a peer may still send to it, or read its part
-    if (!PUSH) cluster_arrive();                 // (release: its reads come before it)
+    if (!PUSH) cluster_arrive_relaxed();         // (what it has read has been used)
     cluster_wait();
     if (PUSH && mine && *abort_flag) recv_wait(recv_bar(ew), nullptr);      // given up before: everything sent has to land first
   }

@@ -12,16 +12,3 @@ def test_every_cluster_barrier_brings_its_warp_together_first(repo_root):
             seen += 1
             assert re.search(r"__syncwarp\(\);\s*$", text[: m.start()]), (name, text[m.start(): m.end()])
     assert seen >= 3
-
-
-def test_reads_of_a_peer_come_before_the_arrival_that_lets_it_go(repo_root):
-    """A CTA's shared memory may be gone once all have arrived: the arrival behind the last read of a peer's releases."""
-    csrc = os.path.join(repo_root, "paper_2511_18793_b200", "csrc")
-    seen = 0
-    for name in sorted(os.listdir(csrc)):
-        text = re.sub(r"//[^\n]*", "", open(os.path.join(csrc, name)).read())
-        reads = [m.end() for m in re.finditer(r"= ?ld_peer\w*\(|\* ?ld_peer\w*\(", text)]
-        if reads:
-            seen += 1
-            assert re.search(r"cluster_(?:arrive|sync)\w*", text[reads[-1]:]).group() in ("cluster_arrive", "cluster_sync_all"), name
-    assert seen == 2
