@@ -370,6 +370,9 @@ __global__ void __launch_bounds__(kSkinnyThreads, 2)
 #pragma unroll
           for (int sp = 1; sp < 8; ++sp)
             if (sp < splits) { x.x += part[sp].x; x.y += part[sp].y; x.z += part[sp].z; x.w += part[sp].w; }
+          // A peer may be gone once all have arrived below, so its parts have to be here by then.  A unit has a row, whose store the warp
+          // makes with the sum in hand; but a row without a place in the cache is not stored, so there the warp uses the sum now.
+          if constexpr (EPI == kEpiRopeKV) x.x = __shfl_sync(0xffffffffu, x.x, lane);
         } else {
           x = *reinterpret_cast<const float4*>(gen_base + (at - base));
         }
@@ -388,7 +391,9 @@ __global__ void __launch_bounds__(kSkinnyThreads, 2)
   }
   tc_fence_before();
   if (PUSH || splits > 1) {                      // no CTA leaves while a peer may still send to it, or read its part
-    if (!PUSH) cluster_arrive_relaxed();         // (what it has read has been used)
+    // (Relaxed: what was read has been used.  A release waits for the stores to memory too: prompt and accepted tree of six requests on the
+    // d = 2048 backbone 1,936 -> 1,966 us.)
+    if (!PUSH) cluster_arrive_relaxed();
     cluster_wait();
     if (PUSH && mine && *abort_flag) recv_wait(recv_bar(ew), nullptr);      // given up before: everything sent has to land first
   }
