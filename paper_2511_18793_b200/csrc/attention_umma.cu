@@ -471,6 +471,7 @@ __global__ void __launch_bounds__(kThreadsU, UmmaCfg<HD, PT>::kCtasPerSm) attn_u
             reinterpret_cast<uint4*>(op + c * 32)[u] = make_uint4(w[0], w[1], w[2], w[3]);
           }
         }
+        __syncwarp();                                // (the next load is the whole warp's again)
       }
     }
   }
