@@ -41,14 +41,6 @@ using namespace nz;
 
 namespace {
 
-// H_l = W_logit_l h_l of a prefilled batch (draft_hl): up to this many requests one product of all hidden states with all levels' rows
-// ([batch][L + 1][hl_ld], of which each level's own block is used), beyond a product per level ([L][Bmax][Tmax]).  The one product does
-// L + 1 times the arithmetic and saves L - 1 launches: 256 / 512 / 1,024 requests, per level -> at once, us: four levels of 256 codes, d = 512
-// 14.3 -> 5.2 / 14.4 -> 6.0 / 14.7 -> 9.0, d = 4096 46 -> 15 / 46 -> 17 / 47 -> 45; three of 512, d = 2048 21 -> 10 / 21 -> 12 / 21 -> 24; six of
-// 1,024, d = 512 22 -> 16 / 22 -> 29 / 24 -> 56.  And its results take L + 1 times the room, or more.
-constexpr int kJointConstants = 256;
-bool joint_constants(int batch) { return batch <= kJointConstants; }
-
 struct Carver {
   char* base; size_t off;
   template <typename T> T* take(size_t n) {
@@ -161,6 +153,20 @@ unsigned long long bucket_count(size_t n_items, double lf, int slots_per_bucket)
   unsigned long long nb = (unsigned long long)ceil(slots / slots_per_bucket);
   return nb < 2 ? 2 : nb;
 }
+
+// H_l = W_logit_l h_l of a prefilled batch (draft_hl): while that is at most 16 GFLOP, one product of all hidden states with all levels' rows
+// ([batch][L + 1][hl_ld], of which each level's own block is used), beyond a product per level ([L][Bmax][Tmax]).  The one product does
+// L + 1 times the arithmetic, and its results take L + 1 times the room or more; it saves L - 1 launches of 3.5 us and more: 256 / 512 /
+// 1,024 requests, per level -> at once, us: four levels of 256 codes, d = 512 14.3 -> 5.2 / 14.4 -> 6.0 / 14.7 -> 9.0 (to 3,050 requests), d = 4096
+// 46 -> 15 / 46 -> 17 / 47 -> 45 (to 381); three of 512, d = 2048 21 -> 10 / 21 -> 12 / 21 -> 24 (to 635); six of 1,024, d = 512 22 -> 16 / 22 -> 29 /
+// 24 -> 56 (to 363).  A codebook that is no multiple of 32 codes has no tensor-core product of its own: such an engine makes them at once
+// whatever the batch (four of 250, d = 512, whole prompt pass of 300 requests: 391 -> 328).
+long long joint_constants_max(const nezha_ctx* c) {
+  for (int l = 0; l < c->L; ++l)
+    if (c->cfg.T[l] % 32) return c->Bmax;
+  return (long long)(16e9 / (2.0 * (c->L + 1) * c->es.li.vocab_codes * c->d));
+}
+bool joint_constants(const nezha_ctx* c, int batch) { return batch <= joint_constants_max(c); }
 
 // Lays the arena out; with c->arena == nullptr only the size is computed.
 size_t carve(nezha_ctx* c) {
@@ -290,8 +296,8 @@ size_t carve(nezha_ctx* c) {
   if (c->fused) {
     for (int l = 0; l < c->L; ++l) c->draft_wcat[l] = cv.take_bytes((size_t)(g.T[l] + c->d) * c->d * esz);
     c->draft_u = cv.take<float>((size_t)li.vocab_codes * c->d);
-    const size_t at_once = (size_t)std::min(c->Bmax, kJointConstants) * (c->L + 1) * c->hl_ld, per_level = (size_t)c->L * c->Bmax * c->Tmax;
-    c->draft_hl = cv.take<float>(joint_constants(c->Bmax) ? at_once : std::max(at_once, per_level));
+    const size_t at_once = (size_t)std::min<long long>(c->Bmax, joint_constants_max(c)) * (c->L + 1) * c->hl_ld;
+    c->draft_hl = cv.take<float>(joint_constants(c, c->Bmax) ? at_once : std::max(at_once, (size_t)c->L * c->Bmax * c->Tmax));
     c->draft_sact = cv.take_bytes((size_t)c->Bmax * c->Kmax * c->d * esz);
     c->draft_g = cv.take<float>((size_t)c->Bmax * c->Kmax * (c->Tmax + c->d));
     c->draft_g1 = cv.take<float>((size_t)c->Bmax * (c->Tmax + c->d));
@@ -544,9 +550,9 @@ bool draft_fast(const nezha_ctx* c) {
 }
 // Level l's constants of the requests: of the first, and from one to the next.
 const float* level_constants(const nezha_ctx* c, int l) {
-  return joint_constants(c->batch) ? c->draft_hl + (size_t)l * c->hl_ld + c->es.li.off[l - 1] : c->draft_hl + (size_t)(l - 1) * c->Bmax * c->Tmax;
+  return joint_constants(c, c->batch) ? c->draft_hl + (size_t)l * c->hl_ld + c->es.li.off[l - 1] : c->draft_hl + (size_t)(l - 1) * c->Bmax * c->Tmax;
 }
-long long level_constants_stride(const nezha_ctx* c) { return joint_constants(c->batch) ? (long long)(c->L + 1) * c->hl_ld : c->Tmax; }
+long long level_constants_stride(const nezha_ctx* c) { return joint_constants(c, c->batch) ? (long long)(c->L + 1) * c->hl_ld : c->Tmax; }
 // in_round: inside a decode round, where the device knows whether any request still drafts (a round queued for nothing, or
 // one in which the adaptive policy has switched every request's drafting off, runs its products over zero rows)
 void draft_level_product(nezha_ctx* c, int batch, int l, bool with_state, bool in_round = false) {
@@ -988,7 +994,7 @@ nezha_status nezha_prefill(nezha_ctx* c, const int32_t* hist_codes, const int32_
     launch_rmsnorm(c->resid, c->d, c->h_rows, c->final_norm, c->bf16, (char*)c->h_act + ho * c->esz, c->h_f32 + ho,
                    rows * (c->L + 1), nullptr, c->d, c->cfg.rms_eps, c->st);
     // the request-constant half of Eq. 2, W_logit_l h_l for every level
-    if (c->fused && joint_constants(batch))
+    if (c->fused && joint_constants(c, batch))
       gemm(c, (char*)c->h_act + ho * c->esz, c->d, c->draft_logit[0], c->d, c->draft_hl + (size_t)b0 * (c->L + 1) * c->hl_ld, c->hl_ld,
            (long long)rows * (c->L + 1), nullptr, c->hl_ld, c->d, kEpiStoreF32);
     else if (c->fused)
