@@ -317,8 +317,12 @@ __global__ void __launch_bounds__(AttnCfg<HD, RW, KW>::kThreads) attn_tc_kernel(
           mma_bf16(o[np * 2 + 1], pf[ks], b2, b3);
         }
       }
+      // This warp is done with slot s: what it read is in its registers before the slot is given back.  Without the fence some matrix loads
+      // of the tile's end were still on their way when the producer's next copy came in: about one pass in a thousand of 64 requests had
+      // 8 or 16 columns of one head from rows of the tile after the next.
+      __threadfence_block();
       __syncwarp();
-      if (lane == 0) mbar_arrive(empty_bar(s));      // this warp is done with slot s
+      if (lane == 0) mbar_arrive(empty_bar(s));
     }
     if (KW > 1 && g > 0) {                           // hand the partial softmax state to warp group 0
       float* dst = merge + ((size_t)((g - 1) * RW + rw) * C::kMergeFloats) * 32 + lane;

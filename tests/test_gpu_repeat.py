@@ -51,3 +51,23 @@ def test_passes_of_few_rows_return_the_same_bits_many_times(n_hist):
             assert torch.equal(a, b)
     assert torch.isfinite(first[0]).all()
     case.eng.close()
+
+
+# A warp gives a tile of K and V back to the copies of the next while its last loads of that tile may be under way.
+@pytest.mark.parametrize("hd,kv_heads,batch,beam,n_hist,level,calls", [
+    (64, 8, 64, 10, 50, 1, 12_000), (64, 8, 64, 10, 50, 2, 12_000),     # 16-row CTAs, two warps that take every second tile
+    (128, 4, 64, 10, 50, 2, 6_000),
+    (64, 2, 64, 12, 50, 1, 6_000), (64, 8, 64, 40, 50, 1, 6_000),       # 48 and 40 rows, every warp all tiles
+    (64, 2, 2, 10, 400, 1, 6_000)])                                     # tiles split over a cluster
+def test_a_pass_returns_the_same_bits_thousands_of_times(hd, kv_heads, batch, beam, n_hist, level, calls):
+    w = synth.scaled(synth.WORKLOADS["small"], n_layers=1, n_q_heads=512 // hd, n_kv_heads=kv_heads, n_items=50_000, batch=batch, beam=beam,
+                     n_hist=n_hist)
+    case = Case(w).prefill()
+    g = torch.Generator(device="cuda").manual_seed(1)
+    prefixes = torch.randint(0, 256, (batch, beam, level), dtype=torch.int32, device="cuda", generator=g)
+    first = case.eng.primary_logits(beam, level, prefixes).clone()
+    bad = torch.zeros((), dtype=torch.int64, device="cuda")
+    for _ in range(calls):
+        bad += (case.eng.primary_logits(beam, level, prefixes) != first).any()
+    assert torch.isfinite(first).all() and int(bad) == 0
+    case.eng.close()
